@@ -159,8 +159,8 @@ int kvcrush_score(const kvcrush_problem_t* problem, const kvcrush_tensor_t* Q, c
  *   Q_new       [n_layers][n_seqs][n_q_heads][head_dim]: stride_token steps from one sequence to the next
  *   K           the cached keys, token-major, same dtype as Q_new (BF16, FP16 or FP32), head_dim <= 256, multiple of 8
  *   scores_dev  in/out [n_layers][n_q_heads][T] float32 running column sums
- * Runs on the CUDA cores (one block per layer, sequence and KV head, which serves the query heads of its group);
- * bound by reading K twice.
+ * One cluster of blocks per layer, sequence and KV head serves the query heads of its group from one read of K
+ * (logits of sequences of about 10^5 keys and more are computed twice).
  */
 int kvcrush_score_decode(const kvcrush_problem_t* problem, const kvcrush_tensor_t* Q_new, const kvcrush_tensor_t* K,
                          float* scores_dev, int32_t* status_dev, void* stream);

@@ -53,6 +53,39 @@ def test_decode_update_matches_oracle(B, dtype, D, Hq, Hkv, seqlens):
             np.testing.assert_allclose(inc_g.sum(axis=1), 1.0, rtol=1e-3)
 
 
+@pytest.mark.parametrize("dtype,D,Hq,Hkv,seqlens", [
+    (inputs.BF16, 128, 12, 1, (16, 17, 255, 2049)),      # 12 query heads of one group: two passes; last tiles of 16, 1, 15
+    (inputs.FP16, 40, 32, 4, (1, 4097)),                 # half a block of 32 channels
+    (inputs.FP16, 200, 2, 2, (300,)),                    # head_dim above 128
+    (inputs.FP32, 24, 9, 1, (5, 1030)),                  # fp32, two passes
+    (inputs.BF16, 64, 1, 1, (20000,)),                   # one unit: the largest cluster
+    (inputs.BF16, 32, 8, 1, (52000, 0, 9)),              # logits of a block beyond shared memory: computed twice
+])
+def test_decode_update_at_the_edges_of_its_split(B, dtype, D, Hq, Hkv, seqlens):
+    """Tiles of 16 keys, passes of 8 heads, clusters of 1 to 8 blocks, stored and recomputed logits: increments within
+    the score tolerance of the float64 oracle plus one float32 ulp of the running sum they are added to."""
+    import torch
+    dev = torch.device("cuda:0")
+    w = inputs.Workload("dece", 1, Hq, Hkv, D, seqlens, dtype, dtype, 0.25, base_seed=170 + D)
+    lis, q, k, _, _ = TL.stack_layers(w, range(1), with_cache=False)
+    cu = w.cu_seqlens
+    q_new = np.ascontiguousarray(q[:, [max(int(cu[s + 1]) - 1, 0) for s in range(len(seqlens))]])
+    base = np.random.Generator(np.random.Philox(6)).random((1, Hq, w.total_tokens)).astype(np.float32)
+    prob = B.Problem(1, Hq, Hkv, D, seqlens, device=dev)
+    scores = torch.from_numpy(base.copy()).to(dev)
+    status = torch.zeros(4, dtype=torch.int32, device=dev)
+    B.kvcrush_score_decode(prob, TL.torch_storage(q_new, dtype, dev), TL.torch_storage(k, dtype, dev), scores, status=status)
+    got = scores.cpu().numpy()[0].astype(np.float64)
+    for s, L in enumerate(seqlens):
+        a, b = int(cu[s]), int(cu[s + 1])
+        if L == 0:
+            continue
+        want = O.decode_update(base[0][:, a:b].astype(np.float64), inputs.widen(q_new[0, s], dtype),
+                               inputs.widen(k[0, a:b], dtype))
+        inc = want - base[0][:, a:b]
+        assert (np.abs(got[:, a:b] - want) <= 1e-5 + 2e-3 * np.abs(inc) + 2.0 ** -23 * np.abs(want)).all(), s
+
+
 def test_prefill_then_decode_rebuilds_the_column_sums(B):
     """Scores of a 600-token prompt from the tensor-core sweeps, then 8 decode steps: the running scores equal the
     column sums of the 608-token causal attention."""
