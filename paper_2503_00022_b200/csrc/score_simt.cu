@@ -2,11 +2,11 @@
 // "attention weights" and "normalized attention score" steps).  Serves fp32 inputs and shapes the
 // tensor-core kernels do not cover (bf16 and fp16 inputs are widened on load); the S x S matrix is never stored.
 //
-//   lse_rows_kernel   one warp per query row j: lanes take keys t, t+32, ..; each lane keeps an
-//                     online (max, sum) pair in the log2 domain; lse2(j) = log2 sum_t 2^(s2(j,t))
-//                     with s2 = q.k * scale * log2(e).
-//   colsum_kernel     one warp per key t: lanes take queries j, j+32, ..; accumulates
-//                     2^(s2(j,t) - lse2(j)) = A(j,t) and reduces over the warp.
+// Two sweeps of one tiled kernel: row log-sum-exps, then column sums.  64 x 64 logit tiles from fp32 copies of both
+// operands in shared memory, 4 x 4 logits a thread, so that a 16-byte shared-memory read feeds eight FMAs (one warp
+// per row and one dot product per lane spent 170 us on 8 heads x 512 tokens of 64 channels, all of it waiting for loads,
+// and 2174 us on 4 layers of 1024 tokens; the two sweeps now take 26 and 180 us).
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -16,7 +16,10 @@ namespace kvc {
 
 namespace {
 
-constexpr int kWarpsPerBlock = 4;
+namespace cg = cooperative_groups;
+
+constexpr int kRows = 64;                    // rows of both operands' tiles
+constexpr int kThreads = 256;
 constexpr int kMaxD = 256;
 
 template <typename T>
@@ -52,117 +55,190 @@ __device__ __forceinline__ void load8<__half>(const __half* p, float (&v)[8]) {
   }
 }
 
+// Rows of a [kRows][D] tile start kPad floats apart from a multiple of 32 banks, so that the 16-byte reads of 16
+// consecutive rows do not meet in a bank.
+constexpr int kPad = 4;
+
+// Stages rows row0 .. row0+kRows-1 of a sequence of L tokens (zeros past its end) as fp32.
 template <typename T>
-__device__ __forceinline__ float dot_row(const float* __restrict__ a_sh, const T* __restrict__ b, int D) {
-  float acc = 0.f;
-  for (int d = 0; d < D; d += 8) {
-    float v[8];
-    load8<T>(b + d, v);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) acc = fmaf(a_sh[d + i], v[i], acc);
-  }
-  return acc;
-}
-
-template <typename T>
-__device__ __forceinline__ void stage_row(float* sh, const T* row, int D, int lane) {
-  for (int d = lane * 8; d < D; d += 32 * 8) {
-    float v[8];
-    load8<T>(row + d, v);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) sh[d + i] = v[i];
-  }
-  __syncwarp();
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-lse_rows_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, float* __restrict__ lse2,
-                float* __restrict__ lse_out) {
-  __shared__ float q_sh[kWarpsPerBlock][kMaxD];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const long long row = (long long)blockIdx.x * kWarpsPerBlock + wib;     // (layer, head, token)
-  if (row >= (long long)s.n_layers * s.Hq * s.T) return;
-  const int tok = (int)(row % s.T);
-  const int h = (int)((row / s.T) % s.Hq);
-  const int layer = (int)(row / ((long long)s.T * s.Hq));
-  const int seq = seq_of_token(s.cu_seqlens, s.n_seqs, tok);
-  const int t0 = __ldg(s.cu_seqlens + seq), t1 = __ldg(s.cu_seqlens + seq + 1);
-  const int t_end = s.causal ? tok + 1 : t1;
-  const int ws = (s.window > 0 && t1 - t0 > s.window) ? t1 - t0 - s.window : 0;   // first voting query of the sequence
-  if (tok - t0 < ws) return;                       // this query does not vote: its log-sum-exp is not needed
-
-  const T* q = static_cast<const T*>(Q.ptr) + layer * Q.sl + (long long)tok * Q.st + h * Q.sh;
-  const T* kbase = static_cast<const T*>(K.ptr) + layer * K.sl + (h / s.G) * K.sh;
-  stage_row<T>(q_sh[wib], q, s.D, lane);
-
-  float m = -INFINITY, sum = 0.f;
-  for (int t = t0 + lane; t < t_end; t += 32) {
-    const float x = dot_row<T>(q_sh[wib], kbase + (long long)t * K.st, s.D) * scale_log2;
-    if (x > m) { sum = sum * exp2f(m - x) + 1.f; m = x; } else { sum += exp2f(x - m); }
-  }
-  float big = m;
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) big = fmaxf(big, __shfl_xor_sync(0xFFFFFFFFu, big, d));
-  float part = (m == -INFINITY) ? 0.f : sum * exp2f(m - big);
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, d);
-  if (lane == 0) {
-    const float v = big + log2f(part);
-    lse2[row] = v;
-    if (lse_out) lse_out[row] = v * 0.69314718055994530942f;
+__device__ __forceinline__ void stage_tile(float* sh, const T* base, long long stride, int row0, int L, int D) {
+  const int vec = D / 8;                                    // 8 channels at a time
+  for (int e = threadIdx.x; e < kRows * vec; e += kThreads) {
+    const int r = e / vec, d = (e - r * vec) * 8;
+    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (row0 + r < L) load8<T>(base + (long long)(row0 + r) * stride + d, v);
+    float4* out = reinterpret_cast<float4*>(sh + r * (D + kPad) + d);
+    out[0] = make_float4(v[0], v[1], v[2], v[3]);
+    out[1] = make_float4(v[4], v[5], v[6], v[7]);
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-colsum_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const float* __restrict__ lse,
-              float lse_mul, float* __restrict__ scores, int normalize) {
-  __shared__ float k_sh[kWarpsPerBlock][kMaxD];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const long long col = (long long)blockIdx.x * kWarpsPerBlock + wib;     // (layer, head, token)
-  if (col >= (long long)s.n_layers * s.Hq * s.T) return;
-  const int tok = (int)(col % s.T);
-  const int h = (int)((col / s.T) % s.Hq);
-  const int layer = (int)(col / ((long long)s.T * s.Hq));
-  const int seq = seq_of_token(s.cu_seqlens, s.n_seqs, tok);
-  const int t0 = __ldg(s.cu_seqlens + seq), t1 = __ldg(s.cu_seqlens + seq + 1);
-  const int ws = (s.window > 0 && t1 - t0 > s.window) ? t1 - t0 - s.window : 0;   // first voting query of the sequence
-  const int j_begin = max(s.causal ? tok : t0, t0 + ws);
+// One sweep over the logits.  A cluster owns kRows rows of the stationary operand of one (layer, head, sequence); its
+// blocks take the streamed operand's tiles in turn, and block 0 adds up what they found (through distributed shared
+// memory, in the order of the blocks).
+//   kColsum = false   stationary queries, streamed keys: (max, sum of 2^(x - max)) of every query row
+//   kColsum = true    stationary keys, streamed queries: sum of 2^(x - lse2(query)) of every key
+// 256 threads as 16 x 16; a thread holds 4 x 4 logits of a 64 x 64 tile.
+template <typename T, bool kColsum>
+__global__ void __launch_bounds__(kThreads)
+simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const float* __restrict__ lse, float lse_mul,
+                  float* __restrict__ lse2_out, float* __restrict__ lse_nat_out, float* __restrict__ scores, int normalize,
+                  int max_tiles) {
+  extern __shared__ float4 dyn4[];
+  float* fix_sh = reinterpret_cast<float*>(dyn4);
+  float* str_sh = fix_sh + kRows * (s.D + kPad);
+  __shared__ float part[2][kRows];                          // this block's maximum (sweep 1) and sum of every row
+  __shared__ float nlse_sh[kRows];                          // sweep 2: minus lse2 of the streamed queries, -inf: no vote
+  cg::cluster_group cluster = cg::this_cluster();
+  const int n_blk = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  int unit = blockIdx.x / n_blk;
+  const int h = unit % s.Hq; unit /= s.Hq;
+  const int layer = unit % s.n_layers; unit /= s.n_layers;
+  const int seq = unit % s.n_seqs, rank_tile = unit / s.n_seqs;
+  const int t0 = __ldg(s.cu_seqlens + seq), L = __ldg(s.cu_seqlens + seq + 1) - t0;
+  const int n_tiles = (L + kRows - 1) / kRows;
+  if (rank_tile >= n_tiles) return;                         // uniform over the cluster, like every exit below
+  // heaviest tiles first: the last query rows, the first keys
+  const int tile = kColsum ? rank_tile : n_tiles - 1 - rank_tile;
+  const int row0 = tile * kRows;
+  const int ws = (s.window > 0 && L > s.window) ? L - s.window : 0;       // first voting query
+  if (!kColsum && row0 + kRows <= ws) return;               // no query of this tile votes
+  const int first = kColsum ? max(s.causal ? tile : 0, ws / kRows) : 0;
+  const int last = kColsum ? n_tiles : (s.causal ? tile + 1 : n_tiles);   // streamed tiles [first, last)
+  const T* qbase = static_cast<const T*>(Q.ptr) + layer * Q.sl + (long long)t0 * Q.st + h * Q.sh;
+  const T* kbase = static_cast<const T*>(K.ptr) + layer * K.sl + (long long)t0 * K.st + (h / s.G) * K.sh;
+  const size_t vec0 = ((size_t)layer * s.Hq + h) * s.T + t0;
+  const float ninf = -INFINITY;
 
-  const T* k = static_cast<const T*>(K.ptr) + layer * K.sl + (long long)tok * K.st + (h / s.G) * K.sh;
-  const T* qbase = static_cast<const T*>(Q.ptr) + layer * Q.sl + h * Q.sh;
-  const float* lse_row = lse + ((long long)layer * s.Hq + h) * s.T;
-  stage_row<T>(k_sh[wib], k, s.D, lane);
-
-  float acc = 0.f;
-  for (int j = j_begin + lane; j < t1; j += 32) {
-    const float x = dot_row<T>(k_sh[wib], qbase + (long long)j * Q.st, s.D) * scale_log2;
-    acc += exp2f(x - __ldg(lse_row + j) * lse_mul);
-  }
+  stage_tile<T>(fix_sh, kColsum ? kbase : qbase, kColsum ? K.st : Q.st, row0, L, s.D);
+  float m[4], sum[4];
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, d);
-  if (lane == 0) scores[col] = normalize ? acc / (float)(t1 - t0 - ws) : acc;
+  for (int i = 0; i < 4; ++i) { m[i] = ninf; sum[i] = 0.f; }
+  for (int u = first + rank; u < last; u += n_blk) {
+    __syncthreads();                                        // the previous tile is done with
+    stage_tile<T>(str_sh, kColsum ? qbase : kbase, kColsum ? Q.st : K.st, u * kRows, L, s.D);
+    if (kColsum && tid < kRows) {
+      const int j = u * kRows + tid;
+      nlse_sh[tid] = j < L && j >= ws ? -(__ldg(lse + vec0 + j) * lse_mul) : ninf;
+    }
+    __syncthreads();
+    float acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    const float* fa = fix_sh + ty * (s.D + kPad);           // stationary rows ty + 16 i, streamed rows tx + 16 j
+    const float* fb = str_sh + tx * (s.D + kPad);
+#pragma unroll 2
+    for (int d = 0; d < s.D; d += 4) {
+      float4 a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        a[i] = *reinterpret_cast<const float4*>(fa + i * 16 * (s.D + kPad) + d);
+        b[i] = *reinterpret_cast<const float4*>(fb + i * 16 * (s.D + kPad) + d);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          acc[i][j] = fmaf(a[i].w, b[j].w, fmaf(a[i].z, b[j].z, fmaf(a[i].y, b[j].y, fmaf(a[i].x, b[j].x, acc[i][j]))));
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = row0 + ty + 16 * i;
+      float x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = u * kRows + tx + 16 * j;
+        const bool in = c < L && (!s.causal || (kColsum ? c >= r : c <= r));
+        x[j] = in ? (kColsum ? fmaf(acc[i][j], scale_log2, nlse_sh[tx + 16 * j]) : acc[i][j] * scale_log2) : ninf;
+      }
+      if constexpr (kColsum) {
+        sum[i] += (exp2f(x[0]) + exp2f(x[1])) + (exp2f(x[2]) + exp2f(x[3]));
+      } else {
+        const float big = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
+        if (big > m[i]) { sum[i] *= exp2f(m[i] - big); m[i] = big; }     // first tile: 0 * 2^-inf
+        if (m[i] != ninf) sum[i] += (exp2f(x[0] - m[i]) + exp2f(x[1] - m[i])) + (exp2f(x[2] - m[i]) + exp2f(x[3] - m[i]));
+      }
+    }
+  }
+  // the 16 threads of a row, then the blocks of the cluster
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float big = m[i];
+    if constexpr (!kColsum) {
+#pragma unroll
+      for (int d = 8; d > 0; d >>= 1) big = fmaxf(big, __shfl_xor_sync(0xFFFFFFFFu, big, d));
+      sum[i] = m[i] == ninf ? 0.f : sum[i] * exp2f(m[i] - big);
+    }
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) sum[i] += __shfl_xor_sync(0xFFFFFFFFu, sum[i], d);
+    if (tx == 0) { part[0][ty + 16 * i] = big; part[1][ty + 16 * i] = sum[i]; }
+  }
+  if (n_blk > 1) cluster.sync(); else __syncthreads();
+  if (rank == 0 && tid < kRows && row0 + tid < L) {
+    const size_t out = vec0 + row0 + tid;
+    float big = ninf, total = 0.f;
+    if constexpr (!kColsum)
+      for (int b = 0; b < n_blk; ++b) big = fmaxf(big, *cluster.map_shared_rank(&part[0][tid], b));
+    for (int b = 0; b < n_blk; ++b) {
+      const float p = *cluster.map_shared_rank(&part[1][tid], b);
+      total += kColsum ? p : p > 0.f ? p * exp2f(*cluster.map_shared_rank(&part[0][tid], b) - big) : 0.f;
+    }
+    if constexpr (kColsum) {
+      scores[out] = normalize ? total / (float)(L - ws) : total;
+    } else if (row0 + tid >= ws) {
+      const float v = big + log2f(total);
+      lse2_out[out] = v;
+      if (lse_nat_out) lse_nat_out[out] = v * 0.69314718055994530942f;
+    }
+  }
+  if (n_blk > 1) cluster.sync();                            // block 0 has read the others' parts
+}
+
+template <typename T, bool kColsum>
+int launch_sweep(const Shape& s, const TensorView& Q, const TensorView& K, float scale_log2, const float* lse, float lse_mul,
+                 float* lse2_out, float* lse_nat_out, float* scores, int normalize, cudaStream_t stream) {
+  const int max_tiles = (s.max_seqlen + kRows - 1) / kRows;
+  const long long units = (long long)max_tiles * s.n_seqs * s.n_layers * s.Hq;
+  // A small problem does not fill the chip with one block per tile of rows: its streamed tiles are shared by up to 8
+  // blocks then (8 heads x 512 tokens: 64 tiles of rows, 4 blocks each; with 8 the second wave starts, 26 -> 37 us).
+  int n_blk = 1;
+  while (n_blk < 8 && 2 * n_blk <= max_tiles && units * n_blk < 148) n_blk *= 2;
+  if (units * n_blk > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
+  const size_t dyn = (size_t)2 * kRows * (s.D + kPad) * sizeof(float);
+  auto kern = simt_sweep_kernel<T, kColsum>;
+  if (dyn > 40 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
+    return KVCRUSH_ERR_CUDA;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(units * n_blk));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = dyn;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)n_blk; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, kern, s, Q, K, scale_log2, lse, lse_mul, lse2_out, lse_nat_out, scores, normalize, max_tiles) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    return KVCRUSH_ERR_CUDA;
+  }
+  return check_launch();
 }
 
 template <typename T>
 int run(const Shape& s, const TensorView& Q, const TensorView& K, float scale_log2, const float* lse_in,
         float lse_in_mul, float* lse2_ws, float* scores, float* lse_out, int normalize, cudaStream_t stream) {
-  const long long rows = (long long)s.n_layers * s.Hq * s.T;
-  if (rows == 0) return KVCRUSH_OK;
-  const long long blocks = (rows + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  if (blocks > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
-  const float* lse = lse_in;
-  float mul = lse_in_mul;
+  if (s.T == 0) return KVCRUSH_OK;
   if (!lse_in) {
-    lse_rows_kernel<T><<<(unsigned)blocks, kWarpsPerBlock * 32, 0, stream>>>(s, Q, K, scale_log2, lse2_ws, lse_out);
-    if (check_launch() != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
-    lse = lse2_ws;
-    mul = 1.f;
+    const int rc = launch_sweep<T, false>(s, Q, K, scale_log2, nullptr, 1.f, lse2_ws, lse_out, nullptr, 0, stream);
+    if (rc != KVCRUSH_OK) return rc;
+    return launch_sweep<T, true>(s, Q, K, scale_log2, lse2_ws, 1.f, nullptr, nullptr, scores, normalize, stream);
   }
-  colsum_kernel<T><<<(unsigned)blocks, kWarpsPerBlock * 32, 0, stream>>>(s, Q, K, scale_log2, lse, mul, scores,
-                                                                          normalize);
-  return check_launch();
+  return launch_sweep<T, true>(s, Q, K, scale_log2, lse_in, lse_in_mul, nullptr, nullptr, scores, normalize, stream);
 }
 
 }  // namespace

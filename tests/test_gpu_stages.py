@@ -408,3 +408,39 @@ def test_pass_replays_from_a_cuda_graph(B):
     torch.cuda.synchronize()
     cp.check_status()
     assert torch.equal(cp.idx, want[0]) and torch.equal(cp.k_out, want[1]) and torch.equal(cp.scores, want[2])
+
+
+@pytest.mark.parametrize("dtype,D,Hq,Hkv,seqlens,causal,window", [
+    (inputs.FP32, 64, 2, 1, (63, 64, 65), True, 0),          # around one tile of 64 rows
+    (inputs.FP32, 8, 1, 1, (1,), True, 0),                   # the smallest problem
+    (inputs.FP32, 128, 1, 1, (1025,), True, 0),              # streamed tiles shared by 8 blocks, last tile of one row
+    (inputs.FP32, 72, 4, 2, (190, 0, 129), False, 0),        # channels not a multiple of the shared-memory bank count
+    (inputs.FP32, 256, 2, 2, (200,), True, 70),              # widest heads, window that cuts a tile
+    (inputs.BF16, 200, 2, 1, (257,), True, 0),               # bf16 too wide for the tensor-core kernels
+])
+def test_cuda_core_scores_at_the_edges_of_their_tiles(B, dtype, D, Hq, Hkv, seqlens, causal, window):
+    """fp32 sums of at most 1025 terms and an exponential of 2 ulp: far inside the score tolerance."""
+    import torch
+    dev = torch.device("cuda:0")
+    w = inputs.Workload("simt", 2, Hq, Hkv, D, seqlens, dtype, dtype, 0.25, base_seed=190 + D, causal=causal)
+    lis, q, k, _, _ = TL.stack_layers(w, range(2), with_cache=False)
+    prob = B.Problem(2, Hq, Hkv, D, seqlens, causal=causal, device=dev, query_window=window)
+    ws = torch.empty(B.kvcrush_workspace_size(prob, B.STAGE_SCORE), dtype=torch.uint8, device=dev)
+    status = torch.zeros(4, dtype=torch.int32, device=dev)
+    scores = torch.full((2, Hq, w.total_tokens), -1.0, device=dev)
+    lse = torch.full_like(scores, 7.0)
+    B.kvcrush_score(prob, TL.torch_storage(q, dtype, dev), TL.torch_storage(k, dtype, dev), scores, lse_out=lse,
+                    impl=B.SCORE_SIMT, workspace=ws, status=status)
+    g, gl = scores.cpu().numpy(), lse.cpu().numpy()
+    assert status.cpu().tolist()[0] == 0
+    cu = w.cu_seqlens
+    for l, li in enumerate(lis):
+        for s, L in enumerate(seqlens):
+            a, b = int(cu[s]), int(cu[s + 1])
+            if L == 0:
+                continue
+            j0 = max(0, L - window) if window else 0
+            c, ol = O.scores(inputs.widen(li.q[a:b], dtype), inputs.widen(li.k[a:b], dtype), causal, rows=(j0, L))
+            assert TL.within_score_tolerance(g[l][:, a:b], c).all(), (l, s)
+            np.testing.assert_allclose(gl[l][:, a + j0:b], ol[:, j0:], rtol=0, atol=2e-5)
+            assert (gl[l][:, a:a + j0] == 7.0).all()                       # rows that do not vote are not written
