@@ -5,6 +5,7 @@
 //                             the k-th largest is found by 12-bit radix histograms over (key - smallest key),
 //                             starting at the top bit in which the row's keys differ at all; one warp ranks the
 //                             last few candidates directly.  Usually one histogram pass.
+//   theta_warp_kernel         the same search by one warp per row, for many short rows.
 //   theta_stream_kernel       the same result for longer rows: MSB-first radix select (4 sweeps of 8 bits) that
 //                             re-reads the row from memory (or from a shared-memory copy) in every sweep.
 //   signature_pack_kernel     one block per (layer, 128 tokens): stages the [heads][tokens] tile of scores in shared
@@ -124,6 +125,104 @@ theta_select_kernel(Shape s, const float* __restrict__ scores, const int32_t* __
     __syncthreads();                                         // hist and found are rewritten by the next step
   }
   if (tid == 0) *out = key_to_float(base + top);
+}
+
+// One warp per row, for rows of up to 32 * kItems tokens: the same search as theta_select_kernel without a block's
+// barriers, and with as many rows in flight as an SM has warps.  Short rows come in large numbers (a serving batch of 16
+// sequences x 32 layers x 32 heads of 736 tokens is 16384 rows), where a block per row spends its time in barriers: the
+// signature stage took 99 us with it and takes 62 us with this kernel.
+constexpr int kRowWarps = 8;
+constexpr int kRowBits = 9;
+constexpr int kRowBins = 1 << kRowBits;
+
+template <int kItems>
+__global__ void __launch_bounds__(kRowWarps * 32)
+theta_warp_kernel(Shape s, const float* __restrict__ scores, const int32_t* __restrict__ sig_keep,
+                  float* __restrict__ theta, unsigned n_rows) {
+  __shared__ alignas(16) uint32_t hist_sh[kRowWarps][kRowBins];
+  __shared__ uint32_t small_sh[kRowWarps][sel::kSmallList];
+  __shared__ uint32_t small_n_sh[kRowWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned r = blockIdx.x * kRowWarps + warp;
+  if (r >= n_rows) return;
+  uint32_t* hist = hist_sh[warp];
+  const int h = r % s.Hq;
+  const int seg = r / s.Hq;                       // layer * n_seqs + seq
+  const int layer = seg / s.n_seqs, seq = seg - layer * s.n_seqs;
+  const int t0 = __ldg(s.cu_seqlens + seq);
+  const int L = __ldg(s.cu_seqlens + seq + 1) - t0;
+  const int keep = __ldg(sig_keep + seg);
+  if (keep <= 0 || keep >= L) {
+    if (lane == 0) theta[r] = keep <= 0 ? __int_as_float(0x7F800000) : __int_as_float(0xFF800000);
+    return;
+  }
+  const float* row = scores + ((size_t)layer * s.Hq + h) * s.T + t0;
+  uint32_t key[kItems];
+  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) key[j] = j * 32 + lane < L ? order_key(__ldg(row + j * 32 + lane)) : 0u;
+#pragma unroll
+  for (int j = 0; j < kItems; ++j)
+    if (j * 32 + lane < L) { lo = min(lo, key[j]); hi = max(hi, key[j]); }
+  const uint32_t base = __reduce_min_sync(sel::kFull, lo), range = __reduce_max_sync(sel::kFull, hi) - base;
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) key[j] -= base;            // slots past the end of the row are left out below
+
+  int rem = range ? 32 - __clz(range) : 0;
+  uint32_t top = 0, k_rem = (uint32_t)keep;
+  while (rem > 0) {
+    const int w = rem < kRowBits ? rem : kRowBits, shift = rem - w;
+    uint4* h4 = reinterpret_cast<uint4*>(hist);
+#pragma unroll
+    for (int i = 0; i < kRowBins / 128; ++i) h4[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+    if (lane == 0) small_n_sh[warp] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < kItems; ++j)
+      if (j * 32 + lane < L && ((key[j] >> 1) >> (rem - 1)) == top) atomicAdd(&hist[(key[j] >> shift) & ((1u << w) - 1u)], 1u);
+    __syncwarp();
+    // lane l owns the kRowBins / 32 bins from kRowBins - 1 - l * 16 downwards (bins above the digit's width are empty)
+    uint32_t c[kRowBins / 32], local = 0;
+#pragma unroll
+    for (int i = 0; i < kRowBins / 128; ++i) {
+      const uint4 v = h4[(31 - lane) * (kRowBins / 128) + (kRowBins / 128 - 1 - i)];
+      c[4 * i] = v.w; c[4 * i + 1] = v.z; c[4 * i + 2] = v.y; c[4 * i + 3] = v.x;
+      local += (v.x + v.y) + (v.z + v.w);
+    }
+    uint32_t incl = local;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t v = __shfl_up_sync(sel::kFull, incl, d);
+      if (lane >= d) incl += v;
+    }
+    uint32_t acc = incl - local, bin = 0, left = 0, live = 0;
+    const bool mine = acc < k_rem && k_rem <= incl;
+    if (mine) {
+      bool found = false;
+#pragma unroll
+      for (int i = 0; i < kRowBins / 32; ++i) {
+        if (!found && k_rem <= acc + c[i]) {
+          found = true;
+          bin = kRowBins - 1 - lane * (kRowBins / 32) - i; left = k_rem - acc; live = c[i];
+        }
+        acc += c[i];
+      }
+    }
+    const int src = __ffs(__ballot_sync(sel::kFull, mine)) - 1;
+    top = (top << w) | __shfl_sync(sel::kFull, bin, src);
+    k_rem = __shfl_sync(sel::kFull, left, src);
+    live = __shfl_sync(sel::kFull, live, src);
+    rem = shift;
+    if (rem > 0 && live <= (uint32_t)sel::kSmallList) {      // few candidates: ranked directly
+#pragma unroll
+      for (int j = 0; j < kItems; ++j)
+        if (j * 32 + lane < L && (key[j] >> rem) == top) small_sh[warp][atomicAdd(&small_n_sh[warp], 1u)] = key[j];
+      __syncwarp();
+      top = sel::warp_rank_select32(lane < (int)live ? small_sh[warp][lane] : 0u, (int)live, k_rem, lane);
+      rem = 0;
+    }
+  }
+  if (lane == 0) theta[r] = key_to_float(base + top);
 }
 
 __global__ void __launch_bounds__(kSelectThreads)
@@ -292,7 +391,14 @@ int launch_signature(const Shape& s, const float* scores, const int32_t* sig_kee
   if (!theta_in) {
     const unsigned blocks = (unsigned)s.n_layers * s.n_seqs * s.Hq;
     const int m = s.max_seqlen;
-    if (m <= 2048) launch_theta<256, 8, 8>(s, scores, sig_keep, theta, blocks, stream);
+    // A warp per row up to 512 tokens (stage at 1024 rows of 400 tokens: 11.8 -> 7.5 us); up to 1024 tokens only for
+    // more rows than the chip holds as blocks (148 x 8): its chain over 32 keys a lane is longer than the block's
+    // (32 rows of 1001 tokens: 8.9 against 7.3 us).
+    const unsigned warp_blocks = (blocks + kRowWarps - 1) / kRowWarps;
+    if (m <= 256) theta_warp_kernel<8><<<warp_blocks, kRowWarps * 32, 0, stream>>>(s, scores, sig_keep, theta, blocks);
+    else if (m <= 512) theta_warp_kernel<16><<<warp_blocks, kRowWarps * 32, 0, stream>>>(s, scores, sig_keep, theta, blocks);
+    else if (m <= 1024 && blocks > 1184) theta_warp_kernel<32><<<warp_blocks, kRowWarps * 32, 0, stream>>>(s, scores, sig_keep, theta, blocks);
+    else if (m <= 2048) launch_theta<256, 8, 8>(s, scores, sig_keep, theta, blocks, stream);
     else if (m <= 4096) launch_theta<512, 8, 4>(s, scores, sig_keep, theta, blocks, stream);
     else if (m <= 8192) launch_theta<512, 16, 4>(s, scores, sig_keep, theta, blocks, stream);
     else if (m <= 16384) launch_theta<512, 32, 1>(s, scores, sig_keep, theta, blocks, stream);

@@ -105,6 +105,16 @@ def test_signature_thresholds_for_rows_beyond_the_register_kernel(B):
     _select_case(B, 4, 2, [33000], [(100, 50)], 1, 3, 0, seed=18)
 
 
+@pytest.mark.parametrize("seqlens,ties", [
+    ([1, 2, 31, 32, 33, 256], 0), ([255, 256, 1, 100], 2),       # 8 keys a lane
+    ([257, 31, 512], 0), ([511, 512, 480], 3),                   # 16
+    ([513, 1023, 1024, 64] * 10, 0), ([1024, 700] * 19, 1),      # 32, more rows than the chip holds as blocks
+])
+def test_thresholds_by_one_warp_per_row_are_exact(B, seqlens, ties):
+    budgets = [(max(1, L // 5), L // 7) for L in seqlens]
+    _select_case(B, 32, 8, seqlens, budgets, 1, ties, 0, seed=230 + len(seqlens))
+
+
 def test_signature_rank_other_than_budget_and_explicit_theta(B):
     import torch
     dev = _dev()
