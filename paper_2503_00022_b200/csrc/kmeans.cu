@@ -25,9 +25,9 @@ namespace kvc {
 
 namespace {
 
-using sel::kThreads;
 using sel::kFull;
 
+constexpr int kThreads = 1024;
 constexpr int kPlanes = 16;            // bit planes of a count: counts up to 65535 (segments of up to 32768 tokens)
 constexpr int kTile = 64;              // clusters staged in shared memory at a time
 constexpr int kAssignThreads = 256;
@@ -133,7 +133,7 @@ kmeans_prepare_kernel(Shape s, KmArgs a) {
   const int n_words = (L + 31) >> 5;
   for (int i = tid; i < n_words; i += kThreads) { imp_mask[i] = 0; zero_mask[i] = 0; }
   __syncthreads();
-  if (b_imp > 0) sel::mark_top_keys(keys, L, b_imp, imp_mask, sc);
+  if (b_imp > 0) sel::mark_top_keys<kThreads>(keys, L, b_imp, imp_mask, sc);
   const int N = L - b_imp;
   for (int i = tid; i < n_words; i += kThreads) {
     const uint32_t valid = (i == n_words - 1 && (L & 31)) ? ((1u << (L & 31)) - 1u) : 0xFFFFFFFFu;
@@ -141,7 +141,7 @@ kmeans_prepare_kernel(Shape s, KmArgs a) {
   }
   __syncthreads();
   int32_t* cand = a.cand + (size_t)layer * s.T + t0;
-  sel::emit_kept(grp_mask, zero_mask, n_words, cand, nullptr, sc);   // grouped tokens in ascending order
+  sel::emit_kept<kThreads>(grp_mask, zero_mask, n_words, cand, nullptr, sc);   // grouped tokens in ascending order
   if (tid == 0) { info[0] = b_rep > 0 ? N : 0; info[1] = b_rep; info[2] = b_imp; info[3] = 0; }
   __syncthreads();
   // initial centroids: the vectors at ranks floor(i * N / k)
@@ -283,11 +283,11 @@ kmeans_finish_kernel(Shape s, KmArgs a) {
   __syncthreads();
   // the important set plus, for the budget that empty clusters left, the most important of the remaining tokens
   const int k_top = b_imp + (k - n_reps);
-  if (k_top > 0) sel::mark_top_keys(keys, L, k_top, imp_mask, sc);
+  if (k_top > 0) sel::mark_top_keys<kThreads>(keys, L, k_top, imp_mask, sc);
   __syncthreads();
   int32_t* out_idx = a.idx + __ldg(a.cu_kept + seg);
   uint8_t* out_kind = a.kind ? a.kind + __ldg(a.cu_kept + seg) : nullptr;
-  sel::emit_kept(imp_mask, rep_mask, n_words, out_idx, out_kind, sc);
+  sel::emit_kept<kThreads>(imp_mask, rep_mask, n_words, out_idx, out_kind, sc);
 }
 
 template <int kMode>

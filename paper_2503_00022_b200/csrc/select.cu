@@ -23,10 +23,10 @@ namespace kvc {
 
 namespace {
 
-using sel::kThreads;
-using sel::kWarps;
 using sel::kFull;
 using sel::head_mask;
+constexpr int kThreads = 1024;
+constexpr int kWarps = kThreads / 32;
 constexpr int kMaxBins = 129;              // Hamming distances 0..128
 
 // Order-preserving 64-bit key of a float64 importance; tokens kept by decree (the first keep_initial and the last
@@ -176,13 +176,13 @@ select_segment_kernel(Shape s, SelectArgs a) {
   }
   const int n_words = (L + 31) >> 5;
   int r_lo, r_hi;                            // contiguous token range of this warp
-  sel::warp_range(L, warp, r_lo, r_hi);
+  sel::warp_range<kThreads>(L, warp, r_lo, r_hi);
 
   for (int i = tid; i < n_words; i += kThreads) { imp_mask[i] = 0; rep_mask[i] = 0; }
   __syncthreads();
 
   // ---- 1. important tokens: the b_imp largest keys, ties to the lower index --------------------
-  if (b_imp > 0) sel::mark_top_keys(keys, L, b_imp, imp_mask, sc);
+  if (b_imp > 0) sel::mark_top_keys<kThreads>(keys, L, b_imp, imp_mask, sc);
 
   // ---- 2-4. representatives of the other tokens ------------------------------------------------
   if (b_rep > 0) {
@@ -409,7 +409,7 @@ select_segment_kernel(Shape s, SelectArgs a) {
   }
 
   // ---- 5. kept = important U representatives, ascending ------------------------------------------
-  sel::emit_kept(imp_mask, rep_mask, n_words, out_idx, out_kind, sc);
+  sel::emit_kept<kThreads>(imp_mask, rep_mask, n_words, out_idx, out_kind, sc);
 }
 
 }  // namespace

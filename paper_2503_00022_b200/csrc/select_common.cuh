@@ -8,8 +8,7 @@
 namespace kvc {
 namespace sel {
 
-constexpr int kThreads = 1024;
-constexpr int kWarps = kThreads / 32;
+constexpr int kMaxWarps = 32;                  // the helpers below take the block's thread count kT, at most 1024
 constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kDigitBits = 11;                 // radix digit of the 64-bit selection
 constexpr int kBins = 1 << kDigitBits;
@@ -17,12 +16,12 @@ constexpr int kSmallList = 32;                 // candidates one warp ranks dire
 
 struct Scratch {
   alignas(16) uint32_t hist[kBins];
-  unsigned long long red[2][kWarps];           // per-warp minimum / maximum
+  unsigned long long red[2][kMaxWarps];          // per-warp minimum / maximum
   unsigned long long small[kSmallList];
   unsigned long long sel_x;                    // result of a search step
   uint32_t sel[3];                             // digit, remaining rank, live keys
   uint32_t small_n;
-  int warp_tot[kWarps];
+  int warp_tot[kMaxWarps];
 };
 
 __device__ __forceinline__ uint32_t head_mask(int Hq, int w) {
@@ -37,9 +36,10 @@ __device__ __forceinline__ int warps_before(const int* tot, int warp, int lane) 
 }
 
 // Contiguous item range of a warp: a multiple of 32 items, so that mask words do not straddle warps.
+template <int kT>
 __device__ __forceinline__ void warp_range(int n, int warp, int& r_lo, int& r_hi) {
   const int n_words = (n + 31) >> 5;
-  const int per_warp = ((n_words + kWarps - 1) / kWarps) * 32;
+  const int per_warp = ((n_words + kT / 32 - 1) / (kT / 32)) * 32;
   r_lo = min(n, warp * per_warp);
   r_hi = min(n, r_lo + per_warp);
 }
@@ -128,16 +128,31 @@ __device__ __forceinline__ uint32_t warp_rank_select32(uint32_t v, int n, uint32
 // the keys' common magnitude -, and as soon as at most 32 candidates are left one warp ranks them directly; then
 // one ordered pass marks the members.  Called by all threads of the block; imp_mask must be zero on entry;
 // 0 < k < n.
+template <int kT>
 __device__ __forceinline__ void mark_top_keys(const unsigned long long* keys, int n, int k, uint32_t* imp_mask,
                                               Scratch& sc) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
+  if (n <= 32) {                                       // one warp ranks every item: larger keys first, then lower index
+    if (warp == 0) {
+      const unsigned long long v = lane < n ? keys[lane] : 0ull;
+      int before = 0;
+      for (int j = 0; j < n; ++j) {
+        const unsigned long long o = __shfl_sync(kFull, v, j);
+        before += o > v || (o == v && j < lane);
+      }
+      const unsigned imp_b = __ballot_sync(kFull, lane < n && before < k);
+      if (lane == 0) imp_mask[0] = imp_b;
+    }
+    __syncthreads();
+    return;
+  }
   int r_lo, r_hi;
-  warp_range(n, warp, r_lo, r_hi);
+  warp_range<kT>(n, warp, r_lo, r_hi);
 
   // smallest and largest key
   unsigned long long lo = ~0ull, hi = 0ull;
-  for (int i = tid; i < n; i += kThreads) {
+  for (int i = tid; i < n; i += kT) {
     const unsigned long long key = keys[i];
     lo = key < lo ? key : lo;
     hi = key > hi ? key : hi;
@@ -150,8 +165,8 @@ __device__ __forceinline__ void mark_top_keys(const unsigned long long* keys, in
   }
   if (lane == 0) { sc.red[0][warp] = lo; sc.red[1][warp] = hi; }
   __syncthreads();
-  lo = sc.red[0][lane];
-  hi = sc.red[1][lane];
+  lo = lane < kT / 32 ? sc.red[0][lane] : ~0ull;
+  hi = lane < kT / 32 ? sc.red[1][lane] : 0ull;
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) {
     const unsigned long long a = __shfl_xor_sync(kFull, lo, d), b = __shfl_xor_sync(kFull, hi, d);
@@ -168,27 +183,27 @@ __device__ __forceinline__ void mark_top_keys(const unsigned long long* keys, in
   bool first = true;
   while (rem > 0) {
     const int w = rem < kDigitBits ? rem : kDigitBits, shift = rem - w, n_bins = 1 << w;
-    for (int i = tid; i < n_bins; i += kThreads) sc.hist[i] = 0;
+    for (int i = tid; i < n_bins; i += kT) sc.hist[i] = 0;
     if (tid == 0) sc.small_n = 0;
     __syncthreads();
     if (first) {                                       // every key counts and has no bits above the digit
-      for (int i = tid; i < n; i += kThreads) atomicAdd(&sc.hist[(uint32_t)((keys[i] - base) >> shift)], 1u);
+      for (int i = tid; i < n; i += kT) atomicAdd(&sc.hist[(uint32_t)((keys[i] - base) >> shift)], 1u);
     } else {
-      for (int i = tid; i < n; i += kThreads) {
+      for (int i = tid; i < n; i += kT) {
         const unsigned long long x = keys[i] - base;
         if (((x >> 1) >> (rem - 1)) == top) atomicAdd(&sc.hist[(uint32_t)(x >> shift) & (uint32_t)(n_bins - 1)], 1u);
       }
     }
     first = false;
     __syncthreads();
-    find_digit_desc<kThreads>(sc.hist, n_bins, k_rem, sc.warp_tot, sc.sel);
+    find_digit_desc<kT>(sc.hist, n_bins, k_rem, sc.warp_tot, sc.sel);
     top = (top << w) | sc.sel[0];
     k_rem = sc.sel[1];
     const uint32_t live = sc.sel[2];
     n_equal = live;                                    // exact once no bits are left
     rem = shift;
     if (rem > 0 && live <= (uint32_t)kSmallList) {     // few candidates: one warp ranks their remaining bits
-      for (int i = tid; i < n; i += kThreads) {
+      for (int i = tid; i < n; i += kT) {
         const unsigned long long x = keys[i] - base;
         if ((x >> rem) == top) sc.small[atomicAdd(&sc.small_n, 1u)] = x;
       }
@@ -240,13 +255,14 @@ __device__ __forceinline__ void mark_top_keys(const unsigned long long* keys, in
 
 // Writes the members of imp_mask | rep_mask in ascending order (kind: 1 for members of rep_mask).
 // Called by all threads of the block after the masks are complete.
+template <int kT>
 __device__ __forceinline__ void emit_kept(const uint32_t* imp_mask, const uint32_t* rep_mask, int n_words,
                                           int32_t* out_idx, uint8_t* out_kind, Scratch& sc) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // every thread takes a contiguous run of mask BYTES (8 items each): with fewer words than threads a word-wise
   // split would leave most threads idle and the others with up to 32 serial stores
   const int n_bytes = 4 * n_words;
-  const int bpt = (n_bytes + kThreads - 1) / kThreads;
+  const int bpt = (n_bytes + kT - 1) / kT;
   const int b_lo = min(n_bytes, tid * bpt), b_hi = min(n_bytes, b_lo + bpt);
   auto byte_of = [](const uint32_t* mask, int b) -> uint32_t { return (mask[b >> 2] >> (8 * (b & 3))) & 0xFFu; };
   int cnt = 0;

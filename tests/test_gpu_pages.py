@@ -77,6 +77,18 @@ def test_pages_match_oracle(B, P, mode):
     _check_pages(cp, scores, Hkv, seqlens, P, b_imp, b_rep, mode, explicit)
 
 
+@pytest.mark.parametrize("P,pages", [(8, [31, 32, 33, 2]), (8, [128, 5]), (8, [129, 100]), (4, [512, 33]), (4, [513])])
+@pytest.mark.parametrize("ties", [0, 2])
+def test_pages_at_the_edges_of_the_block_sizes(B, P, pages, ties):
+    """128, 256 and 1024 threads a segment; up to 32 pages are ranked by one warp, ties included."""
+    seqlens = [P * n - (1 if i % 2 else 0) for i, n in enumerate(pages)]
+    scores = _scores(2, 32, seqlens, 470 + len(pages) + P, ties=ties)
+    b_imp = np.asarray([[max(1, n // 3) for n in pages]], dtype=np.int32)
+    b_rep = np.asarray([[max(1, n // 4) for n in pages]], dtype=np.int32)
+    cp = _run_pages(B, scores, 8, seqlens, P, b_imp, b_rep)
+    _check_pages(cp, scores, 8, seqlens, P, b_imp, b_rep)
+
+
 def test_page_size_one_equals_token_level_kernel(B):
     import torch
     seqlens, Hq, Hkv = [700, 129], 40, 8
