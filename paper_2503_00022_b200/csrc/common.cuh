@@ -46,6 +46,21 @@ __device__ __forceinline__ int seq_of_token(const int32_t* __restrict__ cu, int 
   return lo;
 }
 
+// Segment (layer * n_seqs + seq) that owns row `row` of the kept lists, 0 <= row < cu_kept[n_seg].  All lanes of the warp
+// call it with the same row; 32 boundaries are tested at a time (512 segments: two dependent loads instead of nine).
+__device__ __forceinline__ int warp_segment_of_row(const int32_t* __restrict__ cu_kept, int n_seg, long long row, int lane) {
+  int lo = 0, n = n_seg;               // the segment is in [lo, lo + n)
+  while (n > 1) {
+    const int step = (n + 31) / 32;    // lane i stands for the segments [lo + i * step, ..); lane 0's bound always holds
+    const int at = lo + lane * step;
+    const bool reached = lane * step < n && (lane == 0 || (long long)__ldg(cu_kept + at) <= row);
+    const int i = 31 - __clz(__ballot_sync(0xFFFFFFFFu, reached));
+    n = min(step, n - i * step);
+    lo += i * step;
+  }
+  return lo;
+}
+
 // ---- stage launchers (defined in the per-stage .cu files) -------------------------------------------
 
 // score: SIMT fp32 kernels (any dtype/shape) and tcgen05 kernels (bf16 or fp16, D a multiple of 8 up to 128).

@@ -147,6 +147,54 @@ def test_compact_scores_is_a_gather(B):
     np.testing.assert_array_equal(gp, want)
 
 
+@pytest.mark.parametrize("n_seqs,P", [(1, 0), (33, 0), (70, 0), (33, 8)])
+def test_gathers_find_their_segment_among_many(B, n_seqs, P):
+    """More segments than a warp tests at a time, empty ones and ones without kept rows among them; one tensor alone."""
+    import torch
+    dev = torch.device("cuda:0")
+    g = np.random.Generator(np.random.Philox(40 + n_seqs + P))
+    n_layers, Hq, Hkv, D, unit = 2, 9, 2, 16, max(P, 1)
+    seqlens = [int(x) for x in g.integers(0, 60, size=n_seqs)] if n_seqs > 1 else [50]
+    places = [(L + unit - 1) // unit for L in seqlens]
+    cu = np.concatenate([[0], np.cumsum(seqlens)])
+    idx, cu_kept = [], [0]
+    for seg in range(n_layers * n_seqs):
+        n = places[seg % n_seqs]
+        k = int(g.integers(0, n + 1)) if n_seqs > 1 else n
+        idx.append(np.sort(g.permutation(n)[:k]))
+        cu_kept.append(cu_kept[-1] + k)
+    flat = np.concatenate(idx).astype(np.int32)
+    cuk = np.asarray(cu_kept, dtype=np.int32)
+    rows = int((cuk[n_seqs::n_seqs] - cuk[:-1:n_seqs]).max()) * unit
+    T = int(sum(seqlens))
+    K = g.standard_normal((n_layers, T, Hkv, D)).astype(np.float32)
+    sc = g.random((n_layers, Hq, T)).astype(np.float32)
+    prob = B.Problem(n_layers, Hq, 1, D, seqlens, device=dev)
+    prob_kv = B.Problem(n_layers, Hkv, Hkv, D, seqlens, device=dev)
+    status = torch.zeros(4, dtype=torch.int32, device=dev)
+    dcu, didx = torch.from_numpy(cuk).to(dev), torch.from_numpy(flat).to(dev)
+    ko = torch.full((n_layers, rows, Hkv, D), -1.0, device=dev)
+    so = torch.full((n_layers, Hq, rows), -1.0, device=dev)
+    dK = torch.from_numpy(K).to(dev)
+    if P:
+        B.kvcrush_compact_pages(prob_kv, dK, None, P, dcu, didx, int(cuk[-1]), ko, None, status=status)
+    else:
+        B.kvcrush_compact(prob_kv, dK, None, dcu, didx, int(cuk[-1]), ko, None, status=status)
+    B.kvcrush_compact_scores(prob, torch.from_numpy(sc).to(dev), P, dcu, didx, int(cuk[-1]), so, status=status)
+    want_k, want_s = np.full(ko.shape, -1.0, np.float32), np.full(so.shape, -1.0, np.float32)
+    for seg, kept in enumerate(idx):
+        l, s = divmod(seg, n_seqs)
+        at = (int(cuk[seg]) - int(cuk[l * n_seqs])) * unit
+        for p in kept:
+            for j in range(unit):
+                t = int(p) * unit + j
+                want_k[l, at] = K[l, cu[s] + t] if t < seqlens[s] else 0.0
+                want_s[l, :, at] = sc[l, :, cu[s] + t] if t < seqlens[s] else 0.0
+                at += 1
+    np.testing.assert_array_equal(ko.cpu().numpy(), want_k)
+    np.testing.assert_array_equal(so.cpu().numpy(), want_s)
+
+
 def test_decode_time_paged_eviction_loop(B):
     """Prefill, then decode steps with page-granular eviction whenever the cache outgrows its budget (Table 1's paged
     setting in small: 1 initial page, 4 recent pages, the rest split between important and representative pages).
