@@ -18,19 +18,20 @@
 //
 //   * one CTA per SM lives for the whole launch and pulls work items from an atomic counter, so TMEM
 //     allocation, barrier set-up and pipeline fill are paid once per SM instead of once per item;
-//   * an item is a 512-row block of the stationary operand (four 128-row quarters).  Every streamed
-//     128-row tile is multiplied with all four quarters, which quarters the L2 -> shared-memory traffic per
-//     logit compared with one tile pair per load;
+//   * an item is a 512-row block of the stationary operand (four 128-row quarters; fewer when a launch has few
+//     items, see block_tiles).  Every streamed 128-row tile is multiplied with all four quarters, which quarters
+//     the L2 -> shared-memory traffic per logit compared with one tile pair per load;
 //   * TMEM holds one 128-column accumulator per quarter, owned by one epilogue group: a group needs no merge
 //     with another group, and while it waits for its accumulator to be refilled the other three keep the
 //     special-function unit busy.
 //
 // Roles: warp 0 fetches + decodes items and issues TMA loads; warps 1 and 2 (one lane each) issue the
-// tcgen05.mma of quarters 0-1 and 2-3; warps 3..18 are four epilogue groups (one per quarter) of 128 threads,
+// tcgen05.mma of quarters 0-1 and 2-3; warp 3 idles; warps 4..19 are four epilogue groups (one per quarter) of 128 threads,
 // thread = TMEM lane = one query row (sweep 1) or one key column (sweep 2).  All synchronisation is by mbarriers
 // with bounded waits: a role that gives up sets the CTA's abort flag, every other wait then ends, the CTA
 // reports through the status word, drains its copies, frees TMEM and returns.
 #include <cuda.h>
+#include <math.h>
 
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -43,15 +44,22 @@ using namespace tc;
 
 constexpr int kTile = 128;
 constexpr int kQ = 4;                        // stationary 128-row quarters per work item
-constexpr int kBlockRows = kQ * kTile;       // stationary rows per work item
 constexpr int kEpiWarps = 16;
 #ifndef KVC_ISSUE_WARPS
 #define KVC_ISSUE_WARPS 2
 #endif
 constexpr int kIssueWarps = KVC_ISSUE_WARPS;   // tcgen05.mma issuing threads; each owns kQ / kIssueWarps quarters
 constexpr int kQPerIssuer = kQ / kIssueWarps;
-constexpr int kThreads = 32 * (1 + kIssueWarps) + kEpiWarps * 32;
-constexpr int kRing = 2;                     // streamed tiles in flight
+constexpr int kCtrlWarps = 4;                // one warpgroup: producer, issuers, one idle warp
+constexpr int kThreads = 32 * (kCtrlWarps + kEpiWarps);
+// Registers: 96 a thread at launch (the most 20 warps can have); the control warpgroup gives some back (what its roles
+// need in either sweep) and the epilogue takes 104.
+template <bool kColsum> constexpr int kCtrlRegs = kColsum ? 64 : 48;
+constexpr int kEpiRegs = 104;
+static_assert(kIssueWarps < kCtrlWarps && 32 * kCtrlWarps * kCtrlRegs<true> + 32 * kEpiWarps * kEpiRegs <= kThreads * 96,
+              "register split within the launch's total");
+constexpr int kTiles = 6;                    // 128-row tiles in shared memory: tpb stationary ones, the others a ring of streamed tiles
+constexpr int kMaxRing = kTiles - 1;
 constexpr uint32_t kTmemCols = 512;          // one 128-column fp32 accumulator per quarter
 constexpr int kLseChunk = 16;                // sweep 2: streamed tiles whose row log-sum-exp is staged at once
 
@@ -65,12 +73,13 @@ struct PersistArgs {
   float* scores;           // sweep 2 output
   int normalize;
   int bf16;                // operand type of Q and K: bf16 (1) or fp16 (0)
-  int max_blocks;          // ceil(max_seqlen / kBlockRows)
+  int tpb;                 // 128-row tiles of an item's stationary block: 4, or 2 or 1 when the launch has few items
+  int max_blocks;          // ceil(max_seqlen / (tpb * kTile))
   int n_items;             // (sequence, stationary block) pairs of one (layer, head)
   int total_items;         // n_items * n_layers * Hq
   int n_lh;                // n_layers * Hq
   int tail_lh;             // the last tail_lh (layer, head) pairs are handed out heaviest item first across all of them
-  int* counter;            // work counter, zero at launch
+  int* counter;            // work counter, zero at launch; NULL: items are dealt out in advance (see the producer)
   int32_t* status;
   int withhold_first_item; // diagnostic: the producer warp fetches its first item and then stops before announcing
                            // it or issuing any copy for it, so that every consumer's first wait runs out
@@ -80,15 +89,13 @@ template <int D>
 struct PSmem {
   static constexpr int kTileBytes = kTile * D * 2;
   static constexpr int kBlockBytes = kTile * 128;
-  static constexpr int kFixedOff = 0;                            // the stationary quarters
-  static constexpr int kRingOff = kQ * kTileBytes;
-  static constexpr int kAuxOff = kRingOff + kRing * kTileBytes;
+  static constexpr int kAuxOff = kTiles * kTileBytes;           // the stationary quarters, then the ring, from offset 0
   static constexpr int kAuxBytes = 26624;
   static constexpr int kTotal = kAuxOff + kAuxBytes + 1024;
 };
 
 struct PAux {
-  unsigned long long full[kRing], empty[kRing];
+  unsigned long long full[kMaxRing], empty[kMaxRing];
   unsigned long long fixed_full, fixed_empty;
   unsigned long long acc_full[kQ], acc_empty[kQ];     // [quarter]
   unsigned long long item_full[2], item_empty[2];
@@ -97,59 +104,61 @@ struct PAux {
   unsigned long long drain[kIssueWarps];
   uint32_t tmem_base;
   int abort_flag;
-  int item[2][8];                                     // layer, head, seq, block, n_tiles (layer < 0: no more work)
+  int item[2][8];                                     // layer, head, first tile, tiles, first token, tokens (layer < 0: no more work)
   alignas(16) float lse_chunk[2][kLseChunk * kTile];  // [buffer][streamed tile inside the chunk][query]: minus lse2
   alignas(16) float part[2][kQ][2][kTile];            // [item parity][slot][max, sum][row]: sweep 1, replicated quarters
 };
 
 // Geometry of one work item, derived identically by every role.
-template <bool kColsum>
+template <bool kColsum, bool kSplit>
 struct Geo {
-  int layer, h, hk, t0, L, blk, first_stream, n_iter;
+  int layer, h, hk, t0, L, first_stream, n_iter;
+  int row0, tile0;             // first row of the stationary block inside the sequence, and row0 / kTile
   int ws;                      // first query row that votes (0 without an observation window)
   bool causal;
-  int nq;                      // quarters of the block that hold rows of the sequence
-  // The four accumulator slots normally hold the four quarters.  In sweep 1 with an observation window only the
-  // quarters with voting queries have work; when these are one or two, each is loaded into rep = 4 or 2 slots and
-  // slot s takes the streamed tiles it with it % rep == s % rep, so that all four epilogue groups stay busy.
-  int rep, v0;                 // slots per voting quarter; first voting quarter
-  __device__ __forceinline__ Geo(const Shape& s, const int* it) {
-    layer = it[0]; h = it[1]; hk = h / s.G; blk = it[3];
-    const int seq = it[2], n_tiles = it[4];
-    t0 = __ldg(s.cu_seqlens + seq);
-    L = __ldg(s.cu_seqlens + seq + 1) - t0;
+  int nq;                      // 128-row quarters of the block that hold rows of the sequence
+  // The four accumulator slots normally hold four quarters.  When an item has only one or two (small blocks, the last
+  // block of a sequence, in sweep 1 also an observation window whose queries lie in one or two quarters), each quarter
+  // serves rep = 4 or 2 slots and slot s takes the streamed tiles it with it % rep == s % rep, so that all four epilogue
+  // groups stay busy; the slots' sums are merged at the end of the item.  (kSplit; without it rep is the constant 1.)
+  int rep, v0;                 // slots per quarter; first quarter with work
+  __device__ __forceinline__ Geo(const Shape& s, const volatile int* it, int tpb) {
+    layer = it[0]; h = it[1]; tile0 = it[2]; t0 = it[4]; L = it[5];
+    const int n_tiles = it[3];
+    hk = h / s.G;
+    row0 = tile0 * kTile;
     causal = s.causal != 0;
-    nq = min(kQ, (L - blk * kBlockRows + kTile - 1) / kTile);
+    nq = min(tpb, (L - row0 + kTile - 1) / kTile);
     ws = (s.window > 0 && L > s.window) ? L - s.window : 0;
-    rep = 1; v0 = 0;
+    v0 = 0;
     if (kColsum) {                                                      // stationary keys, streamed query tiles
-      first_stream = max(causal ? kQ * blk : 0, ws / kTile);
+      first_stream = max(causal ? tile0 : 0, ws / kTile);
       n_iter = n_tiles - first_stream;
     } else {                                                            // stationary queries, streamed key tiles
       first_stream = 0;
-      n_iter = causal ? min(kQ * blk + kQ, n_tiles) : n_tiles;
-      if (ws > blk * kBlockRows) v0 = min(nq - 1, (ws - blk * kBlockRows) / kTile);
-      if (s.window > 0) rep = nq - v0 == 1 ? 4 : (nq - v0 == 2 ? 2 : 1);
+      n_iter = causal ? min(tile0 + tpb, n_tiles) : n_tiles;
+      if (ws > row0) v0 = min(nq - 1, (ws - row0) / kTile);
     }
+    rep = !kSplit ? 1 : nq - v0 == 1 ? 4 : nq - v0 == 2 ? 2 : 1;
   }
-  __device__ __forceinline__ int n_slots() const { return rep > 1 ? kQ : nq; }
   __device__ __forceinline__ int quarter(int slot) const { return rep > 1 ? v0 + slot / rep : slot; }
-  // does streamed tile `it` contribute to slot `sl` (causal: the quarter's own tile index is kQ*blk + quarter)
-  __device__ __forceinline__ bool active(int sl, int it) const {
-    const int qd = quarter(sl);
-    if (qd >= nq || qd < v0) return false;                              // no rows, or no voting query
-    if (rep > 1 && it % rep != sl % rep) return false;
-    if (!causal) return true;
-    return kColsum ? first_stream + it >= kQ * blk + qd : it <= kQ * blk + qd;
-  }
-  __device__ __forceinline__ bool diag(int sl, int it) const {
-    const int qd = quarter(sl);
-    return causal && (kColsum ? first_stream + it == kQ * blk + qd : it == kQ * blk + qd);
+  // Streamed tiles of a slot: first, first + rep, .. below end; `diag`: the one that holds the causal diagonal (-1: none).
+  struct Range { int first, end, diag; };
+  __device__ __forceinline__ Range range(int slot) const {
+    const int qd = quarter(slot), rr = slot & (rep - 1), own = tile0 + qd - first_stream;
+    if (qd >= nq || qd < v0) return {0, 0, -1};                         // no rows, or no voting query
+    if (!causal) return {rr, n_iter, -1};
+    if (!kColsum) return {rr, min(n_iter, own + 1), own};
+    const int lo = max(own, 0);
+    return {lo + ((rr - lo) & (rep - 1)), n_iter, own};
   }
 };
 
+// kSplit: items with one or two quarters spread them over all four accumulators.  The column sweep has an instantiation
+// without it for full blocks: carrying it along costs 2 % there (372 against 365 us at 2 layers of 5003 + 3117 tokens,
+// 4 % at ragged 500 to 1000 tokens), while its partial last blocks are its lightest items.
 // kPolls: polls of every bounded barrier wait (a compile-time constant: the epilogue has no register to spare for it).
-template <int D, bool kColsum, uint32_t kPolls>
+template <int D, bool kColsum, bool kSplit, uint32_t kPolls>
 __global__ void __launch_bounds__(kThreads, 1)
 score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const PersistArgs a) {
@@ -158,8 +167,8 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   PAux* aux = reinterpret_cast<PAux*>(smem + SL::kAuxOff);
   volatile int* abort_flag = &aux->abort_flag;
-  const uint32_t fixed_addr = smem_u32(smem + SL::kFixedOff);
-  const uint32_t ring_addr = smem_u32(smem + SL::kRingOff);
+  const int ring = kTiles - a.tpb;
+  const uint32_t fixed_addr = smem_u32(smem), ring_addr = fixed_addr + a.tpb * SL::kTileBytes;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Shape& s = a.s;
 
@@ -167,7 +176,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     if (lane == 0) {
       // a launch that already failed somewhere is not worth finishing
       aux->abort_flag = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
-      for (int i = 0; i < kRing; ++i) { mbar_init(smem_u32(&aux->full[i]), 1); mbar_init(smem_u32(&aux->empty[i]), kIssueWarps); }
+      for (int i = 0; i < kMaxRing; ++i) { mbar_init(smem_u32(&aux->full[i]), 1); mbar_init(smem_u32(&aux->empty[i]), kIssueWarps); }
       mbar_init(smem_u32(&aux->fixed_full), 1);
       mbar_init(smem_u32(&aux->fixed_empty), kIssueWarps);
       for (int i = 0; i < kIssueWarps; ++i) mbar_init(smem_u32(&aux->drain[i]), 1);
@@ -198,9 +207,13 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
   if (dead) {
     // nothing to do
-  } else if (warp == 0) {
+  } else if (warp < kCtrlWarps) {
+  set_max_regs<kCtrlRegs<kColsum>, false>();
+  if (warp == 0) {
     // ------------------------------ work fetch + TMA producer ------------------------------
-    int n_item = 0, n_stream = 0;
+    int n_item = 0, n_stream = 0;     // n_stream: streamed tiles issued
+    int rs = 0;                       // lane 0: ring slot of the next tile
+    uint32_t ring_phase = 0;          //         and its phase
     int issued_item = 0;              // lane 0: items whose stationary load was issued
     bool alive = true;
     while (alive) {
@@ -209,7 +222,10 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       bool ok = true;
       if (lane == 0) {
         ok = mbar_wait(smem_u32(&aux->item_empty[slot]), ((n_item >> 1) & 1) ^ 1, abort_flag, kPolls);
-        if (ok) idx = atomicAdd(a.counter, 1);
+        // Few items: dealt out in advance, heaviest first in snake order (block b takes b, 2n - 1 - b, 2n + b, ..), which
+        // spares the call the memset of the counter.
+        if (ok) idx = a.counter ? atomicAdd(a.counter, 1)
+                                : n_item * (int)gridDim.x + (n_item & 1 ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x);
       }
       ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
       idx = __shfl_sync(0xFFFFFFFFu, idx, 0);
@@ -231,34 +247,36 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         rank = j / a.tail_lh; lh = a.n_lh - a.tail_lh + (j - rank * a.tail_lh);
       }
       int seq, blk, nblk;
-      decode_item(s.cu_seqlens, s.n_seqs, a.max_blocks, rank, !kColsum, lane, seq, blk, nblk, kBlockRows, s.window);
+      decode_item(s.cu_seqlens, s.n_seqs, a.max_blocks, rank, !kColsum, lane, seq, blk, nblk, a.tpb * kTile, s.window);
       if (lane == 0) {
         int* it = aux->item[slot];
-        it[0] = lh / s.Hq; it[1] = lh - it[0] * s.Hq; it[2] = seq; it[3] = blk;
-        it[4] = (__ldg(s.cu_seqlens + seq + 1) - __ldg(s.cu_seqlens + seq) + kTile - 1) / kTile;
+        it[0] = lh / s.Hq; it[1] = lh - it[0] * s.Hq; it[2] = blk * a.tpb;
+        it[4] = __ldg(s.cu_seqlens + seq); it[5] = __ldg(s.cu_seqlens + seq + 1) - it[4];
+        it[3] = (it[5] + kTile - 1) / kTile;
         mbar_arrive(smem_u32(&aux->item_full[slot]));
-        const Geo<kColsum> g(s, it);
+        const Geo<kColsum, kSplit> g(s, it, a.tpb);
         const int head_fixed = kColsum ? g.hk : g.h, head_stream = kColsum ? g.h : g.hk;
         // the stationary buffer is free once every MMA of the previous item has retired
         ok = mbar_wait(smem_u32(&aux->fixed_empty), (n_item & 1) ^ 1, abort_flag, kPolls);
         if (ok) {
-          const int n_slots = g.n_slots();
-          mbar_expect_tx(smem_u32(&aux->fixed_full), n_slots * SL::kTileBytes);
-          for (int sl = 0; sl < n_slots; ++sl)
+          const int n_fixed = g.nq - g.v0;
+          mbar_expect_tx(smem_u32(&aux->fixed_full), n_fixed * SL::kTileBytes);
+          for (int q = 0; q < n_fixed; ++q)
 #pragma unroll
             for (int kb = 0; kb < D / 64; ++kb)
-              tma_load_4d(fixed_addr + sl * SL::kTileBytes + kb * SL::kBlockBytes, map_fixed, smem_u32(&aux->fixed_full),
-                          kb * 64, g.t0 + g.blk * kBlockRows + g.quarter(sl) * kTile, head_fixed, g.layer);
+              tma_load_4d(fixed_addr + q * SL::kTileBytes + kb * SL::kBlockBytes, map_fixed, smem_u32(&aux->fixed_full),
+                          kb * 64, g.t0 + g.row0 + (g.v0 + q) * kTile, head_fixed, g.layer);
           issued_item = n_item + 1;
-          for (int i = 0; ok && i < g.n_iter; ++i, ++n_stream) {
-            const int rs = n_stream % kRing;
-            ok = mbar_wait(smem_u32(&aux->empty[rs]), ((n_stream / kRing) & 1) ^ 1, abort_flag, kPolls);
+          for (int i = 0; ok && i < g.n_iter; ++i) {
+            ok = mbar_wait(smem_u32(&aux->empty[rs]), ring_phase ^ 1, abort_flag, kPolls);
             if (!ok) break;
             mbar_expect_tx(smem_u32(&aux->full[rs]), SL::kTileBytes);
 #pragma unroll
             for (int kb = 0; kb < D / 64; ++kb)
               tma_load_4d(ring_addr + rs * SL::kTileBytes + kb * SL::kBlockBytes, map_stream, smem_u32(&aux->full[rs]),
                           kb * 64, g.t0 + (g.first_stream + i) * kTile, head_stream, g.layer);
+            ++n_stream;
+            if (++rs == ring) { rs = 0; ring_phase ^= 1; }
           }
         }
       }
@@ -268,8 +286,8 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     }
     if (lane == 0 && *abort_flag) {
       // give the copies in flight a bounded time to land before the CTA's shared memory is released
-      for (int q = max(0, n_stream - kRing); q < n_stream; ++q)
-        for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(smem_u32(&aux->full[q % kRing]), (q / kRing) & 1); ++i) {}
+      for (int q = max(0, n_stream - ring); q < n_stream; ++q)
+        for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(smem_u32(&aux->full[q % ring]), (q / ring) & 1); ++i) {}
       if (issued_item > 0)
         for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(smem_u32(&aux->fixed_full), (issued_item - 1) & 1); ++i) {}
     }
@@ -281,30 +299,35 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     if (lane == 0) {
       const int iw = warp - 1;
       const uint32_t idesc = make_idesc(kTile, kTile, a.bf16 != 0);
-      int n_item = 0, n_stream = 0, cnt[kQPerIssuer] = {};
+      int n_item = 0, rs = 0, cnt[kQPerIssuer] = {};
+      uint32_t ring_phase = 0;
       bool ok = true;
       while (ok) {
         const int slot = n_item & 1;
         ok = mbar_wait(smem_u32(&aux->item_full[slot]), (n_item >> 1) & 1, abort_flag, kPolls);
         if (!ok) break;
-        int it[5];
-#pragma unroll
-        for (int i = 0; i < 5; ++i) it[i] = aux->item[slot][i];
-        mbar_arrive(smem_u32(&aux->item_empty[slot]));
+        const volatile int* it = aux->item[slot];
         if (it[0] < 0) break;
-        const Geo<kColsum> g(s, it);
+        const Geo<kColsum, kSplit> g(s, it, a.tpb);
+        mbar_arrive(smem_u32(&aux->item_empty[slot]));
         ok = mbar_wait(smem_u32(&aux->fixed_full), n_item & 1, abort_flag, kPolls);
-        for (int i = 0; ok && i < g.n_iter; ++i, ++n_stream) {
-          const int rs = n_stream % kRing;
+        typename Geo<kColsum, kSplit>::Range rg[kQPerIssuer];
+        uint32_t a_addr[kQPerIssuer];
+#pragma unroll
+        for (int u = 0; u < kQPerIssuer; ++u) {
+          rg[u] = g.range(kQPerIssuer * iw + u);
+          a_addr[u] = fixed_addr + (g.quarter(kQPerIssuer * iw + u) - g.v0) * SL::kTileBytes;
+        }
+        for (int i = 0; ok && i < g.n_iter; ++i) {
           // also when its quarters skip the tile: the wait keeps the issuer from running a whole ring ahead of
           // the other one, whose arrival on empty[rs] must fall into the same phase as this one's
-          ok = mbar_wait(smem_u32(&aux->full[rs]), (n_stream / kRing) & 1, abort_flag, kPolls);
+          ok = mbar_wait(smem_u32(&aux->full[rs]), ring_phase, abort_flag, kPolls);
           if (!ok) break;
 #pragma unroll
           for (int u = 0; u < kQPerIssuer; ++u) {
             if (!ok) break;
             const int qd = kQPerIssuer * iw + u;
-            if (!g.active(qd, i)) continue;
+            if (i < rg[u].first || i >= rg[u].end || ((i - rg[u].first) & (g.rep - 1))) continue;
             const int c = cnt[u]++;                 // the quarter's accumulator is reused every time: phase c & 1
             ok = mbar_wait(smem_u32(&aux->acc_empty[qd]), (c & 1) ^ 1, abort_flag, kPolls);
             if (!ok) break;
@@ -313,7 +336,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 #pragma unroll
             for (int k = 0; k < D / 16; ++k) {
               const uint32_t off = (k >> 2) * SL::kBlockBytes + (k & 3) * 32;
-              umma_bf16(d_tmem, smem_desc_sw128(fixed_addr + qd * SL::kTileBytes + off),
+              umma_bf16(d_tmem, smem_desc_sw128(a_addr[u] + off),
                         smem_desc_sw128(ring_addr + rs * SL::kTileBytes + off), idesc, k > 0);
             }
             umma_commit(smem_u32(&aux->acc_full[qd]));
@@ -321,6 +344,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           if (!ok) break;
           // this issuer is done with the ring slot (a commit with nothing pending arrives at once)
           umma_commit(smem_u32(&aux->empty[rs]));
+          if (++rs == ring) { rs = 0; ring_phase ^= 1; }
         }
         if (!ok) break;
         umma_commit(smem_u32(&aux->fixed_empty));
@@ -332,9 +356,11 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(smem_u32(&aux->drain[iw]), 0); ++i) {}
       }
     }
+  }
   } else {
     // ------------------------------ epilogue groups ------------------------------
-    const int gi = (warp - 1 - kIssueWarps) >> 2;  // group = stationary quarter; it owns that quarter's accumulator
+    set_max_regs<kEpiRegs, true>();
+    const int gi = (warp - kCtrlWarps) >> 2;  // group = stationary quarter; it owns that quarter's accumulator
     const int quarter = warp & 3;                  // TMEM lanes this warp may read
     const int r = quarter * 32 + lane;             // row of the accumulator = TMEM lane = index inside the group
     const uint32_t t_acc = tmem_base + ((uint32_t)(quarter * 32) << 16) + gi * kTile;
@@ -342,7 +368,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     const float scale = a.scale_log2;
     const f32x2 scale2 = splat2(scale);
     const float ninf = __int_as_float(0xFF800000);
-    int n_item = 0, cnt = 0, n_esync = 0;
+    int n_item = 0, cnt = 0, n_esync = 0, n_merge = 0;
     bool ok = true;
 
     // barrier among all 16 epilogue warps; bounded like every other wait
@@ -363,15 +389,12 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       ok = mbar_wait(smem_u32(&aux->item_full[slot]), (n_item >> 1) & 1, abort_flag, kPolls) && ok;
       ok = __all_sync(0xFFFFFFFFu, ok);
       if (!ok) break;
-      int it[5];
-#pragma unroll
-      for (int i = 0; i < 5; ++i) it[i] = aux->item[slot][i];
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&aux->item_empty[slot]));
+      // The item is read again when its results are written, rather than kept in registers, of which there is none to
+      // spare; the slot is handed back after that.
+      const volatile int* it = aux->item[slot];
       if (it[0] < 0) break;
-      const Geo<kColsum> g(s, it);
-      const int row = g.blk * kBlockRows + g.quarter(gi) * kTile + r;   // token of this thread inside the sequence
-      const size_t out = ((size_t)g.layer * s.Hq + g.h) * s.T + g.t0 + row;
+      const Geo<kColsum, kSplit> g(s, it, a.tpb);
+      const auto rg = g.range(gi);
 
       if constexpr (kColsum) {
         const float* lse_row = a.lse + ((size_t)g.layer * s.Hq + g.h) * s.T + g.t0;
@@ -379,7 +402,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         // at a time and once for all four groups: all 16 warps fill the next chunk's buffer, then work through the
         // current chunk, and meet once per chunk (the buffer of chunk k is rewritten as chunk k + 2 only after
         // everybody left chunk k).
-        const int et = tid - 32 * (1 + kIssueWarps);
+        const int et = tid - 32 * kCtrlWarps;
         auto fill = [&](int k) {
           float* dst = aux->lse_chunk[k & 1];
 #pragma unroll
@@ -391,20 +414,20 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         };
         f32x2 acc[2] = {0ull, 0ull};
         const int n_chunks = (g.n_iter + kLseChunk - 1) / kLseChunk;
+        int i = rg.first;
         fill(0);
         epi_sync();
         for (int k = 0; k < n_chunks && ok; ++k) {
           if (k + 1 < n_chunks) fill(k + 1);
-          const int i_end = min(g.n_iter, kLseChunk * (k + 1));
-          for (int i = kLseChunk * k; i < i_end && ok; ++i) {
-            if (!g.active(gi, i)) continue;
+          const int i_end = min(rg.end, kLseChunk * (k + 1));
+          for (; i < i_end; i += g.rep) {
             const int c = cnt++;
             const float* lse_buf = aux->lse_chunk[k & 1] + (i & (kLseChunk - 1)) * kTile;
             ok = mbar_wait(acc_full, c & 1, abort_flag, kPolls) && ok;
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             tc_fence_after();
-            if (g.diag(gi, i))
+            if (i == rg.diag)
               sweep_tile<true>(t_acc, [&](const uint32_t (&v)[16], int p) { colsum_piece<true>(v, lse_buf + p * 16, scale2, r, p * 16, acc); }, release);
             else
               sweep_tile(t_acc, [&](const uint32_t (&v)[16], int p) { colsum_piece<false>(v, lse_buf + p * 16, scale2, r, p * 16, acc); }, release);
@@ -414,22 +437,32 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         ok = __all_sync(0xFFFFFFFFu, ok);
         if (!ok) break;
         float total = sum4(acc);
-        if (row < g.L) {
+        const Geo<kColsum, kSplit> g(s, it, a.tpb);
+        const int row = g.row0 + g.quarter(gi) * kTile + r;    // token of this thread inside the sequence
+        if (g.rep > 1) {                     // slots that share a quarter add up their sums
+          float (*part)[2][kTile] = aux->part[n_merge++ & 1];
+          part[gi][0][r] = total;
+          epi_sync();
+          ok = __all_sync(0xFFFFFFFFu, ok);
+          if (!ok) break;
+          if ((gi & (g.rep - 1)) == 0)
+            for (int u = 1; u < g.rep; ++u) total += part[gi + u][0][r];
+        }
+        if (row < g.L && (gi & (g.rep - 1)) == 0) {
           if (a.normalize) total = total / (float)(g.L - g.ws);
-          a.scores[out] = total;
+          a.scores[((size_t)g.layer * s.Hq + g.h) * s.T + g.t0 + row] = total;
         }
       } else {
         float m = __int_as_float(0xFF800000);                   // running max (log2 domain) of this row
         f32x2 sum2[2] = {0ull, 0ull};                           // packed partial sums of 2^(x - m)
-        for (int i = 0; i < g.n_iter && ok; ++i) {
-          if (!g.active(gi, i)) continue;
+        for (int i = rg.first; i < rg.end; i += g.rep) {
           const int c = cnt++;
           ok = mbar_wait(acc_full, c & 1, abort_flag, kPolls) && ok;
           ok = __all_sync(0xFFFFFFFFu, ok);
           if (!ok) break;
           tc_fence_after();
           // keys of this tile that count for this row: up to the diagonal (causal) and inside the sequence
-          const int n_valid = g.causal ? (g.diag(gi, i) ? r + 1 : kTile) : min(kTile, g.L - i * kTile);
+          const int n_valid = g.causal ? (i == rg.diag ? r + 1 : kTile) : min(kTile, g.L - i * kTile);
           // masked columns, or a row that has no reference yet (its first tile): exact maxima, piece by piece
           if (__any_sync(0xFFFFFFFFu, n_valid < kTile || !(m > -3.0e38f)))
             sweep_tile<true>(t_acc, [&](const uint32_t (&v)[16], int p) { lse_piece<true>(v, scale, scale2, n_valid - p * 16, m, sum2); }, release);
@@ -439,32 +472,37 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         ok = __all_sync(0xFFFFFFFFu, ok);
         if (!ok) break;
         float sum = sum4(sum2);
-        if (s.window > 0) {                  // slots that share a quarter merge their (max, sum) through shared memory
-          float* pm = aux->part[n_item & 1][gi][0];
-          float* ps = aux->part[n_item & 1][gi][1];
-          pm[r] = m;
-          ps[r] = sum;
+        const Geo<kColsum, kSplit> g(s, it, a.tpb);
+        const int row = g.row0 + g.quarter(gi) * kTile + r;
+        if (g.rep > 1) {                     // slots that share a quarter merge their (max, sum)
+          // (alternating buffers: a slot writes one again only after the sync that follows every read of it)
+          float (*part)[2][kTile] = aux->part[n_merge++ & 1];
+          part[gi][0][r] = m;
+          part[gi][1][r] = sum;
           epi_sync();
           ok = __all_sync(0xFFFFFFFFu, ok);
           if (!ok) break;
-          if (g.rep > 1 && gi % g.rep == 0) {
+          if ((gi & (g.rep - 1)) == 0) {
             float big = m;
-            for (int u = 1; u < g.rep; ++u) big = fmaxf(big, aux->part[n_item & 1][gi + u][0][r]);
+            for (int u = 1; u < g.rep; ++u) big = fmaxf(big, part[gi + u][0][r]);
             float tot = sum > 0.f ? sum * ex2(m - big) : 0.f;
             for (int u = 1; u < g.rep; ++u) {
-              const float mu = aux->part[n_item & 1][gi + u][0][r], su = aux->part[n_item & 1][gi + u][1][r];
+              const float mu = part[gi + u][0][r], su = part[gi + u][1][r];
               tot += su > 0.f ? su * ex2(mu - big) : 0.f;
             }
             m = big;
             sum = tot;
           }
         }
-        if (row < g.L && row >= g.ws && (g.rep == 1 || gi % g.rep == 0)) {
+        if (row < g.L && row >= g.ws && (gi & (g.rep - 1)) == 0) {
           const float lse2 = m + log2f(sum);
+          const size_t out = ((size_t)g.layer * s.Hq + g.h) * s.T + g.t0 + row;
           a.lse2_out[out] = lse2;
           if (a.lse_nat_out) a.lse_nat_out[out] = lse2 * 0.69314718055994530942f;
         }
       }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&aux->item_empty[slot]));
       ++n_item;
     }
   }
@@ -478,9 +516,9 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   if (tid == 0 && !dead && *abort_flag) report(a.status, KVCRUSH_DEV_TIMEOUT, kColsum ? KID_SCORE_COLSUM : KID_SCORE_LSE, blockIdx.x, 0);
 }
 
-template <int D, bool kColsum, uint32_t kPolls>
+template <int D, bool kColsum, bool kSplit, uint32_t kPolls>
 int launch_persist_polls(const CUtensorMap& mq, const CUtensorMap& mk, const PersistArgs& a, int n_sms, cudaStream_t stream) {
-  auto kern = score_persist_kernel<D, kColsum, kPolls>;
+  auto kern = score_persist_kernel<D, kColsum, kSplit, kPolls>;
   constexpr int smem = PSmem<D>::kTotal;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return KVCRUSH_ERR_CUDA;
   const int blocks = a.total_items < n_sms ? a.total_items : n_sms;
@@ -488,11 +526,41 @@ int launch_persist_polls(const CUtensorMap& mq, const CUtensorMap& mk, const Per
   return check_launch();
 }
 
-template <int D, bool kColsum>
+template <int D, bool kColsum, bool kSplit>
 int launch_persist(const CUtensorMap& mq, const CUtensorMap& mk, const PersistArgs& a, bool short_waits, int n_sms,
                    cudaStream_t stream) {
-  return short_waits ? launch_persist_polls<D, kColsum, kShortWaitPolls>(mq, mk, a, n_sms, stream)
-                     : launch_persist_polls<D, kColsum, kWaitPolls>(mq, mk, a, n_sms, stream);
+  return short_waits ? launch_persist_polls<D, kColsum, kSplit, kShortWaitPolls>(mq, mk, a, n_sms, stream)
+                     : launch_persist_polls<D, kColsum, kSplit, kWaitPolls>(mq, mk, a, n_sms, stream);
+}
+
+// Tiles of an item's stationary block.  Four 128-row tiles take the most out of every streamed tile, but a launch with
+// few items then ends with one item per SM and the others idle; with two or one, each tile serves two or four
+// accumulator slots and an item is a half or a quarter as long.  Estimated in rounds (one streamed tile against four
+// accumulators): the longest item or the mean load plus what a list schedule loses, times what a round costs more when
+// a streamed tile is used less often, plus what an item costs by itself.  Both sweeps, 32 heads: 1001 tokens (8 KV heads)
+// 45.5 / 32.4 / 31.3 us with 4 / 2 / 1 tiles, 2048 tokens 83.9 / 59.6 / 71.1, 3072 tokens 121 / 115 / 131, 4096 tokens
+// 175 / 185 / 213; 8 heads, 8192 tokens 297 / 166 / 183, 5000 tokens 183 / 103 / 80.
+int block_tiles(const Shape& s, const int32_t* cu_host, int n_sms) {
+  constexpr float kRoundCost[3] = {1.f, 1.2f, 1.45f};
+  const float n_lh = (float)s.n_layers * s.Hq;
+  int best = kQ;
+  float best_cost = 0.f;
+  for (int v = 0, tpb = kQ; tpb >= 1; ++v, tpb /= 2) {
+    float sum = 0.f, longest = 0.f, items = 0.f;
+    for (int i = 0; i < s.n_seqs; ++i) {
+      const int n = (cu_host[i + 1] - cu_host[i] + kTile - 1) / kTile;
+      const int full = n / tpb, q = n - full * tpb;                  // full blocks, tiles of the last one
+      const float tail = n * (q == 3 ? 4 : q) * 0.25f;
+      const float round_tiles = tpb * 0.25f;                         // rounds per streamed tile
+      sum += tail + (s.causal ? round_tiles * tpb * 0.5f * full * (full + 1) : round_tiles * n * full);
+      longest = fmaxf(longest, fmaxf(tail, full ? round_tiles * (s.causal ? full * tpb : n) : 0.f));
+      items += full + (q > 0);
+    }
+    const float per_sm = n_lh / n_sms;
+    const float cost = kRoundCost[v] * fmaxf(longest, 1.15f * sum * per_sm) + 0.4f * ceilf(items * per_sm);
+    if (tpb == kQ || cost < best_cost) { best = tpb; best_cost = cost; }
+  }
+  return best;
 }
 
 }  // namespace
@@ -528,40 +596,50 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
   a.s = s; a.scale_log2 = scale_log2; a.normalize = normalize; a.bf16 = Q.dtype == KVCRUSH_BF16; a.status = status; a.scores = scores;
   const bool sw = diag.short_waits != 0;
   a.withhold_first_item = diag.withhold_first_item;
-  a.max_blocks = (s.max_seqlen + kBlockRows - 1) / kBlockRows;
-  // work items per (layer, head): every 512-row block for the column sweep; for the row sweep only the
-  // blocks that hold voting queries
-  long long items_col = 0, items_row = 0;
-  for (int i = 0; i < s.n_seqs; ++i) {
-    const int len = cu_host[i + 1] - cu_host[i];
-    const int nb = (len + kBlockRows - 1) / kBlockRows;
-    const int first = (s.window > 0 && len > s.window) ? (len - s.window) / kBlockRows : 0;
-    items_col += nb;
-    items_row += nb - first;
-  }
-  if (items_col == 0) return KVCRUSH_OK;
-  if (items_col * s.n_layers * s.Hq > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
-  if (cudaMemsetAsync(counters, 0, 2 * sizeof(int), stream) != cudaSuccess) return KVCRUSH_ERR_CUDA;
+  // Work items per (layer, head): every block of tpb 128-row tiles for the column sweep; for the row sweep only the
+  // blocks that hold voting queries.
+  auto count = [&](int tpb, bool row_sweep) {
+    long long items = 0;
+    for (int i = 0; i < s.n_seqs; ++i) {
+      const int len = cu_host[i + 1] - cu_host[i], rows = tpb * kTile;
+      items += (len + rows - 1) / rows - (row_sweep && s.window > 0 && len > s.window ? (len - s.window) / rows : 0);
+    }
+    return items;
+  };
   a.n_lh = s.n_layers * s.Hq;
-  auto tail_pairs = [&](long long items) {       // pairs whose items make up about four rounds of the grid
-    const long long t = (4LL * n_sms + items - 1) / items;
-    return (int)(t < a.n_lh ? t : a.n_lh);
+  const long long items_all = count(1, false);
+  if (items_all == 0) return KVCRUSH_OK;
+  if (items_all * a.n_lh > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
+  a.tpb = s.window > 0 ? kQ : block_tiles(s, cu_host, n_sms);
+  bool zeroed = false;
+  auto plan = [&](bool row_sweep, int* counter) {
+    const long long items = count(a.tpb, row_sweep);
+    a.max_blocks = (s.max_seqlen + a.tpb * kTile - 1) / (a.tpb * kTile);
+    a.n_items = (int)items;
+    a.total_items = (int)(items * a.n_lh);
+    const long long tail = (4LL * n_sms + items - 1) / items;   // pairs whose items make up about four rounds of the grid
+    a.tail_lh = (int)(tail < a.n_lh ? tail : a.n_lh);
+    a.counter = a.tail_lh == a.n_lh ? nullptr : counter;
+    if (a.counter && !zeroed) {
+      if (cudaMemsetAsync(counters, 0, 2 * sizeof(int), stream) != cudaSuccess) return false;
+      zeroed = true;
+    }
+    return true;
   };
   int rc;
   if (!lse_in) {
-    a.lse2_out = lse2_ws; a.lse_nat_out = lse_out; a.counter = counters;
-    a.n_items = (int)items_row; a.total_items = (int)(items_row * s.n_layers * s.Hq);
-    a.tail_lh = tail_pairs(items_row);
-    rc = s.D > 64 ? launch_persist<128, false>(mq, mk, a, sw, n_sms, stream) : launch_persist<64, false>(mq, mk, a, sw, n_sms, stream);
+    if (!plan(true, counters)) return KVCRUSH_ERR_CUDA;
+    a.lse2_out = lse2_ws; a.lse_nat_out = lse_out;
+    rc = s.D > 64 ? launch_persist<128, false, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<64, false, true>(mq, mk, a, sw, n_sms, stream);
     if (rc != KVCRUSH_OK) return rc;
     a.lse = lse2_ws; a.lse_mul = 1.f;
   } else {
     a.lse = lse_in; a.lse_mul = lse_in_mul;
   }
-  a.counter = counters + 1;
-  a.n_items = (int)items_col; a.total_items = (int)(items_col * s.n_layers * s.Hq);
-  a.tail_lh = tail_pairs(items_col);
-  return s.D > 64 ? launch_persist<128, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<64, true>(mq, mk, a, sw, n_sms, stream);
+  if (!plan(false, counters + 1)) return KVCRUSH_ERR_CUDA;
+  if (a.tpb < kQ)
+    return s.D > 64 ? launch_persist<128, true, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<64, true, true>(mq, mk, a, sw, n_sms, stream);
+  return s.D > 64 ? launch_persist<128, true, false>(mq, mk, a, sw, n_sms, stream) : launch_persist<64, true, false>(mq, mk, a, sw, n_sms, stream);
 }
 
 }  // namespace kvc

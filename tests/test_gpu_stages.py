@@ -279,6 +279,43 @@ def test_score_tensor_matches_oracle(B, w):
     np.testing.assert_allclose(g, scores.cpu().numpy(), rtol=2e-4, atol=1e-6)
 
 
+@pytest.mark.parametrize("layers,Hq,Hkv,D,seqlens,causal", [
+    (16, 32, 8, 64, (513, 640, 768, 897, 1), True),            # four tiles a block; last blocks of 1, 1, 2 and 4 tiles
+    (16, 32, 32, 64, (1100, 300), False),                      # the same without a mask
+    (1, 32, 8, 128, (2048,), True),                            # two tiles a block
+    (1, 32, 8, 128, (1700, 130), True),                        # two, last blocks of 2 tiles with one short
+    (2, 16, 4, 64, (1921,), False),
+    (1, 32, 8, 128, (897,), True),                             # one tile a block, four slots each
+    (1, 8, 8, 64, (5000,), True),                              # one, more items than SMs dealt out in advance
+])
+def test_scores_with_every_block_size(B, layers, Hq, Hkv, D, seqlens, causal):
+    """Blocks of 4, 2 and 1 stationary tiles and their partial last blocks: the CUDA-core kernels on the same inputs agree
+    within the score tolerance's tenth, the oracle on two heads within the tolerance."""
+    import torch
+    dev = _dev()
+    w = inputs.Workload("blk", layers, Hq, Hkv, D, seqlens, inputs.BF16, inputs.BF16, 0.25, base_seed=250 + D, causal=causal)
+    lis, q, k, _, _ = TL.stack_layers(w, range(layers), with_cache=False)
+    prob = B.Problem(layers, Hq, Hkv, D, seqlens, causal=causal, device=dev)
+    dq, dk = TL.torch_storage(q, w.qk_dtype, dev), TL.torch_storage(k, w.qk_dtype, dev)
+    ws = torch.empty(B.kvcrush_workspace_size(prob, B.STAGE_SCORE), dtype=torch.uint8, device=dev)
+    status = torch.zeros(4, dtype=torch.int32, device=dev)
+    got = {}
+    for impl in (B.SCORE_TENSOR, B.SCORE_SIMT):
+        sc, ls = (torch.full((layers, Hq, w.total_tokens), -1.0, dtype=torch.float32, device=dev) for _ in range(2))
+        B.kvcrush_score(prob, dq, dk, sc, lse_out=ls, impl=impl, workspace=ws, status=status)
+        got[impl] = (sc.cpu().numpy(), ls.cpu().numpy())
+    assert status.cpu().tolist()[0] == 0
+    np.testing.assert_allclose(got[B.SCORE_TENSOR][0], got[B.SCORE_SIMT][0], rtol=2e-4, atol=1e-6)
+    np.testing.assert_allclose(got[B.SCORE_TENSOR][1], got[B.SCORE_SIMT][1], rtol=0, atol=2e-4)
+    cu, G = w.cu_seqlens, Hq // Hkv
+    for s, L in enumerate(seqlens):
+        a, b = int(cu[s]), int(cu[s + 1])
+        for h in (0, Hq - 1):
+            c, _ = O.scores(inputs.widen(lis[-1].q[a:b, h:h + 1], w.qk_dtype),
+                            inputs.widen(lis[-1].k[a:b, h // G:h // G + 1], w.qk_dtype), causal)
+            assert TL.within_score_tolerance(got[B.SCORE_TENSOR][0][-1, h:h + 1, a:b], c).all(), (s, h)
+
+
 def test_score_tensor_rejects_fp32_and_auto_falls_back_to_cuda_cores(B):
     import torch
     dev = _dev()
