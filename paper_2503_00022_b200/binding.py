@@ -104,17 +104,32 @@ def _check(rc: int, where: str) -> None:
 
 
 def _ptr(t) -> Optional[int]:
-    return None if t is None else int(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# A short pass is bound by what the host does between its launches, so the marshalling below takes the cheapest way
+# torch offers: the raw handle of the current stream instead of a Stream object (0.2 against 3.4 us a call), one
+# stride() call per tensor (1.0 against 1.6 us).  Issuing a four-stage pass: 57 -> 37 us.
+_dtype_codes: dict = {}
+_raw_stream = None
 
 
 def _stream() -> int:
-    import torch
-    return int(torch.cuda.current_stream().cuda_stream)
+    """Handle of the current device's current stream."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        torch.cuda.init()
+        _raw_stream = (lambda: raw(dev())) if raw and dev else (lambda: int(torch.cuda.current_stream().cuda_stream))
+    return _raw_stream()
 
 
 def dtype_code(torch_dtype) -> int:
-    import torch
-    return {torch.bfloat16: BF16, torch.float16: FP16, torch.float32: FP32}[torch_dtype]
+    if not _dtype_codes:
+        import torch
+        _dtype_codes.update({torch.bfloat16: BF16, torch.float16: FP16, torch.float32: FP32})
+    return _dtype_codes[torch_dtype]
 
 
 class Problem:
@@ -145,8 +160,9 @@ class Problem:
 
 def tensor_struct(t) -> TensorStruct:
     """Descriptor of a torch tensor viewed as [n_layers, tokens, heads, head_dim] (last stride 1)."""
-    assert t.dim() == 4 and t.stride(3) == 1, "expected [layers, tokens, heads, D] with contiguous D"
-    return TensorStruct(int(t.data_ptr()), dtype_code(t.dtype), 0, t.stride(0), t.stride(1), t.stride(2))
+    strides = t.stride()
+    assert len(strides) == 4 and strides[3] == 1, "expected [layers, tokens, heads, D] with contiguous D"
+    return TensorStruct(t.data_ptr(), dtype_code(t.dtype), 0, *strides[:3])
 
 
 def kvcrush_workspace_size(problem: Problem, stage: int) -> int:
