@@ -61,6 +61,42 @@ __device__ __forceinline__ int warp_segment_of_row(const int32_t* __restrict__ c
   return lo;
 }
 
+// ---- launches that overlap their predecessor's end --------------------------------------------------
+// A pass is a chain of short kernels, so every kernel is launched with programmatic stream serialization: its blocks are
+// set up while the kernel before it still runs.  The price is a rule: every kernel launched with launch_chained calls
+// chain_wait before its first access to global memory (the kernel before it, and with that everything earlier in the
+// stream, has then completed and its writes are visible) and chain_trigger after that, never before: a kernel that is
+// set up early must not find work older than its direct predecessor still running.
+// Passes issued one after the other, fp32 layer of 512 tokens 57.4 -> 48.1 us, bf16 layer of 1001 tokens 65.6 -> 58.8 us.
+// A captured launch keeps full dependencies: the launches of a graph are close together as it is, and its programmatic
+// edges cost more than they give (57.5 against 52.9 us for the same layer replayed).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... Params, class... Args>
+int launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t dyn_smem, cudaStream_t stream, int cluster,
+                   Args&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = dyn_smem;
+  cfg.stream = stream;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) cudaGetLastError();
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = capture == cudaStreamCaptureStatusNone;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  if (cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...) != cudaSuccess) {
+    cudaGetLastError();
+    return KVCRUSH_ERR_CUDA;
+  }
+  return KVCRUSH_OK;
+}
+
 // ---- stage launchers (defined in the per-stage .cu files) -------------------------------------------
 
 // score: SIMT fp32 kernels (any dtype/shape) and tcgen05 kernels (bf16 or fp16, D a multiple of 8 up to 128).

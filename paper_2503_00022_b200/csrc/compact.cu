@@ -31,6 +31,8 @@ template <bool kPaged, int kTensors>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 compact_kernel(Shape s, CompactArgs a, const int32_t* __restrict__ cu_kept, const int32_t* __restrict__ idx,
                long long total_kept, int page_size) {
+  chain_wait();
+  chain_trigger();
   const int lane = threadIdx.x & 31;
   const long long out_row = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   // row = position in the kept list (a token, or a page of which this warp copies slot `slot`); 64-bit divisions are slow
@@ -93,6 +95,8 @@ constexpr int kScoreHeads = 8;
 __global__ void __launch_bounds__(256)
 compact_scores_kernel(Shape s, const float* __restrict__ in, float* __restrict__ out, const int32_t* __restrict__ cu_kept,
                       const int32_t* __restrict__ idx, long long total_kept, int page_size, long long out_tokens) {
+  chain_wait();
+  chain_trigger();
   const long long out_row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   const auto row_of = [&](long long r) {
@@ -146,8 +150,8 @@ int launch_gather(const Shape& s, const TensorView& K, const TensorView* V, int 
   if (blocks > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
   auto kern = page_size > 0 ? (V ? compact_kernel<true, 2> : compact_kernel<true, 1>)
                             : (V ? compact_kernel<false, 2> : compact_kernel<false, 1>);
-  kern<<<(unsigned)blocks, kWarpsPerBlock * 32, 0, stream>>>(s, a, cu_kept, idx, total_kept, page_size > 0 ? page_size : 1);
-  return check_launch();
+  return launch_chained(kern, dim3((unsigned)blocks), dim3(kWarpsPerBlock * 32), 0, stream, 1, s, a, cu_kept, idx, total_kept,
+                        page_size > 0 ? page_size : 1);
 }
 
 }  // namespace
@@ -167,9 +171,8 @@ int launch_compact_scores(const Shape& s, const float* scores_in, int page_size,
   const long long blocks = (rows + 255) / 256;
   if (blocks > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
   const dim3 grid((unsigned)blocks, (unsigned)((s.Hq + kScoreHeads - 1) / kScoreHeads));
-  compact_scores_kernel<<<grid, 256, 0, stream>>>(s, scores_in, scores_out, cu_kept, idx, total_kept, ps,
-                                                             out_tokens);
-  return check_launch();
+  return launch_chained(compact_scores_kernel, grid, dim3(256), 0, stream, 1, s, scores_in, scores_out, cu_kept, idx, total_kept, ps,
+                        out_tokens);
 }
 
 int launch_compact_pages(const Shape& s, const TensorView& K, const TensorView* V, int page_size,

@@ -10,6 +10,8 @@ namespace {
 
 __global__ void __launch_bounds__(256)
 pool_scores_kernel(Shape s, const float* __restrict__ in, int radius, float* __restrict__ out) {
+  chain_wait();
+  chain_trigger();
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long n = (long long)s.n_layers * s.Hq * s.T;
   if (gid >= n) return;
@@ -30,8 +32,7 @@ int launch_pool_scores(const Shape& s, const float* scores_in, int kernel, float
   if (n == 0) return KVCRUSH_OK;
   const long long blocks = (n + 255) / 256;
   if (blocks > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
-  pool_scores_kernel<<<(unsigned)blocks, 256, 0, stream>>>(s, scores_in, (kernel - 1) / 2, scores_out);
-  return check_launch();
+  return launch_chained(pool_scores_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, 1, s, scores_in, (kernel - 1) / 2, scores_out);
 }
 
 }  // namespace kvc

@@ -143,6 +143,8 @@ decode_update_kernel(Shape s, TensorView Qn, TensorView K, float scale_log2, flo
   __shared__ float red[2][kHeads][kWarps];
   __shared__ float part[2][kHeads][2];                             // [pass parity][head]: maximum, sum of this block
   __shared__ float fin[kHeads];                                    // factor of the stored exponentials, or log-sum-exp
+  chain_wait();
+  chain_trigger();
   cg::cluster_group cluster = cg::this_cluster();
   const int n_blk = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int unit = blockIdx.x / n_blk;
@@ -295,21 +297,8 @@ int launch_one(const Shape& s, const TensorView& Qn, const TensorView& K, float 
   if (dyn > 32 * 1024 &&
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
     return KVCRUSH_ERR_CUDA;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)((long long)s.n_layers * s.n_seqs * s.Hkv * n_blk));
-  cfg.blockDim = dim3(kWarps * 32);
-  cfg.dynamicSmemBytes = dyn;
-  cfg.stream = stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)n_blk; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, kern, s, Qn, K, scale_log2, scores, cap) != cudaSuccess) {
-    cudaGetLastError();
-    return KVCRUSH_ERR_CUDA;
-  }
-  return check_launch();
+  return launch_chained(kern, dim3((unsigned)((long long)s.n_layers * s.n_seqs * s.Hkv * n_blk)), dim3(kWarps * 32), dyn, stream,
+                        n_blk, s, Qn, K, scale_log2, scores, cap);
 }
 
 template <typename T, int DB>

@@ -89,6 +89,8 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
   float* str_sh = fix_sh + kRows * (s.D + kPad);
   __shared__ float part[2][kRows];                          // this block's maximum (sweep 1) and sum of every row
   __shared__ float nlse_sh[kRows];                          // sweep 2: minus lse2 of the streamed queries, -inf: no vote
+  chain_wait();
+  chain_trigger();
   cg::cluster_group cluster = cg::this_cluster();
   const int n_blk = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -211,22 +213,8 @@ int launch_sweep(const Shape& s, const TensorView& Q, const TensorView& K, float
   auto kern = simt_sweep_kernel<T, kColsum>;
   if (dyn > 40 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
     return KVCRUSH_ERR_CUDA;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(units * n_blk));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = dyn;
-  cfg.stream = stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)n_blk; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, kern, s, Q, K, scale_log2, lse, lse_mul, lse2_out, lse_nat_out, scores, normalize, max_tiles) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return KVCRUSH_ERR_CUDA;
-  }
-  return check_launch();
+  return launch_chained(kern, dim3((unsigned)(units * n_blk)), dim3(kThreads), dyn, stream, n_blk, s, Q, K, scale_log2, lse, lse_mul,
+                        lse2_out, lse_nat_out, scores, normalize, max_tiles);
 }
 
 template <typename T>

@@ -174,8 +174,6 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
   if (warp == 0) {
     if (lane == 0) {
-      // a launch that already failed somewhere is not worth finishing
-      aux->abort_flag = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
       for (int i = 0; i < kMaxRing; ++i) { mbar_init(smem_u32(&aux->full[i]), 1); mbar_init(smem_u32(&aux->empty[i]), kIssueWarps); }
       mbar_init(smem_u32(&aux->fixed_full), 1);
       mbar_init(smem_u32(&aux->fixed_empty), kIssueWarps);
@@ -196,6 +194,10 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     tmem_alloc(smem_u32(&aux->tmem_base), kTmemCols);
     tmem_relinquish();
   }
+  chain_wait();
+  chain_trigger();
+  // a launch that already failed somewhere is not worth finishing
+  if (tid == 0) aux->abort_flag = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -522,8 +524,7 @@ int launch_persist_polls(const CUtensorMap& mq, const CUtensorMap& mk, const Per
   constexpr int smem = PSmem<D>::kTotal;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return KVCRUSH_ERR_CUDA;
   const int blocks = a.total_items < n_sms ? a.total_items : n_sms;
-  kern<<<(unsigned)blocks, kThreads, smem, stream>>>(mq, mk, a);
-  return check_launch();
+  return launch_chained(kern, dim3((unsigned)blocks), dim3(kThreads), smem, stream, 1, mq, mk, a);
 }
 
 template <int D, bool kColsum, bool kSplit>

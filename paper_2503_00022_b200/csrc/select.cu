@@ -40,6 +40,8 @@ __device__ __forceinline__ unsigned long long importance_key(double v, int t, in
 __global__ void __launch_bounds__(256)
 importance_kernel(Shape s, const float* __restrict__ scores, int keep_initial, int keep_recent,
                   unsigned long long* __restrict__ keys) {
+  chain_wait();
+  chain_trigger();
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (gid >= (long long)s.n_layers * s.T) return;
   const int layer = (int)(gid / s.T), tok = (int)(gid - (long long)layer * s.T);
@@ -75,6 +77,8 @@ importance_kernel(Shape s, const float* __restrict__ scores, int keep_initial, i
 __global__ void __launch_bounds__(256)
 importance_keys_kernel(Shape s, const double* __restrict__ imp, int keep_initial, int keep_recent,
                        unsigned long long* __restrict__ keys) {
+  chain_wait();
+  chain_trigger();
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (gid >= (long long)s.n_layers * s.T) return;
   const int tok = (int)(gid % s.T);
@@ -126,6 +130,8 @@ select_segment_kernel(Shape s, SelectArgs a) {
   __shared__ int bin_base[kMaxBins + 1];
   __shared__ int bit_cnt[128];
   __shared__ uint32_t anchor_sh[4];
+  chain_wait();
+  chain_trigger();
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -417,15 +423,15 @@ select_segment_kernel(Shape s, SelectArgs a) {
 int launch_importance(const Shape& s, const float* scores, int keep_initial, int keep_recent,
                       unsigned long long* keys, cudaStream_t stream) {
   const size_t n = (size_t)s.n_layers * s.T;
-  importance_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(s, scores, keep_initial, keep_recent, keys);
-  return check_launch();
+  return launch_chained(importance_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, stream, 1, s, scores, keep_initial,
+                        keep_recent, keys);
 }
 
 int launch_importance_keys(const Shape& s, const double* importance, int keep_initial, int keep_recent,
                            unsigned long long* keys, cudaStream_t stream) {
   const size_t n = (size_t)s.n_layers * s.T;
-  importance_keys_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(s, importance, keep_initial, keep_recent, keys);
-  return check_launch();
+  return launch_chained(importance_keys_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, stream, 1, s, importance,
+                        keep_initial, keep_recent, keys);
 }
 
 size_t select_workspace_bytes(const Shape& s) {
@@ -469,29 +475,16 @@ int launch_select(const Shape& s, const float* scores, const double* importance,
     if (a.stage_keys) {
       a.imp = importance; a.keep_initial = keep_initial; a.keep_recent = keep_recent;
     } else {
-      importance_keys_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(s, importance, keep_initial, keep_recent, keys);
-      if (check_launch() != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
+      if (launch_importance_keys(s, importance, keep_initial, keep_recent, keys, stream) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
       a.keys = keys;
     }
   }
-  if (dyn > 16 * 1024) {     // static + dynamic shared memory above the 48 KB default needs the opt-in
-    cudaError_t e = cudaSuccess;
-    switch (s.W) {
-      case 1: e = cudaFuncSetAttribute(select_segment_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); break;
-      case 2: e = cudaFuncSetAttribute(select_segment_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); break;
-      case 3: e = cudaFuncSetAttribute(select_segment_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); break;
-      default: e = cudaFuncSetAttribute(select_segment_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); break;
-    }
-    if (e != cudaSuccess) return KVCRUSH_ERR_CUDA;
-  }
-  const unsigned n_seg = (unsigned)(s.n_layers * s.n_seqs);
-  switch (s.W) {
-    case 1: select_segment_kernel<1><<<n_seg, kThreads, dyn, stream>>>(s, a); break;
-    case 2: select_segment_kernel<2><<<n_seg, kThreads, dyn, stream>>>(s, a); break;
-    case 3: select_segment_kernel<3><<<n_seg, kThreads, dyn, stream>>>(s, a); break;
-    default: select_segment_kernel<4><<<n_seg, kThreads, dyn, stream>>>(s, a); break;
-  }
-  return check_launch();
+  auto kern = s.W == 1 ? select_segment_kernel<1> : s.W == 2 ? select_segment_kernel<2>
+            : s.W == 3 ? select_segment_kernel<3> : select_segment_kernel<4>;
+  // static + dynamic shared memory above the 48 KB default needs the opt-in
+  if (dyn > 16 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
+    return KVCRUSH_ERR_CUDA;
+  return launch_chained(kern, dim3((unsigned)(s.n_layers * s.n_seqs)), dim3(kThreads), dyn, stream, 1, s, a);
 }
 
 }  // namespace kvc

@@ -65,6 +65,8 @@ select_pages_kernel(Shape s, PageArgs a) {
   uint32_t* counters = anchor + a.PW;                                                // [n_workers][PW * 16] (u16 pairs)
 
   __shared__ sel::Scratch sc;
+  chain_wait();
+  chain_trigger();
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int seg = blockIdx.x;
@@ -248,8 +250,7 @@ int launch_pages(const Shape& s, PageArgs a, size_t fixed, cudaStream_t stream) 
   if (dyn > 32 * 1024 &&
       cudaFuncSetAttribute(select_pages_kernel<kT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
     return KVCRUSH_ERR_CUDA;
-  select_pages_kernel<kT><<<(unsigned)(s.n_layers * s.n_seqs), kT, dyn, stream>>>(s, a);
-  return check_launch();
+  return launch_chained(select_pages_kernel<kT>, dim3((unsigned)(s.n_layers * s.n_seqs)), dim3(kT), dyn, stream, 1, s, a);
 }
 
 }  // namespace

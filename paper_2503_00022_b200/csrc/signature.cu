@@ -48,6 +48,8 @@ theta_select_kernel(Shape s, const float* __restrict__ scores, const int32_t* __
   __shared__ uint32_t found[3];
   __shared__ int warp_tot[32];
 
+  chain_wait();
+  chain_trigger();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int h = blockIdx.x % s.Hq;
   const int seg = blockIdx.x / s.Hq;              // layer * n_seqs + seq
@@ -142,6 +144,8 @@ theta_warp_kernel(Shape s, const float* __restrict__ scores, const int32_t* __re
   __shared__ alignas(16) uint32_t hist_sh[kRowWarps][kRowBins];
   __shared__ uint32_t small_sh[kRowWarps][sel::kSmallList];
   __shared__ uint32_t small_n_sh[kRowWarps];
+  chain_wait();
+  chain_trigger();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned r = blockIdx.x * kRowWarps + warp;
   if (r >= n_rows) return;
@@ -231,6 +235,8 @@ theta_stream_kernel(Shape s, const float* __restrict__ scores, const int32_t* __
   extern __shared__ uint32_t row_keys[];          // the row's order keys when it fits (stage_row), else unused
   __shared__ uint32_t hist[256];
   __shared__ uint32_t sel_prefix, sel_k;
+  chain_wait();
+  chain_trigger();
 
   const int h = blockIdx.x % s.Hq;
   const int seg = blockIdx.x / s.Hq;              // layer * n_seqs + seq
@@ -332,6 +338,8 @@ signature_pack_kernel(Shape s, const float* __restrict__ scores, const float* __
   extern __shared__ float4 tile4[];                   // [Hq][kPackTok] float
   float* tile = reinterpret_cast<float*>(tile4);
   __shared__ float th_sh[128];
+  chain_wait();
+  chain_trigger();
   const int layer = blockIdx.y;
   const int tok0 = blockIdx.x * kPackTok, tok = tok0 + threadIdx.x;
   const int n_tok = min(kPackTok, s.T - tok0);
@@ -376,12 +384,6 @@ signature_pack_kernel(Shape s, const float* __restrict__ scores, const float* __
   if constexpr (kImportance) importance[(size_t)layer * s.T + tok] = __dadd_rn(total, 0.0);       // -0.0 -> +0.0
 }
 
-template <int kT, int kItems, int kMinB>
-void launch_theta(const Shape& s, const float* scores, const int32_t* sig_keep, float* theta, unsigned blocks,
-                  cudaStream_t stream) {
-  theta_select_kernel<kT, kItems, kMinB><<<blocks, kT, 0, stream>>>(s, scores, sig_keep, theta);
-}
-
 }  // namespace
 
 int launch_signature(const Shape& s, const float* scores, const int32_t* sig_keep, const float* theta_in,
@@ -395,14 +397,21 @@ int launch_signature(const Shape& s, const float* scores, const int32_t* sig_kee
     // more rows than the chip holds as blocks (148 x 8): its chain over 32 keys a lane is longer than the block's
     // (32 rows of 1001 tokens: 8.9 against 7.3 us).
     const unsigned warp_blocks = (blocks + kRowWarps - 1) / kRowWarps;
-    if (m <= 256) theta_warp_kernel<8><<<warp_blocks, kRowWarps * 32, 0, stream>>>(s, scores, sig_keep, theta, blocks);
-    else if (m <= 512) theta_warp_kernel<16><<<warp_blocks, kRowWarps * 32, 0, stream>>>(s, scores, sig_keep, theta, blocks);
-    else if (m <= 1024 && blocks > 1184) theta_warp_kernel<32><<<warp_blocks, kRowWarps * 32, 0, stream>>>(s, scores, sig_keep, theta, blocks);
-    else if (m <= 2048) launch_theta<256, 8, 8>(s, scores, sig_keep, theta, blocks, stream);
-    else if (m <= 4096) launch_theta<512, 8, 4>(s, scores, sig_keep, theta, blocks, stream);
-    else if (m <= 8192) launch_theta<512, 16, 4>(s, scores, sig_keep, theta, blocks, stream);
-    else if (m <= 16384) launch_theta<512, 32, 1>(s, scores, sig_keep, theta, blocks, stream);
-    else if (m <= 32768) launch_theta<1024, 32, 1>(s, scores, sig_keep, theta, blocks, stream);
+    auto by_warp = [&](auto kern) {
+      return launch_chained(kern, dim3(warp_blocks), dim3(kRowWarps * 32), 0, stream, 1, s, scores, sig_keep, theta, blocks);
+    };
+    auto by_block = [&](auto kern, int threads) {
+      return launch_chained(kern, dim3(blocks), dim3(threads), 0, stream, 1, s, scores, sig_keep, theta);
+    };
+    int rc;
+    if (m <= 256) rc = by_warp(theta_warp_kernel<8>);
+    else if (m <= 512) rc = by_warp(theta_warp_kernel<16>);
+    else if (m <= 1024 && blocks > 1184) rc = by_warp(theta_warp_kernel<32>);
+    else if (m <= 2048) rc = by_block(theta_select_kernel<256, 8, 8>, 256);
+    else if (m <= 4096) rc = by_block(theta_select_kernel<512, 8, 4>, 512);
+    else if (m <= 8192) rc = by_block(theta_select_kernel<512, 16, 4>, 512);
+    else if (m <= 16384) rc = by_block(theta_select_kernel<512, 32, 1>, 512);
+    else if (m <= 32768) rc = by_block(theta_select_kernel<1024, 32, 1>, 1024);
     else {
       const size_t row_bytes = (size_t)m * sizeof(uint32_t);
       const int stage_row = row_bytes <= 200 * 1024;
@@ -410,25 +419,19 @@ int launch_signature(const Shape& s, const float* scores, const int32_t* sig_kee
       if (dyn > 40 * 1024 &&
           cudaFuncSetAttribute(theta_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
         return KVCRUSH_ERR_CUDA;
-      theta_stream_kernel<<<blocks, kSelectThreads, dyn, stream>>>(s, scores, sig_keep, theta, stage_row);
+      rc = launch_chained(theta_stream_kernel, dim3(blocks), dim3(kSelectThreads), dyn, stream, 1, s, scores, sig_keep, theta, stage_row);
     }
-    if (check_launch() != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
+    if (rc != KVCRUSH_OK) return rc;
     th = theta;
   }
   const dim3 grid((unsigned)((s.T + kPackTok - 1) / kPackTok), (unsigned)s.n_layers);
   const size_t dyn = (size_t)s.Hq * kPackTok * sizeof(float);
   // 16-byte loads need every (layer, head) row to start on a 16-byte boundary
   const int vec_ok = s.T % 4 == 0 && reinterpret_cast<uintptr_t>(scores) % 16 == 0;
-  if (importance) {
-    if (dyn > 48 * 1024 && cudaFuncSetAttribute(signature_pack_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-      return KVCRUSH_ERR_CUDA;
-    signature_pack_kernel<true><<<grid, kPackTok, dyn, stream>>>(s, scores, th, sigs, importance, vec_ok);
-  } else {
-    if (dyn > 48 * 1024 && cudaFuncSetAttribute(signature_pack_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-      return KVCRUSH_ERR_CUDA;
-    signature_pack_kernel<false><<<grid, kPackTok, dyn, stream>>>(s, scores, th, sigs, nullptr, vec_ok);
-  }
-  return check_launch();
+  auto kern = importance ? signature_pack_kernel<true> : signature_pack_kernel<false>;
+  if (dyn > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
+    return KVCRUSH_ERR_CUDA;
+  return launch_chained(kern, grid, dim3(kPackTok), dyn, stream, 1, s, scores, th, sigs, importance, vec_ok);
 }
 
 // ---------------------------------------------------------------------------------------------------
