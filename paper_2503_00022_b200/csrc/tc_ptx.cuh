@@ -453,10 +453,10 @@ inline EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// 4-D view (channel, token, head, layer) of a token-major bf16 or fp16 tensor; box = 64 channels x 128 tokens.
+// 4-D view (channel, token, head, layer) of a token-major bf16 or fp16 tensor; box = 64 channels x `rows` tokens.
 // A stride only matters along an axis longer than 1; there it must be positive (the TMA unit cannot repeat a row)
 // and inside the tensor map's 40-bit byte range.  Returns false for anything the map cannot describe.
-inline bool make_map(CUtensorMap* map, const TensorView& t, int D, int T, int H, int n_layers) {
+inline bool make_map(CUtensorMap* map, const TensorView& t, int D, int T, int H, int n_layers, int rows = 128) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
   const cuuint64_t gdim[4] = {(cuuint64_t)D, (cuuint64_t)T, (cuuint64_t)H, (cuuint64_t)n_layers};
@@ -470,7 +470,7 @@ inline bool make_map(CUtensorMap* map, const TensorView& t, int D, int T, int H,
       gstride[i] = 16;                                // never used to step: any legal value
     }
   }
-  const cuuint32_t box[4] = {64, 128u, 1, 1};
+  const cuuint32_t box[4] = {64, (cuuint32_t)rows, 1, 1};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   return enc(map, t.dtype == KVCRUSH_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(t.ptr), gdim, gstride, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,

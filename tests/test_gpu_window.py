@@ -70,6 +70,48 @@ def test_windowed_scores_match_oracle(B, w, window):
                 np.testing.assert_allclose(g[l][:, a:b].astype(np.float64).sum(axis=1), float(L - j0), rtol=2e-4)
 
 
+@pytest.mark.parametrize("layers,Hq,Hkv,D,seqlens,window,causal,gain", [
+    (10, 16, 16, 64, (300,), 64, True, 1.0),              # one CTA alone (more units than SMs)
+    (1, 4, 4, 128, (128, 129, 1000, 0, 5, 64), 64, True, 1.0),   # several sequences of very different length per cluster
+    (2, 4, 1, 128, (4100,), 32, True, 1.0),               # clusters of 8, last tile of 4 keys
+    (1, 2, 2, 64, (8192,), 33, True, 1.0),                # every accumulator in use
+    (1, 8, 2, 128, (900, 31), 16, False, 1.0),            # 16 columns, no mask
+    (6, 32, 8, 128, (1500,), 7, True, 1.0),               # units in turn on the same accumulators
+    (1, 4, 4, 128, (700, 200), 48, True, 40.0),           # logits far outside [-100, 100]: kept tiles, exact maxima
+    (1, 2, 2, 64, (600,), 64, False, 12.0),               # some tiles kept, some not
+])
+def test_one_pass_window_scores_match_oracle(B, layers, Hq, Hkv, D, seqlens, window, causal, gain):
+    """Windows of up to 64 queries: scores within the score tolerance of the oracle, row log-sum-exp within 3e-4 (scaled by
+    the gain on the queries, as the logits are)."""
+    import torch
+    dev = _dev()
+    w = inputs.Workload("win1", layers, Hq, Hkv, D, seqlens, inputs.BF16, inputs.BF16, 0.25, base_seed=290 + D, causal=causal)
+    lis, q, k, _, _ = TL.stack_layers(w, range(layers), with_cache=False)
+    dq = (TL.torch_storage(q, w.qk_dtype, dev).float() * gain).to(torch.bfloat16)
+    dk = TL.torch_storage(k, w.qk_dtype, dev)
+    hq = dq.cpu().view(torch.int16).numpy().view(np.uint16)
+    prob = B.Problem(layers, Hq, Hkv, D, seqlens, causal=causal, device=dev, query_window=window)
+    ws = torch.empty(B.kvcrush_workspace_size(prob, B.STAGE_SCORE), dtype=torch.uint8, device=dev)
+    status = torch.zeros(4, dtype=torch.int32, device=dev)
+    scores = torch.full((layers, Hq, w.total_tokens), -1.0, dtype=torch.float32, device=dev)
+    lse = torch.full_like(scores, 7.0)
+    for _ in range(2):
+        B.kvcrush_score(prob, dq, dk, scores, lse_out=lse, workspace=ws, status=status)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist()[0] == 0
+    g, gl, cu, G = scores.cpu().numpy(), lse.cpu().numpy(), w.cu_seqlens, Hq // Hkv
+    for l in sorted({0, layers - 1}):
+        for s, L in enumerate(seqlens):
+            a, b = int(cu[s]), int(cu[s + 1])
+            if L == 0:
+                continue
+            j0 = max(0, L - window)
+            c, ol = O.scores(inputs.widen(hq[l, a:b], w.qk_dtype), inputs.widen(lis[l].k[a:b], w.qk_dtype), causal, rows=(j0, L))
+            assert TL.within_score_tolerance(g[l][:, a:b], c).all(), (l, s)
+            np.testing.assert_allclose(gl[l][:, a + j0:b], ol[:, j0:], rtol=0, atol=3e-4 * gain)
+            assert (gl[l][:, a:a + j0] == 7.0).all()
+
+
 @pytest.mark.parametrize("kernel", [1, 3, 7, 33])
 def test_pooling_is_bit_exact(B, kernel):
     import torch
