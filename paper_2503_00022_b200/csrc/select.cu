@@ -16,6 +16,9 @@
 //                               minimising  sum_{h: bit set} (m - 2 n_h)  (= L1 distance to the
 //                               per-bit mean, up to a constant), ties to the lower token
 //                            5. kept = important U representatives, ascending token index
+// A chain of short block-wide steps in one CTA per segment, bound by their latencies (8192 tokens, thousand cycles: staging
+// 4.7, top-k 6.8, sort 7.7, buckets 13 to 21, output 2.9; device time 20.5 -> 18.4 us for 32 such segments, 10.1 -> 8.5 us
+// for one of 1001 tokens); from about 13000 tokens on by instructions and L2 reads (32 segments of 32768 tokens 117 -> 69 us).
 // All decisions are integer or exact float64 comparisons, so the result is unique.
 #include "select_common.cuh"
 
@@ -87,15 +90,15 @@ importance_keys_kernel(Shape s, const double* __restrict__ imp, int keep_initial
   keys[gid] = importance_key(imp[gid], tok - t0, __ldg(s.cu_seqlens + seq + 1) - t0, keep_initial, keep_recent);
 }
 
-// sum over the GW lanes of this lane's group of popc(mine & theirs); lanes without a member hold zeros
+// sum over the GW lanes of the group that starts at lane g0: popc(mine & theirs); lanes without a member hold zeros
 template <int W, int GW>
-__device__ __forceinline__ int group_and_popc(const uint32_t (&mine)[4]) {
-  int shared = 0;
+__device__ __forceinline__ int group_and_popc(const uint32_t (&mine)[4], int g0) {
+  int common = 0;
 #pragma unroll
   for (int u = 0; u < GW; ++u)
 #pragma unroll
-    for (int w = 0; w < W; ++w) shared += __popc(mine[w] & __shfl_sync(kFull, mine[w], u, GW));
-  return shared;
+    for (int w = 0; w < W; ++w) common += __popc(mine[w] & __shfl_sync(kFull, mine[w], g0 + u));
+  return common;
 }
 
 struct SelectArgs {
@@ -112,21 +115,27 @@ struct SelectArgs {
   int32_t* idx;
   uint8_t* kind;
   int32_t* n_kept;                    // optional [n_layers][n_seqs]: tokens kept per segment
-  int32_t* sorted;                    // [n_layers][T] scratch: grouped tokens in (d, t) order
+  int32_t* sorted;                    // [n_layers][T] scratch: grouped tokens in (d, t) order (segments not staged)
   int mask_words;                     // words of one membership mask in shared memory
   int stage_words;                    // max_seqlen rounded up to a multiple of 4 (one staged int32 per token)
-  int stage_sorted, stage_sig, stage_keys;   // which per-segment arrays are copied into shared memory
+  int stage_sig, stage_sorted;        // kLong: which of the two live in shared memory (sorted: as 16-bit indices)
 };
 
-template <int W>                       // signature words per token (compile time: the per-word loops unroll)
+// W: signature words per token (compile time: the per-word loops unroll).
+// kLong: segments whose keys, signatures and sorted order do not all fit in shared memory.  Of those the signatures come
+// first, which the bucket step gathers one by one, then the sorted order as 16-bit indices; the keys' upper halves are
+// copied into the signatures' place while the top k are looked for.
+template <int W, bool kLong>
 __global__ void __launch_bounds__(kThreads, 1)
 select_segment_kernel(Shape s, SelectArgs a) {
-  extern __shared__ uint32_t dyn_smem[];
+  extern __shared__ __align__(16) uint32_t dyn_smem[];
   uint32_t* imp_mask = dyn_smem;
   uint32_t* rep_mask = dyn_smem + a.mask_words;
 
-  __shared__ sel::Scratch sc;
-  __shared__ int warp_hist[kWarps][kMaxBins];
+  // the scratch of the top-k step and the per-warp histograms of the sort are not in use at the same time
+  __shared__ union { sel::Scratch sc; int warp_hist[kWarps][kMaxBins]; } shared;
+  sel::Scratch& sc = shared.sc;
+  int (&warp_hist)[kWarps][kMaxBins] = shared.warp_hist;
   __shared__ int bin_base[kMaxBins + 1];
   __shared__ int bit_cnt[128];
   __shared__ uint32_t anchor_sh[4];
@@ -153,32 +162,33 @@ select_segment_kernel(Shape s, SelectArgs a) {
     return;
   }
 
-  // The segment's arrays are read many times with dependent addresses (8 radix sweeps, two counting-sort
-  // sweeps, one gather per bucket), so whatever fits is first copied into shared memory; the rest is read
-  // through L2.  The pointers below are generic and point to either place.
+  // The segment's arrays are read many times with dependent addresses (radix sweeps, counting-sort sweeps, one gather
+  // per bucket), so whatever fits is first copied into shared memory; the rest is read through L2.  The pointers below
+  // are generic and point to either place.
   const unsigned long long* keys = a.keys ? a.keys + (size_t)layer * s.T + t0 : nullptr;
   const uint32_t* sig = a.sigs + ((size_t)layer * s.T + t0) * W;
-  int32_t* sorted = a.sorted + (size_t)layer * s.T + t0;
-  uint32_t* sort_code = nullptr;         // per token: distance | position among the warp's tokens of that distance << 8
-  {
-    uint32_t* arena = dyn_smem + 2 * a.mask_words;
-    if (a.stage_sorted) { sorted = reinterpret_cast<int32_t*>(arena); arena += a.stage_words; }
-    if (a.stage_sig) {
-      _Pragma("unroll 8") for (int i = tid; i < L * W; i += kThreads) arena[i] = __ldg(sig + i);
-      sig = arena;
-      arena += a.stage_words * W;
+  uint32_t* arena = dyn_smem + 2 * a.mask_words;
+  uint32_t* sig_sh = kLong && !a.stage_sig ? nullptr : arena;
+  if (sig_sh) arena += a.stage_words * W;
+  int32_t* sorted = kLong ? a.sorted + (size_t)layer * s.T + t0 : reinterpret_cast<int32_t*>(arena);
+  uint16_t* sorted16 = kLong && a.stage_sorted ? reinterpret_cast<uint16_t*>(arena) : nullptr;
+  arena += a.stage_words;
+  uint32_t* sort_code = arena;           // !kLong, per token: distance | position among the warp's tokens of that distance << 8
+  auto sorted_at = [&](int i) { return kLong && sorted16 ? (int)sorted16[i] : sorted[i]; };
+  auto stage_sig = [&]() {
+    _Pragma("unroll 8") for (int i = tid; i < L * W; i += kThreads) sig_sh[i] = __ldg(sig + i);
+    sig = sig_sh;
+  };
+  if (!kLong) {
+    stage_sig();
+    unsigned long long* ks = reinterpret_cast<unsigned long long*>(arena);        // dead once the important set is marked
+    if (a.keys) {
+      _Pragma("unroll 8") for (int i = tid; i < L; i += kThreads) ks[i] = keys[i];
+    } else {
+      const double* imp = a.imp + (size_t)layer * s.T + t0;
+      _Pragma("unroll 8") for (int i = tid; i < L; i += kThreads) ks[i] = importance_key(__ldg(imp + i), i, L, a.keep_initial, a.keep_recent);
     }
-    if (a.stage_keys) {
-      unsigned long long* ks = reinterpret_cast<unsigned long long*>(arena);
-      sort_code = reinterpret_cast<uint32_t*>(arena);      // the keys are dead once the important set is marked
-      if (a.keys) {
-        _Pragma("unroll 8") for (int i = tid; i < L; i += kThreads) ks[i] = keys[i];
-      } else {
-        const double* imp = a.imp + (size_t)layer * s.T + t0;
-        _Pragma("unroll 8") for (int i = tid; i < L; i += kThreads) ks[i] = importance_key(__ldg(imp + i), i, L, a.keep_initial, a.keep_recent);
-      }
-      keys = ks;
-    }
+    keys = ks;
   }
   const int n_words = (L + 31) >> 5;
   int r_lo, r_hi;                            // contiguous token range of this warp
@@ -188,11 +198,12 @@ select_segment_kernel(Shape s, SelectArgs a) {
   __syncthreads();
 
   // ---- 1. important tokens: the b_imp largest keys, ties to the lower index --------------------
-  if (b_imp > 0) sel::mark_top_keys<kThreads>(keys, L, b_imp, imp_mask, sc);
+  if (b_imp > 0) sel::mark_top_keys<kThreads>(keys, L, b_imp, imp_mask, sc, kLong ? sig_sh : nullptr);
 
   // ---- 2-4. representatives of the other tokens ------------------------------------------------
   if (b_rep > 0) {
     const int N = L - b_imp;
+    if (kLong && sig_sh) { stage_sig(); __syncthreads(); }
     // anchor
     if (a.anchor_mode == KVCRUSH_ANCHOR_MEAN) {
       for (int i = tid; i < 128; i += kThreads) bit_cnt[i] = 0;
@@ -234,19 +245,23 @@ select_segment_kernel(Shape s, SelectArgs a) {
 
     // counting sort by (d, t): per-warp histograms over contiguous token ranges.  When there is room, the first
     // sweep also notes every token's distance and its position among the warp's tokens of that distance, so that
-    // the second sweep is a plain scatter.
+    // the second sweep is a plain scatter; otherwise the first sweep only counts.
     for (int base = r_lo; base < r_hi; base += 32) {
       const int i = base + lane;
       const bool cand = i < r_hi && !((imp_mask[base >> 5] >> lane) & 1u);
       int d = 0;
       if (cand)
         _Pragma("unroll") for (int w = 0; w < W; ++w) d += __popc((sig[(size_t)i * W + w] ^ anc[w]) & hm[w]);
+      if (kLong) {
+        if (cand) atomicAdd(&warp_hist[warp][d], 1);
+        continue;
+      }
       const unsigned voters = __ballot_sync(kFull, cand);
       unsigned peers = 0;
       if (cand) {
         peers = __match_any_sync(voters, d);
-        if (sort_code) sort_code[i] = (uint32_t)d | ((uint32_t)(warp_hist[warp][d] + __popc(peers & lt_mask)) << 8);
-      } else if (sort_code && i < r_hi) {
+        sort_code[i] = (uint32_t)d | ((uint32_t)(warp_hist[warp][d] + __popc(peers & lt_mask)) << 8);
+      } else if (i < r_hi) {
         sort_code[i] = 0xFFFFFFFFu;
       }
       __syncwarp();
@@ -265,7 +280,7 @@ select_segment_kernel(Shape s, SelectArgs a) {
       for (int b = 1; b <= n_bins; ++b) bin_base[b] += bin_base[b - 1];
     }
     __syncthreads();
-    if (sort_code) {
+    if (!kLong) {
       for (int i = r_lo + lane; i < r_hi; i += 32) {
         const uint32_t c = sort_code[i];
         if (c != 0xFFFFFFFFu) {
@@ -284,7 +299,8 @@ select_segment_kernel(Shape s, SelectArgs a) {
         unsigned peers = 0;
         if (cand) {
           peers = __match_any_sync(voters, d);
-          sorted[bin_base[d] + warp_hist[warp][d] + __popc(peers & lt_mask)] = i;
+          const int pos = bin_base[d] + warp_hist[warp][d] + __popc(peers & lt_mask);
+          if (sorted16) sorted16[pos] = (uint16_t)i; else sorted[pos] = i;
         }
         __syncwarp();
         if (cand && (peers & lt_mask) == 0) warp_hist[warp][d] += __popc(peers);
@@ -298,15 +314,16 @@ select_segment_kernel(Shape s, SelectArgs a) {
     const int q_nr = N / b_rep, r_nr = N - q_nr * b_rep;
     const int m_max = q_nr + (r_nr > 0 ? 1 : 0);                               // largest bucket
     if (m_max <= 16) {
-      // Small buckets (the usual case: N/R is the compression ratio): 32 / gw buckets share a warp, gw = the power
-      // of two that holds a bucket, one lane per member.  sum_{h set in t} n_h = sum over members u of
-      // popc(sig_t & sig_u), so cost(t) = m * popc(sig_t) - 2 * sum_u popc(sig_t & sig_u): gw shuffles inside
-      // the lane group.  |cost| <= 16 * 128 and t < 2^18, so (cost, t) packs into 31 bits and one warp-level
-      // minimum per lane group picks the representative, ties to the lower token.
-      int gw = 2;
-      while (gw < m_max) gw <<= 1;
-      const int per_warp = 32 / gw, sub = lane / gw, j = lane - sub * gw;
-      const unsigned gmask = (0xFFFFFFFFu >> (32 - gw)) << (sub * gw);
+      // Small buckets (the usual case: N/R is the compression ratio): 32 / gw buckets share a warp, one lane per member.
+      // sum_{h set in t} n_h = sum over members u of popc(sig_t & sig_u), so
+      // cost(t) = m * popc(sig_t) - 2 * sum_u popc(sig_t & sig_u): gw shuffles inside the lane group.
+      // |cost| <= 16 * 128 and t < 2^18, so (cost, t) packs into 31 bits and one warp-level minimum per lane group
+      // picks the representative, ties to the lower token.  The step is bound by its shuffles and bit counts, so the group
+      // width follows the bucket closer than the next power of two in long segments (32768 tokens, 3277 buckets of 9: 74
+      // thousand cycles with 16 lanes, 57 with 10; in short ones the wider choice of code costs more than it gives).
+      const int gw = m_max <= 2 ? 2 : m_max <= 4 ? 4 : kLong && m_max <= 6 ? 6 : m_max <= 8 ? 8 : kLong && m_max <= 10 ? 10 : 16;
+      const int per_warp = 32 / gw, sub = lane / gw, j = lane - sub * gw, g0 = sub * gw;   // sub == per_warp: lanes left over
+      const unsigned gmask = sub < per_warp ? (0xFFFFFFFFu >> (32 - gw)) << g0 : 0xFFFFFFFFu << g0;
       // bucket b starts at b*q_nr + frac with b*r_nr = frac*R + rem.  Divisions are slow, so each lane divides once
       // for its first bucket and then steps exactly by the warp's stride of kWarps*per_warp buckets.
       const int first_bkt = warp * per_warp + sub, stride_b = kWarps * per_warp;
@@ -315,22 +332,27 @@ select_segment_kernel(Shape s, SelectArgs a) {
       int frac = (int)(p0 / (unsigned)b_rep), rem = (int)(p0 - (unsigned long long)frac * (unsigned)b_rep);
       const int step_q = (int)(ps / (unsigned)b_rep), step_r = (int)(ps - (unsigned long long)step_q * (unsigned)b_rep);
       for (int bkt = first_bkt; bkt - sub < b_rep; bkt += stride_b) {
-        const bool live = bkt < b_rep;
+        const bool live = sub < per_warp && bkt < b_rep;
         const int lo = live ? bkt * q_nr + frac : 0;
         const int m = live ? q_nr + (rem + r_nr >= b_rep ? 1 : 0) : 0;       // the next bucket's frac is one larger
         frac += step_q;
         rem += step_r;
         if (rem >= b_rep) { rem -= b_rep; ++frac; }
         const bool member = j < m;
-        const int t = member ? sorted[lo + j] : 0;
+        const int t = member ? sorted_at(lo + j) : 0;
         uint32_t mine[4] = {0u, 0u, 0u, 0u};
         _Pragma("unroll") for (int w = 0; w < W; ++w) mine[w] = member ? sig[(size_t)t * W + w] & head_mask(s.Hq, w) : 0u;
         int ones = 0;
         _Pragma("unroll") for (int w = 0; w < W; ++w) ones += __popc(mine[w]);
         // lanes past a bucket's last member hold zeros and add nothing
-        const int shared = gw == 8 ? group_and_popc<W, 8>(mine) : gw == 4 ? group_and_popc<W, 4>(mine)
-                         : gw == 16 ? group_and_popc<W, 16>(mine) : group_and_popc<W, 2>(mine);
-        const int cost = m * ones - 2 * shared;
+        int common;
+        if (gw == 8) common = group_and_popc<W, 8>(mine, g0);
+        else if (gw == 4) common = group_and_popc<W, 4>(mine, g0);
+        else if (gw == 2) common = group_and_popc<W, 2>(mine, g0);
+        else if (kLong && gw == 6) common = group_and_popc<W, 6>(mine, g0);
+        else if (kLong && gw == 10) common = group_and_popc<W, 10>(mine, g0);
+        else common = group_and_popc<W, 16>(mine, g0);
+        const int cost = m * ones - 2 * common;
         const uint32_t key = member ? ((uint32_t)(cost + 4096) << 18) | (uint32_t)t : 0xFFFFFFFFu;
         const uint32_t best = __reduce_min_sync(gmask, key);
         if (j == 0 && live) {
@@ -357,7 +379,7 @@ select_segment_kernel(Shape s, SelectArgs a) {
         // one lane per member.  sum_{h set in t} n_h = sum over members u of popc(sig_t & sig_u), so
         // cost(t) = m * popc(sig_t) - 2 * sum_u popc(sig_t & sig_u): m shuffles instead of one ballot per head
         const bool member = lane < m;
-        const int t = member ? sorted[lo + lane] : 0;
+        const int t = member ? sorted_at(lo + lane) : 0;
         uint32_t mine[4] = {0u, 0u, 0u, 0u};
         _Pragma("unroll") for (int w = 0; w < W; ++w) mine[w] = member ? sig[(size_t)t * W + w] & head_mask(s.Hq, w) : 0u;
         int ones = 0, shared = 0;
@@ -372,7 +394,7 @@ select_segment_kernel(Shape s, SelectArgs a) {
         int n_ones[4] = {0, 0, 0, 0};        // lane b of word w holds n_h for head 32w+b
         for (int c0 = lo; c0 < hi; c0 += 32) {
           const bool member = c0 + lane < hi;
-          const int t = member ? sorted[c0 + lane] : 0;
+          const int t = member ? sorted_at(c0 + lane) : 0;
           _Pragma("unroll") for (int w = 0; w < W; ++w) {
             const uint32_t word = member ? sig[(size_t)t * W + w] : 0u;
             const int nb = min(32, s.Hq - 32 * w);
@@ -384,7 +406,7 @@ select_segment_kernel(Shape s, SelectArgs a) {
         }
         for (int c0 = lo; c0 < hi; c0 += 32) {
           const bool member = c0 + lane < hi;
-          const int t = member ? sorted[c0 + lane] : 0;
+          const int t = member ? sorted_at(c0 + lane) : 0;
           int cost = 0;
           _Pragma("unroll") for (int w = 0; w < W; ++w) {
             const uint32_t word = member ? sig[(size_t)t * W + w] : 0u;
@@ -460,11 +482,15 @@ int launch_select(const Shape& s, const float* scores, const double* importance,
   a.mask_words = ((s.max_seqlen + 31) / 32 + 3) & ~3;
   a.stage_words = (s.max_seqlen + 3) & ~3;
   size_t dyn = (size_t)a.mask_words * 2 * sizeof(uint32_t);
-  const size_t budget = 196 * 1024;     // dynamic shared memory this kernel may take (static part: ~27 KB)
+  const size_t budget = 208 * 1024;     // dynamic shared memory this kernel may take (static part: ~18 KB)
   const size_t per_tok = (size_t)a.stage_words * sizeof(uint32_t);
-  if (dyn + per_tok <= budget) { a.stage_sorted = 1; dyn += per_tok; }
-  if (dyn + per_tok * s.W <= budget) { a.stage_sig = 1; dyn += per_tok * s.W; }
-  if (dyn + 2 * per_tok <= budget) { a.stage_keys = 1; dyn += 2 * per_tok; }
+  const bool long_seg = dyn + per_tok * (s.W + 3) > budget;
+  if (!long_seg) {
+    dyn += per_tok * (s.W + 3);
+  } else {
+    if (dyn + per_tok * s.W <= budget) { a.stage_sig = 1; dyn += per_tok * s.W; }
+    if (s.max_seqlen <= 65536 && dyn + per_tok / 2 <= budget) { a.stage_sorted = 1; dyn += per_tok / 2; }
+  }
   // importance keys: computed here from the scores, or taken from the caller's I(t) - converted while the segment
   // kernel stages them, or by a small kernel when the segments are too long to be staged
   if (!importance) {
@@ -472,17 +498,19 @@ int launch_select(const Shape& s, const float* scores, const double* importance,
     a.keys = keys;
   }
   if (importance) {
-    if (a.stage_keys) {
+    if (!long_seg) {
       a.imp = importance; a.keep_initial = keep_initial; a.keep_recent = keep_recent;
     } else {
       if (launch_importance_keys(s, importance, keep_initial, keep_recent, keys, stream) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
       a.keys = keys;
     }
   }
-  auto kern = s.W == 1 ? select_segment_kernel<1> : s.W == 2 ? select_segment_kernel<2>
-            : s.W == 3 ? select_segment_kernel<3> : select_segment_kernel<4>;
+  auto kern = s.W == 1 ? (long_seg ? select_segment_kernel<1, true> : select_segment_kernel<1, false>)
+            : s.W == 2 ? (long_seg ? select_segment_kernel<2, true> : select_segment_kernel<2, false>)
+            : s.W == 3 ? (long_seg ? select_segment_kernel<3, true> : select_segment_kernel<3, false>)
+                       : (long_seg ? select_segment_kernel<4, true> : select_segment_kernel<4, false>);
   // static + dynamic shared memory above the 48 KB default needs the opt-in
-  if (dyn > 16 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
+  if (dyn > 28 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
     return KVCRUSH_ERR_CUDA;
   return launch_chained(kern, dim3((unsigned)(s.n_layers * s.n_seqs)), dim3(kThreads), dyn, stream, 1, s, a);
 }

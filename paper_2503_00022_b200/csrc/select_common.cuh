@@ -12,13 +12,14 @@ constexpr int kMaxWarps = 32;                  // the helpers below take the blo
 constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kDigitBits = 11;                 // radix digit of the 64-bit selection
 constexpr int kBins = 1 << kDigitBits;
-constexpr int kSmallList = 32;                 // candidates one warp ranks directly
+constexpr int kSmallList = 32;                 // 32-bit candidates one warp ranks directly
+constexpr int kRankList = 256;                 // 64-bit candidates a block ranks directly, at most
 
 struct Scratch {
   alignas(16) uint32_t hist[kBins];
-  unsigned long long red[2][kMaxWarps];          // per-warp minimum / maximum
-  unsigned long long small[kSmallList];
-  unsigned long long sel_x;                    // result of a search step
+  unsigned long long red[kMaxWarps];           // per-warp maximum and minimum of the keys' upper halves
+  unsigned long long small[kRankList];
+  unsigned long long sel_x;                    // result of a ranking
   uint32_t sel[3];                             // digit, remaining rank, live keys
   uint32_t small_n;
   int warp_tot[kMaxWarps];
@@ -90,26 +91,30 @@ __device__ __forceinline__ void find_digit_desc(const uint32_t* hist, int n_bins
   __syncthreads();
 }
 
-// One warp ranks at most 32 candidates held one per lane (lanes >= n hold nothing): returns in every lane the
-// k_rem-th largest value, sets k_out to the rank left among the candidates equal to it and n_equal to their number.
-__device__ __forceinline__ unsigned long long warp_rank_select(unsigned long long v, int n, uint32_t k_rem, int lane,
-                                                               uint32_t& k_out, uint32_t& n_equal) {
-  uint32_t gt = 0, ge = 0;
-  for (int j = 0; j < n; ++j) {
-    const unsigned long long o = __shfl_sync(kFull, v, j);
-    gt += o > v;
-    ge += o >= v;
+// The block ranks the n <= min(kT, kRankList) candidates in sc.small, a thread each: returns the k_rem-th largest value,
+// sets k_out to the rank left among the candidates equal to it and n_equal to their number.  A barrier lies between the
+// list's last update and this call.
+template <int kT>
+__device__ __forceinline__ unsigned long long rank_select(Scratch& sc, int n, uint32_t k_rem, uint32_t& k_out, uint32_t& n_equal) {
+  if ((int)threadIdx.x < n) {
+    const unsigned long long v = sc.small[threadIdx.x];
+    uint32_t gt = 0, ge = 0;
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+      const unsigned long long o = sc.small[j];
+      gt += o > v;
+      ge += o >= v;
+    }
+    if (gt < k_rem && k_rem <= ge) { sc.sel_x = v; sc.sel[1] = k_rem - gt; sc.sel[2] = ge - gt; }   // equal candidates agree
   }
-  const bool hit = lane < n && gt < k_rem && k_rem <= ge;
-  const unsigned who = __ballot_sync(kFull, hit);
-  const int src = __ffs(who) - 1;                     // equal candidates all qualify: any of them
-  const uint32_t gt_src = __shfl_sync(kFull, gt, src);
-  k_out = k_rem - gt_src;
-  n_equal = __shfl_sync(kFull, ge, src) - gt_src;
-  return __shfl_sync(kFull, v, src);
+  __syncthreads();
+  k_out = sc.sel[1];
+  n_equal = sc.sel[2];
+  return sc.sel_x;
 }
 
-// The same for 32-bit candidates (one shuffle per candidate instead of two).
+// One warp ranks at most 32 candidates held one per lane (lanes >= n hold nothing): returns the k_rem-th largest value in
+// every lane.
 __device__ __forceinline__ uint32_t warp_rank_select32(uint32_t v, int n, uint32_t k_rem, int lane) {
   uint32_t gt = 0, ge = 0;
   for (int j = 0; j < n; ++j) {
@@ -122,15 +127,35 @@ __device__ __forceinline__ uint32_t warp_rank_select32(uint32_t v, int n, uint32
   return __shfl_sync(kFull, v, __ffs(who) - 1);
 }
 
+// Calls f(item, index) for items tid, tid + kT, .. of [0, n).  Items outside shared memory come eight loads at a time: they
+// are read through L2, and f's atomics would hold every load back until the one before is used.
+template <int kT, class Load, class F>
+__device__ __forceinline__ void for_items(bool far, int n, Load&& load, F&& f) {
+  if (!far) {
+    for (int i = threadIdx.x; i < n; i += kT) f(load(i), i);
+    return;
+  }
+  for (int i0 = threadIdx.x; i0 < n; i0 += 8 * kT) {
+    decltype(load(0)) v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = load(min(i0 + j * kT, n - 1));
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (i0 + j * kT < n) f(v[j], i0 + j * kT);
+  }
+}
+
 // Sets bit i of imp_mask for the k items with the largest keys[0..n); equal keys are admitted in ascending
-// index order.  Exact: the k-th largest key is found by radix histograms over (key - smallest key), starting at
-// the top bit in which the keys of this segment differ at all - the digits are then spread over the bins whatever
-// the keys' common magnitude -, and as soon as at most 32 candidates are left one warp ranks them directly; then
-// one ordered pass marks the members.  Called by all threads of the block; imp_mask must be zero on entry;
-// 0 < k < n.
+// index order.  Exact.  The first round is a histogram of the keys' upper halves alone (32-bit arithmetic, warp-level
+// minimum and maximum), over (upper half - smallest upper half) from the top bit in which they differ at all, so that the
+// bins are spread whatever the keys' common magnitude; usually at most 256 keys are left in the bin of the k-th largest
+// and are ranked directly (24 of them by one warp with 64-bit shuffles took 3 of the step's 10 thousand cycles).  Otherwise radix rounds over the whole keys follow; then one ordered pass marks the
+// members.  Called by all threads of the block; imp_mask must be zero on entry; 0 < k < n.
+// copy: optional shared memory for n words; keys that are not in shared memory are then read whole only where it matters
+// (the sweeps over 32768 keys took 9 thousand cycles each through L2).
 template <int kT>
 __device__ __forceinline__ void mark_top_keys(const unsigned long long* keys, int n, int k, uint32_t* imp_mask,
-                                              Scratch& sc) {
+                                              Scratch& sc, uint32_t* copy = nullptr) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
   if (n <= 32) {                                       // one warp ranks every item: larger keys first, then lower index
@@ -149,85 +174,105 @@ __device__ __forceinline__ void mark_top_keys(const unsigned long long* keys, in
   }
   int r_lo, r_hi;
   warp_range<kT>(n, warp, r_lo, r_hi);
+  const bool far = !__isShared(keys), far_upper = far && !copy;
+  const auto upper_word = [&](int i) { return reinterpret_cast<const uint32_t*>(keys)[2 * i + 1]; };
+  const auto upper = [&](int i) { return copy ? copy[i] : upper_word(i); };
+  const auto whole = [&](int i) { return keys[i]; };
 
-  // smallest and largest key
-  unsigned long long lo = ~0ull, hi = 0ull;
-  for (int i = tid; i < n; i += kT) {
-    const unsigned long long key = keys[i];
-    lo = key < lo ? key : lo;
-    hi = key > hi ? key : hi;
-  }
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    const unsigned long long a = __shfl_xor_sync(kFull, lo, d), b = __shfl_xor_sync(kFull, hi, d);
-    lo = a < lo ? a : lo;
-    hi = b > hi ? b : hi;
-  }
-  if (lane == 0) { sc.red[0][warp] = lo; sc.red[1][warp] = hi; }
+  // smallest and largest upper half
+  uint32_t lo32 = 0xFFFFFFFFu, hi32 = 0u;
+  for_items<kT>(far, n, upper_word, [&](uint32_t x, int i) {
+    lo32 = min(lo32, x);
+    hi32 = max(hi32, x);
+    if (copy) copy[i] = x;
+  });
+  lo32 = __reduce_min_sync(kFull, lo32);
+  hi32 = __reduce_max_sync(kFull, hi32);
+  if (lane == 0) sc.red[warp] = (unsigned long long)hi32 << 32 | lo32;
+  for (int i = tid; i < kBins; i += kT) sc.hist[i] = 0;
+  if (tid == 0) sc.small_n = 0;
   __syncthreads();
-  lo = lane < kT / 32 ? sc.red[0][lane] : ~0ull;
-  hi = lane < kT / 32 ? sc.red[1][lane] : 0ull;
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    const unsigned long long a = __shfl_xor_sync(kFull, lo, d), b = __shfl_xor_sync(kFull, hi, d);
-    lo = a < lo ? a : lo;
-    hi = b > hi ? b : hi;
+  {
+    const unsigned long long v = sc.red[lane < kT / 32 ? lane : 0];
+    lo32 = __reduce_min_sync(kFull, (uint32_t)v);
+    hi32 = __reduce_max_sync(kFull, (uint32_t)(v >> 32));
   }
-  const unsigned long long base = lo, range = hi - lo;
+  const int bits = hi32 > lo32 ? 32 - __clz(hi32 - lo32) : 1, shift32 = bits > kDigitBits ? bits - kDigitBits : 0;
+  for_items<kT>(far_upper, n, upper, [&](uint32_t x, int) { atomicAdd(&sc.hist[(x - lo32) >> shift32], 1u); });
+  __syncthreads();
+  find_digit_desc<kT>(sc.hist, kBins, (uint32_t)k, sc.warp_tot, sc.sel);
+  const uint32_t digit = sc.sel[0], k_in_bin = sc.sel[1], live0 = sc.sel[2];
 
-  // x = key - base has `rem` significant bits; `top` is the value of the bits of x above them chosen so far
-  int rem = range ? 64 - __clzll((long long)range) : 0;
-  unsigned long long top = 0;
-  uint32_t k_rem = (uint32_t)k;
-  uint32_t n_equal = (uint32_t)n;                      // keys equal to the k-th largest (all of them when range == 0)
-  bool first = true;
-  while (rem > 0) {
-    const int w = rem < kDigitBits ? rem : kDigitBits, shift = rem - w, n_bins = 1 << w;
-    for (int i = tid; i < n_bins; i += kT) sc.hist[i] = 0;
-    if (tid == 0) sc.small_n = 0;
+  unsigned long long kth;                              // the k-th largest key ..
+  uint32_t k_rem, n_equal;                             // .. and how many of the n_equal keys equal to it are admitted
+  constexpr uint32_t kDirect = kT < kRankList ? kT : kRankList;
+  if (live0 <= kDirect) {
+    for_items<kT>(far_upper, n, upper, [&](uint32_t x, int i) {
+      if ((x - lo32) >> shift32 == digit) sc.small[atomicAdd(&sc.small_n, 1u)] = keys[i];
+    });
     __syncthreads();
-    if (first) {                                       // every key counts and has no bits above the digit
-      for (int i = tid; i < n; i += kT) atomicAdd(&sc.hist[(uint32_t)((keys[i] - base) >> shift)], 1u);
-    } else {
-      for (int i = tid; i < n; i += kT) {
-        const unsigned long long x = keys[i] - base;
-        if (((x >> 1) >> (rem - 1)) == top) atomicAdd(&sc.hist[(uint32_t)(x >> shift) & (uint32_t)(n_bins - 1)], 1u);
-      }
-    }
-    first = false;
-    __syncthreads();
-    find_digit_desc<kT>(sc.hist, n_bins, k_rem, sc.warp_tot, sc.sel);
-    top = (top << w) | sc.sel[0];
-    k_rem = sc.sel[1];
-    const uint32_t live = sc.sel[2];
-    n_equal = live;                                    // exact once no bits are left
-    rem = shift;
-    if (rem > 0 && live <= (uint32_t)kSmallList) {     // few candidates: one warp ranks their remaining bits
-      for (int i = tid; i < n; i += kT) {
-        const unsigned long long x = keys[i] - base;
-        if ((x >> rem) == top) sc.small[atomicAdd(&sc.small_n, 1u)] = x;
-      }
+    kth = rank_select<kT>(sc, (int)live0, k_in_bin, k_rem, n_equal);
+  } else {
+    // radix rounds over x = key - base, base = the smallest upper half with zeros below: x has `rem` significant bits;
+    // `top` is the value of the bits of x above them chosen so far.  The first digit is known.
+    const unsigned long long base = (unsigned long long)lo32 << 32;
+    int rem = 32 + shift32;
+    unsigned long long top = digit;
+    k_rem = k_in_bin;
+    n_equal = live0;
+    while (rem > 0) {
+      const int w = rem < kDigitBits ? rem : kDigitBits, shift = rem - w, n_bins = 1 << w;
+      __syncthreads();                                 // sc.sel and sc.hist are rewritten
+      for (int i = tid; i < n_bins; i += kT) sc.hist[i] = 0;
+      if (tid == 0) sc.small_n = 0;
       __syncthreads();
-      if (warp == 0) {
-        uint32_t k_out, n_eq_out;
-        const unsigned long long v = warp_rank_select(lane < (int)live ? sc.small[lane] : 0ull, (int)live, k_rem, lane, k_out, n_eq_out);
-        if (lane == 0) { sc.sel_x = v; sc.sel[1] = k_out; sc.sel[2] = n_eq_out; }
-      }
+      for_items<kT>(far, n, whole, [&](unsigned long long key, int) {
+        const unsigned long long x = key - base;
+        if ((x >> rem) == top) atomicAdd(&sc.hist[(uint32_t)(x >> shift) & (uint32_t)(n_bins - 1)], 1u);
+      });
       __syncthreads();
-      top = sc.sel_x;
+      find_digit_desc<kT>(sc.hist, n_bins, k_rem, sc.warp_tot, sc.sel);
+      top = (top << w) | sc.sel[0];
       k_rem = sc.sel[1];
-      n_equal = sc.sel[2];
-      rem = 0;
+      const uint32_t live = sc.sel[2];
+      n_equal = live;                                  // exact once no bits are left
+      rem = shift;
+      if (rem > 0 && live <= kDirect) {   // few candidates: ranked by their remaining bits
+        for_items<kT>(far, n, whole, [&](unsigned long long key, int) {
+          const unsigned long long x = key - base;
+          if ((x >> rem) == top) sc.small[atomicAdd(&sc.small_n, 1u)] = x;
+        });
+        __syncthreads();
+        uint32_t k_out;
+        top = rank_select<kT>(sc, (int)live, k_rem, k_out, n_equal);
+        k_rem = k_out;
+        rem = 0;
+      }
     }
-    __syncthreads();                                   // sc.sel and sc.hist are rewritten by the next step
+    kth = base + top;
   }
-  // kth = the k-th largest key; k_rem of the n_equal keys equal to it are admitted, in ascending index order
-  const unsigned long long kth = base + top;
-  if (k_rem == n_equal) {                              // no tie is cut (the usual case): everything >= kth is in
+  if (k_rem == n_equal && copy) {                      // no tie is cut (the usual case): everything >= kth is in
+    const uint32_t kth_hi = (uint32_t)(kth >> 32);
     for (int base_i = r_lo; base_i < r_hi; base_i += 32) {
       const int i = base_i + lane;
-      const unsigned imp_b = __ballot_sync(kFull, i < r_hi && keys[i] >= kth);
+      const uint32_t x = i < r_hi ? copy[i] : 0u;
+      const unsigned imp_b = __ballot_sync(kFull, i < r_hi && (x > kth_hi || (x == kth_hi && keys[i] >= kth)));
       if (lane == 0) imp_mask[base_i >> 5] = imp_b;
+    }
+    __syncthreads();
+    return;
+  }
+  if (k_rem == n_equal) {
+    for (int base_i = r_lo; base_i < r_hi; base_i += 8 * 32) {
+      unsigned long long key[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) key[j] = base_i + 32 * j + lane < r_hi ? keys[base_i + 32 * j + lane] : 0ull;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (base_i + 32 * j >= r_hi) break;
+        const unsigned imp_b = __ballot_sync(kFull, base_i + 32 * j + lane < r_hi && key[j] >= kth);
+        if (lane == 0) imp_mask[(base_i >> 5) + j] = imp_b;
+      }
     }
     __syncthreads();
     return;
@@ -236,6 +281,7 @@ __device__ __forceinline__ void mark_top_keys(const unsigned long long* keys, in
   for (int i = r_lo + lane; i < r_hi; i += 32) n_eq += (keys[i] == kth);
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) n_eq += __shfl_xor_sync(kFull, n_eq, d);
+  __syncthreads();                                     // warp_tot may still be read by the digit search
   if (lane == 0) sc.warp_tot[warp] = n_eq;
   __syncthreads();
   int eq_before = 0;

@@ -105,6 +105,18 @@ def test_signature_thresholds_for_rows_beyond_the_register_kernel(B):
     _select_case(B, 4, 2, [33000], [(100, 50)], 1, 3, 0, seed=18)
 
 
+@pytest.mark.parametrize("Hq,L,b_imp,b_rep,ties", [
+    (4, 13088, 900, 1300, 0), (4, 13216, 900, 1300, 0),      # the last segment staged whole, the first that is not
+    (128, 7488, 300, 1500, 0), (128, 7680, 300, 1500, 0),    # the same with four signature words; buckets of 5
+    (4, 33000, 2000, 3300, 0),                               # signatures and 16-bit order in shared memory; buckets of 10
+    (4, 45000, 500, 9000, 0),                                # order in global memory; buckets of 5
+    (4, 66000, 100, 300, 0),                                 # nothing staged, buckets of 220
+    (4, 20000, 700, 1700, 3), (4, 300, 40, 60, 2),           # more than 256 candidates after the first round, ties cut
+])
+def test_select_at_the_edges_of_its_staging(B, Hq, L, b_imp, b_rep, ties):
+    _select_case(B, Hq, Hq, [L], [(b_imp, b_rep)], 1, ties, 0, seed=330 + L % 97)
+
+
 @pytest.mark.parametrize("seqlens,ties", [
     ([1, 2, 31, 32, 33, 256], 0), ([255, 256, 1, 100], 2),       # 8 keys a lane
     ([257, 31, 512], 0), ([511, 512, 480], 3),                   # 16
