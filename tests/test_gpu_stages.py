@@ -121,8 +121,9 @@ def test_select_at_the_edges_of_its_staging(B, Hq, L, b_imp, b_rep, ties):
     ([1, 2, 31, 32, 33, 256], 0), ([255, 256, 1, 100], 2),       # 8 keys a lane
     ([257, 31, 512], 0), ([511, 512, 480], 3),                   # 16
     ([513, 1023, 1024, 64] * 10, 0), ([1024, 700] * 19, 1),      # 32, more rows than the chip holds as blocks
+    ([8193, 8192, 1], 0), ([16385, 40], 2), ([32767], 0),        # upper halves in shared memory; 2: more than 1024 in one bin
 ])
-def test_thresholds_by_one_warp_per_row_are_exact(B, seqlens, ties):
+def test_thresholds_are_exact_for_every_row_kernel(B, seqlens, ties):
     budgets = [(max(1, L // 5), L // 7) for L in seqlens]
     _select_case(B, 32, 8, seqlens, budgets, 1, ties, 0, seed=230 + len(seqlens))
 
