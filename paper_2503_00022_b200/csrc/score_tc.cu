@@ -73,6 +73,7 @@ struct PersistArgs {
   float* scores;           // sweep 2 output
   int normalize;
   int bf16;                // operand type of Q and K: bf16 (1) or fp16 (0)
+  int k_steps;             // 16-channel steps of a dot product; the zeros past the last channel are not multiplied
   int tpb;                 // 128-row tiles of an item's stationary block: 4, or 2 or 1 when the launch has few items
   int max_blocks;          // ceil(max_seqlen / (tpb * kTile))
   int n_items;             // (sequence, stationary block) pairs of one (layer, head)
@@ -337,6 +338,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const uint32_t d_tmem = tmem_base + qd * kTile;
 #pragma unroll
             for (int k = 0; k < D / 16; ++k) {
+              if (k >= a.k_steps) break;
               const uint32_t off = (k >> 2) * SL::kBlockBytes + (k & 3) * 32;
               umma_bf16(d_tmem, smem_desc_sw128(a_addr[u] + off),
                         smem_desc_sw128(ring_addr + rs * SL::kTileBytes + off), idesc, k > 0);
@@ -595,6 +597,7 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
     return KVCRUSH_ERR_CUDA;
   PersistArgs a{};
   a.s = s; a.scale_log2 = scale_log2; a.normalize = normalize; a.bf16 = Q.dtype == KVCRUSH_BF16; a.status = status; a.scores = scores;
+  a.k_steps = (s.D + 15) / 16;
   const bool sw = diag.short_waits != 0;
   if (!lse_in && !sw && !diag.withhold_first_item && score_window_fits(s)) {
     const int rc = launch_score_window(s, Q, maps, scale_log2, scores, lse_out, normalize, status, stream);

@@ -53,6 +53,7 @@ struct WinArgs {
   float* scores;
   int normalize;
   int bf16;
+  int k_steps;               // 16-channel steps of a dot product
   int n_pad;                 // accumulator columns: the window rounded up to 16, 32 or 64
   int ring;
   int n_units;               // n_layers * n_seqs * Hq
@@ -296,9 +297,11 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           used ^= 1u << i;
           tc_fence_after();
 #pragma unroll
-          for (int k = 0; k < D / 16; ++k)
+          for (int k = 0; k < D / 16; ++k) {
+            if (k >= a.k_steps) break;
             umma_bf16(tmem_base + i * n_pad, smem_desc_sw128(ring_addr + rs * kTileBytes + (k >> 2) * kBlockBytes + (k & 3) * 32),
                       smem_desc_sw128(q_addr + qs * q_bytes + (k >> 2) * n_pad * 128 + (k & 3) * 32), idesc, k > 0);
+          }
           umma_commit(smem_u32(&aux->acc_full[i]));
           umma_commit(smem_u32(&aux->k_empty[rs]));
           if (++rs == ring) { rs = 0; ph ^= 1; }
@@ -586,7 +589,7 @@ int launch_score_window(const Shape& s, const TensorView& Q, const ScoreTensorMa
     return KVCRUSH_ERR_CUDA;
   WinArgs a{};
   a.s = s; a.scale_log2 = scale_log2; a.lse_nat_out = lse_out; a.scores = scores; a.normalize = normalize;
-  a.bf16 = Q.dtype == KVCRUSH_BF16; a.status = status;
+  a.bf16 = Q.dtype == KVCRUSH_BF16; a.status = status; a.k_steps = (s.D + 15) / 16;
   a.n_units = s.n_layers * s.n_seqs * s.Hq;
   a.n_pad = 16;
   while (a.n_pad < s.window) a.n_pad *= 2;
