@@ -73,7 +73,6 @@ struct PersistArgs {
   float* scores;           // sweep 2 output
   int normalize;
   int bf16;                // operand type of Q and K: bf16 (1) or fp16 (0)
-  int k_steps;             // 16-channel steps of a dot product; the zeros past the last channel are not multiplied
   int tpb;                 // 128-row tiles of an item's stationary block: 4, or 2 or 1 when the launch has few items
   int max_blocks;          // ceil(max_seqlen / (tpb * kTile))
   int n_items;             // (sequence, stationary block) pairs of one (layer, head)
@@ -158,8 +157,11 @@ struct Geo {
 // kSplit: items with one or two quarters spread them over all four accumulators.  The column sweep has an instantiation
 // without it for full blocks: carrying it along costs 2 % there (372 against 365 us at 2 layers of 5003 + 3117 tokens,
 // 4 % at ragged 500 to 1000 tokens), while its partial last blocks are its lightest items.
+// D: channels of a tile in shared memory (64 or 128); kSteps: 16-channel steps of a dot product that are multiplied (heads
+// of 65 to 96 channels: 6 of 8, the rest is zeros: heads of 96, one sweep of 5003 + 3117 tokens x 8 layers 1418 -> 1355 us;
+// as a run-time bound it cost the full width 0.5 %).
 // kPolls: polls of every bounded barrier wait (a compile-time constant: the epilogue has no register to spare for it).
-template <int D, bool kColsum, bool kSplit, uint32_t kPolls>
+template <int D, int kSteps, bool kColsum, bool kSplit, uint32_t kPolls>
 __global__ void __launch_bounds__(kThreads, 1)
 score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const PersistArgs a) {
@@ -337,8 +339,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + qd * kTile;
 #pragma unroll
-            for (int k = 0; k < D / 16; ++k) {
-              if (k >= a.k_steps) break;
+            for (int k = 0; k < kSteps; ++k) {
               const uint32_t off = (k >> 2) * SL::kBlockBytes + (k & 3) * 32;
               umma_bf16(d_tmem, smem_desc_sw128(a_addr[u] + off),
                         smem_desc_sw128(ring_addr + rs * SL::kTileBytes + off), idesc, k > 0);
@@ -520,20 +521,27 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   if (tid == 0 && !dead && *abort_flag) report(a.status, KVCRUSH_DEV_TIMEOUT, kColsum ? KID_SCORE_COLSUM : KID_SCORE_LSE, blockIdx.x, 0);
 }
 
-template <int D, bool kColsum, bool kSplit, uint32_t kPolls>
+template <int D, int kSteps, bool kColsum, bool kSplit, uint32_t kPolls>
 int launch_persist_polls(const CUtensorMap& mq, const CUtensorMap& mk, const PersistArgs& a, int n_sms, cudaStream_t stream) {
-  auto kern = score_persist_kernel<D, kColsum, kSplit, kPolls>;
+  auto kern = score_persist_kernel<D, kSteps, kColsum, kSplit, kPolls>;
   constexpr int smem = PSmem<D>::kTotal;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return KVCRUSH_ERR_CUDA;
   const int blocks = a.total_items < n_sms ? a.total_items : n_sms;
   return launch_chained(kern, dim3((unsigned)blocks), dim3(kThreads), smem, stream, 1, mq, mk, a);
 }
 
-template <int D, bool kColsum, bool kSplit>
+template <bool kColsum, bool kSplit, uint32_t kPolls>
+int launch_persist_width(const CUtensorMap& mq, const CUtensorMap& mk, const PersistArgs& a, int n_sms, cudaStream_t stream) {
+  if (a.s.D <= 64) return launch_persist_polls<64, 4, kColsum, kSplit, kPolls>(mq, mk, a, n_sms, stream);
+  if (a.s.D <= 96) return launch_persist_polls<128, 6, kColsum, kSplit, kPolls>(mq, mk, a, n_sms, stream);
+  return launch_persist_polls<128, 8, kColsum, kSplit, kPolls>(mq, mk, a, n_sms, stream);
+}
+
+template <bool kColsum, bool kSplit>
 int launch_persist(const CUtensorMap& mq, const CUtensorMap& mk, const PersistArgs& a, bool short_waits, int n_sms,
                    cudaStream_t stream) {
-  return short_waits ? launch_persist_polls<D, kColsum, kSplit, kShortWaitPolls>(mq, mk, a, n_sms, stream)
-                     : launch_persist_polls<D, kColsum, kSplit, kWaitPolls>(mq, mk, a, n_sms, stream);
+  return short_waits ? launch_persist_width<kColsum, kSplit, kShortWaitPolls>(mq, mk, a, n_sms, stream)
+                     : launch_persist_width<kColsum, kSplit, kWaitPolls>(mq, mk, a, n_sms, stream);
 }
 
 // Tiles of an item's stationary block.  Four 128-row tiles take the most out of every streamed tile, but a launch with
@@ -597,7 +605,6 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
     return KVCRUSH_ERR_CUDA;
   PersistArgs a{};
   a.s = s; a.scale_log2 = scale_log2; a.normalize = normalize; a.bf16 = Q.dtype == KVCRUSH_BF16; a.status = status; a.scores = scores;
-  a.k_steps = (s.D + 15) / 16;
   const bool sw = diag.short_waits != 0;
   if (!lse_in && !sw && !diag.withhold_first_item && score_window_fits(s)) {
     const int rc = launch_score_window(s, Q, maps, scale_log2, scores, lse_out, normalize, status, stream);
@@ -638,16 +645,14 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
   if (!lse_in) {
     if (!plan(true, counters)) return KVCRUSH_ERR_CUDA;
     a.lse2_out = lse2_ws; a.lse_nat_out = lse_out;
-    rc = s.D > 64 ? launch_persist<128, false, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<64, false, true>(mq, mk, a, sw, n_sms, stream);
+    rc = launch_persist<false, true>(mq, mk, a, sw, n_sms, stream);
     if (rc != KVCRUSH_OK) return rc;
     a.lse = lse2_ws; a.lse_mul = 1.f;
   } else {
     a.lse = lse_in; a.lse_mul = lse_in_mul;
   }
   if (!plan(false, counters + 1)) return KVCRUSH_ERR_CUDA;
-  if (a.tpb < kQ)
-    return s.D > 64 ? launch_persist<128, true, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<64, true, true>(mq, mk, a, sw, n_sms, stream);
-  return s.D > 64 ? launch_persist<128, true, false>(mq, mk, a, sw, n_sms, stream) : launch_persist<64, true, false>(mq, mk, a, sw, n_sms, stream);
+  return a.tpb < kQ ? launch_persist<true, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<true, false>(mq, mk, a, sw, n_sms, stream);
 }
 
 }  // namespace kvc
