@@ -133,6 +133,28 @@ def test_pooling_is_bit_exact(B, kernel):
         for s in range(len(seqlens)):
             np.testing.assert_array_equal(got[l][:, cu[s]:cu[s + 1]], O.max_pool(scores[l][:, cu[s]:cu[s + 1]], kernel))
 
+@pytest.mark.parametrize("seqlens,kernel", [
+    ([4096], 1), ([4096], 5), ([8192], 7), ([1020], 9), ([4], 7), ([2044, 4], 33),       # quads; the last chunk in two sequences
+    ([1024, 2048], 7), ([2045, 3], 7), ([1, 1023, 4096], 2047),                          # sequences that end inside a quad
+    ([4096] * 80, 7), ([4095, 3, 5000] * 34, 5),                                         # chunks of 1024 tokens
+    ([5000], 12001), ([4999, 2], 12001), ([3], 3),                                       # window too wide for shared memory; odd rows
+])
+def test_pooling_at_the_edges_of_its_chunks(B, seqlens, kernel):
+    import torch
+    dev = _dev()
+    Hq, T = 4, sum(seqlens)
+    scores = np.concatenate([inputs.random_scores(Hq, L, 90 + s) for s, L in enumerate(seqlens)], axis=1)
+    prob = B.Problem(1, Hq, Hq, 16, seqlens, device=dev)
+    out = torch.full((1, Hq, T), -3.0, dtype=torch.float32, device=dev)
+    status = torch.zeros(4, dtype=torch.int32, device=dev)
+    B.kvcrush_pool_scores(prob, torch.from_numpy(scores[None]).to(dev), kernel, out, status=status)
+    torch.cuda.synchronize()
+    a = 0
+    for L in seqlens:
+        np.testing.assert_array_equal(out[0, :, a:a + L].cpu().numpy(), O.max_pool(np.ascontiguousarray(scores[:, a:a + L]), kernel))
+        a += L
+
+
 
 @pytest.mark.parametrize("keep_recent,budgets", [(16, [(40, 30), (20, 10)]), (64, [(10, 5), (64, 64)]), (1, [(1, 1), (0, 9)])])
 def test_keep_recent_selection_is_bit_exact(B, keep_recent, budgets):
