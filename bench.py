@@ -35,12 +35,12 @@ METRIC = "prompt tokens compressed/s (score+select+compact)"
 UNIT = "tokens/s"
 DEFAULT_WORKLOAD = "cfg3_llama2_32l_8k"
 # dram__bytes_read + dram__bytes_write of one sweep launch per layer, from the ncu capture of the 2-layer case:
-# the column-sum sweep read 286.1 MB and wrote 5.5 MB for two layers.  Scaling by the layer count over-states the
+# the column-sum sweep read 290.0 MB and wrote 5.9 MB for two layers.  Scaling by the layer count over-states the
 # full workload a little: the last 37 (layer, head) pairs of a launch are handed out across heads, which costs L2
 # reuse, and they are 37 of 64 pairs in the capture but 37 of 1024 in the full workload.  Valid for the kernel
 # source named in NCU_TRAFFIC_SOURCE only.
-NCU_DRAM_BYTES_PER_LAYER_PER_SWEEP = 145.8e6
-NCU_TRAFFIC_SOURCE = ("ncu capture of score_persist_kernel<128, colsum> at commit 8454247 (2 layers of the workload, scaled by the "
+NCU_DRAM_BYTES_PER_LAYER_PER_SWEEP = 147.9e6
+NCU_TRAFFIC_SOURCE = ("ncu capture of score_persist_kernel<128, colsum> at commit e913ce9 (2 layers of the workload, scaled by the "
                       "layer count: an upper bound, see profiles/)")
 
 
@@ -611,25 +611,29 @@ def run_ours(args, w):
     score_s = stage_ms[0] * 1e-3
     tensor_path = cp.impl != B.SCORE_SIMT and w.qk_dtype in (inputs.BF16, inputs.FP16) and w.head_dim % 8 == 0 and w.head_dim <= 128
     short_tf = work["score_flops"] / score_s / 1e12
+    # score launches per step: two sweeps, or one pass for observation windows of up to 64 queries whose logits fit
+    # the tensor memory of a cluster of eight
+    pad = next((n for n in (16, 32, 64) if args.window <= n), None) if args.window else None
+    n_score = 1 if tensor_path and pad and -(-(-(-max(w.seqlens) // 128)) // 8) * pad <= 512 else 2
     if tensor_path:
         # Headline fraction: the score stage inside the seconds-long loop against the sustained GEMM peak (both at the
         # board's power limit); beside it the K-step loop against the burst peak (both short).
         sus_tf = work["score_flops"] / (sus["score_ms_settled"] * 1e-3) / 1e12 if sus else short_tf
-        launch_ms = (sus["score_ms_settled"] if sus else float(stage_ms[0])) / 2
+        launch_ms = (sus["score_ms_settled"] if sus else float(stage_ms[0])) / n_score
         whole = w.name == DEFAULT_WORKLOAD or w.name.startswith(DEFAULT_WORKLOAD + "_")
         traffic = NCU_DRAM_BYTES_PER_LAYER_PER_SWEEP * w.n_layers if (whole and not args.window) else None
-        roofline = {"bound": "tensor", "kernel": "score_persist_kernel (two sweep launches per step; per-launch figures)",
+        roofline = {"bound": "tensor", "kernel": "score_persist_kernel (two sweep launches per step; per-launch figures)" if n_score == 2 else "score_window_kernel",
                     "achieved": sus_tf, "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                     "frac": sus_tf / peaks["bf16_tflops_sustained"],
                     "timing": ("score stage, CUDA events, settled half of a %.1f s loop of the whole pass" % sus["seconds"]) if sus else "score stage of the timed steps",
                     "peak_source": peaks["source"] + " (sustained bf16: seconds-long loop under the power cap)",
                     "traffic": traffic, "traffic_source": NCU_TRAFFIC_SOURCE if traffic else None,
-                    "algorithmic_flops_per_launch": work["score_flops"] / 2, "launch_ms": launch_ms,
+                    "algorithmic_flops_per_launch": work["score_flops"] / n_score, "launch_ms": launch_ms,
                     "short_loop": {"achieved": short_tf, "peak": peaks["bf16_tflops"], "frac": short_tf / peaks["bf16_tflops"],
-                                   "launch_ms": float(stage_ms[0]) / 2,
+                                   "launch_ms": float(stage_ms[0]) / n_score,
                                    "note": "score stage of the %d timed steps against the burst bf16 peak" % args.steps},
                     "frac_of_nominal_2250": sus_tf / 2250.0,
-                    "exps_per_s": work["exps"] / (2 * launch_ms * 1e-3)}
+                    "exps_per_s": work["exps"] / (n_score * launch_ms * 1e-3)}
         if sus and sus["clocks"]:
             ghz = sus["clocks"]["sm_mhz"] * 1e-3
             roofline["sm_ghz_sustained"] = ghz
@@ -670,9 +674,9 @@ def run_ours(args, w):
         cpu = cpu_baseline_leg(w)
 
     tokens = w.total_tokens * world
-    # kernels of this library per step: two score sweeps, threshold select + signature pack (which also writes the token
+    # kernels of this library per step: the score sweeps, threshold select + signature pack (which also writes the token
     # importance), the segment selection, the gather (+ pooling)
-    launches_per_step = 2 + 2 + (1 if cp.importance is not None else 2) + 1 + (1 if cp.pooled is not None else 0)
+    launches_per_step = n_score + 2 + (1 if cp.importance is not None else 2) + 1 + (1 if cp.pooled is not None else 0)
     line = {
         "metric": METRIC, "value": whole_job_value(w.total_tokens, world, ms_per_step), "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
