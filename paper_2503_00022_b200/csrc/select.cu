@@ -17,9 +17,11 @@
 //                               per-bit mean, up to a constant), ties to the lower token
 //                            5. kept = important U representatives, ascending token index
 // A chain of short block-wide steps in one CTA per segment, bound by their latencies (8192 tokens, thousand cycles: staging
-// 4.7, top-k 6.8, sort 7.7, buckets 13 to 21, output 2.9; device time 20.5 -> 18.4 us for 32 such segments, 10.1 -> 8.5 us
+// 4.7, top-k 6.8, sort 7.7, buckets 13 to 21, output 2.9; device time 20.5 -> 18.4 us for 32 such segments, 10.1 -> 8.2 us
 // for one of 1001 tokens); from about 13000 tokens on by instructions and L2 reads (32 segments of 32768 tokens 117 -> 69 us).
 // All decisions are integer or exact float64 comparisons, so the result is unique.
+#include <type_traits>
+
 #include "select_common.cuh"
 
 namespace kvc {
@@ -28,8 +30,6 @@ namespace {
 
 using sel::kFull;
 using sel::head_mask;
-constexpr int kThreads = 1024;
-constexpr int kWarps = kThreads / 32;
 constexpr int kMaxBins = 129;              // Hamming distances 0..128
 
 // Order-preserving 64-bit key of a float64 importance; tokens kept by decree (the first keep_initial and the last
@@ -125,9 +125,10 @@ struct SelectArgs {
 // kLong: segments whose keys, signatures and sorted order do not all fit in shared memory.  Of those the signatures come
 // first, which the bucket step gathers one by one, then the sorted order as 16-bit indices; the keys' upper halves are
 // copied into the signatures' place while the top k are looked for.
-template <int W, bool kLong>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int W, bool kLong, int kT>
+__global__ void __launch_bounds__(kT, 1024 / kT)
 select_segment_kernel(Shape s, SelectArgs a) {
+  constexpr int kWarps = kT / 32;
   extern __shared__ __align__(16) uint32_t dyn_smem[];
   uint32_t* imp_mask = dyn_smem;
   uint32_t* rep_mask = dyn_smem + a.mask_words;
@@ -155,7 +156,7 @@ select_segment_kernel(Shape s, SelectArgs a) {
 
   if (a.n_kept && tid == 0) a.n_kept[seg] = (int)min((long long)b_imp + b_rep, (long long)L);
   if ((long long)b_imp + b_rep >= L) {             // budget covers the sequence: keep everything
-    for (int i = tid; i < L; i += kThreads) {
+    for (int i = tid; i < L; i += kT) {
       out_idx[i] = i;
       if (out_kind) out_kind[i] = 0;
     }
@@ -176,29 +177,29 @@ select_segment_kernel(Shape s, SelectArgs a) {
   uint32_t* sort_code = arena;           // !kLong, per token: distance | position among the warp's tokens of that distance << 8
   auto sorted_at = [&](int i) { return kLong && sorted16 ? (int)sorted16[i] : sorted[i]; };
   auto stage_sig = [&]() {
-    _Pragma("unroll 8") for (int i = tid; i < L * W; i += kThreads) sig_sh[i] = __ldg(sig + i);
+    _Pragma("unroll 8") for (int i = tid; i < L * W; i += kT) sig_sh[i] = __ldg(sig + i);
     sig = sig_sh;
   };
   if (!kLong) {
     stage_sig();
     unsigned long long* ks = reinterpret_cast<unsigned long long*>(arena);        // dead once the important set is marked
     if (a.keys) {
-      _Pragma("unroll 8") for (int i = tid; i < L; i += kThreads) ks[i] = keys[i];
+      _Pragma("unroll 8") for (int i = tid; i < L; i += kT) ks[i] = keys[i];
     } else {
       const double* imp = a.imp + (size_t)layer * s.T + t0;
-      _Pragma("unroll 8") for (int i = tid; i < L; i += kThreads) ks[i] = importance_key(__ldg(imp + i), i, L, a.keep_initial, a.keep_recent);
+      _Pragma("unroll 8") for (int i = tid; i < L; i += kT) ks[i] = importance_key(__ldg(imp + i), i, L, a.keep_initial, a.keep_recent);
     }
     keys = ks;
   }
   const int n_words = (L + 31) >> 5;
   int r_lo, r_hi;                            // contiguous token range of this warp
-  sel::warp_range<kThreads>(L, warp, r_lo, r_hi);
+  sel::warp_range<kT>(L, warp, r_lo, r_hi);
 
-  for (int i = tid; i < n_words; i += kThreads) { imp_mask[i] = 0; rep_mask[i] = 0; }
+  for (int i = tid; i < n_words; i += kT) { imp_mask[i] = 0; rep_mask[i] = 0; }
   __syncthreads();
 
   // ---- 1. important tokens: the b_imp largest keys, ties to the lower index --------------------
-  if (b_imp > 0) sel::mark_top_keys<kThreads>(keys, L, b_imp, imp_mask, sc, kLong ? sig_sh : nullptr);
+  if (b_imp > 0) sel::mark_top_keys<kT>(keys, L, b_imp, imp_mask, sc, kLong ? sig_sh : nullptr);
 
   // ---- 2-4. representatives of the other tokens ------------------------------------------------
   if (b_rep > 0) {
@@ -206,7 +207,7 @@ select_segment_kernel(Shape s, SelectArgs a) {
     if (kLong && sig_sh) { stage_sig(); __syncthreads(); }
     // anchor
     if (a.anchor_mode == KVCRUSH_ANCHOR_MEAN) {
-      for (int i = tid; i < 128; i += kThreads) bit_cnt[i] = 0;
+      for (int i = tid; i < 128; i += kT) bit_cnt[i] = 0;
       __syncthreads();
       int acc[4] = {0, 0, 0, 0};
       for (int base = r_lo; base < r_hi; base += 32) {
@@ -237,7 +238,7 @@ select_segment_kernel(Shape s, SelectArgs a) {
         word = 0xAAAAAAAAu;
       anchor_sh[tid] = word & head_mask(s.Hq, tid);
     }
-    for (int i = tid; i < kWarps * kMaxBins; i += kThreads) (&warp_hist[0][0])[i] = 0;
+    for (int i = tid; i < kWarps * kMaxBins; i += kT) (&warp_hist[0][0])[i] = 0;
     __syncthreads();
     uint32_t anc[4], hm[4];
     _Pragma("unroll") for (int w = 0; w < 4; ++w) { anc[w] = w < W ? anchor_sh[w] : 0u; hm[w] = w < W ? head_mask(s.Hq, w) : 0u; }
@@ -437,7 +438,7 @@ select_segment_kernel(Shape s, SelectArgs a) {
   }
 
   // ---- 5. kept = important U representatives, ascending ------------------------------------------
-  sel::emit_kept<kThreads>(imp_mask, rep_mask, n_words, out_idx, out_kind, sc);
+  sel::emit_kept<kT>(imp_mask, rep_mask, n_words, out_idx, out_kind, sc);
 }
 
 }  // namespace
@@ -505,14 +506,28 @@ int launch_select(const Shape& s, const float* scores, const double* importance,
       a.keys = keys;
     }
   }
-  auto kern = s.W == 1 ? (long_seg ? select_segment_kernel<1, true> : select_segment_kernel<1, false>)
-            : s.W == 2 ? (long_seg ? select_segment_kernel<2, true> : select_segment_kernel<2, false>)
-            : s.W == 3 ? (long_seg ? select_segment_kernel<3, true> : select_segment_kernel<3, false>)
-                       : (long_seg ? select_segment_kernel<4, true> : select_segment_kernel<4, false>);
-  // static + dynamic shared memory above the 48 KB default needs the opt-in
-  if (dyn > 28 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-    return KVCRUSH_ERR_CUDA;
-  return launch_chained(kern, dim3((unsigned)(s.n_layers * s.n_seqs)), dim3(kThreads), dyn, stream, 1, s, a);
+  auto launch = [&](auto kern, int threads) {
+    // static + dynamic shared memory above the 48 KB default needs the opt-in
+    if (dyn > 28 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
+      return (int)KVCRUSH_ERR_CUDA;
+    return launch_chained(kern, dim3((unsigned)(s.n_layers * s.n_seqs)), dim3(threads), dyn, stream, 1, s, a);
+  };
+  // Threads of a segment: 1024 while every segment has an SM to itself (32 x 8192 tokens 22 us, with 512 threads 27), half as
+  // many up to 1024 tokens, where barriers are most of the work (one segment of 512 tokens 7.7 -> 6.7 us, with 256 threads
+  // 7.5).  Registers let an SM hold 1024 threads, so more segments than SMs take smaller blocks as far as shared memory
+  // holds them: 256 segments of 700 tokens 17.2 -> 10.6 us, 224 of 1900 21.6 -> 15.4, 512 of 4000 62.7 -> 48.1 (with 256
+  // threads 60.7); 512 of 700 tokens 31.9 -> 13.0 (18.9), 512 of 1900 42.0 -> 23.7 (28.6).
+  const long long n_seg = (long long)s.n_layers * s.n_seqs;
+  auto resident = [&](int n) { return n * (dyn + 19 * 1024) <= 227 * 1024; };
+  auto by_words = [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    if (long_seg) return launch(select_segment_kernel<W, true, 1024>, 1024);
+    if (n_seg > 2 * 148 && s.max_seqlen <= 2048 && resident(4)) return launch(select_segment_kernel<W, false, 256>, 256);
+    if ((s.max_seqlen <= 1024 || n_seg > 148) && resident(2)) return launch(select_segment_kernel<W, false, 512>, 512);
+    return launch(select_segment_kernel<W, false, 1024>, 1024);
+  };
+  return s.W == 1 ? by_words(std::integral_constant<int, 1>{}) : s.W == 2 ? by_words(std::integral_constant<int, 2>{})
+       : s.W == 3 ? by_words(std::integral_constant<int, 3>{}) : by_words(std::integral_constant<int, 4>{});
 }
 
 }  // namespace kvc

@@ -117,6 +117,17 @@ def test_select_at_the_edges_of_its_staging(B, Hq, L, b_imp, b_rep, ties):
     _select_case(B, Hq, Hq, [L], [(b_imp, b_rep)], 1, ties, 0, seed=330 + L % 97)
 
 
+@pytest.mark.parametrize("Hq,seqlens,mode,ties", [
+    (8, [1024, 1], 0, 0), (8, [1025, 40], 0, 0), (40, [1000, 33], 2, 1),          # 512 threads, 1024, 512
+    (8, [300, 41, 1500] * 50, 0, 2), (72, [1025, 64] * 75, 2, 0),                 # more segments than SMs: 512
+    (8, [70, 2, 260, 1] * 75, 2, 0), (8, [2048] + [33, 90] * 149, 0, 2),          # more than twice as many: 256
+    (128, [2049] + [64, 20] * 149, 0, 0),                                         # 512 again
+])
+def test_select_in_blocks_of_every_size(B, Hq, seqlens, mode, ties):
+    budgets = [(max(1, L // 6), L // 5) for L in seqlens]
+    _select_case(B, Hq, Hq, seqlens, budgets, 1, ties, mode, seed=370 + len(seqlens))
+
+
 @pytest.mark.parametrize("seqlens,ties", [
     ([1, 2, 31, 32, 33, 256], 0), ([255, 256, 1, 100], 2),       # 8 keys a lane
     ([257, 31, 512], 0), ([511, 512, 480], 3),                   # 16
