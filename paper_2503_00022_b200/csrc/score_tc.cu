@@ -490,10 +490,10 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           if ((gi & (g.rep - 1)) == 0) {
             float big = m;
             for (int u = 1; u < g.rep; ++u) big = fmaxf(big, part[gi + u][0][r]);
-            float tot = sum > 0.f ? sum * ex2(m - big) : 0.f;
+            float tot = sum == 0.f ? 0.f : sum * ex2(m - big);         // 0: a slot without tiles; NaN stays NaN
             for (int u = 1; u < g.rep; ++u) {
               const float mu = part[gi + u][0][r], su = part[gi + u][1][r];
-              tot += su > 0.f ? su * ex2(mu - big) : 0.f;
+              tot += su == 0.f ? 0.f : su * ex2(mu - big);
             }
             m = big;
             sum = tot;

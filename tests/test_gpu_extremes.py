@@ -1,0 +1,64 @@
+"""Scores of inputs that are not finite or lie at the ends of the float range: a NaN logit makes its query's log-sum-exp
+NaN and with it every score the query adds to, a logit of -inf gets the weight 0, a query that does not vote has no
+influence, and weights keep the relative precision of float32 down to the smallest normal number."""
+import numpy as np
+import pytest
+
+from oracle import kvcrush_oracle as O
+import kvc_testlib as TL
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2503_00022_b200 import binding, build
+    build.build()
+    binding.lib()
+    return binding
+
+
+def _normal(shape, seed, dtype):
+    import torch
+    g = np.random.Generator(np.random.Philox(seed))
+    return torch.from_numpy(g.standard_normal(shape).astype(np.float32)).to("cuda:0").to(dtype)
+
+
+def _score(B, q, k, lens, impl, window=0, causal=True, scale=0.0):
+    """(scores, row log-sum-exp; 7.0 where a row is not written) as numpy [layers, Hq, T]."""
+    import torch
+    layers, T, Hq, D = q.shape
+    prob = B.Problem(layers, Hq, k.shape[2], D, lens, causal=causal, softmax_scale=scale, device=q.device, query_window=window)
+    ws = torch.empty(B.kvcrush_workspace_size(prob, B.STAGE_SCORE), dtype=torch.uint8, device=q.device)
+    status = torch.zeros(4, dtype=torch.int32, device=q.device)
+    scores = torch.full((layers, Hq, T), -1.0, dtype=torch.float32, device=q.device)
+    lse = torch.full_like(scores, 7.0)
+    B.kvcrush_score(prob, q, k, scores, lse_out=lse, impl=impl, workspace=ws, status=status)
+    assert status.cpu().tolist()[0] == 0
+    return scores.cpu().numpy(), lse.cpu().numpy()
+
+
+def _decode(B, q_new, k, scale=0.0):
+    import torch
+    layers, L, _, D = k.shape
+    prob = B.Problem(layers, q_new.shape[2], k.shape[2], D, (L,), softmax_scale=scale, device=k.device)
+    scores = torch.zeros((layers, q_new.shape[2], L), dtype=torch.float32, device=k.device)
+    status = torch.zeros(4, dtype=torch.int32, device=k.device)
+    B.kvcrush_score_decode(prob, q_new, k, scores, status=status)
+    return scores.cpu().numpy()
+
+
+# The column of a NaN key is chosen so that its exponential takes the special-function unit: the polynomial that serves
+# columns 6, 7, 14 and 15 of every 16 clamps its argument and with it a NaN.
+@pytest.mark.parametrize("layers,Hq,L,p", [
+    (1, 2, 201, 64), (1, 2, 201, 160),       # blocks of one tile: four slots a quarter
+    (1, 8, 1100, 128), (1, 32, 2052, 513),   # blocks of one or two tiles
+    (8, 32, 2052, 1024),                     # full blocks, the last one with a single tile
+])
+def test_nan_key_reaches_every_row_that_sees_it_on_the_tensor_cores(B, layers, Hq, L, p):
+    import torch
+    q, k = _normal((layers, L, Hq, 128), 1, torch.bfloat16), _normal((layers, L, Hq, 128), 2, torch.bfloat16)
+    k[:, p] = float("nan")
+    s, lse = _score(B, q, k, (L,), B.SCORE_TENSOR)
+    assert np.isfinite(lse[..., :p]).all() and np.isnan(lse[..., p:]).all()
+    assert np.isnan(s).all()
