@@ -161,7 +161,8 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
       } else {
         const float big = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
         if (big > m[i]) { sum[i] *= exp2f(m[i] - big); m[i] = big; }     // first tile: 0 * 2^-inf
-        if (m[i] != ninf) sum[i] += (exp2f(x[0] - m[i]) + exp2f(x[1] - m[i])) + (exp2f(x[2] - m[i]) + exp2f(x[3] - m[i]));
+        const float ref = m[i] == ninf ? 0.f : m[i];                     // no maximum yet: -inf adds 0, NaN makes the sum NaN
+        sum[i] += (exp2f(x[0] - ref) + exp2f(x[1] - ref)) + (exp2f(x[2] - ref) + exp2f(x[3] - ref));
       }
     }
   }
@@ -172,7 +173,7 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
     if constexpr (!kColsum) {
 #pragma unroll
       for (int d = 8; d > 0; d >>= 1) big = fmaxf(big, __shfl_xor_sync(0xFFFFFFFFu, big, d));
-      sum[i] = m[i] == ninf ? 0.f : sum[i] * exp2f(m[i] - big);
+      sum[i] = sum[i] == 0.f ? 0.f : sum[i] * exp2f(m[i] - big);           // 0: nothing seen
     }
 #pragma unroll
     for (int d = 8; d > 0; d >>= 1) sum[i] += __shfl_xor_sync(0xFFFFFFFFu, sum[i], d);
@@ -186,7 +187,7 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
       for (int b = 0; b < n_blk; ++b) big = fmaxf(big, *cluster.map_shared_rank(&part[0][tid], b));
     for (int b = 0; b < n_blk; ++b) {
       const float p = *cluster.map_shared_rank(&part[1][tid], b);
-      total += kColsum ? p : p > 0.f ? p * exp2f(*cluster.map_shared_rank(&part[0][tid], b) - big) : 0.f;
+      total += kColsum ? p : p == 0.f ? 0.f : p * exp2f(*cluster.map_shared_rank(&part[0][tid], b) - big);
     }
     if constexpr (kColsum) {
       scores[out] = normalize ? total / (float)(L - ws) : total;

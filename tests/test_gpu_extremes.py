@@ -62,3 +62,17 @@ def test_nan_key_reaches_every_row_that_sees_it_on_the_tensor_cores(B, layers, H
     s, lse = _score(B, q, k, (L,), B.SCORE_TENSOR)
     assert np.isfinite(lse[..., :p]).all() and np.isnan(lse[..., p:]).all()
     assert np.isnan(s).all()
+
+
+@pytest.mark.parametrize("layers,Hq,L,p,causal", [
+    (1, 1, 600, 70, True), (1, 1, 600, 3, False),     # streamed tiles shared by a cluster
+    (4, 40, 130, 0, True), (4, 40, 130, 127, True),   # one block per tile of rows; a row whose every logit is NaN
+])
+def test_nan_key_reaches_every_row_that_sees_it_on_the_cuda_cores(B, layers, Hq, L, p, causal):
+    import torch
+    q, k = _normal((layers, L, Hq, 64), 3, torch.float32), _normal((layers, L, Hq, 64), 4, torch.float32)
+    k[:, p] = float("nan")
+    s, lse = _score(B, q, k, (L,), B.SCORE_SIMT, causal=causal)
+    first = p if causal else 0
+    assert np.isfinite(lse[..., :first]).all() and np.isnan(lse[..., first:]).all()
+    assert np.isnan(s).all()
