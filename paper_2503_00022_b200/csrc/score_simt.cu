@@ -88,7 +88,7 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
   float* fix_sh = reinterpret_cast<float*>(dyn4);
   float* str_sh = fix_sh + kRows * (s.D + kPad);
   __shared__ float part[2][kRows];                          // this block's maximum (sweep 1) and sum of every row
-  __shared__ float nlse_sh[kRows];                          // sweep 2: minus lse2 of the streamed queries, -inf: no vote
+  __shared__ float nlse_sh[kRows];                          // sweep 2: minus lse2 of the streamed queries that vote
   chain_wait();
   chain_trigger();
   cg::cluster_group cluster = cg::this_cluster();
@@ -153,7 +153,8 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int c = u * kRows + tx + 16 * j;
-        const bool in = c < L && (!s.causal || (kColsum ? c >= r : c <= r));
+        // a query before the window may share the tile: its logits are left out whatever they are (inf and NaN included)
+        const bool in = c < L && (!kColsum || c >= ws) && (!s.causal || (kColsum ? c >= r : c <= r));
         x[j] = in ? (kColsum ? fmaf(acc[i][j], scale_log2, nlse_sh[tx + 16 * j]) : acc[i][j] * scale_log2) : ninf;
       }
       if constexpr (kColsum) {

@@ -76,3 +76,16 @@ def test_nan_key_reaches_every_row_that_sees_it_on_the_cuda_cores(B, layers, Hq,
     first = p if causal else 0
     assert np.isfinite(lse[..., :first]).all() and np.isnan(lse[..., first:]).all()
     assert np.isnan(s).all()
+
+
+def test_queries_that_do_not_vote_have_no_influence_on_the_cuda_cores(B):
+    """The window starts inside a tile of 64 queries; one of the tile's other queries is NaN, one gives infinite logits."""
+    import torch
+    L, window = 200, 50
+    q, k = _normal((1, L, 2, 64), 5, torch.float32), _normal((1, L, 2, 64), 6, torch.float32)
+    want, want_lse = _score(B, q, k, (L,), B.SCORE_SIMT, window=window)
+    q[:, 130] = float("nan")
+    q[:, 140] = 3e38
+    got, got_lse = _score(B, q, k, (L,), B.SCORE_SIMT, window=window)
+    np.testing.assert_array_equal(got, want)
+    np.testing.assert_array_equal(got_lse, want_lse)
