@@ -17,7 +17,8 @@
 // unit behind: half the keys a CTA, the same chain of latencies), windows of 128 queries (645 against 562 us at 4096 tokens).
 //
 // 2^x is taken without a maximum: float32 has the range unless logits are extreme.  32 keys x one column block whose
-// logits leave [-100, 100] keep them, count with their exact maxima in step 1 and take 2^(x - lse2) in step 2.
+// logits leave [-100, 100] or hold a NaN keep them, count with their exact maxima in step 1 and take 2^(x - lse2) in step 2.
+// So a stored 2^x is finite; a query's sum may be NaN, and is then NaN in every key it votes for, and in no other.
 //
 // Roles: warp 0 issues TMA loads, warp 1 the tcgen05.mma; warps 2..17 are four epilogue groups of four warps.  All waits
 // are bounded as in score_tc.cu; all CTAs of a cluster meet once more before they leave, because peers write into their
@@ -148,6 +149,12 @@ __device__ __forceinline__ void tmem_stn(uint32_t taddr, const uint32_t (&v)[32]
         "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]),
         "r"(v[29]), "r"(v[30]), "r"(v[31])
       : "memory");
+}
+// NaN if any of the three is
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
 }
 __device__ __forceinline__ float min3(float a, float b, float c) {
   float d;
@@ -365,7 +372,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         float hi = 0.f, lo = 0.f;
 #pragma unroll
         for (int i = 0; i < NC; i += 2) {
-          hi = max3(hi, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
+          hi = max3_nan(hi, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
           lo = min3(lo, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
         }
         const bool keep = __any_sync(0xFFFFFFFFu, !(hi * scale < 100.f && lo * scale > -100.f));
@@ -419,7 +426,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
               const bool in = cb * NC + c >= first_col((w.tile0 + j) * kTile + r);
               const float xs = in ? __uint_as_float(x) * scale : kNegInf;
               if (step == 0) m = fmaxf(m, xs);
-              else t += m == kNegInf ? 0.f : ex2(xs - m);
+              else t += ex2(xs - (m == kNegInf ? 0.f : m));            // -inf adds 0, NaN stays
             }
 #pragma unroll
             for (int d = 16; d > 0; d >>= 1) {
@@ -444,9 +451,9 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         const float mw = aux->warp_part[cw][ci][0], tw = aux->warp_part[cw][ci][1];
         float m = mw;
         for (int d = 1; d < tpc; d <<= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
-        float t = mw == kNegInf ? 0.f : tw * ex2(mw - m);
+        float t = tw == 0.f ? 0.f : tw * ex2(mw - m);
         for (int d = 1; d < tpc; d <<= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, d);
-        const float l = m == kNegInf ? kNegInf : m + log2f(t);
+        const float l = t == 0.f ? kNegInf : m + log2f(t);
         if (n_cta == 1) {                           // alone: this warp reads it back itself (and a launch without
           if (sub == 0) aux->part[par][0][col] = l; // clusters has no st.async)
           __syncwarp();
@@ -468,7 +475,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         if (sub == 0) {
           const float lse2 = m + log2f(t);
           aux->nlse[col] = col < w.nv ? -lse2 : kNegInf;
-          aux->factor[col] = col < w.nv ? ex2(fminf(-lse2, 126.f)) : 0.f;    // beyond 2^126 no column is below 2^100
+          aux->factor[col] = col < w.nv ? ex2(lse2 < -126.f ? 126.f : -lse2) : 0.f;    // beyond 2^126 no column is below 2^100
           if (rank == 0 && col < w.nv && a.lse_nat_out)
             a.lse_nat_out[((size_t)w.layer * s.Hq + w.h) * s.T + w.t0 + w.q0 + col] = lse2 * 0.69314718055994530942f;
         }
@@ -483,21 +490,31 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       for (int j = gi; j < w.n; j += 4) {
         const int key = (w.tile0 + j) * kTile + r;
         const uint32_t t_acc = t_lane + j * n_pad;
+        const bool edge = s.causal && key - lane + 31 > w.q0;          // a masked column somewhere in the warp's keys
         f32x2 acc[2] = {0ull, 0ull};
         for (int b = 0; b < n_cb; ++b) {
           uint32_t x[NC];
           tmem_ldn(t_acc + b * NC, x);
           tmem_waitn(x);
+          const int c_first = first_col(key) - b * NC;
           if (!aux->kept[j][b][quarter]) {
             const float4* f4 = reinterpret_cast<const float4*>(aux->factor + b * NC);
+            auto add = [&](auto masked) {
 #pragma unroll
-            for (int i = 0; i < NC / 4; ++i) {
-              const float4 f = f4[i];
-              acc[0] = fma2(pack2(x[4 * i], x[4 * i + 1]), pack2f(f.x, f.y), acc[0]);
-              acc[1] = fma2(pack2(x[4 * i + 2], x[4 * i + 3]), pack2f(f.z, f.w), acc[1]);
-            }
+              for (int i = 0; i < NC / 4; ++i) {
+                float4 f = f4[i];
+                if constexpr (decltype(masked)::value) {               // the stored 2^x is 0 there, but 0 * NaN is not
+                  f.x = 4 * i >= c_first ? f.x : 0.f;
+                  f.y = 4 * i + 1 >= c_first ? f.y : 0.f;
+                  f.z = 4 * i + 2 >= c_first ? f.z : 0.f;
+                  f.w = 4 * i + 3 >= c_first ? f.w : 0.f;
+                }
+                acc[0] = fma2(pack2(x[4 * i], x[4 * i + 1]), pack2f(f.x, f.y), acc[0]);
+                acc[1] = fma2(pack2(x[4 * i + 2], x[4 * i + 3]), pack2f(f.z, f.w), acc[1]);
+              }
+            };
+            if (edge) add(std::true_type{}); else add(std::false_type{});
           } else {
-            const int c_first = first_col(key) - b * NC;
             float t = 0.f;
 #pragma unroll
             for (int i = 0; i < NC; ++i)

@@ -89,3 +89,34 @@ def test_queries_that_do_not_vote_have_no_influence_on_the_cuda_cores(B):
     got, got_lse = _score(B, q, k, (L,), B.SCORE_SIMT, window=window)
     np.testing.assert_array_equal(got, want)
     np.testing.assert_array_equal(got_lse, want_lse)
+
+
+@pytest.mark.parametrize("L,window,p", [(100, 16, 50), (1000, 64, 0), (4000, 33, 3333), (300, 64, 290)])
+def test_nan_key_reaches_every_voting_row_of_a_window(B, L, window, p):
+    import torch
+    q, k = _normal((2, L, 4, 128), 7, torch.bfloat16), _normal((2, L, 4, 128), 8, torch.bfloat16)
+    k[:, p] = float("nan")
+    s, lse = _score(B, q, k, (L,), B.SCORE_TENSOR, window=window)
+    first = max(L - window, p)                                  # first voting row that sees the key
+    assert np.isfinite(lse[..., L - window:first]).all() and np.isnan(lse[..., first:]).all()
+    assert (lse[..., :L - window] == 7.0).all()
+    assert np.isnan(s).all()
+
+
+@pytest.mark.parametrize("what", ["nan", "inf"])
+def test_a_query_without_finite_sum_touches_the_keys_it_sees_only(B, what):
+    """A NaN query, and one with a single logit of +inf (no other of its logits is out of range).  Blocks that see the NaN
+    recompute their weights instead of reading stored ones, a quarter of which come from a polynomial of 7.5e-5."""
+    import torch
+    L, window, j = 300, 64, 270
+    q, k = _normal((1, L, 2, 64), 9, torch.bfloat16), _normal((1, L, 2, 64), 10, torch.bfloat16)
+    q[..., 0], k[..., 0] = 0.0, 0.0
+    want, _ = _score(B, q, k, (L,), B.SCORE_TENSOR, window=window)
+    if what == "nan":
+        q[:, j] = float("nan")
+    else:
+        q[:, j, :, 0], k[:, 17, :, 0] = 1e30, 1e30
+    s, lse = _score(B, q, k, (L,), B.SCORE_TENSOR, window=window)
+    assert np.isnan(lse[..., j]).all() and np.isfinite(np.delete(lse, j, axis=-1)).all()
+    assert np.isnan(s[..., :j + 1]).all()
+    np.testing.assert_allclose(s[..., j + 1:], want[..., j + 1:], rtol=1e-4)
