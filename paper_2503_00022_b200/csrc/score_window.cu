@@ -18,7 +18,8 @@
 //
 // 2^x is taken without a maximum: float32 has the range unless logits are extreme.  32 keys x one column block whose
 // logits leave [-100, 100] or hold a NaN keep them, count with their exact maxima in step 1 and take 2^(x - lse2) in step 2.
-// So a stored 2^x is finite; a query's sum may be NaN, and is then NaN in every key it votes for, and in no other.
+// So a stored 2^x is finite; a query's sum may be NaN, and is then NaN in every key it votes for, and in no other.  For a
+// query whose lse2 is above 126, 2^-lse2 would be flushed to zero: the stored 2^x are multiplied by its square root twice.
 //
 // Roles: warp 0 issues TMA loads, warp 1 the tcgen05.mma; warps 2..17 are four epilogue groups of four warps.  All waits
 // are bounded as in score_tc.cu; all CTAs of a cluster meet once more before they leave, because peers write into their
@@ -487,6 +488,9 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
       // ---- step 2: every key's sum over the queries ----
       tc_fence_after();
+      bool deep = false;                            // a query with lse2 > 126 (its factor is zero)
+      for (int c = lane; c < w.nv; c += 32) deep |= aux->nlse[c] < -126.f;
+      deep = __any_sync(0xFFFFFFFFu, deep);
       for (int j = gi; j < w.n; j += 4) {
         const int key = (w.tile0 + j) * kTile + r;
         const uint32_t t_acc = t_lane + j * n_pad;
@@ -497,7 +501,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           tmem_ldn(t_acc + b * NC, x);
           tmem_waitn(x);
           const int c_first = first_col(key) - b * NC;
-          if (!aux->kept[j][b][quarter]) {
+          if (!deep && !aux->kept[j][b][quarter]) {
             const float4* f4 = reinterpret_cast<const float4*>(aux->factor + b * NC);
             auto add = [&](auto masked) {
 #pragma unroll
@@ -515,10 +519,17 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             };
             if (edge) add(std::true_type{}); else add(std::false_type{});
           } else {
+            const bool keep = aux->kept[j][b][quarter];
             float t = 0.f;
 #pragma unroll
-            for (int i = 0; i < NC; ++i)
-              t += i >= c_first ? ex2(fmaf(__uint_as_float(x[i]), scale, aux->nlse[b * NC + i])) : 0.f;
+            for (int i = 0; i < NC; ++i) {
+              const float x_i = __uint_as_float(x[i]), nl = aux->nlse[b * NC + i];
+              float e;
+              if (keep) e = ex2(fmaf(x_i, scale, nl));
+              else if (nl < -126.f) { const float root = ex2(0.5f * nl); e = x_i * root * root; }
+              else e = x_i * aux->factor[b * NC + i];
+              t += i >= c_first ? e : 0.f;
+            }
             acc[0] = add2(acc[0], pack2f(t, 0.f));
           }
         }

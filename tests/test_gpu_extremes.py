@@ -120,3 +120,21 @@ def test_a_query_without_finite_sum_touches_the_keys_it_sees_only(B, what):
     assert np.isnan(lse[..., j]).all() and np.isfinite(np.delete(lse, j, axis=-1)).all()
     assert np.isnan(s[..., :j + 1]).all()
     np.testing.assert_allclose(s[..., j + 1:], want[..., j + 1:], rtol=1e-4)
+
+
+@pytest.mark.parametrize("window,shallow", [(16, 0), (40, 0), (16, 8), (40, 20)])
+def test_small_weights_of_a_window_keep_their_value_beside_a_huge_logit(B, window, shallow):
+    """32 keys with logits of 110 (2^158) fill one block; the others' logits of 60 to 63 stay in the range that is stored as
+    2^x.  Their weights of e^-50 have to come out as such: exponentials of 7.5e-5, logits rounded by 2^-24 of 158.  The first
+    `shallow` of the voting queries see half of every logit."""
+    import torch
+    L = 512
+    q, k = torch.zeros((1, L, 1, 64), device="cuda:0"), torch.zeros((1, L, 1, 64), device="cuda:0")
+    q[..., 0] = 1.0
+    q[:, L - window:L - window + shallow, :, 0] = 0.5
+    k[0, :, 0, 0] = 60.0 + 0.25 * (torch.arange(L, device="cuda:0") % 13)
+    k[0, 64:96, 0, 0] = 110.0
+    q, k = q.to(torch.bfloat16), k.to(torch.bfloat16)
+    s, _ = _score(B, q, k, (L,), B.SCORE_TENSOR, window=window, scale=1.0)
+    want, _ = O.scores(q[0].double().cpu().numpy(), k[0].double().cpu().numpy(), True, scale=1.0, rows=(L - window, L))
+    np.testing.assert_allclose(s[0, 0], want[0], rtol=3e-4)
