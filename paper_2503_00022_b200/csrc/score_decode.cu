@@ -159,6 +159,8 @@ decode_update_kernel(Shape s, TensorView Qn, TensorView K, float scale_log2, flo
   const int lo = min(L, rank * per * kRows), hi = min(L, lo + per * kRows);
   const T* kbase = static_cast<const T*>(K.ptr) + layer * K.sl + hk * K.sh + (long long)t0 * K.st;
   const float ninf = __int_as_float(0xFF800000);
+  // What a logit's exponential is relative to.  Without a maximum all logits are -inf, which adds 0, or NaN, which has to stay.
+  auto reference = [&](float maximum) { return maximum == ninf ? 0.f : maximum; };
 
   int parity = 0;
   for (int g0 = 0; g0 < s.G; g0 += kHeads, parity ^= 1) {          // the group's query heads, 8 at a time
@@ -195,7 +197,7 @@ decode_update_kernel(Shape s, TensorView Qn, TensorView K, float scale_log2, flo
             sum[i & 1] = sum[i & 1] * exp2f(mx[i & 1] - v) + 1.f;
             mx[i & 1] = v;
           } else {
-            sum[i & 1] += exp2f(v - mx[i & 1]);
+            sum[i & 1] += exp2f(v - reference(mx[i & 1]));
           }
         }
       }
@@ -206,7 +208,7 @@ decode_update_kernel(Shape s, TensorView Qn, TensorView K, float scale_log2, flo
 #pragma unroll
       for (int d = 4; d < 32; d <<= 1) big = fmaxf(big, __shfl_xor_sync(kAll, big, d));
       if constexpr (!kStore) {
-        float p = mx[j] == ninf ? 0.f : sum[j] * exp2f(mx[j] - big);
+        float p = sum[j] == 0.f ? 0.f : sum[j] * exp2f(mx[j] - big);
 #pragma unroll
         for (int d = 4; d < 32; d <<= 1) p += __shfl_xor_sync(kAll, p, d);
         if (g == 0) red[1][2 * c + j][warp] = p;
@@ -222,8 +224,9 @@ decode_update_kernel(Shape s, TensorView Qn, TensorView K, float scale_log2, flo
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) m = fmaxf(m, red[0][h][w]);
         float p = 0.f;
+        const float ref = reference(m);
         for (int i = tid; i < hi - lo; i += kWarps * 32) {
-          const float e = exp2f(x_sh[h * cap + i] - m);
+          const float e = exp2f(x_sh[h * cap + i] - ref);
           x_sh[h * cap + i] = e;
           p += e;
         }
@@ -238,9 +241,9 @@ decode_update_kernel(Shape s, TensorView Qn, TensorView K, float scale_log2, flo
       for (int w = 0; w < kWarps; ++w) m = fmaxf(m, red[0][tid][w]);
       for (int w = 0; w < kWarps; ++w) {
         const float sw = red[1][tid][w];
-        p += kStore ? sw : red[0][tid][w] == ninf ? 0.f : sw * exp2f(red[0][tid][w] - m);
+        p += kStore ? sw : sw == 0.f ? 0.f : sw * exp2f(red[0][tid][w] - m);
       }
-      part[parity][tid][0] = m;                                    // -inf for a block without keys
+      part[parity][tid][0] = m;                                    // -inf: no key, or none with a logit above -inf
       part[parity][tid][1] = p;
     }
     // also keeps a block from rewriting `part` two passes later while a peer still reads it
@@ -257,7 +260,7 @@ decode_update_kernel(Shape s, TensorView Qn, TensorView K, float scale_log2, flo
       float all_m = m;
 #pragma unroll
       for (int d = 1; d < kMaxCluster; d <<= 1) all_m = fmaxf(all_m, __shfl_xor_sync(kAll, all_m, d));
-      p = m == ninf ? 0.f : p * exp2f(m - all_m);
+      p = p == 0.f ? 0.f : p * exp2f(m - all_m);
 #pragma unroll
       for (int d = 1; d < kMaxCluster; d <<= 1) p += __shfl_xor_sync(kAll, p, d);
       // stored exponentials are relative to this block's maximum

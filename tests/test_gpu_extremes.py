@@ -138,3 +138,28 @@ def test_small_weights_of_a_window_keep_their_value_beside_a_huge_logit(B, windo
     s, _ = _score(B, q, k, (L,), B.SCORE_TENSOR, window=window, scale=1.0)
     want, _ = O.scores(q[0].double().cpu().numpy(), k[0].double().cpu().numpy(), True, scale=1.0, rows=(L - window, L))
     np.testing.assert_allclose(s[0, 0], want[0], rtol=3e-4)
+
+
+@pytest.mark.parametrize("dtype,L,Hq", [("float32", 2048, 2), ("bfloat16", 2048, 2), ("bfloat16", 52000, 8)])
+def test_decode_keys_with_logits_of_minus_infinity_get_no_weight(B, dtype, L, Hq):
+    """A stretch of keys longer than one block's part, and (52000 keys x 8 heads) the variant without stored logits."""
+    import torch
+    q, k = _normal((1, 1, Hq, 64), 11, torch.float32), _normal((1, L, 1, 64), 12, torch.float32)
+    q[..., 0], k[..., 0] = 1e30, 0.0
+    n = L // 8 * 3
+    k[:, n:2 * n, :, 0] = -1e30                                  # product -1e60: -inf in float32
+    q, k = q.to(getattr(torch, dtype)), k.to(getattr(torch, dtype))
+    got = _decode(B, q, k)[0]
+    assert (got[:, n:2 * n] == 0.0).all()
+    rest = torch.cat([k[0, :n], k[0, 2 * n:]]).double().cpu().numpy()
+    want = O.decode_update(np.zeros((Hq, L - n)), q[0, 0].double().cpu().numpy(), rest)
+    np.testing.assert_allclose(np.delete(got, np.s_[n:2 * n], axis=1), want, rtol=1e-4)
+
+
+@pytest.mark.parametrize("L,Hq,first,last", [(2048, 2, 5, 6), (2048, 2, 256, 512), (52000, 8, 5, 6), (52000, 8, 6512, 13024)])
+def test_decode_nan_keys_reach_every_score_of_the_sequence(B, L, Hq, first, last):
+    """A single key, and all the keys of the second of a cluster's eight blocks."""
+    import torch
+    q, k = _normal((1, 1, Hq, 64), 13, torch.bfloat16), _normal((1, L, 1, 64), 14, torch.bfloat16)
+    k[:, first:last] = float("nan")
+    assert np.isnan(_decode(B, q, k)).all()
