@@ -163,3 +163,22 @@ def test_decode_nan_keys_reach_every_score_of_the_sequence(B, L, Hq, first, last
     q, k = _normal((1, 1, Hq, 64), 13, torch.bfloat16), _normal((1, L, 1, 64), 14, torch.bfloat16)
     k[:, first:last] = float("nan")
     assert np.isnan(_decode(B, q, k)).all()
+
+
+def test_decode_adds_weights_below_the_smallest_normal_number(B):
+    """Logits of 0 (one key) and -88 to -100: weights down to e^-100 = 2^-144.  Their last place is 2^-149: two of it from the
+    exponential, half of it each from the factor of the block and from the product.  A second step adds the same again."""
+    import torch
+    L = 400
+    q, k = torch.zeros((1, 1, 1, 8), device="cuda:0"), torch.zeros((1, L, 1, 8), device="cuda:0")
+    q[..., 0] = 1.0
+    k[0, 1:, 0, 0] = -88.0 - 12.0 * torch.arange(1, L, device="cuda:0") / L
+    prob = B.Problem(1, 1, 1, 8, (L,), softmax_scale=1.0, device="cuda:0")
+    scores = torch.zeros((1, 1, L), dtype=torch.float32, device="cuda:0")
+    status = torch.zeros(4, dtype=torch.int32, device="cuda:0")
+    w = np.exp(k[0, :, 0, 0].double().cpu().numpy())
+    w /= w.sum()
+    for n in (1, 2):
+        B.kvcrush_score_decode(prob, q, k, scores, status=status)
+        got = scores.cpu().numpy()[0, 0].astype(np.float64)
+        assert (np.abs(got - n * w) <= 1e-5 * n * w + 3 * n * 2.0 ** -149).all()
