@@ -23,7 +23,7 @@
 //
 // Roles: warp 0 issues TMA loads, warp 1 the tcgen05.mma; warps 2..17 are four epilogue groups of four warps.  All waits
 // are bounded as in score_tc.cu; all CTAs of a cluster meet once more before they leave, because peers write into their
-// shared memory.
+// shared memory, and one that gave up then waits for the stores that were on their way to it.
 #include <cuda.h>
 
 #include <atomic>
@@ -60,6 +60,7 @@ struct WinArgs {
   int ring;
   int n_units;               // n_layers * n_seqs * Hq
   int32_t* status;
+  int withhold_first_item;   // diagnostic: the producer stops before its first copy, so that every consumer's first wait runs out
 };
 
 struct WAux {
@@ -69,6 +70,7 @@ struct WAux {
   unsigned long long epi_bar, part_full[2], drain;
   uint32_t tmem_base;
   int abort_flag;
+  int n_unit;                                           // units whose sums this CTA has received
   alignas(16) float nlse[kMaxN];                        // minus log2 sum of the window's queries, -inf: no vote
   alignas(16) float factor[kMaxN];                      // 2^nlse
   unsigned char kept[kMaxSlots][4][4];                  // [tile][column block][lane quarter]: logits were kept
@@ -90,8 +92,8 @@ __device__ __forceinline__ void peer_store_async(uint32_t addr, float v, uint32_
                : "memory");
 }
 // mbar_wait for a barrier that other CTAs complete
-__device__ __forceinline__ bool cluster_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  for (uint32_t i = 0; i < kWaitPolls; ++i) {
+__device__ __forceinline__ bool cluster_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t polls) {
+  for (uint32_t i = 0; i < polls; ++i) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -103,6 +105,16 @@ __device__ __forceinline__ bool cluster_wait(uint32_t bar, uint32_t parity, vola
   }
   *abort_flag = 1;
   return false;
+}
+// one poll of a barrier that other CTAs complete
+__device__ __forceinline__ bool cluster_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
 }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -201,8 +213,8 @@ struct Unit {
   }
 };
 
-// NC: columns of one epilogue thread in step 1.
-template <int D, int NC>
+// NC: columns of one epilogue thread in step 1.  kPolls: polls of every bounded wait.
+template <int D, int NC, uint32_t kPolls>
 __global__ void __launch_bounds__(kThreads, 1)
 score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const WinArgs a) {
   constexpr int kTileBytes = kTile * D * 2, kBlockBytes = kTile * 128;
@@ -239,6 +251,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   }
   chain_wait();
   chain_trigger();
+  if (tid == 0) aux->n_unit = 0;
   if (tid == 0) aux->abort_flag = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
   tc_fence_before();
   __syncthreads();
@@ -254,12 +267,12 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     if (lane == 0) {
       int rs = 0, n_q = 0, n_k = 0;
       uint32_t ph = 0;
-      bool ok = true;
+      bool ok = !a.withhold_first_item;
       for (int u = first_unit; ok && u < a.n_units; u += unit_step) {
         const Unit w(s, u, rank, n_cta);
         if (w.n == 0) continue;
         const int qs = n_q & 1;
-        ok = mbar_wait(smem_u32(&aux->q_empty[qs]), ((n_q >> 1) & 1) ^ 1, abort_flag, kWaitPolls);
+        ok = mbar_wait(smem_u32(&aux->q_empty[qs]), ((n_q >> 1) & 1) ^ 1, abort_flag, kPolls);
         if (!ok) break;
         mbar_expect_tx(smem_u32(&aux->q_full[qs]), q_bytes);
 #pragma unroll
@@ -267,7 +280,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           tma_load_4d(q_addr + qs * q_bytes + kb * n_pad * 128, &map_q, smem_u32(&aux->q_full[qs]), kb * 64, w.t0 + w.q0, w.h, w.layer);
         ++n_q;
         for (int i = 0; i < w.n; ++i) {
-          ok = mbar_wait(smem_u32(&aux->k_empty[rs]), ph ^ 1, abort_flag, kWaitPolls);
+          ok = mbar_wait(smem_u32(&aux->k_empty[rs]), ph ^ 1, abort_flag, kPolls);
           if (!ok) break;
           mbar_expect_tx(smem_u32(&aux->k_full[rs]), kTileBytes);
 #pragma unroll
@@ -297,10 +310,10 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         const Unit w(s, u, rank, n_cta);
         if (w.n == 0) continue;
         const int qs = n_q & 1;
-        ok = mbar_wait(smem_u32(&aux->q_full[qs]), (n_q >> 1) & 1, abort_flag, kWaitPolls);
+        ok = mbar_wait(smem_u32(&aux->q_full[qs]), (n_q >> 1) & 1, abort_flag, kPolls);
         for (int i = 0; ok && i < w.n; ++i) {
-          ok = mbar_wait(smem_u32(&aux->k_full[rs]), ph, abort_flag, kWaitPolls) &&
-               mbar_wait(smem_u32(&aux->acc_empty[i]), ((used >> i) & 1) ^ 1, abort_flag, kWaitPolls);
+          ok = mbar_wait(smem_u32(&aux->k_full[rs]), ph, abort_flag, kPolls) &&
+               mbar_wait(smem_u32(&aux->acc_empty[i]), ((used >> i) & 1) ^ 1, abort_flag, kPolls);
           if (!ok) break;
           used ^= 1u << i;
           tc_fence_after();
@@ -339,12 +352,12 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     auto epi_sync = [&]() {
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&aux->epi_bar));
-      ok = mbar_wait(smem_u32(&aux->epi_bar), n_sync & 1, abort_flag, kWaitPolls) && ok;
+      ok = mbar_wait(smem_u32(&aux->epi_bar), n_sync & 1, abort_flag, kPolls) && ok;
       ++n_sync;
       ok = __all_sync(0xFFFFFFFFu, ok);
     };
     auto wait_acc = [&](int i) {
-      ok = mbar_wait(smem_u32(&aux->acc_full[i]), (used >> i) & 1, abort_flag, kWaitPolls) && ok;
+      ok = mbar_wait(smem_u32(&aux->acc_full[i]), (used >> i) & 1, abort_flag, kPolls) && ok;
       ok = __all_sync(0xFFFFFFFFu, ok);
       tc_fence_after();
       return ok;
@@ -464,7 +477,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         }
       }
       if (n_cta > 1) {
-        ok = cluster_wait(smem_u32(&aux->part_full[par]), (n_unit >> 1) & 1, abort_flag) && ok;
+        ok = cluster_wait(smem_u32(&aux->part_full[par]), (n_unit >> 1) & 1, abort_flag, kPolls) && ok;
         ok = __all_sync(0xFFFFFFFFu, ok);
       }
       if (col < n_pad) {
@@ -545,26 +558,34 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       if (w.n > 0) used ^= 0xFFFFFFFFu >> (32 - w.n);
       ++n_unit;
     }
+    if (et == 0) aux->n_unit = n_unit;
   }
 
   __syncwarp();
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();                               // nobody leaves while a peer may still write into its shared memory
+  if (tid == 0 && n_cta > 1 && *abort_flag) {
+    // The barrier does not order the peers' asynchronous stores.  After it none of them sends any more, and what they have
+    // sent belongs to the unit this CTA gave up in or the next: a bounded time for it to land.  (A CTA that did not give
+    // up has received everything that is sent to it.)
+    for (int u = aux->n_unit; u < aux->n_unit + 2; ++u)
+      for (uint32_t i = 0; i < kDrainPolls && !cluster_test(smem_u32(&aux->part_full[u & 1]), (u >> 1) & 1); ++i) {}
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kCols);
   }
-  if (tid == 0 && !dead && *abort_flag) report(a.status, KVCRUSH_DEV_TIMEOUT, KID_SCORE_COLSUM, blockIdx.x, 0);
+  if (tid == 0 && !dead && *abort_flag) report(a.status, KVCRUSH_DEV_TIMEOUT, KID_SCORE_WINDOW, blockIdx.x, 0);
 }
 
 constexpr int kMaxDevices = 64;
 
 // Clusters of n_cta blocks that run at the same time (write-once cache per device: the answer depends on nothing else).
-template <int D, int NC>
+template <int D, int NC, uint32_t kPolls>
 int resident_clusters(int log_cta, int smem) {
   static std::atomic<int> known[kMaxDevices][4];
-  auto kern = score_window_kernel<D, NC>;
+  auto kern = score_window_kernel<D, NC, kPolls>;
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
   if ((n = known[dev][log_cta].load(std::memory_order_relaxed)) > 0) return n;
@@ -586,15 +607,21 @@ int resident_clusters(int log_cta, int smem) {
   return n;
 }
 
-template <int D, int NC>
-int launch_window(const CUtensorMap& mq, const CUtensorMap& mk, const WinArgs& a, int log_cta, cudaStream_t stream) {
+template <int D, int NC, uint32_t kPolls>
+int launch_window_polls(const CUtensorMap& mq, const CUtensorMap& mk, const WinArgs& a, int log_cta, cudaStream_t stream) {
   constexpr int smem = kSmemTiles * kTile * D * 2 + kAuxBytes + 1024;
-  auto kern = score_window_kernel<D, NC>;
-  const int clusters = resident_clusters<D, NC>(log_cta, smem);
+  auto kern = score_window_kernel<D, NC, kPolls>;
+  const int clusters = resident_clusters<D, NC, kPolls>(log_cta, smem);
   if (clusters < 1) return KVCRUSH_ERR_UNSUPPORTED;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return KVCRUSH_ERR_CUDA;
   const int n = clusters < a.n_units ? clusters : a.n_units;
   return launch_chained(kern, dim3((unsigned)n << log_cta), dim3(kThreads), smem, stream, 1 << log_cta, mq, mk, a);
+}
+
+template <int D, int NC>
+int launch_window(const CUtensorMap& mq, const CUtensorMap& mk, const WinArgs& a, int log_cta, bool short_waits, cudaStream_t stream) {
+  return short_waits ? launch_window_polls<D, NC, kShortWaitPolls>(mq, mk, a, log_cta, stream)
+                     : launch_window_polls<D, NC, kWaitPolls>(mq, mk, a, log_cta, stream);
 }
 
 }  // namespace
@@ -610,7 +637,7 @@ bool score_window_fits(const Shape& s) {
 }
 
 int launch_score_window(const Shape& s, const TensorView& Q, const ScoreTensorMaps& maps, float scale_log2, float* scores,
-                        float* lse_out, int normalize, int32_t* status, cudaStream_t stream) {
+                        float* lse_out, int normalize, int32_t* status, const ScoreDiag& diag, cudaStream_t stream) {
   int dev = 0, n_sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sms < 1)
@@ -618,6 +645,7 @@ int launch_score_window(const Shape& s, const TensorView& Q, const ScoreTensorMa
   WinArgs a{};
   a.s = s; a.scale_log2 = scale_log2; a.lse_nat_out = lse_out; a.scores = scores; a.normalize = normalize;
   a.bf16 = Q.dtype == KVCRUSH_BF16; a.status = status; a.k_steps = (s.D + 15) / 16;
+  a.withhold_first_item = diag.withhold_first_item;
   a.n_units = s.n_layers * s.n_seqs * s.Hq;
   a.n_pad = 16;
   while (a.n_pad < s.window) a.n_pad *= 2;
@@ -630,8 +658,9 @@ int launch_score_window(const Shape& s, const TensorView& Q, const ScoreTensorMa
   int log_cta = 0;
   auto per = [&]() { return (tiles + (1 << log_cta) - 1) >> log_cta; };
   while (log_cta < 3 && (per() * a.n_pad > kCols || (per() > 1 && (a.n_units << (log_cta + 1)) <= n_sms))) ++log_cta;
-  if (s.D > 64) return a.n_pad == 16 ? launch_window<128, 16>(mq, mk, a, log_cta, stream) : launch_window<128, 32>(mq, mk, a, log_cta, stream);
-  return a.n_pad == 16 ? launch_window<64, 16>(mq, mk, a, log_cta, stream) : launch_window<64, 32>(mq, mk, a, log_cta, stream);
+  const bool sw = diag.short_waits != 0;
+  if (s.D > 64) return a.n_pad == 16 ? launch_window<128, 16>(mq, mk, a, log_cta, sw, stream) : launch_window<128, 32>(mq, mk, a, log_cta, sw, stream);
+  return a.n_pad == 16 ? launch_window<64, 16>(mq, mk, a, log_cta, sw, stream) : launch_window<64, 32>(mq, mk, a, log_cta, sw, stream);
 }
 
 }  // namespace kvc

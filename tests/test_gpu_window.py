@@ -112,6 +112,49 @@ def test_one_pass_window_scores_match_oracle(B, layers, Hq, Hkv, D, seqlens, win
             assert (gl[l][:, a:a + j0] == 7.0).all()
 
 
+@pytest.mark.parametrize("L,window", [
+    (100, 16),                                            # one CTA alone
+    (1000, 64),                                           # a cluster of 8, one tile of keys each
+    (1100, 64),                                           # a cluster of 8, three CTAs without keys: their sums are on the way
+])
+def test_one_pass_window_waits_that_run_out_are_reported(B, L, window):
+    """The bounded waits of the one-pass window kernel, made to run out through the library's diagnostic entry point: no CTA
+    issues a copy, so every CTA's consumers give up, the clusters meet, tensor memory is freed and the kernel (id 4: the
+    dispatch took this one) returns with the status word set and the outputs untouched.  Afterwards the public entry point
+    gives the oracle's scores on the same context."""
+    import ctypes
+    import torch
+    dev = _dev()
+    fn = B.lib().kvcrush_diag_score
+    vp, i32 = ctypes.c_void_p, ctypes.c_int
+    fn.restype = i32
+    fn.argtypes = [ctypes.POINTER(B.ProblemStruct), ctypes.POINTER(B.TensorStruct), ctypes.POINTER(B.TensorStruct),
+                   vp, vp, vp, i32, i32, vp, ctypes.c_size_t, vp, vp, i32, i32]
+    w = inputs.Workload("win_out", 1, 1, 1, 128, (L,), inputs.BF16, inputs.BF16, 0.25, base_seed=56)
+    lis, q, k, _, _ = TL.stack_layers(w, range(1), with_cache=False)
+    prob = B.Problem(1, 1, 1, 128, w.seqlens, device=dev, query_window=window)
+    dq, dk = TL.torch_storage(q, w.qk_dtype, dev), TL.torch_storage(k, w.qk_dtype, dev)
+    qs, ks = B.tensor_struct(dq), B.tensor_struct(dk)
+    scores = torch.full((1, 1, L), -5.0, dtype=torch.float32, device=dev)
+    lse = torch.full_like(scores, -7.0)
+    ws = torch.empty(B.kvcrush_workspace_size(prob, B.STAGE_SCORE), dtype=torch.uint8, device=dev)
+    status = torch.zeros(4, dtype=torch.int32, device=dev)
+    stream = int(torch.cuda.current_stream().cuda_stream)
+    rc = fn(prob.ref, ctypes.byref(qs), ctypes.byref(ks), None, scores.data_ptr(), lse.data_ptr(), 0, B.SCORE_TENSOR,
+            ws.data_ptr(), ws.numel(), status.data_ptr(), stream, 1, 1)
+    assert rc == B.OK
+    torch.cuda.synchronize()
+    st = status.cpu().tolist()
+    assert st[0] == B.DEV_TIMEOUT and st[1] == 4 and 0 <= st[2] < 8, st
+    assert bool((scores == -5.0).all()) and bool((lse == -7.0).all())
+    status.zero_()
+    B.kvcrush_score(prob, dq, dk, scores, lse_out=lse, workspace=ws, status=status)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist()[0] == 0
+    c, _ = O.scores(inputs.widen(lis[0].q, w.qk_dtype), inputs.widen(lis[0].k, w.qk_dtype), True, rows=(L - window, L))
+    assert TL.within_score_tolerance(scores.cpu().numpy()[0], c).all()
+
+
 @pytest.mark.parametrize("kernel", [1, 3, 7, 33])
 def test_pooling_is_bit_exact(B, kernel):
     import torch
