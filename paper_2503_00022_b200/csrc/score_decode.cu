@@ -139,7 +139,7 @@ template <typename T, int DB, int kWarps, bool kStore>
 __global__ void __launch_bounds__(kWarps * 32)
 decode_update_kernel(Shape s, TensorView Qn, TensorView K, float scale_log2, float* __restrict__ scores, int cap) {
   extern __shared__ float x_sh[];                                  // [heads of the pass][cap]
-  __shared__ float q_sh[sizeof(T) == 4 ? kHeads * kMaxD : 1];
+  __shared__ alignas(16) float q_sh[sizeof(T) == 4 ? kHeads * kMaxD : 4];   // read as float4
   __shared__ float red[2][kHeads][kWarps];
   __shared__ float part[2][kHeads][2];                             // [pass parity][head]: maximum, sum of this block
   __shared__ float fin[kHeads];                                    // factor of the stored exponentials, or log-sum-exp

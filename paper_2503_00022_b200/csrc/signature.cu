@@ -140,7 +140,7 @@ constexpr int kListKeys = 1024;
 __global__ void __launch_bounds__(1024, 2)
 theta_upper_kernel(Shape s, const float* __restrict__ scores, const int32_t* __restrict__ sig_keep, float* __restrict__ theta) {
   constexpr int kT = 1024;
-  extern __shared__ uint16_t upper[];             // [max_seqlen]
+  extern __shared__ __align__(16) uint16_t upper[];   // [max_seqlen], read in pairs
   __shared__ alignas(16) uint32_t hist[kThetaBins];
   __shared__ uint32_t list[kListKeys];
   __shared__ uint32_t red[32], list_n, found[3];
