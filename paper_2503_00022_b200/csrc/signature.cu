@@ -541,7 +541,7 @@ int launch_signature(const Shape& s, const float* scores, const int32_t* sig_kee
   // 16-byte loads need every (layer, head) row to start on a 16-byte boundary
   const int vec_ok = s.T % 4 == 0 && reinterpret_cast<uintptr_t>(scores) % 16 == 0;
   auto kern = importance ? signature_pack_kernel<true> : signature_pack_kernel<false>;
-  if (dyn > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
+  if (dyn > 40 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
     return KVCRUSH_ERR_CUDA;
   return launch_chained(kern, grid, dim3(kPackTok), dyn, stream, 1, s, scores, th, sigs, importance, vec_ok);
 }

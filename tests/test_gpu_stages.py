@@ -77,6 +77,9 @@ def _select_case(B, Hq, Hkv, seqlens, budgets, n_layers, ties, mode, seed, sig_k
     (40, 10, [777, 1025], [(64, 32), (100, 101)], 2, 1),           # two signature words, MEAN anchor
     (128, 16, [600], [(50, 70)], 0, 2),                            # four words, explicit (random) anchor
     (4, 1, [300, 300], [(0, 30), (30, 0)], 3, 0),                  # pure KVCrush / pure H2O
+    (95, 95, [300], [(40, 30)], 0, 0),                             # a tile of scores just below, at and above 48 KB of
+    (96, 96, [300], [(40, 30)], 0, 0),                             # shared memory
+    (97, 97, [300], [(40, 30)], 0, 0),
     (16, 16, [100, 1, 64], [(60, 60), (1, 0), (3, 1)], 0, 1),      # budget >= length keeps all; L = 1
     (32, 32, [5000], [(10, 1)], 0, 0),                             # one huge bucket
     (32, 32, [2500], [(20, 2)], 2, 1),
