@@ -97,6 +97,16 @@ int launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t dyn_
   return KVCRUSH_OK;
 }
 
+// Lets a kernel be launched with up to `bound` bytes of dynamic shared memory.  The attribute belongs to the kernel, not to
+// the launch, so every call sets the same bound: with the size of the launch at hand, two threads with different sizes took
+// the larger one's permission away between setting it and launching.
+template <class Kernel>
+int allow_dynamic_smem(Kernel kernel, int bound) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bound) == cudaSuccess) return KVCRUSH_OK;
+  cudaGetLastError();
+  return KVCRUSH_ERR_CUDA;
+}
+
 // ---- stage launchers (defined in the per-stage .cu files) -------------------------------------------
 
 // score: SIMT fp32 kernels (any dtype/shape) and tcgen05 kernels (bf16 or fp16, D a multiple of 8 up to 128).

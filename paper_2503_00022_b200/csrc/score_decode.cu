@@ -31,6 +31,7 @@ constexpr int kHeads = 8;                    // query heads of one pass over the
 constexpr int kRows = 16;                    // keys of one tile
 constexpr int kMaxCluster = 8;
 constexpr int kMaxD = 256;
+constexpr int kMaxStored = 200 * 1024;       // bytes of logits a block keeps in shared memory, at most
 constexpr unsigned kAll = 0xFFFFFFFFu;
 
 // One tile: keys t .. t+15 (rows beyond t_end read as zeros) against 8 heads.  Lane = 4 * g + c holds the pieces of keys g
@@ -305,9 +306,7 @@ template <typename T, int DB, int kWarps, bool kStore>
 int launch_one(const Shape& s, const TensorView& Qn, const TensorView& K, float scale_log2, float* scores, int n_blk, int cap,
                size_t dyn, cudaStream_t stream) {
   auto kern = decode_update_kernel<T, DB, kWarps, kStore>;
-  if (dyn > 32 * 1024 &&
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-    return KVCRUSH_ERR_CUDA;
+  if (dyn > 32 * 1024 && allow_dynamic_smem(kern, kMaxStored) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
   return launch_chained(kern, dim3((unsigned)((long long)s.n_layers * s.n_seqs * s.Hkv * n_blk)), dim3(kWarps * 32), dyn, stream,
                         n_blk, s, Qn, K, scale_log2, scores, cap);
 }
@@ -329,7 +328,7 @@ int launch_width(const Shape& s, const TensorView& Qn, const TensorView& K, floa
   // Small blocks, so that while some of an SM's blocks exchange sums and write, the others read: 4 warps 351 us against
   // 358 us with 8 at 32 x 32 x 8192 keys, 169 against 214 us at 32 x 16 x 680 keys.  Where only one or two blocks fit
   // an SM it takes 8 warps to have enough loads in flight.
-  if (dyn > 200 * 1024) return launch_one<T, DB, 4, false>(s, Qn, K, scale_log2, scores, n_blk, cap, 0, stream);
+  if (dyn > kMaxStored) return launch_one<T, DB, 4, false>(s, Qn, K, scale_log2, scores, n_blk, cap, 0, stream);
   if (dyn > 64 * 1024) return launch_one<T, DB, 8, true>(s, Qn, K, scale_log2, scores, n_blk, cap, dyn, stream);
   return launch_one<T, DB, 4, true>(s, Qn, K, scale_log2, scores, n_blk, cap, dyn, stream);
 }

@@ -213,8 +213,7 @@ int launch_sweep(const Shape& s, const TensorView& Q, const TensorView& K, float
   if (units * n_blk > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
   const size_t dyn = (size_t)2 * kRows * (s.D + kPad) * sizeof(float);
   auto kern = simt_sweep_kernel<T, kColsum>;
-  if (dyn > 40 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-    return KVCRUSH_ERR_CUDA;
+  if (dyn > 40 * 1024 && allow_dynamic_smem(kern, 2 * kRows * (kMaxD + kPad) * (int)sizeof(float)) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
   return launch_chained(kern, dim3((unsigned)(units * n_blk)), dim3(kThreads), dyn, stream, n_blk, s, Q, K, scale_log2, lse, lse_mul,
                         lse2_out, lse_nat_out, scores, normalize, max_tiles);
 }

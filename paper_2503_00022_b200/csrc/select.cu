@@ -508,8 +508,7 @@ int launch_select(const Shape& s, const float* scores, const double* importance,
   }
   auto launch = [&](auto kern, int threads) {
     // static + dynamic shared memory above the 48 KB default needs the opt-in
-    if (dyn > 28 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-      return (int)KVCRUSH_ERR_CUDA;
+    if (dyn > 28 * 1024 && allow_dynamic_smem(kern, (int)budget) != KVCRUSH_OK) return (int)KVCRUSH_ERR_CUDA;
     return launch_chained(kern, dim3((unsigned)(s.n_layers * s.n_seqs)), dim3(threads), dyn, stream, 1, s, a);
   };
   // Threads of a segment: 1024 while every segment has an SM to itself (32 x 8192 tokens 22 us, with 512 threads 27), half as

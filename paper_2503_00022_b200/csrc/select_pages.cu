@@ -247,9 +247,7 @@ int launch_pages(const Shape& s, PageArgs a, size_t fixed, cudaStream_t stream) 
   if (a.n_workers > kT / 32) a.n_workers = kT / 32;
   if (a.n_workers < 2) return KVCRUSH_ERR_UNSUPPORTED;
   const size_t dyn = fixed + per_worker * a.n_workers;
-  if (dyn > 32 * 1024 &&
-      cudaFuncSetAttribute(select_pages_kernel<kT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-    return KVCRUSH_ERR_CUDA;
+  if (dyn > 32 * 1024 && allow_dynamic_smem(select_pages_kernel<kT>, (int)budget) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
   return launch_chained(select_pages_kernel<kT>, dim3((unsigned)(s.n_layers * s.n_seqs)), dim3(kT), dyn, stream, 1, s, a);
 }
 

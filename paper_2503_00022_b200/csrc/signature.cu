@@ -520,17 +520,15 @@ int launch_signature(const Shape& s, const float* scores, const int32_t* sig_kee
     else if (m <= 8192) rc = by_block(theta_select_kernel<512, 16, 4>, 512);
     else if (m <= 32768) {
       const size_t dyn = ((size_t)m * sizeof(uint16_t) + 15) / 16 * 16;
-      if (cudaFuncSetAttribute(theta_upper_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-        return KVCRUSH_ERR_CUDA;
+      if (allow_dynamic_smem(theta_upper_kernel, 32768 * (int)sizeof(uint16_t)) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
       rc = launch_chained(theta_upper_kernel, dim3(blocks), dim3(1024), dyn, stream, 1, s, scores, sig_keep, theta);
     }
     else {
       const size_t row_bytes = (size_t)m * sizeof(uint32_t);
-      const int stage_row = row_bytes <= 200 * 1024;
+      constexpr int kMaxRow = 200 * 1024;
+      const int stage_row = row_bytes <= kMaxRow;
       const size_t dyn = stage_row ? row_bytes : 0;
-      if (dyn > 40 * 1024 &&
-          cudaFuncSetAttribute(theta_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-        return KVCRUSH_ERR_CUDA;
+      if (stage_row && allow_dynamic_smem(theta_stream_kernel, kMaxRow) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
       rc = launch_chained(theta_stream_kernel, dim3(blocks), dim3(kSelectThreads), dyn, stream, 1, s, scores, sig_keep, theta, stage_row);
     }
     if (rc != KVCRUSH_OK) return rc;
@@ -541,8 +539,7 @@ int launch_signature(const Shape& s, const float* scores, const int32_t* sig_kee
   // 16-byte loads need every (layer, head) row to start on a 16-byte boundary
   const int vec_ok = s.T % 4 == 0 && reinterpret_cast<uintptr_t>(scores) % 16 == 0;
   auto kern = importance ? signature_pack_kernel<true> : signature_pack_kernel<false>;
-  if (dyn > 40 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-    return KVCRUSH_ERR_CUDA;
+  if (dyn > 40 * 1024 && allow_dynamic_smem(kern, 128 * kPackTok * (int)sizeof(float)) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
   return launch_chained(kern, grid, dim3(kPackTok), dyn, stream, 1, s, scores, th, sigs, importance, vec_ok);
 }
 

@@ -457,6 +457,58 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_context_stays_usable(B
     np.testing.assert_allclose(lse.cpu().numpy()[0], ol, rtol=0, atol=2e-4)
 
 
+@pytest.mark.parametrize("stage,small,large", [("signature", 9000, 32000), ("decode", 24000, 40000), ("simt", 128, 256)])
+def test_threads_with_different_sizes_do_not_take_each_others_launches_away(B, stage, small, large):
+    """Two threads issue calls whose kernels take different amounts of dynamic shared memory, on streams of their own, by raw
+    calls and with a short interpreter switch interval, so that they meet between setting the kernel's limit and launching."""
+    import ctypes
+    import sys
+    import threading
+    import torch
+    dev, lib = _dev(), B.lib()
+
+    def job(n):
+        stream, status = torch.cuda.Stream(), torch.zeros(4, dtype=torch.int32, device=dev)
+        tail = (status.data_ptr(), ctypes.c_void_p(stream.cuda_stream))
+        if stage == "signature":
+            prob = B.Problem(1, 1, 1, 16, [n], device=dev)
+            bufs = (torch.rand((1, 1, n), device=dev), torch.tensor([[n // 4]], dtype=torch.int32, device=dev),
+                    torch.empty((1, n, 1), dtype=torch.int32, device=dev), torch.empty((1, 1, 1), device=dev))
+            sc, keep, sigs, theta = (x.data_ptr() for x in bufs)
+            fn, args = lib.kvcrush_signature, (prob.ref, sc, keep, None, sigs, theta, None, None, 0, *tail)
+        elif stage == "decode":
+            prob = B.Problem(1, 8, 1, 64, [n], device=dev)
+            bufs = (torch.ones((1, 1, 8, 64), dtype=torch.bfloat16, device=dev), torch.ones((1, n, 1, 64), dtype=torch.bfloat16, device=dev),
+                    torch.zeros((1, 8, n), device=dev))
+            views = B.tensor_struct(bufs[0]), B.tensor_struct(bufs[1])
+            fn, args = lib.kvcrush_score_decode, (prob.ref, *map(ctypes.byref, views), bufs[2].data_ptr(), *tail)
+        else:
+            prob = B.Problem(1, 1, 1, n, [64], device=dev)
+            bufs = (torch.ones((1, 64, 1, n), device=dev), torch.empty((1, 1, 64), device=dev),
+                    torch.empty(B.kvcrush_workspace_size(prob, B.STAGE_SCORE), dtype=torch.uint8, device=dev))
+            view = B.tensor_struct(bufs[0])
+            fn, args = lib.kvcrush_score, (prob.ref, ctypes.byref(view), ctypes.byref(view), None, bufs[1].data_ptr(), None, 0,
+                                           B.SCORE_SIMT, bufs[2].data_ptr(), bufs[2].numel(), *tail)
+        return lambda: fn(*args), (prob, bufs, status, stream)
+
+    jobs = [job(small), job(large)]
+    assert all(call() == B.OK for call, _ in jobs)
+    torch.cuda.synchronize()
+    failed = []
+    interval = sys.getswitchinterval()
+    sys.setswitchinterval(1e-6)
+    try:
+        threads = [threading.Thread(target=lambda c=call: failed.append(sum(c() != B.OK for _ in range(20000)))) for call, _ in jobs]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+    finally:
+        sys.setswitchinterval(interval)
+    torch.cuda.synchronize()
+    assert failed == [0, 0]
+
+
 def test_pass_replays_from_a_cuda_graph(B):
     """The four stages enqueue kernels and one memset only, so a pass can be recorded once and replayed on new
     contents of the same tensors; the replayed result equals a direct run."""
