@@ -107,8 +107,8 @@ int score_entry(const kvcrush_problem_t* problem, const kvcrush_tensor_t* Q, con
   if (plan == TENSOR_PLAN_NO_ENCODER) return KVCRUSH_ERR_UNSUPPORTED;
   if (plan == TENSOR_PLAN_NO) {
     if (impl == KVCRUSH_SCORE_TENSOR) return KVCRUSH_ERR_UNSUPPORTED;
-    return launch_score_simt(s, q, k, scale_log2, lse_in_dev, log2e, lse2_ws, scores_dev, lse_out_dev, normalize,
-                             status_dev, st);
+    return launch_score_simt(s, problem->cu_seqlens_host, q, k, scale_log2, lse_in_dev, log2e, lse2_ws, scores_dev, lse_out_dev,
+                             normalize, status_dev, st);
   }
   return launch_score_tensor(s, problem->cu_seqlens_host, q, maps, scale_log2, lse_in_dev, log2e, lse2_ws, counters,
                              scores_dev, lse_out_dev, normalize, status_dev, diag, st);

@@ -111,7 +111,7 @@ int allow_dynamic_smem(Kernel kernel, int bound) {
 
 // score: SIMT fp32 kernels (any dtype/shape) and tcgen05 kernels (bf16 or fp16, D a multiple of 8 up to 128).
 // lse2_ws: [n_layers][Hq][T] float32 row log-sum-exp in the log2 domain (written unless lse_in is given).
-int launch_score_simt(const Shape& s, const TensorView& Q, const TensorView& K, float scale_log2,
+int launch_score_simt(const Shape& s, const int32_t* cu_host, const TensorView& Q, const TensorView& K, float scale_log2,
                       const float* lse_in, float lse_in_mul, float* lse2_ws, float* scores, float* lse_out,
                       int normalize, int32_t* status, cudaStream_t stream);
 // Decode step: scores[l][h][t] += attention of sequence(t)'s new query (Q_new's token axis = sequence) to key t.

@@ -79,11 +79,13 @@ __device__ __forceinline__ void stage_tile(float* sh, const T* base, long long s
 //   kColsum = false   stationary queries, streamed keys: (max, sum of 2^(x - max)) of every query row
 //   kColsum = true    stationary keys, streamed queries: sum of 2^(x - lse2(query)) of every key
 // 256 threads as 16 x 16; a thread holds 4 x 4 logits of a 64 x 64 tile.
+// Grid: (slot, layer, head) x the cluster's blocks.  Sequence i owns the slots cu[i] / kRows + i up to the next one's first:
+// at least as many as it has tiles, and in all only T / kRows + n_seqs of them, found without a table.
 template <typename T, bool kColsum>
 __global__ void __launch_bounds__(kThreads)
 simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const float* __restrict__ lse, float lse_mul,
                   float* __restrict__ lse2_out, float* __restrict__ lse_nat_out, float* __restrict__ scores, int normalize,
-                  int max_tiles) {
+                  int layer0, int n_layers) {
   extern __shared__ float4 dyn4[];
   float* fix_sh = reinterpret_cast<float*>(dyn4);
   float* str_sh = fix_sh + kRows * (s.D + kPad);
@@ -96,9 +98,14 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   int unit = blockIdx.x / n_blk;
   const int h = unit % s.Hq; unit /= s.Hq;
-  const int layer = unit % s.n_layers; unit /= s.n_layers;
-  const int seq = unit % s.n_seqs, rank_tile = unit / s.n_seqs;
+  const int layer = layer0 + unit % n_layers; unit /= n_layers;
+  int seq = 0;
+  for (int end = s.n_seqs; end - seq > 1;) {                // unit is the slot: the last sequence whose first slot is not above it
+    const int mid = (seq + end) >> 1;
+    if (__ldg(s.cu_seqlens + mid) / kRows + mid <= unit) seq = mid; else end = mid;
+  }
   const int t0 = __ldg(s.cu_seqlens + seq), L = __ldg(s.cu_seqlens + seq + 1) - t0;
+  const int rank_tile = unit - (t0 / kRows + seq);
   const int n_tiles = (L + kRows - 1) / kRows;
   if (rank_tile >= n_tiles) return;                         // uniform over the cluster, like every exit below
   // heaviest tiles first: the last query rows, the first keys
@@ -202,46 +209,55 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
 }
 
 template <typename T, bool kColsum>
-int launch_sweep(const Shape& s, const TensorView& Q, const TensorView& K, float scale_log2, const float* lse, float lse_mul,
+int launch_sweep(const Shape& s, const int32_t* cu_host, const TensorView& Q, const TensorView& K, float scale_log2, const float* lse, float lse_mul,
                  float* lse2_out, float* lse_nat_out, float* scores, int normalize, cudaStream_t stream) {
   const int max_tiles = (s.max_seqlen + kRows - 1) / kRows;
-  const long long units = (long long)max_tiles * s.n_seqs * s.n_layers * s.Hq;
+  long long tiles = 0;
+  for (int i = 0; i < s.n_seqs; ++i) tiles += (cu_host[i + 1] - cu_host[i] + kRows - 1) / kRows;
+  const long long units = tiles * s.n_layers * s.Hq;
   // A small problem does not fill the chip with one block per tile of rows: its streamed tiles are shared by up to 8
   // blocks then (8 heads x 512 tokens: 64 tiles of rows, 4 blocks each; with 8 the second wave starts, 26 -> 37 us).
   int n_blk = 1;
   while (n_blk < 8 && 2 * n_blk <= max_tiles && units * n_blk < 148) n_blk *= 2;
-  if (units * n_blk > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
+  const long long slots = s.n_seqs == 1 ? max_tiles : (long long)s.T / kRows + s.n_seqs, per_layer = slots * s.Hq * n_blk;
+  if (per_layer > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
   const size_t dyn = (size_t)2 * kRows * (s.D + kPad) * sizeof(float);
   auto kern = simt_sweep_kernel<T, kColsum>;
   if (dyn > 40 * 1024 && allow_dynamic_smem(kern, 2 * kRows * (kMaxD + kPad) * (int)sizeof(float)) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
-  return launch_chained(kern, dim3((unsigned)(units * n_blk)), dim3(kThreads), dyn, stream, n_blk, s, Q, K, scale_log2, lse, lse_mul,
-                        lse2_out, lse_nat_out, scores, normalize, max_tiles);
+  const int layers = (int)(0x7FFFFFFFLL / per_layer < s.n_layers ? 0x7FFFFFFFLL / per_layer : s.n_layers);    // of one launch
+  for (int layer0 = 0; layer0 < s.n_layers; layer0 += layers) {
+    const int n = s.n_layers - layer0 < layers ? s.n_layers - layer0 : layers;
+    const int rc = launch_chained(kern, dim3((unsigned)(per_layer * n)), dim3(kThreads), dyn, stream, n_blk, s, Q, K, scale_log2,
+                                  lse, lse_mul, lse2_out, lse_nat_out, scores, normalize, layer0, n);
+    if (rc != KVCRUSH_OK) return rc;
+  }
+  return KVCRUSH_OK;
 }
 
 template <typename T>
-int run(const Shape& s, const TensorView& Q, const TensorView& K, float scale_log2, const float* lse_in,
+int run(const Shape& s, const int32_t* cu_host, const TensorView& Q, const TensorView& K, float scale_log2, const float* lse_in,
         float lse_in_mul, float* lse2_ws, float* scores, float* lse_out, int normalize, cudaStream_t stream) {
   if (s.T == 0) return KVCRUSH_OK;
   if (!lse_in) {
-    const int rc = launch_sweep<T, false>(s, Q, K, scale_log2, nullptr, 1.f, lse2_ws, lse_out, nullptr, 0, stream);
+    const int rc = launch_sweep<T, false>(s, cu_host, Q, K, scale_log2, nullptr, 1.f, lse2_ws, lse_out, nullptr, 0, stream);
     if (rc != KVCRUSH_OK) return rc;
-    return launch_sweep<T, true>(s, Q, K, scale_log2, lse2_ws, 1.f, nullptr, nullptr, scores, normalize, stream);
+    return launch_sweep<T, true>(s, cu_host, Q, K, scale_log2, lse2_ws, 1.f, nullptr, nullptr, scores, normalize, stream);
   }
-  return launch_sweep<T, true>(s, Q, K, scale_log2, lse_in, lse_in_mul, nullptr, nullptr, scores, normalize, stream);
+  return launch_sweep<T, true>(s, cu_host, Q, K, scale_log2, lse_in, lse_in_mul, nullptr, nullptr, scores, normalize, stream);
 }
 
 }  // namespace
 
-int launch_score_simt(const Shape& s, const TensorView& Q, const TensorView& K, float scale_log2,
+int launch_score_simt(const Shape& s, const int32_t* cu_host, const TensorView& Q, const TensorView& K, float scale_log2,
                       const float* lse_in, float lse_in_mul, float* lse2_ws, float* scores, float* lse_out,
                       int normalize, int32_t* /*status*/, cudaStream_t stream) {
   if (s.D > kMaxD || s.D % 8 != 0) return KVCRUSH_ERR_UNSUPPORTED;
   if (Q.dtype == KVCRUSH_FP32)
-    return run<float>(s, Q, K, scale_log2, lse_in, lse_in_mul, lse2_ws, scores, lse_out, normalize, stream);
+    return run<float>(s, cu_host, Q, K, scale_log2, lse_in, lse_in_mul, lse2_ws, scores, lse_out, normalize, stream);
   if (Q.dtype == KVCRUSH_BF16)
-    return run<__nv_bfloat16>(s, Q, K, scale_log2, lse_in, lse_in_mul, lse2_ws, scores, lse_out, normalize, stream);
+    return run<__nv_bfloat16>(s, cu_host, Q, K, scale_log2, lse_in, lse_in_mul, lse2_ws, scores, lse_out, normalize, stream);
   if (Q.dtype == KVCRUSH_FP16)
-    return run<__half>(s, Q, K, scale_log2, lse_in, lse_in_mul, lse2_ws, scores, lse_out, normalize, stream);
+    return run<__half>(s, cu_host, Q, K, scale_log2, lse_in, lse_in_mul, lse2_ws, scores, lse_out, normalize, stream);
   return KVCRUSH_ERR_UNSUPPORTED;
 }
 

@@ -182,3 +182,25 @@ def test_decode_adds_weights_below_the_smallest_normal_number(B):
         B.kvcrush_score_decode(prob, q, k, scores, status=status)
         got = scores.cpu().numpy()[0, 0].astype(np.float64)
         assert (np.abs(got - n * w) <= 1e-5 * n * w + 3 * n * 2.0 ** -149).all()
+
+
+def test_one_long_and_many_short_sequences_on_the_cuda_cores(B):
+    """512 tiles of rows x 4096 sequences x 4096 heads would be more blocks than a grid holds; the work is small (a window of
+    one query).  Layers and heads share their rows, so every slice gives the same scores."""
+    import torch
+    layers, Hq, long_len, n_short = 32, 128, 32768, 4095
+    T = long_len + n_short
+    q = _normal((1, T, 1, 8), 15, torch.float32).expand(layers, T, Hq, 8)
+    k = _normal((1, T, 1, 8), 16, torch.float32).expand(layers, T, Hq, 8)
+    lens = (long_len,) + (1,) * n_short
+    prob = B.Problem(layers, Hq, Hq, 8, lens, device="cuda:0", query_window=1)
+    ws = torch.empty(B.kvcrush_workspace_size(prob, B.STAGE_SCORE), dtype=torch.uint8, device="cuda:0")
+    status = torch.zeros(4, dtype=torch.int32, device="cuda:0")
+    scores = torch.full((layers, Hq, T), -1.0, dtype=torch.float32, device="cuda:0")
+    B.kvcrush_score(prob, q, k, scores, impl=B.SCORE_SIMT, workspace=ws, status=status)
+    assert bool((scores == scores[:1, :1]).all())
+    got = scores[0, 0].cpu().numpy()
+    want, _ = O.scores(q[0, :long_len, :1].double().cpu().numpy(), k[0, :long_len, :1].double().cpu().numpy(), True,
+                       rows=(long_len - 1, long_len))
+    assert TL.within_score_tolerance(got[:long_len], want[0]).all()
+    np.testing.assert_allclose(got[long_len:], 1.0, rtol=1e-6)
