@@ -539,6 +539,9 @@ def test_pass_replays_from_a_cuda_graph(B):
 @pytest.mark.parametrize("dtype,D,Hq,Hkv,seqlens,causal,window", [
     (inputs.FP32, 64, 2, 1, (63, 64, 65), True, 0),          # around one tile of 64 rows
     (inputs.FP32, 8, 1, 1, (1,), True, 0),                   # the smallest problem
+    (inputs.FP32, 64, 2, 1, (15, 0, 16, 1), True, 0),        # a logit a thread: no sequence above 16 tokens
+    (inputs.FP32, 40, 2, 2, (16, 31, 17, 32), False, 0),     # 2 x 2 logits a thread: none above 32
+    (inputs.FP32, 64, 1, 1, (30, 16, 33), True, 10),
     (inputs.FP32, 128, 1, 1, (1025,), True, 0),              # streamed tiles shared by 8 blocks, last tile of one row
     (inputs.FP32, 72, 4, 2, (190, 0, 129), False, 0),        # channels not a multiple of the shared-memory bank count
     (inputs.FP32, 256, 2, 2, (200,), True, 70),              # widest heads, window that cuts a tile
