@@ -546,30 +546,49 @@ int launch_persist(const CUtensorMap& mq, const CUtensorMap& mk, const PersistAr
 
 // Tiles of an item's stationary block.  Four 128-row tiles take the most out of every streamed tile, but a launch with
 // few items then ends with one item per SM and the others idle; with two or one, each tile serves two or four
-// accumulator slots and an item is a half or a quarter as long.  Estimated in rounds (one streamed tile against four
-// accumulators): the longest item or the mean load plus what a list schedule loses, times what a round costs more when
-// a streamed tile is used less often, plus what an item costs by itself.  Both sweeps, 32 heads: 1001 tokens (8 KV heads)
-// 45.5 / 32.4 / 31.3 us with 4 / 2 / 1 tiles, 2048 tokens 83.9 / 59.6 / 71.1, 3072 tokens 121 / 115 / 131, 4096 tokens
-// 175 / 185 / 213; 8 heads, 8192 tokens 297 / 166 / 183, 5000 tokens 183 / 103 / 80.
-int block_tiles(const Shape& s, const int32_t* cu_host, int n_sms) {
-  constexpr float kRoundCost[3] = {1.f, 1.2f, 1.45f};
+// accumulator slots and an item is a half or a quarter as long.  The time of the call's sweeps is estimated in us from the
+// rounds of the items (one streamed tile against four accumulators) and what an item costs by itself: a launch takes its
+// longest item, or an SM's mean load and a part of the shortest item.  Blocks of less than four tiles have to win by 5 %.
+// The constants are a fit to 400 problems (1 to 1024 heads, 60 to 8192 tokens, batches of up to 64 sequences) timed with each
+// block size: the choice is 0.4 % behind the best on average, 15 % at worst (heads of 200 tokens), and never slower than four
+// tiles.  32 heads, 4 / 2 / 1 tiles: 1001 tokens 45 / 33 / 31 us, 2048 tokens 80 / 56 / 66, 4096 tokens 168 / 173 / 204; 8 heads,
+// 3000 tokens 115 / 72 / 78; 1024 heads, 300 tokens 115 / 159 / 186; 256 heads, 12 sequences of 200 to 800 tokens 575 / 731 / 988.
+int block_tiles(const Shape& s, const int32_t* cu_host, int n_sms, bool row_sweep) {
+  constexpr float kRound[3] = {2.2f, 2.35f, 2.55f}, kItem[3] = {1.2f, 3.1f, 3.1f};
+  constexpr float kShortest = 0.55f, kFixed = 3.5f, kCounter = 3.f, kMargin = 1.05f;
+  constexpr float kShare[5] = {0.f, 0.25f, 0.5f, 1.f, 1.f};          // rounds per streamed tile of a block, by its tiles
   const float n_lh = (float)s.n_layers * s.Hq;
   int best = kQ;
   float best_cost = 0.f;
   for (int v = 0, tpb = kQ; tpb >= 1; ++v, tpb /= 2) {
-    float sum = 0.f, longest = 0.f, items = 0.f;
-    for (int i = 0; i < s.n_seqs; ++i) {
-      const int n = (cu_host[i + 1] - cu_host[i] + kTile - 1) / kTile;
-      const int full = n / tpb, q = n - full * tpb;                  // full blocks, tiles of the last one
-      const float tail = n * (q == 3 ? 4 : q) * 0.25f;
-      const float round_tiles = tpb * 0.25f;                         // rounds per streamed tile
-      sum += tail + (s.causal ? round_tiles * tpb * 0.5f * full * (full + 1) : round_tiles * n * full);
-      longest = fmaxf(longest, fmaxf(tail, full ? round_tiles * (s.causal ? full * tpb : n) : 0.f));
-      items += full + (q > 0);
+    float cost = 0.f;
+    for (int sweep = row_sweep ? 0 : 1; sweep < 2; ++sweep) {
+      float sum = 0.f, longest = 0.f, shortest = 1e9f, items = 0.f;
+      auto block = [&](float n_streamed, float share) {
+        const float rounds = fmaxf(1.f, n_streamed * share);
+        longest = fmaxf(longest, rounds);
+        shortest = fminf(shortest, rounds);
+        return rounds;
+      };
+      for (int i = 0; i < s.n_seqs; ++i) {
+        const int n = (cu_host[i + 1] - cu_host[i] + kTile - 1) / kTile;
+        const int full = n / tpb, q = n - full * tpb;                // full blocks, tiles of the last one
+        if (full > 0) {                                              // from the least streamed tiles to the most
+          const int most = !s.causal ? n : sweep == 0 ? full * tpb : n;
+          const int least = !s.causal ? n : sweep == 0 ? tpb : n - (full - 1) * tpb;
+          block((float)least, kShare[tpb]);
+          block((float)most, kShare[tpb]);
+          sum += 0.5f * full * (least + most) * kShare[tpb];
+        }
+        if (q > 0) sum += block(s.causal && sweep == 1 ? (float)q : (float)n, sweep == 1 && tpb == kQ ? 1.f : kShare[q]);
+        items += full + (q > 0);
+      }
+      const float item = kItem[v], mean = (kRound[v] * sum + item * items) * n_lh / n_sms;
+      longest = kRound[v] * longest + item;
+      cost += kFixed + (items * n_lh <= n_sms ? longest : fmaxf(longest, mean + kShortest * (kRound[v] * shortest + item)));
+      if (sweep == 1 && items * n_lh > 2 * n_sms) cost += kCounter;
     }
-    const float per_sm = n_lh / n_sms;
-    const float cost = kRoundCost[v] * fmaxf(longest, 1.15f * sum * per_sm) + 0.4f * ceilf(items * per_sm);
-    if (tpb == kQ || cost < best_cost) { best = tpb; best_cost = cost; }
+    if (tpb == kQ || cost < best_cost) { best = tpb; best_cost = tpb == kQ ? cost / kMargin : cost; }
   }
   return best;
 }
@@ -626,7 +645,7 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
   const long long items_all = count(1, false);
   if (items_all == 0) return KVCRUSH_OK;
   if (items_all * a.n_lh > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
-  a.tpb = s.window > 0 ? kQ : block_tiles(s, cu_host, n_sms);
+  a.tpb = s.window > 0 ? kQ : block_tiles(s, cu_host, n_sms, !lse_in);
   bool zeroed = false;
   auto plan = [&](bool row_sweep, int* counter) {
     const long long items = count(a.tpb, row_sweep);
