@@ -97,6 +97,14 @@ int launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t dyn_
   return KVCRUSH_OK;
 }
 
+// Streaming multiprocessors of the current device.
+inline int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) return n;
+  cudaGetLastError();
+  return 1;
+}
+
 // Lets a kernel be launched with up to `bound` bytes of dynamic shared memory.  The attribute belongs to the kernel, not to
 // the launch, so every call sets the same bound: with the size of the launch at hand, two threads with different sizes took
 // the larger one's permission away between setting it and launching.

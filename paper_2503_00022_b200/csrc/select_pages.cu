@@ -278,11 +278,21 @@ int launch_select_pages(const Shape& s, const float* scores, const double* impor
   a.sort_cap = 32;
   while (a.sort_cap < a.np_cap) a.sort_cap <<= 1;
   const size_t fixed = (size_t)a.np_cap * 8 + (size_t)a.sort_cap * 4 + (size_t)a.np_cap / 32 * 8 + (size_t)a.PW * 4;
-  // Few pages need few threads: with small blocks several segments share an SM and barriers are cheap (512 segments of
-  // 23 pages: 77 us with 1024 threads each, 25 us with 128).
-  if (max_pages <= 128) return launch_pages<128>(s, a, fixed, stream);
-  if (max_pages <= 512) return launch_pages<256>(s, a, fixed, stream);
-  return launch_pages<1024>(s, a, fixed, stream);
+  // Few pages need few threads, and many segments have to share an SM, which holds 1024 threads of this kernel (128 / 256 /
+  // 512 / 1024 threads, a quarter of the pages kept; one segment of 23 pages 16 / 16 / 16 / 17 us, of 64 21 / 14 / 15 / 16,
+  // of 128 34 / 22 / 17 / 18, of 256 65 / 37 / 26 / 23, of 512 127 / 70 / 44 / 37).  288 segments of 256 pages 70 / 44 / 37 / 47,
+  // 512 segments of 64 pages 31 / 23 / 33 / 63, of 256 101 / 67 / 71 / 92, of 512 196 / 129 / 126 / 146; 1200 segments of 23
+  // pages 33 / 48 / 81 / 148, of 125 87 / 83 / 98 / 167.
+  const long long n_seg = (long long)s.n_layers * s.n_seqs;
+  const int per_sm = (int)((n_seg + sm_count() - 1) / sm_count());
+  const int wanted = max_pages <= 32 ? 128 : max_pages <= 80 ? 256 : max_pages <= 160 ? 512 : 1024;
+  const int shared = per_sm <= 1 ? 1024 : per_sm <= 2 ? 512 : max_pages > 256 ? 512 : per_sm > 4 && max_pages <= 100 ? 128 : 256;
+  switch (wanted < shared ? wanted : shared) {
+    case 128: return launch_pages<128>(s, a, fixed, stream);
+    case 256: return launch_pages<256>(s, a, fixed, stream);
+    case 512: return launch_pages<512>(s, a, fixed, stream);
+    default: return launch_pages<1024>(s, a, fixed, stream);
+  }
 }
 
 }  // namespace kvc

@@ -89,6 +89,21 @@ def test_pages_at_the_edges_of_the_block_sizes(B, P, pages, ties):
     _check_pages(cp, scores, 8, seqlens, P, b_imp, b_rep)
 
 
+@pytest.mark.parametrize("layers,pages", [
+    (1, [80, 33]), (1, [81, 160]), (1, [161, 100]),              # 256, 512 and 1024 threads a segment
+    (100, [90, 33]), (100, [161, 5]),                            # two segments an SM: 512 threads
+    (200, [60, 35]), (200, [257, 3]), (200, [129, 20]),          # three: 256 threads, and 512 for many pages
+    (400, [35, 2]), (400, [101, 6]),                             # more: 128 threads, and 256
+])
+def test_page_blocks_follow_the_number_of_segments(B, layers, pages):
+    seqlens = [4 * n - (1 if i % 2 else 0) for i, n in enumerate(pages)]
+    scores = np.tile(_scores(2, 4, seqlens, 480 + len(pages) + layers, ties=3), ((layers + 1) // 2, 1, 1))[:layers]
+    b_imp = np.asarray([[max(1, n // 3) for n in pages]], dtype=np.int32)
+    b_rep = np.asarray([[max(1, n // 4) for n in pages]], dtype=np.int32)
+    cp = _run_pages(B, scores, 2, seqlens, 4, b_imp, b_rep)
+    _check_pages(cp, scores, 2, seqlens, 4, b_imp, b_rep)
+
+
 def test_page_size_one_equals_token_level_kernel(B):
     import torch
     seqlens, Hq, Hkv = [700, 129], 40, 8
