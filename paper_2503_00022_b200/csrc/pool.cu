@@ -3,9 +3,9 @@
 // odd width `kernel`, clipped to t's own sequence.
 //
 // Bound by latency and by the two passes over the scores.  A block takes a chunk of 1024 tokens (256 when that
-// would leave SMs idle: one layer of 700 + 300 tokens 2.6 -> 2.1 us) of one (layer, head) row: it stages
-// them and the window's overhang in shared memory, all loads in flight together.  Where the rows allow 16-byte accesses and
-// the chunk lies in one sequence, places outside the sequence hold NaN, which fmaxf passes over, and a thread takes four
+// would leave SMs idle: one layer of 700 + 300 tokens 2.6 -> 2.1 us; 1024 rows of 2000 tokens 11.5 against 6.5 us) of one
+// (layer, head) row: it stages them and the window's overhang in shared memory, all loads in flight together, 16 bytes wide
+// where the rows allow it.  Where then the chunk lies in one sequence, places outside the sequence hold NaN, which fmaxf passes over, and a thread takes four
 // neighbouring outputs from 16-byte reads.  32 x 32 rows of 8192 tokens, width 7: 20 us against 42 us with one output a
 // thread, whose window came from L1 behind a 64-bit division.
 #include "common.cuh"
@@ -29,6 +29,8 @@ pool_scores_kernel(Shape s, const float* __restrict__ in, int radius, int chunk,
   const int t_end = min(t0 + chunk, s.T);
   const float* src = in + (size_t)row * s.T;
   float* dst = out + (size_t)row * s.T;
+  int first = max(t0 - radius, 0);                               // stage[0] is the row's element `first`
+  bool staged = false;
   if constexpr (kStaged) {
     if (quads) {
       const int pad = (radius + 3) / 4, n_quads = chunk / 4 + 2 * pad, q0 = t0 / 4 - pad;    // stage4[0] is the row's quad q0
@@ -40,16 +42,7 @@ pool_scores_kernel(Shape s, const float* __restrict__ in, int radius, int chunk,
       }
       const int seq = seq_of_token(s.cu_seqlens, s.n_seqs, t0);
       const int a = __ldg(s.cu_seqlens + seq), b = __ldg(s.cu_seqlens + seq + 1);
-      if (t_end <= b) {
-        auto put = [&](int i, float4 x) {
-          const int t = 4 * (q0 + i);
-          const float none = __int_as_float(0x7FFFFFFF);
-          if (t < a || t >= b) x.x = none;
-          if (t + 1 < a || t + 1 >= b) x.y = none;
-          if (t + 2 < a || t + 2 >= b) x.z = none;
-          if (t + 3 < a || t + 3 >= b) x.w = none;
-          stage4[i] = x;
-        };
+      auto stage_all = [&](auto&& put) {
 #pragma unroll
         for (int j = 0; j < 2; ++j)
           if (tid + j * kThreads < n_quads) put(tid + j * kThreads, v[j]);
@@ -58,6 +51,17 @@ pool_scores_kernel(Shape s, const float* __restrict__ in, int radius, int chunk,
           put(i, q >= 0 && 4 * q < s.T ? __ldg(reinterpret_cast<const float4*>(src) + q) : float4{});
         }
         __syncthreads();
+      };
+      if (t_end <= b) {
+        stage_all([&](int i, float4 x) {
+          const int t = 4 * (q0 + i);
+          const float none = __int_as_float(0x7FFFFFFF);
+          if (t < a || t >= b) x.x = none;
+          if (t + 1 < a || t + 1 >= b) x.y = none;
+          if (t + 2 < a || t + 2 >= b) x.z = none;
+          if (t + 3 < a || t + 3 >= b) x.w = none;
+          stage4[i] = x;
+        });
         if (t0 + 4 * tid >= t_end) return;
         float m[4];
 #pragma unroll
@@ -81,9 +85,11 @@ pool_scores_kernel(Shape s, const float* __restrict__ in, int radius, int chunk,
         reinterpret_cast<float4*>(dst)[t0 / 4 + tid] = make_float4(m[0], m[1], m[2], m[3]);
         return;
       }
+      stage_all([&](int i, float4 x) { stage4[i] = x; });
+      first = 4 * q0;
+      staged = true;
     }
   }
-  const int first = max(t0 - radius, 0), last = min(t_end - 1 + radius, s.T - 1);
   int t = t0 + tid, seq = 0, seq_first = 0, seq_end = 0;
   if (t < t_end) {
     seq = seq_of_token(s.cu_seqlens, s.n_seqs, t);
@@ -91,9 +97,12 @@ pool_scores_kernel(Shape s, const float* __restrict__ in, int radius, int chunk,
     seq_end = __ldg(s.cu_seqlens + seq + 1);
   }
   if constexpr (kStaged) {
+    if (!staged) {
+      const int last = min(t_end - 1 + radius, s.T - 1);
 #pragma unroll 5
-    for (int u = first + tid; u <= last; u += kThreads) stage[u - first] = __ldg(src + u);
-    __syncthreads();
+      for (int u = first + tid; u <= last; u += kThreads) stage[u - first] = __ldg(src + u);
+      __syncthreads();
+    }
   }
   auto at = [&](int u) { return kStaged ? stage[u - first] : __ldg(src + u); };
   for (; t < t_end; t += kThreads) {
@@ -111,7 +120,7 @@ pool_scores_kernel(Shape s, const float* __restrict__ in, int radius, int chunk,
 int launch_pool_scores(const Shape& s, const float* scores_in, int kernel, float* scores_out, cudaStream_t stream) {
   const int radius = (kernel - 1) / 2;
   const long long rows = (long long)s.n_layers * s.Hq;
-  const int chunk = rows * (s.T / kMaxChunk) >= 8 * 148 ? kMaxChunk : kThreads;
+  const int chunk = rows * ((s.T + kMaxChunk - 1) / kMaxChunk) >= 8 * sm_count() ? kMaxChunk : kThreads;
   const int n_chunks = (s.T + chunk - 1) / chunk;
   const long long blocks = rows * n_chunks;
   if (blocks == 0) return KVCRUSH_OK;
