@@ -145,8 +145,8 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
 
 // Observation windows of up to 64 queries in one pass over the keys (tensor cores); score_window_fits: does it apply.
 bool score_window_fits(const Shape& s);
-int launch_score_window(const Shape& s, const TensorView& Q, const ScoreTensorMaps& maps, float scale_log2, float* scores,
-                        float* lse_out, int normalize, int32_t* status, const ScoreDiag& diag, cudaStream_t stream);
+int launch_score_window(const Shape& s, const int32_t* cu_host, const TensorView& Q, const ScoreTensorMaps& maps,
+                        float scale_log2, float* scores, float* lse_out, int normalize, int32_t* status, const ScoreDiag& diag, cudaStream_t stream);
 
 // importance: optional out [n_layers][T] float64, the token importance I(t) of stage 3 (written from the same loads).
 int launch_signature(const Shape& s, const float* scores, const int32_t* sig_keep, const float* theta_in,

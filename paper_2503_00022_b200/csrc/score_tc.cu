@@ -632,7 +632,7 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
   a.s = s; a.scale_log2 = scale_log2; a.normalize = normalize; a.bf16 = Q.dtype == KVCRUSH_BF16; a.status = status; a.scores = scores;
   const bool sw = diag.short_waits != 0;
   if (!lse_in && score_window_fits(s)) {
-    const int rc = launch_score_window(s, Q, maps, scale_log2, scores, lse_out, normalize, status, diag, stream);
+    const int rc = launch_score_window(s, cu_host, Q, maps, scale_log2, scores, lse_out, normalize, status, diag, stream);
     // no room for its clusters on this GPU: two sweeps (but not for a diagnostic call, which tests the kernel a call takes)
     if (rc != KVCRUSH_ERR_UNSUPPORTED || sw || diag.withhold_first_item) return rc;
   }

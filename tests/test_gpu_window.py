@@ -77,6 +77,9 @@ def test_windowed_scores_match_oracle(B, w, window):
     (1, 2, 2, 64, (8192,), 33, True, 1.0),                # every accumulator in use
     (1, 8, 2, 128, (900, 31), 16, False, 1.0),            # 16 columns, no mask
     (6, 32, 8, 128, (1500,), 7, True, 1.0),               # units in turn on the same accumulators
+    (1, 4, 2, 128, (300, 2500, 0, 5000, 90, 1100), 64, True, 1.0),       # one launch for lengths that need clusters of 1 to 8
+    (6, 16, 2, 128, (300, 2500, 0, 5000, 90, 1100), 64, True, 1.0),      # a launch for each cluster size
+    (20, 6, 3, 64, (1025, 1024, 2049, 31), 40, False, 1.0),              # the same at the edges between the sizes
     (1, 4, 4, 128, (700, 200), 48, True, 40.0),           # logits far outside [-100, 100]: kept tiles, exact maxima
     (1, 2, 2, 64, (600,), 64, False, 12.0),               # some tiles kept, some not
 ])
