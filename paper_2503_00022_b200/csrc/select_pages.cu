@@ -285,7 +285,7 @@ int launch_select_pages(const Shape& s, const float* scores, const double* impor
   // pages 33 / 48 / 81 / 148, of 125 87 / 83 / 98 / 167.
   const long long n_seg = (long long)s.n_layers * s.n_seqs;
   const int per_sm = (int)((n_seg + sm_count() - 1) / sm_count());
-  const int wanted = max_pages <= 32 ? 128 : max_pages <= 80 ? 256 : max_pages <= 160 ? 512 : 1024;
+  const int wanted = max_pages <= 16 ? 128 : max_pages <= 48 ? 256 : max_pages <= 160 ? 512 : 1024;
   const int shared = per_sm <= 1 ? 1024 : per_sm <= 2 ? 512 : max_pages > 256 ? 512 : per_sm > 4 && max_pages <= 100 ? 128 : 256;
   switch (wanted < shared ? wanted : shared) {
     case 128: return launch_pages<128>(s, a, fixed, stream);
