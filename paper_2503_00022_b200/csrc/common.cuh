@@ -73,19 +73,20 @@ __device__ __forceinline__ int warp_segment_of_row(const int32_t* __restrict__ c
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// overlap = false: the kernel starts when its predecessor has ended.
 template <class... Params, class... Args>
-int launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t dyn_smem, cudaStream_t stream, int cluster,
-                   Args&&... args) {
+int launch_kernel(bool overlap, void (*kernel)(Params...), dim3 grid, dim3 block, size_t dyn_smem, cudaStream_t stream, int cluster,
+                  Args&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = dyn_smem;
   cfg.stream = stream;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) cudaGetLastError();
+  if (overlap && cudaStreamIsCapturing(stream, &capture) != cudaSuccess) cudaGetLastError();
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = capture == cudaStreamCaptureStatusNone;
+  at[0].val.programmaticStreamSerializationAllowed = overlap && capture == cudaStreamCaptureStatusNone;
   at[1].id = cudaLaunchAttributeClusterDimension;
   at[1].val.clusterDim.x = (unsigned)cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
@@ -95,6 +96,11 @@ int launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t dyn_
     return KVCRUSH_ERR_CUDA;
   }
   return KVCRUSH_OK;
+}
+template <class... Params, class... Args>
+int launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t dyn_smem, cudaStream_t stream, int cluster,
+                   Args&&... args) {
+  return launch_kernel(true, kernel, grid, block, dyn_smem, stream, cluster, static_cast<Args&&>(args)...);
 }
 
 // Streaming multiprocessors of the current device.
