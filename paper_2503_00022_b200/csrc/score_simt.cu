@@ -80,13 +80,15 @@ __device__ __forceinline__ void stage_tile(float* sh, const T* base, long long s
 //   kColsum = true    stationary keys, streamed queries: sum of 2^(x - lse2(query)) of every key
 // 256 threads as 16 x 16; a thread holds N x N logits of a tile: 4 x 4, or 1 x 1 or 2 x 2 where no sequence is longer than
 // 16 or 32 tokens and the rest of the 64 x 64 would be zeros (300 sequences of 5 tokens, 2 layers x 8 heads: 237 -> 70 us).
-// Grid: (slot, layer, head) x the cluster's blocks.  Sequence i owns the slots cu[i] / kRows + i up to the next one's first:
-// at least as many as it has tiles, and in all only T / kRows + n_seqs of them, found without a table.
+// Grid: (slot, layer, head) x the cluster's blocks.  In a batch of sequences of similar length slots are (tile, sequence)
+// pairs, the heaviest tiles of all sequences first (4 layers x 8 heads x 6 sequences of 600 tokens: 424 us, sequence by sequence
+// 453).  Otherwise (by_seq) sequence i owns the slots cu[i] / kRows + i up to the next one's first: at least as many as it has
+// tiles, and in all only T / kRows + n_seqs of them, found without a table.
 template <typename T, bool kColsum, int N>
 __global__ void __launch_bounds__(kThreads)
 simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const float* __restrict__ lse, float lse_mul,
                   float* __restrict__ lse2_out, float* __restrict__ lse_nat_out, float* __restrict__ scores, int normalize,
-                  int layer0, int n_layers) {
+                  int layer0, int n_layers, int by_seq) {
   extern __shared__ float4 dyn4[];
   float* fix_sh = reinterpret_cast<float*>(dyn4);
   float* str_sh = fix_sh + 16 * N * (s.D + kPad);
@@ -100,13 +102,17 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
   int unit = blockIdx.x / n_blk;
   const int h = unit % s.Hq; unit /= s.Hq;
   const int layer = layer0 + unit % n_layers; unit /= n_layers;
-  int seq = 0;
-  for (int end = s.n_seqs; end - seq > 1;) {                // unit is the slot: the last sequence whose first slot is not above it
-    const int mid = (seq + end) >> 1;
-    if (__ldg(s.cu_seqlens + mid) / kRows + mid <= unit) seq = mid; else end = mid;
+  int seq = 0;                                              // unit is the slot
+  if (!by_seq) {
+    seq = unit % s.n_seqs;
+  } else {
+    for (int end = s.n_seqs; end - seq > 1;) {              // the last sequence whose first slot is not above it
+      const int mid = (seq + end) >> 1;
+      if (__ldg(s.cu_seqlens + mid) / kRows + mid <= unit) seq = mid; else end = mid;
+    }
   }
   const int t0 = __ldg(s.cu_seqlens + seq), L = __ldg(s.cu_seqlens + seq + 1) - t0;
-  const int rank_tile = unit - (t0 / kRows + seq);
+  const int rank_tile = by_seq ? unit - (t0 / kRows + seq) : unit / s.n_seqs;
   const int n_tiles = (L + kRows - 1) / kRows;
   if (rank_tile >= n_tiles) return;                         // uniform over the cluster, like every exit below
   // heaviest tiles first: the last query rows, the first keys
@@ -220,7 +226,9 @@ int launch_sweep(const Shape& s, const int32_t* cu_host, const TensorView& Q, co
   // blocks then (8 heads x 512 tokens: 64 tiles of rows, 4 blocks each; with 8 the second wave starts, 26 -> 37 us).
   int n_blk = 1;
   while (n_blk < 8 && 2 * n_blk <= max_tiles && units * n_blk < 148) n_blk *= 2;
-  const long long slots = s.n_seqs == 1 ? max_tiles : (long long)s.T / kRows + s.n_seqs, per_layer = slots * s.Hq * n_blk;
+  const long long pairs = (long long)max_tiles * s.n_seqs;
+  const int by_seq = 8 * pairs > 9 * tiles;
+  const long long slots = by_seq ? (long long)s.T / kRows + s.n_seqs : pairs, per_layer = slots * s.Hq * n_blk;
   if (per_layer > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
   const size_t dyn = (size_t)2 * 16 * N * (s.D + kPad) * sizeof(float);
   auto kern = simt_sweep_kernel<T, kColsum, N>;
@@ -234,7 +242,7 @@ int launch_sweep(const Shape& s, const int32_t* cu_host, const TensorView& Q, co
   for (int layer0 = 0; layer0 < s.n_layers; layer0 += layers) {
     const int n = s.n_layers - layer0 < layers ? s.n_layers - layer0 : layers;
     const int rc = launch_kernel(overlap, kern, dim3((unsigned)(per_layer * n)), dim3(kThreads), dyn, stream, n_blk, s, Q, K, scale_log2,
-                                  lse, lse_mul, lse2_out, lse_nat_out, scores, normalize, layer0, n);
+                                  lse, lse_mul, lse2_out, lse_nat_out, scores, normalize, layer0, n, by_seq);
     if (rc != KVCRUSH_OK) return rc;
   }
   return KVCRUSH_OK;
