@@ -161,7 +161,8 @@ int kvcrush_score(const kvcrush_problem_t* problem, const kvcrush_tensor_t* Q, c
  *   K           the cached keys, token-major, same dtype as Q_new (BF16, FP16 or FP32), head_dim <= 256, multiple of 8
  *   scores_dev  in/out [n_layers][n_q_heads][T] float32 running column sums
  * One cluster of blocks per layer, sequence and KV head serves the query heads of its group from one read of K
- * (logits of sequences of about 10^5 keys and more are computed twice).
+ * (logits are computed twice in sequences of more than 409600 keys over the query heads of a group, of which at most 8
+ * count: 51200 keys at 8 heads).
  */
 int kvcrush_score_decode(const kvcrush_problem_t* problem, const kvcrush_tensor_t* Q_new, const kvcrush_tensor_t* K,
                          float* scores_dev, int32_t* status_dev, void* stream);

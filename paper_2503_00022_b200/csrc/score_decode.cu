@@ -134,7 +134,7 @@ __device__ __forceinline__ void for_tiles(const T* __restrict__ kbase, long long
 }
 
 // Grid: one cluster per (layer, sequence, KV head).  DB: 32-channel blocks of a key row.  kStore: the block's logits fit
-// in shared memory (cap tokens per head); else (sequences of about 10^5 tokens and more) the second step computes them
+// in shared memory (cap tokens per head); else (from 51 201 keys on at 8 query heads a pass, 409 601 at one) the second step computes them
 // again from K.
 template <typename T, int DB, int kWarps, bool kStore>
 __global__ void __launch_bounds__(kWarps * 32)
@@ -320,8 +320,9 @@ int launch_width(const Shape& s, const TensorView& Qn, const TensorView& K, floa
   auto bytes = [&](int n_blk) { return (size_t)n_heads * tokens(n_blk) * sizeof(float); };
   // Blocks per unit: enough of them for about eight per SM (the last wave is then a small part of the run), none with
   // fewer than 256 keys, and at most 16 KB of logits a block while the cluster can grow.
+  const int n_sms = sm_count();
   int n_blk = 1;
-  while (n_blk < kMaxCluster && tokens(n_blk) > 256 && (units * n_blk < 8 * 148 || bytes(n_blk) > 16 * 1024)) n_blk *= 2;
+  while (n_blk < kMaxCluster && tokens(n_blk) > 256 && (units * n_blk < 8 * n_sms || bytes(n_blk) > 16 * 1024)) n_blk *= 2;
   if (units * n_blk > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
   const size_t dyn = bytes(n_blk);
   const int cap = tokens(n_blk);

@@ -224,8 +224,9 @@ int launch_sweep(const Shape& s, const int32_t* cu_host, const TensorView& Q, co
   const long long units = tiles * s.n_layers * s.Hq;
   // A small problem does not fill the chip with one block per tile of rows: its streamed tiles are shared by up to 8
   // blocks then (8 heads x 512 tokens: 64 tiles of rows, 4 blocks each; with 8 the second wave starts, 26 -> 37 us).
+  const int n_sms = sm_count();
   int n_blk = 1;
-  while (n_blk < 8 && 2 * n_blk <= max_tiles && units * n_blk < 148) n_blk *= 2;
+  while (n_blk < 8 && 2 * n_blk <= max_tiles && units * n_blk < n_sms) n_blk *= 2;
   const long long pairs = (long long)max_tiles * s.n_seqs;
   const int by_seq = 8 * pairs > 9 * tiles;
   const long long slots = by_seq ? (long long)s.T / kRows + s.n_seqs : pairs, per_layer = slots * s.Hq * n_blk;
@@ -237,7 +238,7 @@ int launch_sweep(const Shape& s, const int32_t* cu_host, const TensorView& Q, co
   // than a block an SM pays for that unless its blocks are short: 2 layers x 8 heads, 500 + 300 + 700 tokens, both sweeps 146
   // against 109 us; 8 heads x 512 tokens, two tiles a block, whole pass 46 against 47 us.
   const int streamed = s.window > 0 && s.window / kRows + 2 < max_tiles ? s.window / kRows + 2 : max_tiles;
-  const bool overlap = per_layer * s.n_layers <= sm_count() || (per_layer * s.n_layers <= 2 * sm_count() && streamed <= 2 * n_blk);
+  const bool overlap = per_layer * s.n_layers <= n_sms || (per_layer * s.n_layers <= 2 * n_sms && streamed <= 2 * n_blk);
   const int layers = (int)(0x7FFFFFFFLL / per_layer < s.n_layers ? 0x7FFFFFFFLL / per_layer : s.n_layers);    // of one launch
   for (int layer0 = 0; layer0 < s.n_layers; layer0 += layers) {
     const int n = s.n_layers - layer0 < layers ? s.n_layers - layer0 : layers;

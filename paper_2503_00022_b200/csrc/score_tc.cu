@@ -624,10 +624,7 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
   if (!(scale_log2 > 0.f)) return KVCRUSH_ERR_UNSUPPORTED;
   const CUtensorMap& mq = *reinterpret_cast<const CUtensorMap*>(maps.q);
   const CUtensorMap& mk = *reinterpret_cast<const CUtensorMap*>(maps.k);
-  int dev = 0, n_sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sms < 1)
-    return KVCRUSH_ERR_CUDA;
+  const int n_sms = sm_count();
   PersistArgs a{};
   a.s = s; a.scale_log2 = scale_log2; a.normalize = normalize; a.bf16 = Q.dtype == KVCRUSH_BF16; a.status = status; a.scores = scores;
   const bool sw = diag.short_waits != 0;

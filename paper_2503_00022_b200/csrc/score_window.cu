@@ -687,7 +687,10 @@ int launch_score_window(const Shape& s, const int32_t* cu_host, const TensorView
     longest[need] = len > longest[need] ? len : longest[need];
     largest = need > largest ? need : largest;
   }
-  auto rounds = [&](long long n, int log_cta) { return (n + (n_sms >> log_cta) - 1) / (n_sms >> log_cta); };
+  auto rounds = [&](long long n, int log_cta) {
+    const int clusters = n_sms >> log_cta > 0 ? n_sms >> log_cta : 1;
+    return (n + clusters - 1) / clusters;
+  };
   long long apart = 0, together = 0;
   for (int need = 0; need < 4; ++need) { apart += rounds(units[need], need); together += units[need]; }
   const bool split = rounds(together, largest) >= apart + 2;

@@ -517,12 +517,13 @@ int launch_select(const Shape& s, const float* scores, const double* importance,
   // holds them: 256 segments of 700 tokens 17.2 -> 10.6 us, 224 of 1900 21.6 -> 15.4, 512 of 4000 62.7 -> 48.1 (with 256
   // threads 60.7); 512 of 700 tokens 31.9 -> 13.0 (18.9), 512 of 1900 42.0 -> 23.7 (28.6).
   const long long n_seg = (long long)s.n_layers * s.n_seqs;
+  const int n_sms = sm_count();
   auto resident = [&](int n) { return n * (dyn + 19 * 1024) <= 227 * 1024; };
   auto by_words = [&](auto w) {
     constexpr int W = decltype(w)::value;
     if (long_seg) return launch(select_segment_kernel<W, true, 1024>, 1024);
-    if (n_seg > 2 * 148 && s.max_seqlen <= 2048 && resident(4)) return launch(select_segment_kernel<W, false, 256>, 256);
-    if ((s.max_seqlen <= 1024 || n_seg > 148) && resident(2)) return launch(select_segment_kernel<W, false, 512>, 512);
+    if (n_seg > 2 * n_sms && s.max_seqlen <= 2048 && resident(4)) return launch(select_segment_kernel<W, false, 256>, 256);
+    if ((s.max_seqlen <= 1024 || n_seg > n_sms) && resident(2)) return launch(select_segment_kernel<W, false, 512>, 512);
     return launch(select_segment_kernel<W, false, 1024>, 1024);
   };
   return s.W == 1 ? by_words(std::integral_constant<int, 1>{}) : s.W == 2 ? by_words(std::integral_constant<int, 2>{})

@@ -502,7 +502,7 @@ int launch_signature(const Shape& s, const float* scores, const int32_t* sig_kee
     const unsigned blocks = (unsigned)s.n_layers * s.n_seqs * s.Hq;
     const int m = s.max_seqlen;
     // A warp per row up to 512 tokens (stage at 1024 rows of 400 tokens: 11.8 -> 7.5 us); up to 1024 tokens only for
-    // more rows than the chip holds as blocks (148 x 8): its chain over 32 keys a lane is longer than the block's
+    // more rows than the chip holds as blocks (8 an SM): its chain over 32 keys a lane is longer than the block's
     // (32 rows of 1001 tokens: 8.9 against 7.3 us).
     const unsigned warp_blocks = (blocks + kRowWarps - 1) / kRowWarps;
     auto by_warp = [&](auto kern) {
@@ -514,7 +514,7 @@ int launch_signature(const Shape& s, const float* scores, const int32_t* sig_kee
     int rc;
     if (m <= 256) rc = by_warp(theta_warp_kernel<8>);
     else if (m <= 512) rc = by_warp(theta_warp_kernel<16>);
-    else if (m <= 1024 && blocks > 1184) rc = by_warp(theta_warp_kernel<32>);
+    else if (m <= 1024 && blocks > 8u * (unsigned)sm_count()) rc = by_warp(theta_warp_kernel<32>);
     else if (m <= 2048) rc = by_block(theta_select_kernel<256, 8, 8>, 256);
     else if (m <= 4096) rc = by_block(theta_select_kernel<512, 8, 4>, 512);
     else if (m <= 8192) rc = by_block(theta_select_kernel<512, 16, 4>, 512);

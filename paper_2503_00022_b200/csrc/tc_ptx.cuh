@@ -132,7 +132,7 @@ __device__ __forceinline__ f32x2 exp2_sfu2(f32x2 x) {
   unpack2(x, a, b);
   return pack2f(ex2(a), ex2(b));
 }
-// 2^x for a pair on the FMA pipe, x <= ~0 (any magnitude): round-to-nearest split x = n + f, f in [-0.5, 0.5],
+// 2^x for a pair on the FMA pipe, x below 127 (the result has to be a normal number; smaller x count as -125): round-to-nearest split x = n + f, f in [-0.5, 0.5],
 // cubic minimax polynomial for 2^f (relative error 7.5e-5), exponent bits of n added to the result.
 // The special-function unit delivers 16 ex2 per clock per SM and is the busiest unit of both sweeps; a
 // share of the exponentials can go down this path instead, at 6 packed + 6 scalar instructions a pair.
