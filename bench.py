@@ -15,6 +15,7 @@ no exchange step, so there is no collective on the data path (weak scaling).
 from __future__ import annotations
 
 import argparse
+import ctypes
 import json
 import os
 import subprocess
@@ -58,9 +59,9 @@ def measured_peaks():
 # workload arithmetic (algorithmic work, independent of how the kernels do it)
 # ---------------------------------------------------------------------------------------------
 
-def algorithmic_work(w: inputs.Workload, window: int = 0):
+def algorithmic_work(w: inputs.Workload, window: int = 0, sweeps: int = 2):
     """Per step (all layers).  Causal entries per head = L(L+1)/2 (rows of the observation window only when
-    window > 0); 2*D flops each; two sweeps."""
+    window > 0); 2*D flops and one exponential each and sweep."""
     def ent(L):
         ws = L - window if 0 < window < L else 0
         return (L * (L + 1) // 2 - ws * (ws + 1) // 2) if w.causal else (L - ws) * L
@@ -73,7 +74,10 @@ def algorithmic_work(w: inputs.Workload, window: int = 0):
     T, W = w.total_tokens, (w.n_q_heads + 31) // 32
     signature_bytes = (4 * w.n_q_heads + 4 * W) * T * w.n_layers
     select_bytes = (4 * w.n_q_heads + 4 * W) * T * w.n_layers + 4 * kept * w.n_layers
-    return dict(score_flops=2 * flops_per_sweep, exps=2 * entries * w.n_q_heads * w.n_layers,
+    voting = sum(min(L, window) if window else L for L in w.seqlens)
+    score_bytes = w.n_layers * (w.head_dim * inputs.storage_itemsize(w.qk_dtype) * (voting * w.n_q_heads + T * w.n_kv_heads)
+                                + 4 * w.n_q_heads * (T + voting))                    # Q and K once, scores and lse written
+    return dict(score_flops=sweeps * flops_per_sweep, exps=sweeps * entries * w.n_q_heads * w.n_layers, score_bytes=score_bytes,
                 compact_bytes=compact_bytes, signature_bytes=signature_bytes, select_bytes=select_bytes, kept=kept)
 
 
@@ -604,25 +608,32 @@ def run_ours(args, w):
         return
 
     peaks = measured_peaks()
-    work = algorithmic_work(w, args.window)
+    tensor_path = cp.impl != B.SCORE_SIMT and w.qk_dtype in (inputs.BF16, inputs.FP16) and w.head_dim % 8 == 0 and w.head_dim <= 128
+    # score launches per step and sweeps over the logits, as the library decides: two sweeps, or one pass over the keys
+    one_pass = ctypes.c_int(0)
+    n_score = B.lib().kvcrush_diag_score_kernels(prob.ref, ctypes.byref(one_pass)) if tensor_path else 2
+    work = algorithmic_work(w, args.window, 1 if one_pass.value else 2)
     if args.page_size:                                    # rows actually gathered: kept pages x page size
         eb = inputs.storage_itemsize(w.cache_dtype)
         work["compact_bytes"] = 2 * 2 * cp.total_kept * args.page_size * w.n_kv_heads * w.head_dim * eb
     score_s = stage_ms[0] * 1e-3
-    tensor_path = cp.impl != B.SCORE_SIMT and w.qk_dtype in (inputs.BF16, inputs.FP16) and w.head_dim % 8 == 0 and w.head_dim <= 128
     short_tf = work["score_flops"] / score_s / 1e12
-    # score launches per step: two sweeps, or one pass for observation windows of up to 64 queries whose logits fit
-    # the tensor memory of a cluster of eight
-    pad = next((n for n in (16, 32, 64) if args.window <= n), None) if args.window else None
-    n_score = 1 if tensor_path and pad and -(-(-(-max(w.seqlens) // 128)) // 8) * pad <= 512 else 2
-    if tensor_path:
+    if one_pass.value:
+        # bound by reading K once
+        score_ms = sus["score_ms_settled"] if sus else float(stage_ms[0])
+        gbs = work["score_bytes"] / (score_ms * 1e-3) / 1e9
+        roofline = {"bound": "hbm", "kernel": "score_window_kernel (%d launches per step)" % n_score, "achieved": gbs,
+                    "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"], "peak_source": peaks["source"],
+                    "traffic": None, "algorithmic_bytes": work["score_bytes"], "algorithmic_flops": work["score_flops"],
+                    "launch_ms": score_ms / n_score, "exps_per_s": work["exps"] / (score_ms * 1e-3)}
+    elif tensor_path:
         # Headline fraction: the score stage inside the seconds-long loop against the sustained GEMM peak (both at the
         # board's power limit); beside it the K-step loop against the burst peak (both short).
         sus_tf = work["score_flops"] / (sus["score_ms_settled"] * 1e-3) / 1e12 if sus else short_tf
         launch_ms = (sus["score_ms_settled"] if sus else float(stage_ms[0])) / n_score
         whole = w.name == DEFAULT_WORKLOAD or w.name.startswith(DEFAULT_WORKLOAD + "_")
         traffic = NCU_DRAM_BYTES_PER_LAYER_PER_SWEEP * w.n_layers if (whole and not args.window) else None
-        roofline = {"bound": "tensor", "kernel": "score_persist_kernel (two sweep launches per step; per-launch figures)" if n_score == 2 else "score_window_kernel",
+        roofline = {"bound": "tensor", "kernel": "score_persist_kernel (two sweep launches per step; per-launch figures)",
                     "achieved": sus_tf, "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                     "frac": sus_tf / peaks["bf16_tflops_sustained"],
                     "timing": ("score stage, CUDA events, settled half of a %.1f s loop of the whole pass" % sus["seconds"]) if sus else "score stage of the timed steps",

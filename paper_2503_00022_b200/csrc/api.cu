@@ -143,6 +143,18 @@ int kvcrush_diag_score(const kvcrush_problem_t* problem, const kvcrush_tensor_t*
                      status_dev, stream, diag);
 }
 
+// Not part of the public ABI: kernels that kvcrush_score launches for a problem that the tensor-core kernels take, without
+// lse_in_dev (two sweeps, or the one-pass window kernel once for every cluster size), or a negative error code.
+// *one_pass: which of the two.
+int kvcrush_diag_score_kernels(const kvcrush_problem_t* problem, int* one_pass) {
+  Shape s;
+  const int rc = make_shape(problem, &s);
+  if (rc != KVCRUSH_OK) return rc;
+  if (!one_pass) return KVCRUSH_ERR_INVALID_ARG;
+  *one_pass = score_window_fits(s);
+  return *one_pass ? score_window_launches(s, problem->cu_seqlens_host) : 2;
+}
+
 int kvcrush_score_decode(const kvcrush_problem_t* problem, const kvcrush_tensor_t* Q_new, const kvcrush_tensor_t* K,
                          float* scores_dev, int32_t* status_dev, void* stream) {
   Shape s;

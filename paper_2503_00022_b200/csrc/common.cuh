@@ -150,7 +150,9 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
                         cudaStream_t stream);
 
 // Observation windows of up to 64 queries in one pass over the keys (tensor cores); score_window_fits: does it apply.
+// score_window_launches: kernels it then takes.
 bool score_window_fits(const Shape& s);
+int score_window_launches(const Shape& s, const int32_t* cu_host);
 int launch_score_window(const Shape& s, const int32_t* cu_host, const TensorView& Q, const ScoreTensorMaps& maps,
                         float scale_log2, float* scores, float* lse_out, int normalize, int32_t* status, const ScoreDiag& diag, cudaStream_t stream);
 

@@ -643,16 +643,59 @@ int launch_window(const CUtensorMap& mq, const CUtensorMap& mk, const WinArgs& a
                      : launch_window_polls<D, NC, kWaitPolls>(mq, mk, a, units, log_cta, stream);
 }
 
+int pad_window(int window) {
+  int n_pad = 16;
+  while (n_pad < window) n_pad *= 2;
+  return n_pad;
+}
+
+// CTAs per cluster: as few as hold the logits, more while the launch would leave SMs idle.  A batch whose sequences need
+// clusters of different sizes is launched once for each size, longest first, if that spares at least two rounds of the
+// chip: 8192 and 15 x 300 tokens (4 layers x 32 heads, 64 queries) 744 -> 198 us (the two sweeps 348), 4200 and 4000 tokens
+// (1 layer) 45 us together, 47 apart.
+struct Plan {
+  int cta_tokens;            // keys whose logits one CTA holds
+  long long units[4], together;      // (layer, sequence, head)s by the log2 of the cluster size they need, and all of them
+  int longest[4], largest;   // longest sequence of a size, largest size
+  bool split;
+};
+Plan plan_launches(const Shape& s, const int32_t* cu_host, int n_sms, int n_pad) {
+  Plan p{};
+  p.cta_tokens = kCols / n_pad * kTile;
+  for (int i = 0; i < s.n_seqs; ++i) {
+    const int len = cu_host[i + 1] - cu_host[i];
+    if (len == 0) continue;
+    int need = 0;
+    while (len > p.cta_tokens << need) ++need;
+    p.units[need] += (long long)s.n_layers * s.Hq;
+    p.longest[need] = len > p.longest[need] ? len : p.longest[need];
+    p.largest = need > p.largest ? need : p.largest;
+  }
+  auto rounds = [&](long long n, int log_cta) {
+    const int clusters = n_sms >> log_cta > 0 ? n_sms >> log_cta : 1;
+    return (n + clusters - 1) / clusters;
+  };
+  long long apart = 0;
+  for (int need = 0; need < 4; ++need) { apart += rounds(p.units[need], need); p.together += p.units[need]; }
+  p.split = rounds(p.together, p.largest) >= apart + 2;
+  return p;
+}
+
 }  // namespace
 
 // The one-pass kernel takes windows of up to 64 queries when the logits of a cluster's keys fit its TMEM: sequences of
 // up to 65536 / (window rounded up) x 8 tokens; the rest goes to the two sweeps.
 bool score_window_fits(const Shape& s) {
   if (s.window < 1 || s.window > kMaxN || s.max_seqlen < 1) return false;
-  int n_pad = 16;
-  while (n_pad < s.window) n_pad *= 2;
   const int tiles = (s.max_seqlen + kTile - 1) / kTile;
-  return (tiles + kMaxCluster - 1) / kMaxCluster * n_pad <= kCols && (long long)s.n_layers * s.n_seqs * s.Hq <= 0x7FFFFFFFLL / kMaxCluster;
+  return (tiles + kMaxCluster - 1) / kMaxCluster * pad_window(s.window) <= kCols && (long long)s.n_layers * s.n_seqs * s.Hq <= 0x7FFFFFFFLL / kMaxCluster;
+}
+
+int score_window_launches(const Shape& s, const int32_t* cu_host) {
+  const Plan p = plan_launches(s, cu_host, sm_count(), pad_window(s.window));
+  int n = 0;
+  for (int need = 0; need < 4; ++need) n += p.units[need] > 0;
+  return p.split ? n : 1;
 }
 
 int launch_score_window(const Shape& s, const int32_t* cu_host, const TensorView& Q, const ScoreTensorMaps& maps, float scale_log2, float* scores,
@@ -662,8 +705,7 @@ int launch_score_window(const Shape& s, const int32_t* cu_host, const TensorView
   a.bf16 = Q.dtype == KVCRUSH_BF16; a.status = status; a.k_steps = (s.D + 15) / 16;
   a.withhold_first_item = diag.withhold_first_item;
   a.n_units = s.n_layers * s.n_seqs * s.Hq;
-  a.n_pad = 16;
-  while (a.n_pad < s.window) a.n_pad *= 2;
+  a.n_pad = pad_window(s.window);
   a.ring = kMaxRing;                                // two query buffers of n_pad rows take the sixth tile at most
   CUtensorMap mq;
   if (!make_map(&mq, Q, s.D, s.T, s.Hq, s.n_layers, a.n_pad)) return KVCRUSH_ERR_UNSUPPORTED;
@@ -671,41 +713,20 @@ int launch_score_window(const Shape& s, const int32_t* cu_host, const TensorView
   const bool sw = diag.short_waits != 0;
   auto launch = s.D > 64 ? (a.n_pad == 16 ? launch_window<128, 16> : launch_window<128, 32>)
                          : (a.n_pad == 16 ? launch_window<64, 16> : launch_window<64, 32>);
-  // CTAs per cluster: as few as hold the logits, more while the launch would leave SMs idle.  A batch whose sequences need
-  // clusters of different sizes is launched once for each size, longest first, if that spares at least two rounds of the
-  // chip: 8192 and 15 x 300 tokens (4 layers x 32 heads, 64 queries) 744 -> 202 us (the two sweeps 348), 4200 and 4000 tokens
-  // (1 layer) 45 us together, 47 apart.
-  const int n_sms = sm_count(), cta_tokens = kCols / a.n_pad * kTile;
-  long long units[4] = {0, 0, 0, 0};
-  int longest[4] = {0, 0, 0, 0}, largest = 0;
-  for (int i = 0; i < s.n_seqs; ++i) {
-    const int len = cu_host[i + 1] - cu_host[i];
-    if (len == 0) continue;
-    int need = 0;
-    while (len > cta_tokens << need) ++need;
-    units[need] += (long long)s.n_layers * s.Hq;
-    longest[need] = len > longest[need] ? len : longest[need];
-    largest = need > largest ? need : largest;
-  }
-  auto rounds = [&](long long n, int log_cta) {
-    const int clusters = n_sms >> log_cta > 0 ? n_sms >> log_cta : 1;
-    return (n + clusters - 1) / clusters;
-  };
-  long long apart = 0, together = 0;
-  for (int need = 0; need < 4; ++need) { apart += rounds(units[need], need); together += units[need]; }
-  const bool split = rounds(together, largest) >= apart + 2;
-  for (int need = largest; need >= 0; --need) {
-    const long long n = split ? units[need] : together;
+  const int n_sms = sm_count();
+  const Plan plan = plan_launches(s, cu_host, n_sms, a.n_pad);
+  for (int need = plan.largest; need >= 0; --need) {
+    const long long n = plan.split ? plan.units[need] : plan.together;
     if (n == 0) continue;
-    if (split) {
-      a.min_len = need == 0 ? 1 : (cta_tokens << (need - 1)) + 1;
-      a.max_len = cta_tokens << need;
+    if (plan.split) {
+      a.min_len = need == 0 ? 1 : (plan.cta_tokens << (need - 1)) + 1;
+      a.max_len = plan.cta_tokens << need;
     }
-    const int tiles = (longest[need] + kTile - 1) / kTile;
+    const int tiles = (plan.longest[need] + kTile - 1) / kTile;
     int log_cta = need;
     while (log_cta < 3 && (tiles + (1 << log_cta) - 1) >> log_cta > 1 && n << (log_cta + 1) <= n_sms) ++log_cta;
     const int rc = launch(mq, mk, a, (int)n, log_cta, sw, stream);
-    if (rc != KVCRUSH_OK || !split) return rc;
+    if (rc != KVCRUSH_OK || !plan.split) return rc;
   }
   return KVCRUSH_OK;
 }

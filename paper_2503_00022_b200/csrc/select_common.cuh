@@ -150,7 +150,8 @@ __device__ __forceinline__ void for_items(bool far, int n, Load&& load, F&& f) {
 // minimum and maximum), over (upper half - smallest upper half) from the top bit in which they differ at all, so that the
 // bins are spread whatever the keys' common magnitude; usually at most 256 keys are left in the bin of the k-th largest
 // and are ranked directly (24 of them by one warp with 64-bit shuffles took 3 of the step's 10 thousand cycles).
-// Otherwise radix rounds over the whole keys follow; then one ordered pass marks the members.  Called by all threads of the block; imp_mask must be zero on entry; 0 < k < n.
+// Otherwise radix rounds over the whole keys follow; then one ordered pass marks the members.  Called by all threads of the
+// block; imp_mask must be zero on entry; 0 < k < n.
 // copy: optional shared memory for n words; keys that are not in shared memory are then read whole only where it matters
 // (the sweeps over 32768 keys took 9 thousand cycles each through L2).
 template <int kT>

@@ -115,6 +115,17 @@ def test_one_pass_window_scores_match_oracle(B, layers, Hq, Hkv, D, seqlens, win
             assert (gl[l][:, a:a + j0] == 7.0).all()
 
 
+@pytest.mark.parametrize("layers,seqlens,window,want", [
+    (4, (8192,), 64, (1, 1)), (4, (8192,) + (300,) * 15, 64, (2, 1)), (1, (4200, 4000), 64, (1, 1)),
+    (4, (8193,), 64, (2, 0)), (4, (8192,), 65, (2, 0)), (4, (8192,), 0, (2, 0)),
+])
+def test_score_kernel_count_follows_the_dispatch(B, layers, seqlens, window, want):
+    import ctypes
+    prob = B.Problem(layers, 32, 32, 128, seqlens, device=_dev(), query_window=window)
+    one_pass = ctypes.c_int(-1)
+    assert (B.lib().kvcrush_diag_score_kernels(prob.ref, ctypes.byref(one_pass)), one_pass.value) == want
+
+
 @pytest.mark.parametrize("L,window", [
     (100, 16),                                            # one CTA alone
     (1000, 64),                                           # a cluster of 8, one tile of keys each
