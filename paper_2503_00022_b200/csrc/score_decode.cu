@@ -322,7 +322,9 @@ int launch_width(const Shape& s, const TensorView& Qn, const TensorView& K, floa
   // fewer than 256 keys, and at most 16 KB of logits a block while the cluster can grow.
   const int n_sms = sm_count();
   int n_blk = 1;
-  while (n_blk < kMaxCluster && tokens(n_blk) > 256 && (units * n_blk < 8 * n_sms || bytes(n_blk) > 16 * 1024)) n_blk *= 2;
+  while (n_blk < kMaxCluster && 2 * units * n_blk <= 0x7FFFFFFFLL && tokens(n_blk) > 256 &&
+         (units * n_blk < 8 * n_sms || bytes(n_blk) > 16 * 1024))
+    n_blk *= 2;
   if (units * n_blk > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
   const size_t dyn = bytes(n_blk);
   const int cap = tokens(n_blk);
