@@ -277,15 +277,18 @@ decode_update_kernel(Shape s, TensorView Qn, TensorView K, float scale_log2, flo
       for (int h = 0; h < n_heads; ++h) {
         float* out = scores + ((long long)layer * s.Hq + h0 + h) * s.T + t0 + lo;
         const float f = fin[h];
+        bool tiny = false;
 #pragma unroll 4
         for (int i = tid; i < hi - lo; i += kWarps * 32) {
           const float v = x_sh[h * cap + i] * f;
-          if (v < 0x1p-100f) {
-            if (v > 0.f) __stcg(out + i, __ldcg(out + i) + v);
-          } else {
-            atomicAdd(out + i, v);
-          }
+          if (!(v < 0x1p-100f)) atomicAdd(out + i, v);
+          tiny |= v < 0x1p-100f && v > 0.f;
         }
+        if (tiny)
+          for (int i = tid; i < hi - lo; i += kWarps * 32) {
+            const float v = x_sh[h * cap + i] * f;
+            if (v < 0x1p-100f && v > 0.f) __stcg(out + i, __ldcg(out + i) + v);
+          }
       }
     } else {
       for_tiles<T, DB, kWarps>(kbase, K.st, lo, hi, s.D, warp, lane, qr, q_sh, [&](int t, const float (&x)[4]) {

@@ -20,6 +20,7 @@
 // logits leave [-100, 100] or hold a NaN keep them, count with their exact maxima in step 1 and take 2^(x - lse2) in step 2.
 // So a stored 2^x is finite; a query's sum may be NaN, and is then NaN in every key it votes for, and in no other.  For a
 // query whose lse2 is above 126, 2^-lse2 would be flushed to zero: the stored 2^x are multiplied by its square root twice.
+// A unit with such a query, or one whose sum is NaN, takes step 2 value by value.
 //
 // Roles: warp 0 issues TMA loads, warp 1 the tcgen05.mma; warps 2..17 are four epilogue groups of four warps.  All waits
 // are bounded as in score_tc.cu; all CTAs of a cluster meet once more before they leave, because peers write into their
@@ -72,6 +73,7 @@ struct WAux {
   uint32_t tmem_base;
   int abort_flag;
   int n_unit;                                           // units whose sums this CTA has received
+  int by_value;                                         // 1 + the last unit with a query whose lse2 is above 126 or NaN
   alignas(16) float nlse[kMaxN];                        // minus log2 sum of the window's queries, -inf: no vote
   alignas(16) float factor[kMaxN];                      // 2^nlse
   unsigned char kept[kMaxSlots][4][4];                  // [tile][column block][lane quarter]: logits were kept
@@ -269,7 +271,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   }
   chain_wait();
   chain_trigger();
-  if (tid == 0) aux->n_unit = 0;
+  if (tid == 0) aux->n_unit = aux->by_value = 0;
   if (tid == 0) aux->abort_flag = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
   tc_fence_before();
   __syncthreads();
@@ -507,6 +509,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         if (sub == 0) {
           const float lse2 = m + log2f(t);
           aux->nlse[col] = col < w.nv ? -lse2 : kNegInf;
+          if (col < w.nv && !(lse2 <= 126.f)) aux->by_value = n_unit + 1;
           aux->factor[col] = col < w.nv ? ex2(lse2 < -126.f ? 126.f : -lse2) : 0.f;    // beyond 2^126 no column is below 2^100
           if (rank == 0 && col < w.nv && a.lse_nat_out)
             a.lse_nat_out[((size_t)w.layer * s.Hq + w.h) * s.T + w.t0 + w.q0 + col] = lse2 * 0.69314718055994530942f;
@@ -519,37 +522,25 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
       // ---- step 2: every key's sum over the queries ----
       tc_fence_after();
-      bool deep = false;                            // a query with lse2 > 126 (its factor is zero)
-      for (int c = lane; c < w.nv; c += 32) deep |= aux->nlse[c] < -126.f;
-      deep = __any_sync(0xFFFFFFFFu, deep);
+      const bool by_value = aux->by_value == n_unit + 1;
       for (int j = gi; j < w.n; j += 4) {
         const int key = (w.tile0 + j) * kTile + r;
         const uint32_t t_acc = t_lane + j * n_pad;
-        const bool edge = s.causal && key - lane + 31 > w.q0;          // a masked column somewhere in the warp's keys
         f32x2 acc[2] = {0ull, 0ull};
         for (int b = 0; b < n_cb; ++b) {
           uint32_t x[NC];
           tmem_ldn(t_acc + b * NC, x);
           tmem_waitn(x);
-          const int c_first = first_col(key) - b * NC;
-          if (!deep && !aux->kept[j][b][quarter]) {
+          if (!by_value && !aux->kept[j][b][quarter]) {
             const float4* f4 = reinterpret_cast<const float4*>(aux->factor + b * NC);
-            auto add = [&](auto masked) {
 #pragma unroll
-              for (int i = 0; i < NC / 4; ++i) {
-                float4 f = f4[i];
-                if constexpr (decltype(masked)::value) {               // the stored 2^x is 0 there, but 0 * NaN is not
-                  f.x = 4 * i >= c_first ? f.x : 0.f;
-                  f.y = 4 * i + 1 >= c_first ? f.y : 0.f;
-                  f.z = 4 * i + 2 >= c_first ? f.z : 0.f;
-                  f.w = 4 * i + 3 >= c_first ? f.w : 0.f;
-                }
-                acc[0] = fma2(pack2(x[4 * i], x[4 * i + 1]), pack2f(f.x, f.y), acc[0]);
-                acc[1] = fma2(pack2(x[4 * i + 2], x[4 * i + 3]), pack2f(f.z, f.w), acc[1]);
-              }
-            };
-            if (edge) add(std::true_type{}); else add(std::false_type{});
+            for (int i = 0; i < NC / 4; ++i) {
+              const float4 f = f4[i];
+              acc[0] = fma2(pack2(x[4 * i], x[4 * i + 1]), pack2f(f.x, f.y), acc[0]);
+              acc[1] = fma2(pack2(x[4 * i + 2], x[4 * i + 3]), pack2f(f.z, f.w), acc[1]);
+            }
           } else {
+            const int c_first = first_col(key) - b * NC;
             const bool keep = aux->kept[j][b][quarter];
             float t = 0.f;
 #pragma unroll
