@@ -300,11 +300,11 @@ __device__ __forceinline__ void mark_top_keys(const unsigned long long* keys, in
   __syncthreads();
 }
 
-// Writes the members of imp_mask | rep_mask in ascending order (kind: 1 for members of rep_mask).
+// Writes the members of imp_mask | rep_mask in ascending order (kind: 1 for members of rep_mask), counted from item `first`.
 // Called by all threads of the block after the masks are complete.
 template <int kT>
 __device__ __forceinline__ void emit_kept(const uint32_t* imp_mask, const uint32_t* rep_mask, int n_words,
-                                          int32_t* out_idx, uint8_t* out_kind, Scratch& sc) {
+                                          int32_t* out_idx, uint8_t* out_kind, Scratch& sc, int first = 0) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // every thread takes a contiguous run of mask BYTES (8 items each): with fewer words than threads a word-wise
   // split would leave most threads idle and the others with up to 32 serial stores
@@ -331,7 +331,7 @@ __device__ __forceinline__ void emit_kept(const uint32_t* imp_mask, const uint32
     while (bits) {
       const int k = __ffs(bits) - 1;
       bits &= bits - 1;
-      out_idx[pos] = 8 * b + k;
+      out_idx[pos] = first + 8 * b + k;
       if (out_kind) out_kind[pos] = (rep >> k) & 1u;
       ++pos;
     }

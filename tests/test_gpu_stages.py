@@ -131,6 +131,19 @@ def test_select_in_blocks_of_every_size(B, Hq, seqlens, mode, ties):
     _select_case(B, Hq, Hq, seqlens, budgets, 1, ties, mode, seed=370 + len(seqlens))
 
 
+@pytest.mark.parametrize("Hq,layers,seqlens,b_imp,b_rep,mode,ties,share", [
+    (32, 1, [8192], 800, 1200, 0, 0, True), (8, 3, [8193, 31, 1], 900, 1300, 1, 0, True),    # four blocks; parts of 32 tokens and none
+    (8, 1, [8200], 300, 3, 0, 0, True), (8, 1, [16385], 100, 1, 2, 0, True),                 # fewer buckets than blocks: order in global memory
+    (128, 1, [9000], 400, 1700, 1, 0, True), (72, 2, [17001, 100], 0, 2900, 2, 2, False),    # four and three signature words; nothing important
+    (32, 5, [8222], 500, 0, 0, 0, True), (40, 8, [8233], 333, 2222, 0, 3, True),             # no buckets; ties cut across blocks
+    (4, 2, [20000], 700, 1700, 0, 2, False), (4, 1, [45000], 500, 9000, 0, 0, True),         # eight blocks
+    (4, 32, [8195], 700, 600, 0, 0, True), (4, 33, [8195], 700, 600, 0, 0, True),            # as many segments as take clusters, and one more
+])
+def test_select_by_a_cluster_of_blocks(B, Hq, layers, seqlens, b_imp, b_rep, mode, ties, share):
+    budgets = [(b_imp, b_rep)] + [(max(1, L // 6), L // 5) for L in seqlens[1:]]
+    _select_case(B, Hq, Hq, seqlens, budgets, layers, ties, mode, seed=410 + Hq + layers, share_importance=share)
+
+
 @pytest.mark.parametrize("seqlens,ties", [
     ([1, 2, 31, 32, 33, 256], 0), ([255, 256, 1, 100], 2),       # 8 keys a lane
     ([257, 31, 512], 0), ([511, 512, 480], 3),                   # 16
