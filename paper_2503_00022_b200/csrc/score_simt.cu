@@ -5,7 +5,8 @@
 // Two sweeps of one tiled kernel: row log-sum-exps, then column sums.  64 x 64 logit tiles from fp32 copies of both
 // operands in shared memory, 4 x 4 logits a thread, so that a 16-byte shared-memory read feeds eight FMAs (one warp
 // per row and one dot product per lane spent 170 us on 8 heads x 512 tokens of 64 channels, all of it waiting for loads,
-// and 2174 us on 4 layers of 1024 tokens; the two sweeps now take 26 and 180 us).
+// and 2174 us on 4 layers of 1024 tokens; the two sweeps now take 26 and 180 us one after the other).  The column sweep
+// stages its tiles and forms its first logits while the row sweep ends: whole pass of 8 heads x 512 tokens 44.8 -> 39.8 us.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -27,14 +28,14 @@ __device__ __forceinline__ void load8(const T* p, float (&v)[8]);
 
 template <>
 __device__ __forceinline__ void load8<float>(const float* p, float (&v)[8]) {
-  const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-  const float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  const float4 a = __ldcg(reinterpret_cast<const float4*>(p));
+  const float4 b = __ldcg(reinterpret_cast<const float4*>(p) + 1);
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 
 template <>
 __device__ __forceinline__ void load8<__nv_bfloat16>(const __nv_bfloat16* p, float (&v)[8]) {
-  const uint4 r = __ldg(reinterpret_cast<const uint4*>(p));
+  const uint4 r = __ldcg(reinterpret_cast<const uint4*>(p));
   const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -45,7 +46,7 @@ __device__ __forceinline__ void load8<__nv_bfloat16>(const __nv_bfloat16* p, flo
 
 template <>
 __device__ __forceinline__ void load8<__half>(const __half* p, float (&v)[8]) {
-  const uint4 r = __ldg(reinterpret_cast<const uint4*>(p));
+  const uint4 r = __ldcg(reinterpret_cast<const uint4*>(p));
   const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -88,14 +89,16 @@ template <typename T, bool kColsum, int N>
 __global__ void __launch_bounds__(kThreads)
 simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const float* __restrict__ lse, float lse_mul,
                   float* __restrict__ lse2_out, float* __restrict__ lse_nat_out, float* __restrict__ scores, int normalize,
-                  int layer0, int n_layers, int by_seq) {
+                  int layer0, int n_layers, int by_seq, int early) {
   extern __shared__ float4 dyn4[];
   float* fix_sh = reinterpret_cast<float*>(dyn4);
   float* str_sh = fix_sh + 16 * N * (s.D + kPad);
   __shared__ float part[2][kRows];                          // this block's maximum (sweep 1) and sum of every row
   __shared__ float nlse_sh[kRows];                          // sweep 2: minus lse2 of the streamed queries that vote
-  chain_wait();
-  chain_trigger();
+  if (!kColsum || !early) {                                 // early: sweep 1 of the same call is the launch before
+    chain_wait();
+    chain_trigger();
+  }
   cg::cluster_group cluster = cg::this_cluster();
   const int n_blk = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -134,10 +137,6 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
   for (int u = first + rank; u < last; u += n_blk) {
     __syncthreads();                                        // the previous tile is done with
     stage_tile<T, 16 * N>(str_sh, kColsum ? qbase : kbase, kColsum ? Q.st : K.st, u * kRows, L, s.D);
-    if (kColsum && tid < kRows) {
-      const int j = u * kRows + tid;
-      nlse_sh[tid] = j < L && j >= ws ? -(__ldg(lse + vec0 + j) * lse_mul) : ninf;
-    }
     __syncthreads();
     float acc[N][N];
 #pragma unroll
@@ -159,6 +158,17 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
 #pragma unroll
         for (int j = 0; j < N; ++j)
           acc[i][j] = fmaf(a[i].w, b[j].w, fmaf(a[i].z, b[j].z, fmaf(a[i].y, b[j].y, fmaf(a[i].x, b[j].x, acc[i][j]))));
+    }
+    if constexpr (kColsum) {                                // the row log-sum-exp is needed only now
+      if (early && u == first + rank) {
+        chain_wait();
+        chain_trigger();
+      }
+      if (tid < kRows) {
+        const int j = u * kRows + tid;
+        nlse_sh[tid] = j < L && j >= ws ? -(__ldcg(lse + vec0 + j) * lse_mul) : ninf;
+      }
+      __syncthreads();
     }
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -217,7 +227,7 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
 
 template <typename T, bool kColsum, int N>
 int launch_sweep(const Shape& s, const int32_t* cu_host, const TensorView& Q, const TensorView& K, float scale_log2, const float* lse, float lse_mul,
-                 float* lse2_out, float* lse_nat_out, float* scores, int normalize, cudaStream_t stream) {
+                 float* lse2_out, float* lse_nat_out, float* scores, int normalize, bool early, cudaStream_t stream) {
   const int max_tiles = (s.max_seqlen + kRows - 1) / kRows;
   long long tiles = 0;
   for (int i = 0; i < s.n_seqs; ++i) tiles += (cu_host[i + 1] - cu_host[i] + kRows - 1) / kRows;
@@ -243,7 +253,7 @@ int launch_sweep(const Shape& s, const int32_t* cu_host, const TensorView& Q, co
   for (int layer0 = 0; layer0 < s.n_layers; layer0 += layers) {
     const int n = s.n_layers - layer0 < layers ? s.n_layers - layer0 : layers;
     const int rc = launch_kernel(overlap, kern, dim3((unsigned)(per_layer * n)), dim3(kThreads), dyn, stream, n_blk, s, Q, K, scale_log2,
-                                  lse, lse_mul, lse2_out, lse_nat_out, scores, normalize, layer0, n, by_seq);
+                                  lse, lse_mul, lse2_out, lse_nat_out, scores, normalize, layer0, n, by_seq, early && overlap && layer0 == 0);
     if (rc != KVCRUSH_OK) return rc;
   }
   return KVCRUSH_OK;
@@ -253,11 +263,11 @@ template <typename T, int N>
 int run_tiles(const Shape& s, const int32_t* cu_host, const TensorView& Q, const TensorView& K, float scale_log2, const float* lse_in,
               float lse_in_mul, float* lse2_ws, float* scores, float* lse_out, int normalize, cudaStream_t stream) {
   if (!lse_in) {
-    const int rc = launch_sweep<T, false, N>(s, cu_host, Q, K, scale_log2, nullptr, 1.f, lse2_ws, lse_out, nullptr, 0, stream);
+    const int rc = launch_sweep<T, false, N>(s, cu_host, Q, K, scale_log2, nullptr, 1.f, lse2_ws, lse_out, nullptr, 0, false, stream);
     if (rc != KVCRUSH_OK) return rc;
-    return launch_sweep<T, true, N>(s, cu_host, Q, K, scale_log2, lse2_ws, 1.f, nullptr, nullptr, scores, normalize, stream);
+    return launch_sweep<T, true, N>(s, cu_host, Q, K, scale_log2, lse2_ws, 1.f, nullptr, nullptr, scores, normalize, true, stream);
   }
-  return launch_sweep<T, true, N>(s, cu_host, Q, K, scale_log2, lse_in, lse_in_mul, nullptr, nullptr, scores, normalize, stream);
+  return launch_sweep<T, true, N>(s, cu_host, Q, K, scale_log2, lse_in, lse_in_mul, nullptr, nullptr, scores, normalize, false, stream);
 }
 
 template <typename T>

@@ -586,3 +586,36 @@ def test_cuda_core_scores_at_the_edges_of_their_tiles(B, dtype, D, Hq, Hkv, seql
             assert TL.within_score_tolerance(g[l][:, a:b], c).all(), (l, s)
             np.testing.assert_allclose(gl[l][:, a + j0:b], ol[:, j0:], rtol=0, atol=2e-5)
             assert (gl[l][:, a:a + j0] == 7.0).all()                       # rows that do not vote are not written
+
+
+@pytest.mark.parametrize("layers,Hq,Hkv,D,seqlens,dtype", [
+    (1, 8, 8, 64, [512], "float32"), (2, 4, 2, 32, [130, 1, 257], "float32"),               # CUDA cores, with and without clusters
+    (1, 32, 8, 128, [1001], "bfloat16"), (1, 16, 16, 64, [300, 128, 700], "float16"),       # tensor cores, items dealt out in advance
+    (2, 32, 8, 96, [1500, 1100], "bfloat16"),                                               # by the counter
+])
+def test_a_pass_follows_inputs_written_just_before_it(B, layers, Hq, Hkv, D, seqlens, dtype):
+    """Kernels of a call that read its inputs before the kernel in front of them has ended: queries, keys and scores written by
+    the launch before the call give what they give after a synchronisation, bit for bit."""
+    import torch
+    dev, dt = _dev(), getattr(torch, dtype)
+    T = sum(seqlens)
+    prob = B.Problem(layers, Hq, Hkv, D, seqlens, device=dev)
+    keep = np.asarray([[max(1, L // 8) for L in seqlens]], dtype=np.int32)
+    cp = B.CompressionPass(prob, keep, keep, cache_dtype=dt)
+    g = torch.Generator(device=dev).manual_seed(11)
+    new = lambda h: torch.randn((layers, T, h, D), generator=g, device=dev).to(dt)
+    q, k, v = new(Hq), new(Hkv), new(Hkv)
+    outs = lambda: [x.clone() for x in (cp.scores, cp.theta, cp.sigs, cp.importance, cp.idx, cp.k_out, cp.v_out)]
+    for _ in range(4):
+        q2, k2 = new(Hq), new(Hkv)
+        cp.run(q, k, k, v)                       # the old inputs are in every cache
+        q.copy_(q2)
+        k.copy_(k2)
+        cp.run(q, k, k, v)
+        got = outs()
+        torch.cuda.synchronize()
+        cp.run(q, k, k, v)
+        torch.cuda.synchronize()
+        cp.check_status()
+        for a, b in zip(got, outs()):
+            assert torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
