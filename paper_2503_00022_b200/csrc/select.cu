@@ -478,8 +478,7 @@ select_cluster_kernel(Shape s, SelectArgs a) {
   __shared__ int all_bits[C][128];
   __shared__ int all_equal[C], all_kept[C];
   cluster_arrive();                                  // (waited for below: all blocks have started)
-  chain_wait();
-  chain_trigger();
+  chain_wait();                                      // (chain_trigger: at the end)
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -894,6 +893,7 @@ select_cluster_kernel(Shape s, SelectArgs a) {
     const int total = __reduce_add_sync(kFull, lane < kWarps ? sc.warp_tot[lane] : 0);
     if (lane < C) *peer_of(&all_kept[rank], lane) = total;
   }
+  chain_trigger();                                   // blocks of the next kernel, set up earlier, would crowd on the SMs without a cluster
   cluster_barrier();                                 // from here on nobody touches a peer's memory
   int before = 0;
   for (int c = 0; c < rank; ++c) before += all_kept[c];
@@ -929,8 +929,9 @@ size_t cluster_bytes(const Shape& s, int cap) { return (size_t)cap / 4 + (size_t
 // 70.7 / 34.1 / 81.  Twice as many take two rounds of half the time: 36 of 8192 19.6 / 35.7, but 64 of 32768 74.8 / 67.1.
 int select_cluster_size(const Shape& s, long long n_seg, int n_sms) {
   auto fits = [&](int c) { return cluster_bytes(s, cluster_tokens(s, c)) <= (size_t)kClusterSmem; };
-  if (s.max_seqlen < 8192) return 0;
-  if (s.max_seqlen > 16384 && n_seg * 8 <= n_sms * 4 / 5 && fits(8)) return 8;
+  const bool few = n_seg * 8 <= n_sms * 4 / 5;
+  if (s.max_seqlen < (few ? 8192 : 12288)) return 0;
+  if (s.max_seqlen > 16384 && few && fits(8)) return 8;
   if (n_seg * 4 <= n_sms * (s.max_seqlen > 24576 ? 7 / 4.0 : 7 / 8.0) && fits(4)) return 4;
   return 0;
 }

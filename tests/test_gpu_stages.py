@@ -137,7 +137,7 @@ def test_select_in_blocks_of_every_size(B, Hq, seqlens, mode, ties):
     (128, 1, [9000], 400, 1700, 1, 0, True), (72, 2, [17001, 100], 0, 2900, 2, 2, False),    # four and three signature words; nothing important
     (32, 5, [8222], 500, 0, 0, 0, True), (40, 8, [8233], 333, 2222, 0, 3, True),             # no buckets; ties cut across blocks
     (4, 2, [20000], 700, 1700, 0, 2, False), (4, 1, [45000], 500, 9000, 0, 0, True),         # eight blocks
-    (4, 32, [8195], 700, 600, 0, 0, True), (4, 33, [8195], 700, 600, 0, 0, True),            # as many segments as take clusters, and one more
+    (4, 32, [12300], 700, 900, 0, 0, True), (4, 33, [12300], 700, 900, 0, 0, True),          # as many segments as take clusters, and one more
 ])
 def test_select_by_a_cluster_of_blocks(B, Hq, layers, seqlens, b_imp, b_rep, mode, ties, share):
     budgets = [(b_imp, b_rep)] + [(max(1, L // 6), L // 5) for L in seqlens[1:]]
