@@ -8,13 +8,16 @@
 //   step 1  puts 2^x in the logit's place, sums it over its keys for every query and exchanges the sums through
 //           distributed shared memory,
 //   step 2  adds 2^x * 2^-lse2(query) over the queries of every key, from the same accumulators.
-// The CTAs live for the whole launch; while step 2 works on one unit the next unit's keys are already on their way, and
-// its tiles are multiplied as their accumulators become free, so the loads hardly pause.
-// Measured, 32 layers x 32 heads x 8192 tokens of 128 channels (2.1 GB of keys): 16 queries 382 us, 32 queries 481 us, 64
-// queries 705 us, where the two sweeps take 1150, 1155 and 1122 us; 1000 tokens, 64 queries 77 against 172 us.  With 64
-// queries a cluster of 8 needs all its accumulators for one unit, and the chain load - sum - exchange - add is no longer
-// hidden by the next unit's loads.  Taken back: clusters of 16 with two units in TMEM (1056 us, and 1277 us with step 2 one
-// unit behind: half the keys a CTA, the same chain of latencies), windows of 128 queries (645 against 562 us at 4096 tokens).
+// The CTAs live for the whole launch.  Sixteen warps do step 1, four others the exchange and step 2; they hand units on through
+// barriers, and unit after unit takes the next accumulators round and round, so that loads, products, exponentials and sums of
+// up to three units overlap.  (With all warps at one unit's steps in turn the chain exponentials - exchange - sums was the
+// time.)  For a launch's last unit all of them share step 2.
+// Measured, 32 layers x 32 heads x 8192 tokens of 128 channels (2.1 GB of keys): 16 queries 352 us, 32 queries 430 us, 64
+// queries 633 us (with one group of warps for all steps 375, 512, 732; the two sweeps 1150, 1155 and 1122); 1000 tokens, 64
+// queries 71.5 us (79.6; 172), 8 layers of 5003 + 3117 tokens 184 (238), 8 layers x 40 heads of 12000 tokens, 32 queries 221 (293).
+// With 64 queries a cluster of 8 needs all its accumulators for one unit, and step 1 of the next one follows step 2 tile by
+// tile.  Taken back: clusters of 16 with two units in TMEM (1056 us, and 1277 with step 2 one unit behind: half the keys a CTA,
+// the same chain of latencies), windows of 128 queries (645 against 562 us at 4096 tokens, with one group of warps).
 //
 // 2^x is taken without a maximum: float32 has the range unless logits are extreme.  32 keys x one column block whose
 // logits leave [-100, 100] or hold a NaN keep them, count with their exact maxima in step 1 and take 2^(x - lse2) in step 2.
@@ -22,7 +25,8 @@
 // query whose lse2 is above 126, 2^-lse2 would be flushed to zero: the stored 2^x are multiplied by its square root twice.
 // A unit with such a query, or one whose sum is NaN, takes step 2 value by value.
 //
-// Roles: warp 0 issues TMA loads, warp 1 the tcgen05.mma; warps 2..17 are four epilogue groups of four warps.  All waits
+// Roles: warp 0 issues TMA loads, warp 1 the tcgen05.mma; warps 4..19 are the four groups of step 1, warps 20..23 the group of
+// the exchange and step 2.  All waits
 // are bounded as in score_tc.cu; all CTAs of a cluster meet once more before they leave, because peers write into their
 // shared memory, and one that gave up then waits for the stores that were on their way to it.
 #include <cuda.h>
@@ -40,9 +44,16 @@ using namespace tc;
 
 constexpr int kTile = 128;
 constexpr int kCols = 512;                   // TMEM columns
-constexpr int kCtrlWarps = 2;
-constexpr int kEpiWarps = 16;
-constexpr int kThreads = 32 * (kCtrlWarps + kEpiWarps);
+constexpr int kCtrlWarps = 4;                // one warpgroup: producer, issuer, two idle warps
+constexpr int kExpWarps = 16;                // four groups of four: step 1
+constexpr int kSumWarps = 4;                 // one group: exchange and step 2
+constexpr int kThreads = 32 * (kCtrlWarps + kExpWarps + kSumWarps);
+constexpr int kNC = 16;                      // columns of a step-1 thread
+// Registers: 80 a thread at launch (the most 24 warps can have); the control warpgroup gives some to the group of step 2.  With
+// 48 and 112 the producer and the issuer spill: 732 us instead of 633 for 64 queries of 8192 tokens.
+constexpr int kLaunchRegs = 80, kCtrlRegs = 64, kSumRegs = 96;
+static_assert(32 * (kCtrlWarps * kCtrlRegs + kExpWarps * kLaunchRegs + kSumWarps * kSumRegs) <= kThreads * kLaunchRegs,
+              "register split within the launch's total");
 constexpr int kMaxRing = 5;                  // key tiles in flight
 constexpr int kMaxSlots = 32;                // accumulators (windows of up to 16 queries)
 constexpr int kMaxCluster = 8;
@@ -57,7 +68,6 @@ struct WinArgs {
   int normalize;
   int bf16;
   int k_steps;               // 16-channel steps of a dot product
-  int n_pad;                 // accumulator columns: the window rounded up to 16, 32 or 64
   int ring;
   int n_units;               // n_layers * n_seqs * Hq
   int min_len, max_len;      // > 0: this launch takes the sequences of min_len to max_len tokens
@@ -69,15 +79,17 @@ struct WAux {
   unsigned long long k_full[kMaxRing], k_empty[kMaxRing];
   unsigned long long q_full[2], q_empty[2];
   unsigned long long acc_full[kMaxSlots], acc_empty[kMaxSlots];
-  unsigned long long epi_bar, part_full[2], drain;
+  unsigned long long sums_full[2], sums_empty[2];       // [unit parity]: warp_part and kept
+  unsigned long long sum_bar, part_full[2], last_unit, drain;
   uint32_t tmem_base;
   int abort_flag;
   int n_unit;                                           // units whose sums this CTA has received
-  int by_value;                                         // 1 + the last unit with a query whose lse2 is above 126 or NaN
-  alignas(16) float nlse[kMaxN];                        // minus log2 sum of the window's queries, -inf: no vote
-  alignas(16) float factor[kMaxN];                      // 2^nlse
-  unsigned char kept[kMaxSlots][4][4];                  // [tile][column block][lane quarter]: logits were kept
-  float warp_part[kEpiWarps][32][2];                    // (maximum, sum) of a warp's columns
+  int any_kept[2];                                      // [unit parity] 1 + the last unit that kept logits
+  int last_by_value;                                    // the last unit's step 2 goes value by value
+  alignas(16) float nlse[kSumWarps][kMaxN];             // [warp of step 2] minus log2 sum of the window's queries, -inf: no vote
+  alignas(16) float factor[kSumWarps][kMaxN];           // 2^nlse
+  uint32_t kept[2][kExpWarps];                          // [unit parity] tiles (bits) whose logits a warp of step 1 kept
+  float warp_part[2][kExpWarps][kNC][2];                // [unit parity] (maximum, sum) of a warp's columns
   float part[2][kMaxCluster][kMaxN];                    // [unit parity][CTA of the cluster][query]: log2 sum, -inf: no key
 };
 constexpr int kAuxBytes = 26624;
@@ -123,30 +135,7 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// 16 or 32 consecutive columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ldn(uint32_t taddr, uint32_t (&v)[16]) { tmem_ld16(taddr, v); }
-__device__ __forceinline__ void tmem_waitn(uint32_t (&v)[16]) { tmem_wait16(v); }
-__device__ __forceinline__ void tmem_ldn(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, "
-      "%24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]),
-        "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]),
-        "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_waitn(uint32_t (&v)[32]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
-                 "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
-                 "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
-                 "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
-               :: "memory");
-}
-// the same columns written (asynchronous: tcgen05.wait::st)
+// 16 columns written (asynchronous: tcgen05.wait::st)
 __device__ __forceinline__ void tmem_stn(uint32_t taddr, const uint32_t (&v)[16]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
@@ -155,26 +144,10 @@ __device__ __forceinline__ void tmem_stn(uint32_t taddr, const uint32_t (&v)[16]
         "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
       : "memory");
 }
-__device__ __forceinline__ void tmem_stn(uint32_t taddr, const uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, "
-      "%25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]),
-        "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]),
-        "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]),
-        "r"(v[29]), "r"(v[30]), "r"(v[31])
-      : "memory");
-}
-// NaN if any of the three is
-__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+// the largest magnitude, NaN if any of the three is
+__device__ __forceinline__ float max3_abs(float a, float b, float c) {
   float d;
-  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-__device__ __forceinline__ float min3(float a, float b, float c) {
-  float d;
-  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(fabsf(b)), "f"(fabsf(c)));
   return d;
 }
 
@@ -222,18 +195,20 @@ struct Unit {
   }
 };
 
-// NC: columns of one epilogue thread in step 1.  kPolls: polls of every bounded wait.
-template <int D, int NC, uint32_t kPolls>
+// NP: accumulator columns, the window rounded up to 16, 32 or 64.  kPolls: polls of every bounded wait.
+template <int D, int NP, uint32_t kPolls>
 __global__ void __launch_bounds__(kThreads, 1)
 score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const WinArgs a) {
+  constexpr int kSlots = kCols / NP;                // accumulators; unit after unit takes the next ones, round and round
   constexpr int kTileBytes = kTile * D * 2, kBlockBytes = kTile * 128;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   WAux* aux = reinterpret_cast<WAux*>(smem + kSmemTiles * kTileBytes);
   volatile int* abort_flag = &aux->abort_flag;
   const uint32_t ring_addr = smem_u32(smem);
-  const int ring = a.ring, n_pad = a.n_pad;
-  const uint32_t q_bytes = (uint32_t)n_pad * D * 2, q_addr = ring_addr + ring * kTileBytes;
+  const int ring = a.ring;
+  constexpr uint32_t q_bytes = NP * D * 2;
+  const uint32_t q_addr = ring_addr + ring * kTileBytes;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Shape& s = a.s;
   uint32_t rank, n_cta;
@@ -258,12 +233,15 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       mbar_init(smem_u32(&aux->q_full[i]), 1);
       mbar_init(smem_u32(&aux->q_empty[i]), 1);
       mbar_init(smem_u32(&aux->part_full[i]), 1);
+      mbar_init(smem_u32(&aux->sums_full[i]), kExpWarps);
+      mbar_init(smem_u32(&aux->sums_empty[i]), kSumWarps);
     }
-    for (int i = 0; i < kMaxSlots; ++i) { mbar_init(smem_u32(&aux->acc_full[i]), 1); mbar_init(smem_u32(&aux->acc_empty[i]), 4); }
-    mbar_init(smem_u32(&aux->epi_bar), kEpiWarps);
+    for (int i = 0; i < kMaxSlots; ++i) { mbar_init(smem_u32(&aux->acc_full[i]), 1); mbar_init(smem_u32(&aux->acc_empty[i]), kSumWarps); }
+    mbar_init(smem_u32(&aux->sum_bar), kSumWarps);
+    mbar_init(smem_u32(&aux->last_unit), kSumWarps);
     mbar_init(smem_u32(&aux->drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    for (int i = 0; i < 2; ++i) mbar_expect_tx(smem_u32(&aux->part_full[i]), n_cta * n_pad * 4);
+    for (int i = 0; i < 2; ++i) mbar_expect_tx(smem_u32(&aux->part_full[i]), n_cta * NP * 4);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   } else if (warp == 1) {
     tmem_alloc(smem_u32(&aux->tmem_base), kCols);
@@ -271,7 +249,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   }
   chain_wait();
   chain_trigger();
-  if (tid == 0) aux->n_unit = aux->by_value = 0;
+  if (tid == 0) aux->n_unit = aux->any_kept[0] = aux->any_kept[1] = aux->last_by_value = 0;
   if (tid == 0) aux->abort_flag = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
   tc_fence_before();
   __syncthreads();
@@ -282,7 +260,9 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
   if (dead) {
     // nothing to do
-  } else if (warp == 0) {
+  } else if (warp < kCtrlWarps) {
+  set_max_regs<kCtrlRegs, false>();
+  if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
     if (lane == 0) {
       int rs = 0, n_q = 0, n_k = 0;
@@ -297,7 +277,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         mbar_expect_tx(smem_u32(&aux->q_full[qs]), q_bytes);
 #pragma unroll
         for (int kb = 0; kb < D / 64; ++kb)
-          tma_load_4d(q_addr + qs * q_bytes + kb * n_pad * 128, &map_q, smem_u32(&aux->q_full[qs]), kb * 64, w.t0 + w.q0, w.h, w.layer);
+          tma_load_4d(q_addr + qs * q_bytes + kb * NP * 128, &map_q, smem_u32(&aux->q_full[qs]), kb * 64, w.t0 + w.q0, w.h, w.layer);
         ++n_q;
         for (int i = 0; i < w.n; ++i) {
           ok = mbar_wait(smem_u32(&aux->k_empty[rs]), ph ^ 1, abort_flag, kPolls);
@@ -322,28 +302,28 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
     if (lane == 0) {
-      const uint32_t idesc = make_idesc(kTile, n_pad, a.bf16 != 0);
+      const uint32_t idesc = make_idesc(kTile, NP, a.bf16 != 0);
       int rs = 0, n_q = 0;
-      uint32_t ph = 0, used = 0;                    // bit i of used: phase of accumulator i
+      uint32_t ph = 0, n_acc = 0;                   // accumulators handed out
       bool ok = true;
       for (int u = unit_from(blockIdx.x / n_cta); ok && u < a.n_units; u = unit_from(u + unit_step)) {
         const Unit w(s, u, rank, n_cta, by_seq);
         if (w.n == 0) continue;
         const int qs = n_q & 1;
         ok = mbar_wait(smem_u32(&aux->q_full[qs]), (n_q >> 1) & 1, abort_flag, kPolls);
-        for (int i = 0; ok && i < w.n; ++i) {
+        for (int i = 0; ok && i < w.n; ++i, ++n_acc) {
+          const int slot = n_acc & (kSlots - 1);
           ok = mbar_wait(smem_u32(&aux->k_full[rs]), ph, abort_flag, kPolls) &&
-               mbar_wait(smem_u32(&aux->acc_empty[i]), ((used >> i) & 1) ^ 1, abort_flag, kPolls);
+               mbar_wait(smem_u32(&aux->acc_empty[slot]), (n_acc / kSlots & 1) ^ 1, abort_flag, kPolls);
           if (!ok) break;
-          used ^= 1u << i;
           tc_fence_after();
 #pragma unroll
           for (int k = 0; k < D / 16; ++k) {
             if (k >= a.k_steps) break;
-            umma_bf16(tmem_base + i * n_pad, smem_desc_sw128(ring_addr + rs * kTileBytes + (k >> 2) * kBlockBytes + (k & 3) * 32),
-                      smem_desc_sw128(q_addr + qs * q_bytes + (k >> 2) * n_pad * 128 + (k & 3) * 32), idesc, k > 0);
+            umma_bf16(tmem_base + slot * NP, smem_desc_sw128(ring_addr + rs * kTileBytes + (k >> 2) * kBlockBytes + (k & 3) * 32),
+                      smem_desc_sw128(q_addr + qs * q_bytes + (k >> 2) * NP * 128 + (k & 3) * 32), idesc, k > 0);
           }
-          umma_commit(smem_u32(&aux->acc_full[i]));
+          umma_commit(smem_u32(&aux->acc_full[slot]));
           umma_commit(smem_u32(&aux->k_empty[rs]));
           if (++rs == ring) { rs = 0; ph ^= 1; }
         }
@@ -356,218 +336,300 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(smem_u32(&aux->drain), 0); ++i) {}
       }
     }
+  }
   } else {
-    // ------------------------------ epilogue groups ------------------------------
-    const int ew = warp - kCtrlWarps, gi = ew >> 2, quarter = warp & 3, et = tid - 32 * kCtrlWarps;
+    const int quarter = warp & 3;
     const int r = quarter * 32 + lane;              // TMEM lane: key of the tile
     const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
     const float scale = a.scale_log2;
-    const f32x2 scale2 = splat2(scale);
-    const int n_cb = n_pad / NC, cb = gi & (n_cb - 1);             // step 1: this group's column block ..
-    const int tpc = 16 / n_cb;                                     // warps that share a column
-    const int j0 = gi / n_cb, j_step = 4 / n_cb;                   // .. and its tiles
-    uint32_t used = 0;
-    int n_sync = 0, n_unit = 0;
+    constexpr int n_cb = NP / kNC, j_step = 4 / n_cb;   // column blocks of step 1, and groups that share one
+    uint32_t n_acc = 0;                             // accumulators taken by earlier units
+    int n_unit = 0;
     bool ok = true;
-    auto epi_sync = [&]() {
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&aux->epi_bar));
-      ok = mbar_wait(smem_u32(&aux->epi_bar), n_sync & 1, abort_flag, kPolls) && ok;
-      ++n_sync;
+    auto slot_of = [&](int j) { return (int)((n_acc + j) & (kSlots - 1)); };
+    auto wait_for = [&](unsigned long long& bar, uint32_t parity) {
+      ok = mbar_wait(smem_u32(&bar), parity, abort_flag, kPolls) && ok;
       ok = __all_sync(0xFFFFFFFFu, ok);
-    };
-    auto wait_acc = [&](int i) {
-      ok = mbar_wait(smem_u32(&aux->acc_full[i]), (used >> i) & 1, abort_flag, kPolls) && ok;
-      ok = __all_sync(0xFFFFFFFFu, ok);
-      tc_fence_after();
       return ok;
     };
 
-    for (int u = unit_from(blockIdx.x / n_cta); u < a.n_units; u = unit_from(u + unit_step)) {
-      const Unit w(s, u, rank, n_cta, by_seq);
-      if (w.L == 0) continue;
-      // first column (query) that key `key` may vote under
-      auto first_col = [&](int key) { return key >= w.L ? kMaxN : s.causal ? key - w.q0 : 0; };
-
-      // ---- step 1: 2^x in the logit's place, summed over this warp's keys per query ----
-      f32x2 sum2[NC / 2];
-#pragma unroll
-      for (int i = 0; i < NC / 2; ++i) sum2[i] = 0ull;
-      uint32_t kept = 0;                            // tiles of this warp that keep their logits
-      int warp_first = kMaxN;                       // first column with a key of this warp
-      for (int j = j0; j < w.n; j += j_step) {
-        if (!wait_acc(j)) break;
-        const uint32_t t_acc = t_lane + j * n_pad + cb * NC;
-        uint32_t v[NC];
-        tmem_ldn(t_acc, v);
-        const int key_first = first_col((w.tile0 + j) * kTile + r), c_first = key_first - cb * NC;
-        warp_first = min(warp_first, __reduce_min_sync(0xFFFFFFFFu, key_first));
-        tmem_waitn(v);
-        float hi = 0.f, lo = 0.f;
-#pragma unroll
-        for (int i = 0; i < NC; i += 2) {
-          hi = max3_nan(hi, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
-          lo = min3(lo, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
-        }
-        const bool keep = __any_sync(0xFFFFFFFFu, !(hi * scale < 100.f && lo * scale > -100.f));
-        if (lane == 0) aux->kept[j][cb][quarter] = keep;
-        if (keep) { kept |= 1u << j; continue; }
-        auto exps = [&](auto mixed) {
-#pragma unroll
-          for (int i = 0; i < NC / 2; ++i) {
-            const f32x2 x = mul2(pack2(v[2 * i], v[2 * i + 1]), scale2);
-            const f32x2 e = decltype(mixed)::value && (i & 3) == 3 ? exp2_poly2(x) : exp2_sfu2(x);
-            sum2[i] = add2(sum2[i], e);
-            float e0, e1;
-            unpack2(e, e0, e1);
-            v[2 * i] = __float_as_uint(e0);
-            v[2 * i + 1] = __float_as_uint(e1);
-          }
-        };
-        if (__any_sync(0xFFFFFFFFu, c_first > 0)) {
-#pragma unroll
-          for (int i = 0; i < NC; ++i) v[i] = i >= c_first ? v[i] : 0xFF800000u;
-          exps(std::false_type{});                  // no vote: exactly 2^-inf = 0
-        } else {
-          exps(std::true_type{});
-        }
-        tmem_stn(t_acc, v);
-      }
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      if (!ok) break;
-      float v[NC];
-#pragma unroll
-      for (int i = 0; i < NC / 2; ++i) unpack2(sum2[i], v[2 * i], v[2 * i + 1]);
-      const float sum = column_sums<NC>(v, lane);
-      const int my_col = NC == 32 ? lane : lane >> 1;
-      const bool has_keys = cb * NC + my_col >= warp_first && sum > 0.f;
-      if (NC == 32 || (lane & 1) == 0) {
-        aux->warp_part[ew][my_col][0] = has_keys ? 0.f : kNegInf;
-        aux->warp_part[ew][my_col][1] = has_keys ? sum : 0.f;
-      }
-      if (kept) {                                   // add the kept tiles, column by column with exact maxima
-        __syncwarp();
+    auto store = [&](const Unit& w, int j, float total) {
+      const int key = (w.tile0 + j) * kTile + r;
+      if (key < w.L) a.scores[((size_t)w.layer * s.Hq + w.h) * s.T + w.t0 + key] = a.normalize ? total / (float)w.nv : total;
+    };
+    // Step 2 of one tile, value by value: logits were kept in the unit, or a query's 2^-lse2 is not a normal number (or NaN).
+    auto by_value_tile = [&](const Unit& w, int j, int par, int copy) {
+      const int slot = slot_of(j), key = (w.tile0 + j) * kTile + r;
+      const int c_first = key >= w.L ? kMaxN : s.causal ? key - w.q0 : 0;
+      float total = 0.f;
 #pragma unroll 1
-        for (int c = 0; c < NC; ++c) {
-          float m = aux->warp_part[ew][c][0], t = 0.f;
-          const float m0 = m, t0 = aux->warp_part[ew][c][1];
-          for (int step = 0; step < 2; ++step) {
-            for (int j = j0; j < w.n; j += j_step) {
-              if (!((kept >> j) & 1u)) continue;
-              uint32_t x;
-              asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(x) : "r"(t_lane + j * n_pad + cb * NC + c) : "memory");
-              asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(x) :: "memory");
-              const bool in = cb * NC + c >= first_col((w.tile0 + j) * kTile + r);
-              const float xs = in ? __uint_as_float(x) * scale : kNegInf;
-              if (step == 0) m = fmaxf(m, xs);
-              else t += ex2(xs - (m == kNegInf ? 0.f : m));            // -inf adds 0, NaN stays
-            }
+      for (int b = 0; b < n_cb; ++b) {
+        uint32_t x[kNC];
+        tmem_ld16(t_lane + slot * NP + b * kNC, x);
+        tmem_wait16(x);
+        const bool keep = aux->kept[par][4 * (b + n_cb * (j & (j_step - 1))) + quarter] >> j & 1u;
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) {
-              if (step == 0) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
-              else t += __shfl_xor_sync(0xFFFFFFFFu, t, d);
-            }
-          }
-          if (m0 != kNegInf) t += t0 * ex2(m0 - m);
-          if (lane == 0) { aux->warp_part[ew][c][0] = m; aux->warp_part[ew][c][1] = t; }
-          __syncwarp();
+        for (int i = 0; i < kNC; ++i) {
+          const float x_i = __uint_as_float(x[i]), nl = aux->nlse[copy][b * kNC + i];
+          float e;
+          if (keep) e = ex2(fmaf(x_i, scale, nl));
+          else if (nl < -126.f) { const float root = ex2(0.5f * nl); e = x_i * root * root; }
+          else e = x_i * aux->factor[copy][b * kNC + i];
+          total += b * kNC + i >= c_first ? e : 0.f;
         }
       }
-      tc_fence_before();
-      epi_sync();
-      if (!ok) break;
+      return total;
+    };
 
-      // ---- the CTA's sums to every CTA of the cluster, then the row log-sum-exp ----
-      // Threads (column, i): i stands first for one of the 16 / n_cb warps that summed the column, then for a CTA.
-      const int par = n_unit & 1, col = et / tpc, sub = et & (tpc - 1);
-      if (col < n_pad) {                            // uniform over a warp
-        const int cw = 4 * (col / NC + n_cb * (sub >> 2)) + (sub & 3), ci = col & (NC - 1);
-        const float mw = aux->warp_part[cw][ci][0], tw = aux->warp_part[cw][ci][1];
-        float m = mw;
-        for (int d = 1; d < tpc; d <<= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
-        float t = tw == 0.f ? 0.f : tw * ex2(mw - m);
-        for (int d = 1; d < tpc; d <<= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, d);
-        const float l = t == 0.f ? kNegInf : m + log2f(t);
-        if (n_cta == 1) {                           // alone: this warp reads it back itself (and a launch without
-          if (sub == 0) aux->part[par][0][col] = l; // clusters has no st.async)
-          __syncwarp();
-        } else {
-          for (int p = sub; p < (int)n_cta; p += tpc)
-            peer_store_async(peer_addr(smem_u32(&aux->part[par][rank][col]), p), l, peer_addr(smem_u32(&aux->part_full[par]), p));
-        }
-      }
-      if (n_cta > 1) {
-        ok = cluster_wait(smem_u32(&aux->part_full[par]), (n_unit >> 1) & 1, abort_flag, kPolls) && ok;
-        ok = __all_sync(0xFFFFFFFFu, ok);
-      }
-      if (col < n_pad) {
-        float m = kNegInf, t = 0.f;
-        for (int p = sub; p < (int)n_cta; p += tpc) m = fmaxf(m, aux->part[par][p][col]);
-        for (int d = 1; d < tpc; d <<= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
-        for (int p = sub; p < (int)n_cta; p += tpc) t += ex2(aux->part[par][p][col] - m);      // -inf: adds nothing
-        for (int d = 1; d < tpc; d <<= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, d);
-        if (sub == 0) {
-          const float lse2 = m + log2f(t);
-          aux->nlse[col] = col < w.nv ? -lse2 : kNegInf;
-          if (col < w.nv && !(lse2 <= 126.f)) aux->by_value = n_unit + 1;
-          aux->factor[col] = col < w.nv ? ex2(lse2 < -126.f ? 126.f : -lse2) : 0.f;    // beyond 2^126 no column is below 2^100
-          if (rank == 0 && col < w.nv && a.lse_nat_out)
-            a.lse_nat_out[((size_t)w.layer * s.Hq + w.h) * s.T + w.t0 + w.q0 + col] = lse2 * 0.69314718055994530942f;
-        }
-      }
-      epi_sync();
-      if (!ok) break;
-      // armed again for the unit after the next: a peer sends that only when it has this CTA's sums of the next unit
-      if (et == 0 && n_cta > 1) mbar_expect_tx(smem_u32(&aux->part_full[par]), n_cta * n_pad * 4);
-
-      // ---- step 2: every key's sum over the queries ----
-      tc_fence_after();
-      const bool by_value = aux->by_value == n_unit + 1;
-      for (int j = gi; j < w.n; j += 4) {
-        const int key = (w.tile0 + j) * kTile + r;
-        const uint32_t t_acc = t_lane + j * n_pad;
-        f32x2 acc[2] = {0ull, 0ull};
-        for (int b = 0; b < n_cb; ++b) {
-          uint32_t x[NC];
-          tmem_ldn(t_acc + b * NC, x);
-          tmem_waitn(x);
-          if (!by_value && !aux->kept[j][b][quarter]) {
-            const float4* f4 = reinterpret_cast<const float4*>(aux->factor + b * NC);
+    if (warp < kCtrlWarps + kExpWarps) {
+      // ------------------------------ step 1: 2^x in the logit's place, summed over this warp's keys per query ------
+      const int ew = warp - kCtrlWarps, gi = ew >> 2;
+      const f32x2 scale2 = splat2(scale);
+      const int cb = gi & (n_cb - 1), j0 = gi / n_cb;   // this group's column block and first tile
+      for (int u = unit_from(blockIdx.x / n_cta); u < a.n_units; u = unit_from(u + unit_step)) {
+        const Unit w(s, u, rank, n_cta, by_seq);
+        if (w.L == 0) continue;
+        const int par = n_unit & 1;
+        const int key_end = s.causal ? min(w.L, w.q0 + cb * kNC + 1) : w.L;   // keys below vote under every column of the block
+        // first column (query) that key `key` may vote under
+        auto first_col = [&](int key) { return key >= w.L ? kMaxN : s.causal ? key - w.q0 : 0; };
+        f32x2 sum2[kNC / 2];
 #pragma unroll
-            for (int i = 0; i < NC / 4; ++i) {
-              const float4 f = f4[i];
-              acc[0] = fma2(pack2(x[4 * i], x[4 * i + 1]), pack2f(f.x, f.y), acc[0]);
-              acc[1] = fma2(pack2(x[4 * i + 2], x[4 * i + 3]), pack2f(f.z, f.w), acc[1]);
+        for (int i = 0; i < kNC / 2; ++i) sum2[i] = 0ull;
+        uint32_t kept = 0;                          // tiles of this warp that keep their logits
+        for (int j = j0; j < w.n; j += j_step) {
+          const int slot = slot_of(j);
+          if (!wait_for(aux->acc_full[slot], (n_acc + j) / kSlots & 1)) break;
+          tc_fence_after();
+          const uint32_t t_acc = t_lane + slot * NP + cb * kNC;
+          uint32_t v[kNC];
+          tmem_ld16(t_acc, v);
+          tmem_wait16(v);
+          float hi = 0.f;
+#pragma unroll
+          for (int i = 0; i < kNC; i += 2) hi = max3_abs(hi, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
+          if (__any_sync(0xFFFFFFFFu, !(hi * scale < 100.f))) { kept |= 1u << j; continue; }
+          auto exps = [&](auto mixed) {
+#pragma unroll
+            for (int i = 0; i < kNC / 2; ++i) {
+              const f32x2 x = mul2(pack2(v[2 * i], v[2 * i + 1]), scale2);
+              const f32x2 e = decltype(mixed)::value && (i & 3) == 3 ? exp2_poly2(x) : exp2_sfu2(x);
+              sum2[i] = add2(sum2[i], e);
+              float e0, e1;
+              unpack2(e, e0, e1);
+              v[2 * i] = __float_as_uint(e0);
+              v[2 * i + 1] = __float_as_uint(e1);
             }
+          };
+          const int tile_key = (w.tile0 + j) * kTile;
+          if (tile_key + kTile > key_end) {         // uniform over the group
+            const int c_first = first_col(tile_key + r) - cb * kNC;
+#pragma unroll
+            for (int i = 0; i < kNC; ++i) v[i] = i >= c_first ? v[i] : 0xFF800000u;
+            exps(std::false_type{});                // no vote: exactly 2^-inf = 0
           } else {
-            const int c_first = first_col(key) - b * NC;
-            const bool keep = aux->kept[j][b][quarter];
-            float t = 0.f;
+            exps(std::true_type{});
+          }
+          tmem_stn(t_acc, v);
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        if (!ok) break;
+        float v[kNC];
 #pragma unroll
-            for (int i = 0; i < NC; ++i) {
-              const float x_i = __uint_as_float(x[i]), nl = aux->nlse[b * NC + i];
-              float e;
-              if (keep) e = ex2(fmaf(x_i, scale, nl));
-              else if (nl < -126.f) { const float root = ex2(0.5f * nl); e = x_i * root * root; }
-              else e = x_i * aux->factor[b * NC + i];
-              t += i >= c_first ? e : 0.f;
+        for (int i = 0; i < kNC / 2; ++i) unpack2(sum2[i], v[2 * i], v[2 * i + 1]);
+        const float sum = column_sums<kNC>(v, lane);
+        if (!wait_for(aux->sums_empty[par], (n_unit >> 1 & 1) ^ 1)) break;
+        float (*part)[2] = aux->warp_part[par][ew];
+        if ((lane & 1) == 0) {
+          part[lane >> 1][0] = sum > 0.f ? 0.f : kNegInf;
+          part[lane >> 1][1] = sum;
+        }
+        if (lane == 0) aux->kept[par][ew] = kept;
+        if (kept) {                                 // add the kept tiles, column by column with exact maxima
+          if (lane == 0) aux->any_kept[par] = n_unit + 1;
+          __syncwarp();
+#pragma unroll 1
+          for (int c = 0; c < kNC; ++c) {
+            float m = part[c][0], t = 0.f;
+            const float m0 = m, t0 = part[c][1];
+            for (int step = 0; step < 2; ++step) {
+              for (int j = j0; j < w.n; j += j_step) {
+                if (!((kept >> j) & 1u)) continue;
+                uint32_t x;
+                asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];"
+                             : "=r"(x) : "r"(t_lane + slot_of(j) * NP + cb * kNC + c) : "memory");
+                asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(x) :: "memory");
+                const bool in = cb * kNC + c >= first_col((w.tile0 + j) * kTile + r);
+                const float xs = in ? __uint_as_float(x) * scale : kNegInf;
+                if (step == 0) m = fmaxf(m, xs);
+                else t += ex2(xs - (m == kNegInf ? 0.f : m));          // -inf adds 0, NaN stays
+              }
+#pragma unroll
+              for (int d = 16; d > 0; d >>= 1) {
+                if (step == 0) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
+                else t += __shfl_xor_sync(0xFFFFFFFFu, t, d);
+              }
             }
-            acc[0] = add2(acc[0], pack2f(t, 0.f));
+            if (m0 != kNegInf) t += t0 * ex2(m0 - m);
+            __syncwarp();
+            if (lane == 0) { part[c][0] = m; part[c][1] = t; }
           }
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&aux->acc_empty[j]));
-        if (key < w.L) {
-          const float total = sum4(acc);
-          a.scores[((size_t)w.layer * s.Hq + w.h) * s.T + w.t0 + key] = a.normalize ? total / (float)w.nv : total;
+        if (lane == 0) mbar_arrive(smem_u32(&aux->sums_full[par]));
+        if (unit_from(u + unit_step) >= a.n_units) {    // the last unit: nothing else to do than to share its step 2
+          if (!wait_for(aux->last_unit, 0)) break;
+          tc_fence_after();
+          const bool by_value = aux->last_by_value != 0;
+          for (int j = 1 + gi; j < w.n; j += 5) {
+            f32x2 acc[2] = {0ull, 0ull};
+            if (!by_value) {
+#pragma unroll
+              for (int b = 0; b < n_cb; ++b) {
+                uint32_t x[kNC];
+                tmem_ld16(t_lane + slot_of(j) * NP + b * kNC, x);
+                tmem_wait16(x);
+                const float4* f4 = reinterpret_cast<const float4*>(aux->factor[0] + b * kNC);
+#pragma unroll
+                for (int i = 0; i < kNC / 4; ++i) {
+                  const float4 f = f4[i];
+                  acc[0] = fma2(pack2(x[4 * i], x[4 * i + 1]), pack2f(f.x, f.y), acc[0]);
+                  acc[1] = fma2(pack2(x[4 * i + 2], x[4 * i + 3]), pack2f(f.z, f.w), acc[1]);
+                }
+              }
+            }
+            store(w, j, by_value ? by_value_tile(w, j, par, 0) : sum4(acc));
+          }
         }
+        n_acc += w.n;
+        ++n_unit;
       }
-      if (!ok) break;
-      if (w.n > 0) used ^= 0xFFFFFFFFu >> (32 - w.n);
-      ++n_unit;
+    } else {
+      // ------------------------------ exchange, then step 2: every key's sum over the queries -----------------------
+      set_max_regs<kSumRegs, true>();
+      const int st = tid - 32 * (kCtrlWarps + kExpWarps);
+      constexpr int tpc = 32 * kSumWarps / NP;      // threads of a column: i stands first for warps that summed it, then for CTAs
+      const int col = st / tpc, sub = st & (tpc - 1);
+      for (int u = unit_from(blockIdx.x / n_cta); u < a.n_units; u = unit_from(u + unit_step)) {
+        const Unit w(s, u, rank, n_cta, by_seq);
+        if (w.L == 0) continue;
+        const int par = n_unit & 1;
+        if (!wait_for(aux->sums_full[par], n_unit >> 1 & 1)) break;
+        // ---- the CTA's sums to every CTA of the cluster, then the row log-sum-exp ----
+        {
+          float mw[2], tw[2];                       // 16 / n_cb warps share a column: two for each of its threads
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int x = sub + i * tpc, ew = 4 * (col / kNC + n_cb * (x >> 2)) + (x & 3);
+            mw[i] = aux->warp_part[par][ew][col & (kNC - 1)][0];
+            tw[i] = aux->warp_part[par][ew][col & (kNC - 1)][1];
+          }
+          float m = fmaxf(mw[0], mw[1]);
+#pragma unroll
+          for (int d = 1; d < tpc; d <<= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
+          float t = (tw[0] == 0.f ? 0.f : tw[0] * ex2(mw[0] - m)) + (tw[1] == 0.f ? 0.f : tw[1] * ex2(mw[1] - m));
+#pragma unroll
+          for (int d = 1; d < tpc; d <<= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, d);
+          const float l = t == 0.f ? kNegInf : m + log2f(t);
+          if (n_cta == 1) {                         // alone (a launch without clusters has no st.async)
+            if (sub == 0) aux->part[par][0][col] = l;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&aux->sum_bar));
+            wait_for(aux->sum_bar, n_unit & 1);
+          } else {
+            for (int p = sub; p < (int)n_cta; p += tpc)
+              peer_store_async(peer_addr(smem_u32(&aux->part[par][rank][col]), p), l, peer_addr(smem_u32(&aux->part_full[par]), p));
+            ok = cluster_wait(smem_u32(&aux->part_full[par]), n_unit >> 1 & 1, abort_flag, kPolls) && ok;
+            ok = __all_sync(0xFFFFFFFFu, ok);
+          }
+          if (!ok) break;
+        }
+        // every warp by itself, which spares the group a barrier
+        bool by_value = aux->any_kept[par] == n_unit + 1;
+#pragma unroll
+        for (int c0 = 0; c0 < NP; c0 += 32) {
+          const int c = c0 + lane;
+          if (NP < 32 && c >= NP) break;
+          float l[kMaxCluster], m = kNegInf, t = 0.f;
+#pragma unroll
+          for (int p = 0; p < kMaxCluster; ++p) {
+            l[p] = p < (int)n_cta ? aux->part[par][p][c] : kNegInf;
+            m = fmaxf(m, l[p]);
+          }
+#pragma unroll
+          for (int p = 0; p < kMaxCluster; ++p) t += ex2(l[p] - m);                       // -inf: adds nothing
+          const float lse2 = m + log2f(t);
+          aux->nlse[st >> 5][c] = c < w.nv ? -lse2 : kNegInf;
+          aux->factor[st >> 5][c] = c < w.nv ? ex2(lse2 < -126.f ? 126.f : -lse2) : 0.f;  // beyond 2^126 no column is below 2^100
+          by_value = by_value || (c < w.nv && !(lse2 <= 126.f));
+          if (rank == 0 && st < 32 && c < w.nv && a.lse_nat_out)
+            a.lse_nat_out[((size_t)w.layer * s.Hq + w.h) * s.T + w.t0 + w.q0 + c] = lse2 * 0.69314718055994530942f;
+        }
+        by_value = __any_sync(0xFFFFFFFFu, by_value);
+        __syncwarp();
+        // armed again for the unit after the next: a peer sends that only when it has this CTA's sums of the next unit
+        if (st == 0 && n_cta > 1) mbar_expect_tx(smem_u32(&aux->part_full[par]), n_cta * NP * 4);
+
+        const bool last = unit_from(u + unit_step) >= a.n_units;      // then step 1's groups take four tiles of five
+        if (last) {
+          if (st == 0) aux->last_by_value = by_value;
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&aux->last_unit));
+        }
+        const int j_all = last ? 5 : 1;             // this group's tiles: every j_all-th
+        tc_fence_after();
+        auto finish = [&](int j, float total) {     // the tile's accumulator goes back, its sums go out
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&aux->acc_empty[slot_of(j)]));
+          store(w, j, total);
+        };
+        if (!by_value) {
+          // pieces of 16 columns, the load of the next one in flight while one is added
+          const float4* f4 = reinterpret_cast<const float4*>(aux->factor[st >> 5]);
+          uint32_t x[kNC], next[kNC];
+          if (w.n > 0) {
+            tmem_ld16(t_lane + slot_of(0) * NP, x);
+            tmem_wait16(x);
+          }
+          for (int j = 0; j < w.n; j += j_all) {
+            f32x2 acc[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+            for (int b = 0; b < n_cb; ++b) {
+              const bool more = b + 1 < n_cb || j + j_all < w.n;
+              if (more) tmem_ld16(t_lane + (b + 1 < n_cb ? slot_of(j) * NP + (b + 1) * kNC : slot_of(j + j_all) * NP), next);
+#pragma unroll
+              for (int i = 0; i < kNC / 4; ++i) {
+                const float4 f = f4[b * (kNC / 4) + i];
+                acc[2 * (i & 1)] = fma2(pack2(x[4 * i], x[4 * i + 1]), pack2f(f.x, f.y), acc[2 * (i & 1)]);
+                acc[2 * (i & 1) + 1] = fma2(pack2(x[4 * i + 2], x[4 * i + 3]), pack2f(f.z, f.w), acc[2 * (i & 1) + 1]);
+              }
+              if (b + 1 < n_cb) {
+                tmem_wait16(next);
+#pragma unroll
+                for (int i = 0; i < kNC; ++i) x[i] = next[i];
+              }
+            }
+            const f32x2 sums[2] = {add2(acc[0], acc[2]), add2(acc[1], acc[3])};
+            finish(j, sum4(sums));
+            if (j + j_all < w.n) {
+              tmem_wait16(next);
+#pragma unroll
+              for (int i = 0; i < kNC; ++i) x[i] = next[i];
+            }
+          }
+        } else {
+          for (int j = 0; j < w.n; j += j_all) finish(j, by_value_tile(w, j, par, st >> 5));
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&aux->sums_empty[par]));
+        n_acc += w.n;
+        ++n_unit;
+      }
+      if (st == 0) aux->n_unit = n_unit;
     }
-    if (et == 0) aux->n_unit = n_unit;
   }
 
   __syncwarp();
@@ -591,10 +653,10 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 constexpr int kMaxDevices = 64;
 
 // Clusters of n_cta blocks that run at the same time (write-once cache per device: the answer depends on nothing else).
-template <int D, int NC, uint32_t kPolls>
+template <int D, int NP, uint32_t kPolls>
 int resident_clusters(int log_cta, int smem) {
   static std::atomic<int> known[kMaxDevices][4];
-  auto kern = score_window_kernel<D, NC, kPolls>;
+  auto kern = score_window_kernel<D, NP, kPolls>;
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
   if ((n = known[dev][log_cta].load(std::memory_order_relaxed)) > 0) return n;
@@ -616,22 +678,22 @@ int resident_clusters(int log_cta, int smem) {
   return n;
 }
 
-template <int D, int NC, uint32_t kPolls>
+template <int D, int NP, uint32_t kPolls>
 int launch_window_polls(const CUtensorMap& mq, const CUtensorMap& mk, const WinArgs& a, int units, int log_cta, cudaStream_t stream) {
   constexpr int smem = kSmemTiles * kTile * D * 2 + kAuxBytes + 1024;
-  auto kern = score_window_kernel<D, NC, kPolls>;
-  const int clusters = resident_clusters<D, NC, kPolls>(log_cta, smem);
+  auto kern = score_window_kernel<D, NP, kPolls>;
+  const int clusters = resident_clusters<D, NP, kPolls>(log_cta, smem);
   if (clusters < 1) return KVCRUSH_ERR_UNSUPPORTED;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return KVCRUSH_ERR_CUDA;
   const int n = clusters < units ? clusters : units;
   return launch_chained(kern, dim3((unsigned)n << log_cta), dim3(kThreads), smem, stream, 1 << log_cta, mq, mk, a);
 }
 
-template <int D, int NC>
+template <int D, int NP>
 int launch_window(const CUtensorMap& mq, const CUtensorMap& mk, const WinArgs& a, int units, int log_cta, bool short_waits,
                   cudaStream_t stream) {
-  return short_waits ? launch_window_polls<D, NC, kShortWaitPolls>(mq, mk, a, units, log_cta, stream)
-                     : launch_window_polls<D, NC, kWaitPolls>(mq, mk, a, units, log_cta, stream);
+  return short_waits ? launch_window_polls<D, NP, kShortWaitPolls>(mq, mk, a, units, log_cta, stream)
+                     : launch_window_polls<D, NP, kWaitPolls>(mq, mk, a, units, log_cta, stream);
 }
 
 int pad_window(int window) {
@@ -696,16 +758,16 @@ int launch_score_window(const Shape& s, const int32_t* cu_host, const TensorView
   a.bf16 = Q.dtype == KVCRUSH_BF16; a.status = status; a.k_steps = (s.D + 15) / 16;
   a.withhold_first_item = diag.withhold_first_item;
   a.n_units = s.n_layers * s.n_seqs * s.Hq;
-  a.n_pad = pad_window(s.window);
+  const int n_pad = pad_window(s.window);
   a.ring = kMaxRing;                                // two query buffers of n_pad rows take the sixth tile at most
   CUtensorMap mq;
-  if (!make_map(&mq, Q, s.D, s.T, s.Hq, s.n_layers, a.n_pad)) return KVCRUSH_ERR_UNSUPPORTED;
+  if (!make_map(&mq, Q, s.D, s.T, s.Hq, s.n_layers, n_pad)) return KVCRUSH_ERR_UNSUPPORTED;
   const CUtensorMap& mk = *reinterpret_cast<const CUtensorMap*>(maps.k);
   const bool sw = diag.short_waits != 0;
-  auto launch = s.D > 64 ? (a.n_pad == 16 ? launch_window<128, 16> : launch_window<128, 32>)
-                         : (a.n_pad == 16 ? launch_window<64, 16> : launch_window<64, 32>);
+  auto launch = s.D > 64 ? (n_pad == 16 ? launch_window<128, 16> : n_pad == 32 ? launch_window<128, 32> : launch_window<128, 64>)
+                         : (n_pad == 16 ? launch_window<64, 16> : n_pad == 32 ? launch_window<64, 32> : launch_window<64, 64>);
   const int n_sms = sm_count();
-  const Plan plan = plan_launches(s, cu_host, n_sms, a.n_pad);
+  const Plan plan = plan_launches(s, cu_host, n_sms, n_pad);
   for (int need = plan.largest; need >= 0; --need) {
     const long long n = plan.split ? plan.units[need] : plan.together;
     if (n == 0) continue;

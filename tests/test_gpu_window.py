@@ -115,6 +115,35 @@ def test_one_pass_window_scores_match_oracle(B, layers, Hq, Hkv, D, seqlens, win
             assert (gl[l][:, a:a + j0] == 7.0).all()
 
 
+@pytest.mark.parametrize("layers,Hq,Hkv,D,seqlens,window,gain", [
+    (12, 32, 4, 64, (700,), 64, 1.0),                     # a CTA alone, two or three units of 6 tiles through 8 accumulators
+    (12, 16, 16, 64, (2000, 0, 90), 32, 1.0),             # clusters of 1 whose units differ, 16 accumulators
+    (9, 32, 32, 64, (1100,), 16, 60.0),                   # logits kept in every unit, 9 tiles through 32 accumulators
+    (2, 40, 8, 128, (7000,), 64, 30.0),                   # clusters of 8, 7 tiles or 6 a CTA
+])
+def test_units_that_follow_each_other_through_the_accumulators(B, layers, Hq, Hkv, D, seqlens, window, gain):
+    """More units than clusters: the exponentials of a unit run beside the sums of the one before, accumulators are taken round
+    and round, all warps share the last unit.  The CUDA-core kernels on the same inputs agree within the score tolerance."""
+    import torch
+    dev = _dev()
+    g = torch.Generator(device=dev).manual_seed(5)
+    T = sum(seqlens)
+    q = (torch.randn((layers, T, Hq, D), generator=g, device=dev) * gain).to(torch.bfloat16)
+    k = torch.randn((layers, T, Hkv, D), generator=g, device=dev).to(torch.bfloat16)
+    prob = B.Problem(layers, Hq, Hkv, D, seqlens, device=dev, query_window=window)
+    ws = torch.empty(B.kvcrush_workspace_size(prob, B.STAGE_SCORE), dtype=torch.uint8, device=dev)
+    status = torch.zeros(4, dtype=torch.int32, device=dev)
+    got = []
+    for impl in (B.SCORE_TENSOR, B.SCORE_TENSOR, B.SCORE_SIMT):
+        scores = torch.full((layers, Hq, T), -1.0, dtype=torch.float32, device=dev)
+        B.kvcrush_score(prob, q, k, scores, impl=impl, workspace=ws, status=status)
+        got.append(scores)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist()[0] == 0
+    assert torch.equal(got[0], got[1])
+    assert TL.within_score_tolerance(got[0].cpu().numpy(), got[2].cpu().numpy()).all()
+
+
 @pytest.mark.parametrize("layers,seqlens,window,want", [
     (4, (8192,), 64, (1, 1)), (4, (8192,) + (300,) * 15, 64, (2, 1)), (1, (4200, 4000), 64, (1, 1)),
     (4, (8193,), 64, (2, 0)), (4, (8192,), 65, (2, 0)), (4, (8192,), 0, (2, 0)),
