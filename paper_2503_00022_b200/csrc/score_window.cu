@@ -12,9 +12,9 @@
 // barriers, and unit after unit takes the next accumulators round and round, so that loads, products, exponentials and sums of
 // up to three units overlap.  (With all warps at one unit's steps in turn the chain exponentials - exchange - sums was the
 // time.)  For a launch's last unit all of them share step 2.
-// Measured, 32 layers x 32 heads x 8192 tokens of 128 channels (2.1 GB of keys): 16 queries 352 us, 32 queries 430 us, 64
-// queries 633 us (with one group of warps for all steps 375, 512, 732; the two sweeps 1150, 1155 and 1122); 1000 tokens, 64
-// queries 71.5 us (79.6; 172), 8 layers of 5003 + 3117 tokens 184 (238), 8 layers x 40 heads of 12000 tokens, 32 queries 221 (293).
+// Measured, 32 layers x 32 heads x 8192 tokens of 128 channels (2.1 GB of keys): 16 queries 351 us, 32 queries 434 us, 64
+// queries 606 us (with one group of warps for all steps 375, 512, 732; the two sweeps 1150, 1155 and 1122); 1000 tokens, 64
+// queries 69.4 us (79.6; 172), 8 layers of 5003 + 3117 tokens 178 (238), 8 layers x 40 heads of 12000 tokens, 32 queries 222 (293).
 // With 64 queries a cluster of 8 needs all its accumulators for one unit, and step 1 of the next one follows step 2 tile by
 // tile.  Taken back: clusters of 16 with two units in TMEM (1056 us, and 1277 with step 2 one unit behind: half the keys a CTA,
 // the same chain of latencies), windows of 128 queries (645 against 562 us at 4096 tokens, with one group of warps).
@@ -25,8 +25,9 @@
 // query whose lse2 is above 126, 2^-lse2 would be flushed to zero: the stored 2^x are multiplied by its square root twice.
 // A unit with such a query, or one whose sum is NaN, takes step 2 value by value.
 //
-// Roles: warp 0 issues TMA loads, warp 1 the tcgen05.mma; warps 4..19 are the four groups of step 1, warps 20..23 the group of
-// the exchange and step 2.  All waits
+// Roles: warp 0 issues TMA loads, warp 1 the tcgen05.mma; warps 4..7 are the group of the exchange and step 2, warps 8..23 the
+// four groups of step 1.  (Step 2, on which the accumulators wait, before step 1 in the order of the warps, and without copies
+// between its two buffers: 64 queries of 8192 tokens 632 -> 606 us, of 4096 292 -> 280; 32 queries of 8192 431 -> 434.)  All waits
 // are bounded as in score_tc.cu; all CTAs of a cluster meet once more before they leave, because peers write into their
 // shared memory, and one that gave up then waits for the stores that were on their way to it.
 #include <cuda.h>
@@ -50,7 +51,7 @@ constexpr int kSumWarps = 4;                 // one group: exchange and step 2
 constexpr int kThreads = 32 * (kCtrlWarps + kExpWarps + kSumWarps);
 constexpr int kNC = 16;                      // columns of a step-1 thread
 // Registers: 80 a thread at launch (the most 24 warps can have); the control warpgroup gives some to the group of step 2.  With
-// 48 and 112 the producer and the issuer spill: 732 us instead of 633 for 64 queries of 8192 tokens.
+// 48 and 112 the producer and the issuer spill: 714 us instead of 633 for 64 queries of 8192 tokens.
 constexpr int kLaunchRegs = 80, kCtrlRegs = 64, kSumRegs = 96;
 static_assert(32 * (kCtrlWarps * kCtrlRegs + kExpWarps * kLaunchRegs + kSumWarps * kSumRegs) <= kThreads * kLaunchRegs,
               "register split within the launch's total");
@@ -381,9 +382,9 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       return total;
     };
 
-    if (warp < kCtrlWarps + kExpWarps) {
+    if (warp >= kCtrlWarps + kSumWarps) {
       // ------------------------------ step 1: 2^x in the logit's place, summed over this warp's keys per query ------
-      const int ew = warp - kCtrlWarps, gi = ew >> 2;
+      const int ew = warp - kCtrlWarps - kSumWarps, gi = ew >> 2;
       const f32x2 scale2 = splat2(scale);
       const int cb = gi & (n_cb - 1), j0 = gi / n_cb;   // this group's column block and first tile
       for (int u = unit_from(blockIdx.x / n_cta); u < a.n_units; u = unit_from(u + unit_step)) {
@@ -508,7 +509,7 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     } else {
       // ------------------------------ exchange, then step 2: every key's sum over the queries -----------------------
       set_max_regs<kSumRegs, true>();
-      const int st = tid - 32 * (kCtrlWarps + kExpWarps);
+      const int st = tid - 32 * kCtrlWarps;
       constexpr int tpc = 32 * kSumWarps / NP;      // threads of a column: i stands first for warps that summed it, then for CTAs
       const int col = st / tpc, sub = st & (tpc - 1);
       for (int u = unit_from(blockIdx.x / n_cta); u < a.n_units; u = unit_from(u + unit_step)) {
@@ -589,35 +590,34 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         if (!by_value) {
           // pieces of 16 columns, the load of the next one in flight while one is added
           const float4* f4 = reinterpret_cast<const float4*>(aux->factor[st >> 5]);
-          uint32_t x[kNC], next[kNC];
+          uint32_t x[2][kNC];
           if (w.n > 0) {
-            tmem_ld16(t_lane + slot_of(0) * NP, x);
-            tmem_wait16(x);
+            tmem_ld16(t_lane + slot_of(0) * NP, x[0]);
+            tmem_wait16(x[0]);
           }
           for (int j = 0; j < w.n; j += j_all) {
+            const bool more = j + j_all < w.n;
             f32x2 acc[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
             for (int b = 0; b < n_cb; ++b) {
-              const bool more = b + 1 < n_cb || j + j_all < w.n;
-              if (more) tmem_ld16(t_lane + (b + 1 < n_cb ? slot_of(j) * NP + (b + 1) * kNC : slot_of(j + j_all) * NP), next);
+              if (b + 1 < n_cb) tmem_ld16(t_lane + slot_of(j) * NP + (b + 1) * kNC, x[(b + 1) & 1]);
+              else if (more) tmem_ld16(t_lane + slot_of(j + j_all) * NP, x[(b + 1) & 1]);
 #pragma unroll
               for (int i = 0; i < kNC / 4; ++i) {
                 const float4 f = f4[b * (kNC / 4) + i];
-                acc[2 * (i & 1)] = fma2(pack2(x[4 * i], x[4 * i + 1]), pack2f(f.x, f.y), acc[2 * (i & 1)]);
-                acc[2 * (i & 1) + 1] = fma2(pack2(x[4 * i + 2], x[4 * i + 3]), pack2f(f.z, f.w), acc[2 * (i & 1) + 1]);
+                acc[2 * (i & 1)] = fma2(pack2(x[b & 1][4 * i], x[b & 1][4 * i + 1]), pack2f(f.x, f.y), acc[2 * (i & 1)]);
+                acc[2 * (i & 1) + 1] = fma2(pack2(x[b & 1][4 * i + 2], x[b & 1][4 * i + 3]), pack2f(f.z, f.w), acc[2 * (i & 1) + 1]);
               }
-              if (b + 1 < n_cb) {
-                tmem_wait16(next);
-#pragma unroll
-                for (int i = 0; i < kNC; ++i) x[i] = next[i];
-              }
+              if (b + 1 < n_cb) tmem_wait16(x[(b + 1) & 1]);
             }
             const f32x2 sums[2] = {add2(acc[0], acc[2]), add2(acc[1], acc[3])};
             finish(j, sum4(sums));
-            if (j + j_all < w.n) {
-              tmem_wait16(next);
+            if (more) {
+              tmem_wait16(x[n_cb & 1]);
+              if constexpr (n_cb == 1) {
 #pragma unroll
-              for (int i = 0; i < kNC; ++i) x[i] = next[i];
+                for (int i = 0; i < kNC; ++i) x[0][i] = x[1][i];
+              }
             }
           }
         } else {
