@@ -202,3 +202,36 @@ def test_paged_pass_end_to_end_with_reduced_cache(B):
                 want = O.compact_pages(cache[a:b], idx, P)
                 assert got.tobytes() == want.tobytes(), (name, l, s)
     assert 12 in cp.kept(0, 1)                               # the short last page of sequence 1 is there
+
+
+@pytest.mark.parametrize("layers,Hq,seqlens,P", [
+    (32, 12, [736] * 16, 32), (32, 19, [733, 31, 1] * 9, 8),         # heads in one and in two or three groups a thread
+])
+def test_scores_of_many_kept_pages_are_gathered(B, layers, Hq, seqlens, P):
+    """As many rows as fill the chip by themselves: bit for bit what indexing gives, zeros past a sequence's end."""
+    import torch
+    dev = torch.device("cuda:0")
+    T, cu = sum(seqlens), np.concatenate([[0], np.cumsum(seqlens)])
+    pages = [(L + P - 1) // P for L in seqlens]
+    keep = np.asarray([[max(1, n - 1) for n in pages]], dtype=np.int32)
+    scores = torch.rand((layers, Hq, T), generator=torch.Generator(device=dev).manual_seed(3), device=dev)
+    prob = B.Problem(layers, Hq, Hq, 16, seqlens, device=dev)
+    cp = B.CompressionPass(prob, keep, np.zeros_like(keep), page_size=P)
+    cp.signature(scores)
+    cp.select(scores)
+    n_out = int(keep.sum()) * P
+    out = torch.full((layers, Hq, n_out), -1.0, device=dev)
+    B.kvcrush_compact_scores(prob, scores, cp.page_size, cp.cu_kept, cp.idx, cp.total_kept, out, status=cp.status)
+    torch.cuda.synchronize()
+    cp.check_status()
+    idx, host = cp.idx.cpu().numpy(), scores.cpu().numpy()
+    want = np.zeros((layers, Hq, n_out), dtype=np.float32)
+    for l in range(layers):
+        at = 0
+        for s, L in enumerate(seqlens):
+            seg = l * len(seqlens) + s
+            for page in idx[int(cp.cu_kept_host[seg]):int(cp.cu_kept_host[seg + 1])]:
+                n = min(P, L - int(page) * P)
+                want[l, :, at:at + n] = host[l, :, cu[s] + page * P:cu[s] + page * P + n]
+                at += P
+    np.testing.assert_array_equal(out.cpu().numpy(), want)
