@@ -373,7 +373,8 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         for (int i = 0; i < kNC; ++i) {
           const float x_i = __uint_as_float(x[i]), nl = aux->nlse[copy][b * kNC + i];
           float e;
-          if (keep) e = ex2(fmaf(x_i, scale, nl));
+          if (nl == kNegInf) e = 0.f;               // no voting query, whatever the logit is (inf and NaN included)
+          else if (keep) e = ex2(fmaf(x_i, scale, nl));
           else if (nl < -126.f) { const float root = ex2(0.5f * nl); e = x_i * root * root; }
           else e = x_i * aux->factor[copy][b * kNC + i];
           total += b * kNC + i >= c_first ? e : 0.f;

@@ -122,6 +122,31 @@ def test_a_query_without_finite_sum_touches_the_keys_it_sees_only(B, what):
     np.testing.assert_allclose(s[..., j + 1:], want[..., j + 1:], rtol=1e-4)
 
 
+@pytest.mark.parametrize("lens,window", [
+    ((300, 200), 40), ((300, 200), 20), ((300, 200), 5),     # the window ends inside its 64, 32 or 16 columns
+    ((50, 300, 37), 64), ((1100, 900), 40),                  # a sequence shorter than the window; a cluster of CTAs
+])
+@pytest.mark.parametrize("bad", [float("nan"), 3e38])
+def test_queries_of_the_next_sequence_have_no_influence_on_a_window(B, lens, window, bad):
+    """The columns behind a window's last query hold the next sequence's first queries; here those give NaN or infinite
+    logits.  Blocks that hold such logits recompute the others' weights instead of reading stored ones, a quarter of which
+    come from a polynomial of 7.5e-5: in the sums over keys and over queries."""
+    import torch
+    T = sum(lens)
+    q, k = _normal((1, T, 2, 64), 21, torch.bfloat16), _normal((1, T, 2, 64), 22, torch.bfloat16)
+    want, want_lse = _score(B, q, k, lens, B.SCORE_TENSOR, window=window)
+    ends = np.cumsum(lens)
+    for e in ends[:-1]:
+        q[:, e] = bad                                        # votes in its own sequence only where that is as short as the window
+        q[:, e + 2] = -bad
+    got, got_lse = _score(B, q, k, lens, B.SCORE_TENSOR, window=window)
+    first = ends[0]
+    np.testing.assert_allclose(got_lse[..., :first], want_lse[..., :first], rtol=0, atol=1e-4)
+    np.testing.assert_allclose(got[..., :first], want[..., :first], rtol=2e-4)
+    if len(lens) == 2:                                       # those queries do not vote: the second sequence is as before
+        np.testing.assert_allclose(got[..., first:], want[..., first:], rtol=2e-4)
+
+
 @pytest.mark.parametrize("window,shallow", [(16, 0), (40, 0), (16, 8), (40, 20)])
 def test_small_weights_of_a_window_keep_their_value_beside_a_huge_logit(B, window, shallow):
     """32 keys with logits of 110 (2^158) fill one block; the others' logits of 60 to 63 stay in the range that is stored as
