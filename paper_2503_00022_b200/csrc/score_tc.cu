@@ -26,7 +26,8 @@
 //     special-function unit busy.
 //
 // Roles: warp 0 fetches + decodes items and issues TMA loads; warps 1 and 2 (one lane each) issue the
-// tcgen05.mma of quarters 0-1 and 2-3; warp 3 idles; warps 4..19 are four epilogue groups (one per quarter) of 128 threads,
+// tcgen05.mma of quarters 0-1 and 2-3; warp 3 overwrites the queries of the column sweep's streamed tiles that do not
+// vote (see there) and idles in the row sweep; warps 4..19 are four epilogue groups (one per quarter) of 128 threads,
 // thread = TMEM lane = one query row (sweep 1) or one key column (sweep 2).  All synchronisation is by mbarriers
 // with bounded waits: a role that gives up sets the CTA's abort flag, every other wait then ends, the CTA
 // reports through the status word, drains its copies, frees TMEM and returns.
@@ -50,13 +51,14 @@ constexpr int kEpiWarps = 16;
 #endif
 constexpr int kIssueWarps = KVC_ISSUE_WARPS;   // tcgen05.mma issuing threads; each owns kQ / kIssueWarps quarters
 constexpr int kQPerIssuer = kQ / kIssueWarps;
-constexpr int kCtrlWarps = 4;                // one warpgroup: producer, issuers, one idle warp
+constexpr int kCtrlWarps = 4;                // one warpgroup: producer, issuers, the warp for non-voting queries
+constexpr int kEdgeWarp = 3;
 constexpr int kThreads = 32 * (kCtrlWarps + kEpiWarps);
 // Registers: 96 a thread at launch (the most 20 warps can have); the control warpgroup gives some back (what its roles
 // need in either sweep) and the epilogue takes 104.
 template <bool kColsum> constexpr int kCtrlRegs = kColsum ? 64 : 48;
 constexpr int kEpiRegs = 104;
-static_assert(kIssueWarps < kCtrlWarps && 32 * kCtrlWarps * kCtrlRegs<true> + 32 * kEpiWarps * kEpiRegs <= kThreads * 96,
+static_assert(kIssueWarps < kEdgeWarp && 32 * kCtrlWarps * kCtrlRegs<true> + 32 * kEpiWarps * kEpiRegs <= kThreads * 96,
               "register split within the launch's total");
 constexpr int kTiles = 6;                    // 128-row tiles in shared memory: tpb stationary ones, the others a ring of streamed tiles
 constexpr int kMaxRing = kTiles - 1;
@@ -101,6 +103,7 @@ struct PSmem {
 
 struct PAux {
   unsigned long long full[kMaxRing], empty[kMaxRing];
+  unsigned long long edge_full[kMaxRing];             // sweep 2: a tile with queries that do not vote has landed
   unsigned long long fixed_full, fixed_empty;
   unsigned long long acc_full[kQ], acc_empty[kQ];     // [quarter]
   unsigned long long item_full[kMaxItemSlots], item_empty[kMaxItemSlots];
@@ -146,6 +149,13 @@ struct Geo {
     }
     rep = !kSplit ? 1 : nq - v0 == 1 ? 4 : nq - v0 == 2 ? 2 : 1;
   }
+  // Sweep 2: the rows [lo, end) of streamed tile i hold queries that vote; the others belong to the next sequence or come
+  // before the window.  Only the first and the last tile of an item can have such rows.
+  struct Voters { int lo, end; __device__ __forceinline__ bool all() const { return lo == 0 && end == kTile; } };
+  __device__ __forceinline__ Voters voters(int i) const {
+    const int j0 = (first_stream + i) * kTile;
+    return {max(0, ws - j0), min(kTile, L - j0)};
+  }
   __device__ __forceinline__ int quarter(int slot) const { return rep > 1 ? v0 + slot / rep : slot; }
   // Streamed tiles of a slot: first, first + rep, .. below end; `diag`: the one that holds the causal diagonal (-1: none).
   struct Range { int first, end, diag; };
@@ -185,7 +195,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
   if (warp == 0) {
     if (lane == 0) {
-      for (int i = 0; i < kMaxRing; ++i) { mbar_init(smem_u32(&aux->full[i]), 1); mbar_init(smem_u32(&aux->empty[i]), kIssueWarps); }
+      for (int i = 0; i < kMaxRing; ++i) { mbar_init(smem_u32(&aux->full[i]), 1); mbar_init(smem_u32(&aux->empty[i]), kIssueWarps); mbar_init(smem_u32(&aux->edge_full[i]), 1); }
       mbar_init(smem_u32(&aux->fixed_full), 1);
       mbar_init(smem_u32(&aux->fixed_empty), kIssueWarps);
       for (int i = 0; i < kIssueWarps; ++i) mbar_init(smem_u32(&aux->drain[i]), 1);
@@ -196,7 +206,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       mbar_init(smem_u32(&aux->epi_bar), kEpiWarps);
       for (int i = 0; i < kSlots; ++i) {
         mbar_init(smem_u32(&aux->item_full[i]), 1);
-        mbar_init(smem_u32(&aux->item_empty[i]), kIssueWarps + kEpiWarps);
+        mbar_init(smem_u32(&aux->item_empty[i]), kIssueWarps + kEpiWarps + (kColsum ? 1 : 0));
       }
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -229,6 +239,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     int n_item = 0, n_stream = 0;     // n_stream: streamed tiles issued
     int rs = 0;                       // lane 0: ring slot of the next tile
     uint32_t ring_phase = 0;          //         and its phase
+    uint32_t edge_last = 0, edge_phase = 0;   // lane 0, bit per ring slot: its tile is announced by edge_full; phase of that
     int issued_item = 0;              // lane 0: items whose stationary load was issued
     bool alive = true;
     while (alive) {
@@ -285,10 +296,19 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           for (int i = 0; ok && i < g.n_iter; ++i) {
             ok = mbar_wait(smem_u32(&aux->empty[rs]), ring_phase ^ 1, abort_flag, kPolls);
             if (!ok) break;
-            mbar_expect_tx(smem_u32(&aux->full[rs]), SL::kTileBytes);
+            uint32_t landed = smem_u32(&aux->full[rs]);
+            if constexpr (kColsum) {               // edge_full first, the edge warp passes it on to `full`
+              edge_last &= ~(1u << rs);
+              if (!g.voters(i).all()) {
+                landed = smem_u32(&aux->edge_full[rs]);
+                edge_last |= 1u << rs;
+                edge_phase ^= 1u << rs;
+              }
+            }
+            mbar_expect_tx(landed, SL::kTileBytes);
 #pragma unroll
             for (int kb = 0; kb < D / 64; ++kb)
-              tma_load_4d(ring_addr + rs * SL::kTileBytes + kb * SL::kBlockBytes, map_stream, smem_u32(&aux->full[rs]),
+              tma_load_4d(ring_addr + rs * SL::kTileBytes + kb * SL::kBlockBytes, map_stream, landed,
                           kb * 64, g.t0 + (g.first_stream + i) * kTile, head_stream, g.layer);
             ++n_stream;
             if (++rs == ring) { rs = 0; ring_phase ^= 1; }
@@ -301,8 +321,13 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     }
     if (lane == 0 && *abort_flag) {
       // give the copies in flight a bounded time to land before the CTA's shared memory is released
-      for (int q = max(0, n_stream - ring); q < n_stream; ++q)
-        for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(smem_u32(&aux->full[q % ring]), (q / ring) & 1); ++i) {}
+      for (int q = max(0, n_stream - ring); q < n_stream; ++q) {
+        const int slot = q % ring;
+        const bool edge = edge_last >> slot & 1u;
+        const uint32_t bar = smem_u32(edge ? &aux->edge_full[slot] : &aux->full[slot]);
+        const uint32_t parity = edge ? (edge_phase >> slot & 1u) ^ 1u : (uint32_t)(q / ring) & 1u;
+        for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(bar, parity); ++i) {}
+      }
       if (issued_item > 0)
         for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(smem_u32(&aux->fixed_full), (issued_item - 1) & 1); ++i) {}
     }
@@ -370,6 +395,51 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         umma_commit(smem_u32(&aux->drain[iw]));
         for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(smem_u32(&aux->drain[iw]), 0); ++i) {}
       }
+    }
+  } else if (kColsum && warp == kEdgeWarp) {
+    // ------------------------------ queries that do not vote ------------------------------
+    // A weight of 2^(x - inf) is 0 only while x is finite or -inf: a NaN or an infinite logit of the next sequence's first
+    // queries, or of one before the window, would reach every key of the block.  So their rows take the values of the tile's
+    // last query that votes before the products are formed: it sees every key whose sum this tile adds to, so that what is
+    // not finite then is not finite in its own right.  (Masked in the epilogue instead, which has no instruction to spare:
+    // heads of 96, 5003 + 3117 tokens, both sweeps 2546 -> 2634 us, 64 sequences of 130 tokens 3895 -> 4380, and 1 % where there
+    // is nothing to mask.)
+    int n_item = 0, rs = 0;
+    uint32_t phase = 0;               // bit per ring slot: phase of edge_full
+    bool ok = true;
+    while (ok) {
+      const int slot = n_item % kSlots;
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&aux->item_full[slot]), (n_item / kSlots) & 1, abort_flag, kPolls));
+      if (!ok) break;
+      const volatile int* it = aux->item[slot];
+      if (it[0] < 0) break;
+      const Geo<kColsum, kSplit> g(s, it, a.tpb);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&aux->item_empty[slot]));
+      for (int i = 0; i < g.n_iter; i += max(1, g.n_iter - 1)) {         // the first and the last tile
+        const auto v = g.voters(i);
+        if (v.all()) continue;
+        const int q = (rs + i) % ring;
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&aux->edge_full[q]), phase >> q & 1u, abort_flag, kPolls));
+        if (!ok) break;
+        phase ^= 1u << q;
+        // a lane keeps one 16-byte piece of every 64 channels; the swizzle has piece c of row r at place c ^ (r & 7)
+        uint4* tile = reinterpret_cast<uint4*>(smem + (a.tpb + q) * SL::kTileBytes);
+        const int piece = lane & 7, from = v.end - 1, n_rows = v.lo + kTile - v.end;
+        uint4 val[D / 64];
+#pragma unroll
+        for (int kb = 0; kb < D / 64; ++kb) val[kb] = tile[kb * (SL::kBlockBytes / 16) + from * 8 + (piece ^ (from & 7))];
+        for (int e = lane >> 3; e < n_rows; e += 4) {
+          const int row = e < v.lo ? e : e - v.lo + v.end;
+#pragma unroll
+          for (int kb = 0; kb < D / 64; ++kb) tile[kb * (SL::kBlockBytes / 16) + row * 8 + (piece ^ (row & 7))] = val[kb];
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // read by tcgen05.mma
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&aux->full[q]));
+      }
+      rs = (rs + g.n_iter) % ring;
+      ++n_item;
     }
   }
   } else {

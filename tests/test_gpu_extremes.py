@@ -91,6 +91,30 @@ def test_queries_that_do_not_vote_have_no_influence_on_the_cuda_cores(B):
     np.testing.assert_array_equal(got_lse, want_lse)
 
 
+@pytest.mark.parametrize("lens,window,causal", [
+    ((200, 150), 0, True), ((200, 150), 0, False), ((1001, 130, 77), 0, True),     # the next sequence's queries in the last tile
+    ((1001, 600), 100, True), ((300, 400), 260, True),                             # and queries before the window in the first one
+])
+@pytest.mark.parametrize("layers,Hq", [(1, 2), (16, 32)])                          # blocks of one or two tiles, full blocks
+@pytest.mark.parametrize("bad", [float("nan"), 3e38])
+def test_queries_that_do_not_vote_have_no_influence_on_the_tensor_cores(B, lens, window, causal, layers, Hq, bad):
+    """Tiles of the column sweep hold the next sequence's first queries and queries before the window; here those give NaN or
+    infinite logits.  The row sweep may take another reference for the rows beside them, and the polynomial that serves a
+    quarter of its exponentials is off by 7.5e-5 to either side, by the fraction of its argument."""
+    import torch
+    T = sum(lens)
+    q, k = _normal((layers, T, Hq, 64), 23, torch.bfloat16), _normal((layers, T, Hq, 64), 24, torch.bfloat16)
+    want, want_lse = _score(B, q, k, lens, B.SCORE_TENSOR, window=window, causal=causal)
+    first = lens[0]
+    at = [first + i for i in range(0, 40, 3)]                # in both exponentials' columns
+    if window:
+        at += [first - window - 1 - i for i in range(0, 40, 3)]
+    q[:, at] = bad
+    got, got_lse = _score(B, q, k, lens, B.SCORE_TENSOR, window=window, causal=causal)
+    np.testing.assert_allclose(got_lse[..., :first], want_lse[..., :first], rtol=0, atol=1.5e-4)
+    np.testing.assert_allclose(got[..., :first], want[..., :first], rtol=2e-4)
+
+
 @pytest.mark.parametrize("L,window,p", [(100, 16, 50), (1000, 64, 0), (4000, 33, 3333), (300, 64, 290)])
 def test_nan_key_reaches_every_voting_row_of_a_window(B, L, window, p):
     import torch
