@@ -131,14 +131,15 @@ int kvcrush_score(const kvcrush_problem_t* problem, const kvcrush_tensor_t* Q, c
 // every CTA stop after fetching its first work item, before announcing it and before issuing any copy, so that the
 // other roles' first waits run out with nothing in flight: the kernels return normally with
 // status = {KVCRUSH_DEV_TIMEOUT, kernel id, block, 0}.  With an observation window of up to 64 queries the kernel is the
-// one-pass kernel; either flag then makes the call fail rather than fall back to the two sweeps.
+// one-pass kernel; either flag then makes the call fail rather than fall back to the two sweeps.  withhold_first_item == 2: only
+// the first CTA of the row sweep stops, the others and the column sweep go on.
 int kvcrush_diag_score(const kvcrush_problem_t* problem, const kvcrush_tensor_t* Q, const kvcrush_tensor_t* K,
                        const float* lse_in_dev, float* scores_dev, float* lse_out_dev, int normalize, int impl,
                        void* workspace, size_t workspace_bytes, int32_t* status_dev, void* stream,
                        int short_waits, int withhold_first_item) {
   ScoreDiag diag{};
   diag.short_waits = short_waits != 0;
-  diag.withhold_first_item = withhold_first_item != 0;
+  diag.withhold_first_item = withhold_first_item;
   return score_entry(problem, Q, K, lse_in_dev, scores_dev, lse_out_dev, normalize, impl, workspace, workspace_bytes,
                      status_dev, stream, diag);
 }

@@ -66,13 +66,15 @@ __device__ __forceinline__ int warp_segment_of_row(const int32_t* __restrict__ c
 // set up while the kernel before it still runs.  The price is a rule: every kernel launched with launch_chained calls
 // chain_wait before its first access to global memory (the kernel before it, and with that everything earlier in the
 // stream, has then completed and its writes are visible) and chain_trigger after that, never before: a kernel that is
-// set up early must not find work older than its direct predecessor still running.
+// set up early must not find work older than its direct predecessor still running.  For the same reason a grid must not end
+// before the one in front of it, which only a chain_wait prevents: not on the path of an error either.
 // Passes issued one after the other, fp32 layer of 512 tokens 57.4 -> 48.1 us, bf16 layer of 1001 tokens 65.6 -> 58.8 us.
 // A captured launch keeps full dependencies: the launches of a graph are close together as it is, and its programmatic
 // edges cost more than they give (57.5 against 52.9 us for the same layer replayed).
 // Inside a call that launches two kernels one after the other, the second may read what neither of them writes (the call's
 // inputs) before it waits, since the first has waited: everything before it has ended when the second is set up.  It reads
-// past the L1 cache then (__ldcg, TMA), which may hold lines from before.
+// past the L1 cache then (__ldcg, TMA), which may hold lines from before.  A block without work may leave such a kernel without
+// chain_wait where another block of the grid has work, and waits.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -143,7 +145,7 @@ int score_tensor_plan(const Shape& s, const TensorView& Q, const TensorView& K, 
 // Diagnostics of one launch (all zero in normal use).
 struct ScoreDiag {
   int short_waits;           // run the kernels instantiated with a short limit on every bounded barrier wait
-  int withhold_first_item;   // the producer warp of every CTA stops before announcing its first work item
+  int withhold_first_item;   // the producer warp stops before announcing its first work item: 1 in every CTA, 2 in the row sweep's first
 };
 // `counters`: two ints of caller scratch (work counters of the two persistent sweeps).
 size_t score_tensor_counter_bytes();

@@ -89,7 +89,8 @@ struct PersistArgs {
   int* counter;            // work counter, zero at launch; NULL: items are dealt out in advance (see the producer)
   int32_t* status;
   int withhold_first_item; // diagnostic: the producer warp fetches its first item and then stops before announcing
-                           // it or issuing any copy for it, so that every consumer's first wait runs out
+                           // it or issuing any copy for it, so that every consumer's first wait runs out (2: in the first
+                           // CTA of the row sweep only)
 };
 
 template <int D>
@@ -231,7 +232,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   const CUtensorMap* map_stream = kColsum ? &map_q : &map_k;
 
   if (dead) {
-    // nothing to do
+    if constexpr (kEarly) chain_wait();            // the row sweep's other CTAs may still run: no later kernel may start beside them
   } else if (warp < kCtrlWarps) {
   set_max_regs<kCtrlRegs<kColsum>, false>();
   if (warp == 0) {
@@ -260,7 +261,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (lane == 0) { aux->item[slot][0] = -1; mbar_arrive(smem_u32(&aux->item_full[slot])); }
         break;
       }
-      if (a.withhold_first_item) break;        // nothing is in flight: the consumers' bounded waits end the CTA
+      if (a.withhold_first_item == 1 || (a.withhold_first_item && !kColsum && blockIdx.x == 0)) break;   // nothing is in flight: the consumers' bounded waits end the CTA
       // (layer, head)-major order keeps the CTAs that run together on a few heads (their Q and K stay in L2); the
       // last pairs are taken weight-major instead, so that the launch does not end with a few CTAs on the heaviest
       // items of the last head while the others idle (a launch with few items is all tail)

@@ -431,7 +431,7 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_context_stays_usable(B
     the public header) the producer warp fetches its work item and then stops before announcing it and before issuing
     any copy, and the kernels run in their instantiation with a short poll limit.  Nothing is in flight, so the
     consumers' first waits expire, the block flags the status word, frees its tensor memory and the kernel returns
-    normally; the second sweep, enqueued by the same call, finds the status word set and leaves at once.  The outputs
+    normally; the second sweep, enqueued by the same call, waits for the first, finds the status word set and leaves.  The outputs
     stay untouched, and the same problem goes through the public entry point once the word is cleared."""
     import ctypes
     import torch
@@ -468,6 +468,42 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_context_stays_usable(B
     c, ol = TL.oracle_scores_layer(w, lis[0])
     assert TL.within_score_tolerance(scores.cpu().numpy()[0], c).all()
     np.testing.assert_allclose(lse.cpu().numpy()[0], ol, rtol=0, atol=2e-4)
+
+
+def test_no_kernel_starts_beside_a_row_sweep_whose_first_block_gave_up(B):
+    """The first block of the row sweep gives up (see above) while the others are in the middle of long items.  The column
+    sweep of the same call is set up meanwhile, block after block on SMs that become free, finds the status word set and
+    leaves; the kernel after the call must find every row log-sum-exp of the others written all the same."""
+    import ctypes
+    import torch
+    dev = _dev()
+    fn = B.lib().kvcrush_diag_score
+    vp, i32 = ctypes.c_void_p, ctypes.c_int
+    fn.restype = i32
+    fn.argtypes = [ctypes.POINTER(B.ProblemStruct), ctypes.POINTER(B.TensorStruct), ctypes.POINTER(B.TensorStruct),
+                   vp, vp, vp, i32, i32, vp, ctypes.c_size_t, vp, vp, i32, i32]
+    Hq, L = 1, 75776                                         # 296 blocks of 256 rows, two for each SM: about 0.7 ms, a limit 0.3
+    g = torch.Generator(device=dev).manual_seed(12)
+    q, k = (torch.randn((1, L, Hq, 64), generator=g, device=dev).to(torch.bfloat16) for _ in range(2))
+    prob = B.Problem(1, Hq, Hq, 64, (L,), device=dev)
+    qs, ks = B.tensor_struct(q), B.tensor_struct(k)
+    ws = torch.empty(B.kvcrush_workspace_size(prob, B.STAGE_SCORE), dtype=torch.uint8, device=dev)
+    scores = torch.full((1, Hq, L), -5.0, device=dev)
+    lse, seen = torch.full_like(scores, -7.0), torch.empty_like(scores)
+    status, status2 = (torch.zeros(4, dtype=torch.int32, device=dev) for _ in range(2))
+    stream = int(torch.cuda.current_stream().cuda_stream)
+    assert fn(prob.ref, ctypes.byref(qs), ctypes.byref(ks), None, scores.data_ptr(), lse.data_ptr(), 0, B.SCORE_TENSOR,
+              ws.data_ptr(), ws.numel(), status.data_ptr(), stream, 1, 2) == B.OK
+    B.kvcrush_pool_scores(prob, lse, 1, seen, status=status2, stream=stream)      # a copy by a kernel of the library
+    torch.cuda.synchronize()
+    assert status.tolist()[:3] == [B.DEV_TIMEOUT, 1, 0]
+    written = lse != -7.0
+    assert 0.5 < written.float().mean().item() < 1.0                     # the first block's items are missing
+    assert torch.equal(seen, lse)
+    status.zero_()
+    B.kvcrush_score(prob, q, k, scores, lse_out=seen, impl=B.SCORE_TENSOR, workspace=ws, status=status)
+    torch.cuda.synchronize()
+    assert status.tolist()[0] == 0 and torch.equal(seen[written], lse[written])
 
 
 @pytest.mark.parametrize("stage,small,large", [("signature", 9000, 32000), ("decode", 24000, 40000), ("simt", 128, 256)])
