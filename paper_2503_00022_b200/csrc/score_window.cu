@@ -12,9 +12,9 @@
 // barriers, and unit after unit takes the next accumulators round and round, so that loads, products, exponentials and sums of
 // up to three units overlap.  (With all warps at one unit's steps in turn the chain exponentials - exchange - sums was the
 // time.)  For a launch's last unit all of them share step 2.
-// Measured, 32 layers x 32 heads x 8192 tokens of 128 channels (2.1 GB of keys): 16 queries 351 us, 32 queries 434 us, 64
-// queries 606 us (with one group of warps for all steps 375, 512, 732; the two sweeps 1150, 1155 and 1122); 1000 tokens, 64
-// queries 69.4 us (79.6; 172), 8 layers of 5003 + 3117 tokens 178 (238), 8 layers x 40 heads of 12000 tokens, 32 queries 222 (293).
+// Measured, 32 layers x 32 heads x 8192 tokens of 128 channels (2.1 GB of keys): 16 queries 354 us, 32 queries 434 us, 64
+// queries 596 us (with one group of warps for all steps 375, 512, 732; the two sweeps 1150, 1155 and 1122); 1000 tokens, 64
+// queries 68.6 us (79.6; 172), 8 layers of 5003 + 3117 tokens 176 (238), 8 layers x 40 heads of 12000 tokens, 32 queries 223 (293).
 // With 64 queries a cluster of 8 needs all its accumulators for one unit, and step 1 of the next one follows step 2 tile by
 // tile.  Taken back: clusters of 16 with two units in TMEM (1056 us, and 1277 with step 2 one unit behind: half the keys a CTA,
 // the same chain of latencies), windows of 128 queries (645 against 562 us at 4096 tokens, with one group of warps).
@@ -23,7 +23,10 @@
 // logits leave [-100, 100] or hold a NaN keep them, count with their exact maxima in step 1 and take 2^(x - lse2) in step 2.
 // So a stored 2^x is finite; a query's sum may be NaN, and is then NaN in every key it votes for, and in no other.  For a
 // query whose lse2 is above 126, 2^-lse2 would be flushed to zero: the stored 2^x are multiplied by its square root twice.
-// A unit with such a query, or one whose sum is NaN, takes step 2 value by value.
+// A unit with such a query, with one whose sum is NaN, or with kept logits takes step 2 value by value, with one decision for
+// 16 values (a branch for each made one kept block cost a unit ten times its step 2).  8 layers x 32 heads x 8192 tokens, 64
+// queries, four keys with logits of 75: 1021 -> 473 us (with one group of warps for all steps 540), one in 128 keys 1277 -> 743
+// (760), all queries times 60: 981 -> 755 (768), logits of 95 959 -> 480 (625); the rest is step 1's sums with exact maxima.
 //
 // Roles: warp 0 issues TMA loads, warp 1 the tcgen05.mma; warps 4..7 are the group of the exchange and step 2, warps 8..23 the
 // four groups of step 1.  (Step 2, on which the accumulators wait, before step 1 in the order of the warps, and without copies
@@ -88,7 +91,8 @@ struct WAux {
   int any_kept[2];                                      // [unit parity] 1 + the last unit that kept logits
   int last_by_value;                                    // the last unit's step 2 goes value by value
   alignas(16) float nlse[kSumWarps][kMaxN];             // [warp of step 2] minus log2 sum of the window's queries, -inf: no vote
-  alignas(16) float factor[kSumWarps][kMaxN];           // 2^nlse
+  alignas(16) float factor[kSumWarps][kMaxN];           // 2^nlse, or its root if that is below the normal numbers ..
+  alignas(16) float factor2[kSumWarps][kMaxN];          // .. and then the root again, else 1
   uint32_t kept[2][kExpWarps];                          // [unit parity] tiles (bits) whose logits a warp of step 1 kept
   float warp_part[2][kExpWarps][kNC][2];                // [unit parity] (maximum, sum) of a warp's columns
   float part[2][kMaxCluster][kMaxN];                    // [unit parity][CTA of the cluster][query]: log2 sum, -inf: no key
@@ -362,25 +366,40 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     auto by_value_tile = [&](const Unit& w, int j, int par, int copy) {
       const int slot = slot_of(j), key = (w.tile0 + j) * kTile + r;
       const int c_first = key >= w.L ? kMaxN : s.causal ? key - w.q0 : 0;
-      float total = 0.f;
+      float total[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
       for (int b = 0; b < n_cb; ++b) {
         uint32_t x[kNC];
         tmem_ld16(t_lane + slot * NP + b * kNC, x);
         tmem_wait16(x);
         const bool keep = aux->kept[par][4 * (b + n_cb * (j & (j_step - 1))) + quarter] >> j & 1u;
+        const int first = c_first - b * kNC;
+        if (keep) {
 #pragma unroll
-        for (int i = 0; i < kNC; ++i) {
-          const float x_i = __uint_as_float(x[i]), nl = aux->nlse[copy][b * kNC + i];
-          float e;
-          if (nl == kNegInf) e = 0.f;               // no voting query, whatever the logit is (inf and NaN included)
-          else if (keep) e = ex2(fmaf(x_i, scale, nl));
-          else if (nl < -126.f) { const float root = ex2(0.5f * nl); e = x_i * root * root; }
-          else e = x_i * aux->factor[copy][b * kNC + i];
-          total += b * kNC + i >= c_first ? e : 0.f;
+          for (int i = 0; i < kNC; i += 4) {
+            const float4 n4 = *reinterpret_cast<const float4*>(&aux->nlse[copy][b * kNC + i]);
+            const float nl[4] = {n4.x, n4.y, n4.z, n4.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {           // -inf: no voting query, whatever the logit is (inf and NaN included)
+              const float e = ex2(fmaf(__uint_as_float(x[i + k]), scale, nl[k]));
+              total[k] += i + k >= first && nl[k] != kNegInf ? e : 0.f;
+            }
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < kNC; i += 4) {
+            const float4 f4 = *reinterpret_cast<const float4*>(&aux->factor[copy][b * kNC + i]);
+            const float4 g4 = *reinterpret_cast<const float4*>(&aux->factor2[copy][b * kNC + i]);
+            const float f[4] = {f4.x, f4.y, f4.z, f4.w}, g[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float e = __uint_as_float(x[i + k]) * f[k] * g[k];
+              total[k] += i + k >= first ? e : 0.f;
+            }
+          }
         }
       }
-      return total;
+      return (total[0] + total[1]) + (total[2] + total[3]);
     };
 
     if (warp >= kCtrlWarps + kSumWarps) {
@@ -563,7 +582,10 @@ score_window_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           for (int p = 0; p < kMaxCluster; ++p) t += ex2(l[p] - m);                       // -inf: adds nothing
           const float lse2 = m + log2f(t);
           aux->nlse[st >> 5][c] = c < w.nv ? -lse2 : kNegInf;
-          aux->factor[st >> 5][c] = c < w.nv ? ex2(lse2 < -126.f ? 126.f : -lse2) : 0.f;  // beyond 2^126 no column is below 2^100
+          const bool tiny = lse2 > 126.f;
+          const float f = ex2(lse2 < -126.f ? 126.f : tiny ? -0.5f * lse2 : -lse2);       // beyond 2^126 no column is below 2^100
+          aux->factor[st >> 5][c] = c < w.nv ? f : 0.f;
+          aux->factor2[st >> 5][c] = tiny ? f : 1.f;
           by_value = by_value || (c < w.nv && !(lse2 <= 126.f));
           if (rank == 0 && st < 32 && c < w.nv && a.lse_nat_out)
             a.lse_nat_out[((size_t)w.layer * s.Hq + w.h) * s.T + w.t0 + w.q0 + c] = lse2 * 0.69314718055994530942f;

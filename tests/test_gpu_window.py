@@ -144,6 +144,37 @@ def test_units_that_follow_each_other_through_the_accumulators(B, layers, Hq, Hk
     assert TL.within_score_tolerance(got[0].cpu().numpy(), got[2].cpu().numpy()).all()
 
 
+def test_a_few_logits_out_of_range_cost_what_their_sums_cost(B):
+    """Four keys of every head whose logits of 75 are kept beside the stored exponentials (a head's attention sinks): their sums
+    are formed one column after the other, the other keys go on as they are.  2.9 times the time of logits in range; value by
+    value in the whole unit with a branch for each it was 6.3 times."""
+    import torch
+    dev = _dev()
+    layers, H, L, D = 4, 32, 8192, 128
+    g = torch.Generator(device=dev).manual_seed(6)
+    q, k = (torch.randn((layers, L, H, D), generator=g, device=dev).to(torch.bfloat16) for _ in range(2))
+    q[..., 0], k[..., 0] = 8.0, 0.0
+    prob = B.Problem(layers, H, H, D, (L,), device=dev, query_window=64)
+    ws = torch.empty(B.kvcrush_workspace_size(prob, B.STAGE_SCORE), dtype=torch.uint8, device=dev)
+    status = torch.zeros(4, dtype=torch.int32, device=dev)
+    scores = torch.empty((layers, H, L), dtype=torch.float32, device=dev)
+    times = []
+    for sink in (0.0, 75.0):
+        k[:, :4, :, 0] = sink * D ** 0.5 / 8.0
+        best = []
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(5):
+                B.kvcrush_score(prob, q, k, scores, impl=B.SCORE_TENSOR, workspace=ws, status=status)
+            b.record()
+            torch.cuda.synchronize()
+            best.append(a.elapsed_time(b))
+        times.append(min(best))
+    assert status.tolist()[0] == 0
+    assert times[1] < 4.5 * times[0]
+
+
 @pytest.mark.parametrize("layers,seqlens,window,want", [
     (4, (8192,), 64, (1, 1)), (4, (8192,) + (300,) * 15, 64, (2, 1)), (1, (4200, 4000), 64, (1, 1)),
     (4, (8193,), 64, (2, 0)), (4, (8192,), 65, (2, 0)), (4, (8192,), 0, (2, 0)),
