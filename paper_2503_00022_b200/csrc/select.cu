@@ -994,14 +994,13 @@ int launch_select(const Shape& s, const float* scores, const double* importance,
     const int cap = cluster_tokens(s, cluster);
     const size_t cluster_dyn = cluster_bytes(s, cap);
     a.stage_words = cap;
-    auto launch = [&](auto kern, int threads) {
+    auto launch = [&](auto kern) {
       if (allow_dynamic_smem(kern, kClusterSmem) != KVCRUSH_OK) return (int)KVCRUSH_ERR_CUDA;
-      return launch_chained(kern, dim3((unsigned)(n_seg * cluster)), dim3(threads), cluster_dyn, stream, cluster, s, a);
+      return launch_chained(kern, dim3((unsigned)(n_seg * cluster)), dim3(1024), cluster_dyn, stream, cluster, s, a);
     };
     auto by_words = [&](auto w) {
       constexpr int W = decltype(w)::value;
-      return cluster == 4 ? launch(select_cluster_kernel<W, 4, 1024>, 1024)
-           : cap > 1024 ? launch(select_cluster_kernel<W, 8, 1024>, 1024) : launch(select_cluster_kernel<W, 8, 512>, 512);
+      return cluster == 4 ? launch(select_cluster_kernel<W, 4, 1024>) : launch(select_cluster_kernel<W, 8, 1024>);
     };
     return s.W == 1 ? by_words(std::integral_constant<int, 1>{}) : s.W == 2 ? by_words(std::integral_constant<int, 2>{})
          : s.W == 3 ? by_words(std::integral_constant<int, 3>{}) : by_words(std::integral_constant<int, 4>{});
