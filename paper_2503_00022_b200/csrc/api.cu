@@ -156,6 +156,14 @@ int kvcrush_diag_score_kernels(const kvcrush_problem_t* problem, int* one_pass) 
   return *one_pass ? score_window_launches(s, problem->cu_seqlens_host) : 2;
 }
 
+// Not part of the public ABI: blocks that kvcrush_select gives a segment of this problem on a device of n_sms multiprocessors
+// that runs clusters of up to largest_cluster of them (0: none), or a negative error code.
+int kvcrush_diag_select_blocks(const kvcrush_problem_t* problem, int n_sms, int largest_cluster) {
+  Shape s;
+  const int rc = make_shape(problem, &s);
+  return rc != KVCRUSH_OK ? rc : select_blocks_of_a_segment(s, n_sms, largest_cluster);
+}
+
 int kvcrush_score_decode(const kvcrush_problem_t* problem, const kvcrush_tensor_t* Q_new, const kvcrush_tensor_t* K,
                          float* scores_dev, int32_t* status_dev, void* stream) {
   Shape s;

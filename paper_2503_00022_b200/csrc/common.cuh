@@ -166,6 +166,8 @@ int launch_signature(const Shape& s, const float* scores, const int32_t* sig_kee
                      uint32_t* sigs, float* theta, double* importance, cudaStream_t stream);
 
 size_t select_workspace_bytes(const Shape& s);
+// Blocks that launch_select gives a segment on a device of n_sms multiprocessors that runs clusters of up to largest_cluster.
+int select_blocks_of_a_segment(const Shape& s, int n_sms, int largest_cluster);
 // importance: optional [n_layers][T] float64 I(t) from the signature stage; NULL: computed from the scores.
 int launch_select(const Shape& s, const float* scores, const double* importance, const uint32_t* sigs,
                   const int32_t* budget_imp,

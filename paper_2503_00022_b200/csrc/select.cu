@@ -22,6 +22,7 @@
 // Few segments of 8192 tokens or more take select_cluster_kernel, four or eight blocks a segment: 32 of 32768 tokens, with the
 // keys' conversion, 71 -> 34 us.
 // All decisions are integer or exact float64 comparisons, so the result is unique.
+#include <atomic>
 #include <type_traits>
 
 #include "select_common.cuh"
@@ -448,7 +449,9 @@ select_segment_kernel(Shape s, SelectArgs a) {
 // range of the tokens (keys, signatures, masks) and a range of the buckets; what they exchange goes through distributed
 // shared memory: extremes and histogram of the keys, the few candidates at the k-th largest, counts of the distances, the
 // tokens and signatures in (d, t) order - each sent straight to the block that owns its bucket, so that the bucket step
-// reads its signatures in order - and the representatives' bits.  Seven or eight cluster barriers in all.
+// reads its signatures in order - and the representatives' bits.  Eight cluster barriers as a rule (start, key range, histogram,
+// candidates, distances, order, representatives, counts), one more each for a mean anchor and for a tie that is cut, two more
+// for every further radix round (more than 256 candidates).
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_barrier() { cluster_arrive(); cluster_wait(); }
@@ -926,17 +929,61 @@ size_t cluster_bytes(const Shape& s, int cap) { return (size_t)cap / 4 + (size_t
 // work than barriers, and while its blocks find SMs (about 33 clusters of four, 15 of eight).  One block / cluster of 4 / of 8:
 // 1 segment of 4096 tokens 13.6 / 15.0 / 15.3 us, of 8192 19.2 / 17.9 / 17.9, of 16384 36.4 / 22.6 / 22.5, of 32768 65.8 / 32.0 /
 // 26.7; 8 of 20000 51.1 / 29.3 / 26.7; 32 of 4096 14.1 / 16.4 / 46, of 8192 19.5 / 19.2 / 53, of 16384 38.6 / 24.0 / 68, of 32768
-// 70.7 / 34.1 / 81.  Twice as many take two rounds of half the time: 36 of 8192 19.6 / 35.7, but 64 of 32768 74.8 / 67.1.
-int select_cluster_size(const Shape& s, long long n_seg, int n_sms) {
+// 70.7 / 34.1 / 81.  Twice as many take two rounds of half the time: 36 of 8192 19.6 / 35.7, but 64 of 32768 74.8 / 67.1, of 25000
+// 60.9 / 56.2.  The longest segment decides in ragged batches as well: one of 30000 and 60 of 1000 62.4 / 30.3, 64 between 1000 and
+// 32768 70.6 / 60.7, 64 between 8000 and 25000 57.0 / 52.6, one of 12300 and 15 of 500 33.1 / 20.4 (whole selection, 8 heads).
+// held(c): the device runs clusters of c such blocks at all.
+template <class Held>
+int select_cluster_size(const Shape& s, long long n_seg, int n_sms, Held&& held) {
   auto fits = [&](int c) { return cluster_bytes(s, cluster_tokens(s, c)) <= (size_t)kClusterSmem; };
   const bool few = n_seg * 8 <= n_sms * 4 / 5;
   if (s.max_seqlen < (few ? 8192 : 12288)) return 0;
-  if (s.max_seqlen > 16384 && few && fits(8)) return 8;
-  if (n_seg * 4 <= n_sms * (s.max_seqlen > 24576 ? 7 / 4.0 : 7 / 8.0) && fits(4)) return 4;
+  if (s.max_seqlen > 16384 && few && fits(8) && held(8)) return 8;
+  if (n_seg * 4 <= n_sms * (s.max_seqlen > 24576 ? 7 / 4.0 : 7 / 8.0) && fits(4) && held(4)) return 4;
   return 0;
 }
 
+template <int W, int C>
+constexpr auto cluster_kernel = select_cluster_kernel<W, C, 1024>;
+
+// Whether this device runs a cluster of C blocks with all the shared memory they may take (write-once cache per device: the
+// answer depends on nothing else).
+template <int W, int C>
+bool holds_cluster() {
+  constexpr int kMaxDevices = 64;
+  static std::atomic<int> known[kMaxDevices];                  // 1: yes, 2: no
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return false; }
+  if (const int k = known[dev].load(std::memory_order_relaxed)) return k == 1;
+  if (allow_dynamic_smem(cluster_kernel<W, C>, kClusterSmem) != KVCRUSH_OK) return false;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(C);
+  cfg.blockDim = dim3(1024);
+  cfg.dynamicSmemBytes = kClusterSmem;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&n, cluster_kernel<W, C>, &cfg) != cudaSuccess) { cudaGetLastError(); return false; }
+  known[dev].store(n > 0 ? 1 : 2, std::memory_order_relaxed);
+  return n > 0;
+}
+bool holds_cluster(int words, int cluster) {
+  switch (words) {
+    case 1: return cluster == 4 ? holds_cluster<1, 4>() : holds_cluster<1, 8>();
+    case 2: return cluster == 4 ? holds_cluster<2, 4>() : holds_cluster<2, 8>();
+    case 3: return cluster == 4 ? holds_cluster<3, 4>() : holds_cluster<3, 8>();
+    default: return cluster == 4 ? holds_cluster<4, 4>() : holds_cluster<4, 8>();
+  }
+}
+
 }  // namespace
+
+int select_blocks_of_a_segment(const Shape& s, int n_sms, int largest_cluster) {
+  const int n = select_cluster_size(s, (long long)s.n_layers * s.n_seqs, n_sms, [&](int c) { return c <= largest_cluster; });
+  return n > 0 ? n : 1;
+}
 
 size_t select_workspace_bytes(const Shape& s) {
   const size_t n = (size_t)s.n_layers * s.T;
@@ -975,7 +1022,7 @@ int launch_select(const Shape& s, const float* scores, const double* importance,
   }
   const long long n_seg = (long long)s.n_layers * s.n_seqs;
   const int n_sms = sm_count();
-  const int cluster = select_cluster_size(s, n_seg, n_sms);
+  const int cluster = select_cluster_size(s, n_seg, n_sms, [&](int c) { return holds_cluster(s.W, c); });
   // importance keys: computed here from the scores, or taken from the caller's I(t) - converted while the segment
   // kernel stages them, or by a small kernel when the segments are too long to be staged
   if (!importance) {
@@ -1000,7 +1047,7 @@ int launch_select(const Shape& s, const float* scores, const double* importance,
     };
     auto by_words = [&](auto w) {
       constexpr int W = decltype(w)::value;
-      return cluster == 4 ? launch(select_cluster_kernel<W, 4, 1024>) : launch(select_cluster_kernel<W, 8, 1024>);
+      return cluster == 4 ? launch(cluster_kernel<W, 4>) : launch(cluster_kernel<W, 8>);
     };
     return s.W == 1 ? by_words(std::integral_constant<int, 1>{}) : s.W == 2 ? by_words(std::integral_constant<int, 2>{})
          : s.W == 3 ? by_words(std::integral_constant<int, 3>{}) : by_words(std::integral_constant<int, 4>{});

@@ -126,6 +126,20 @@ def test_entry_points_reject_bad_arguments_before_launch(lib):
     assert lib.kvcrush_compact(r(p), r(t), None, 0x100, 0x100, -1, r(t), None, 0x100, None) == B.ERR_INVALID_ARG
 
 
+@pytest.mark.parametrize("n_layers,length,q_heads,blocks", [
+    (1, 8191, 8, 1), (1, 8192, 8, 4), (14, 8192, 8, 4), (15, 12287, 8, 1), (32, 12288, 8, 4), (33, 24576, 8, 1), (64, 24577, 8, 4),
+    (65, 24577, 8, 1), (1, 16385, 8, 8), (14, 90112, 8, 8), (1, 100000, 8, 1), (1, 40000, 128, 1), (1, 36000, 128, 8),
+])
+def test_selection_takes_clusters_only_where_the_device_runs_them(lib, n_layers, length, q_heads, blocks):
+    """As many blocks a segment as the rule says on a full chip; one where the device (a slice of it) has no room for a cluster,
+    four where it has none for eight."""
+    p = _problem(cu=[0, length], n_layers=n_layers, n_q_heads=q_heads)
+    ask = lambda largest: lib.kvcrush_diag_select_blocks(ctypes.byref(p), 148, largest)
+    assert ask(8) == blocks
+    assert ask(4) in ((1, 4) if blocks == 8 else (blocks,))
+    assert ask(0) == 1
+
+
 def _no_cuda_device():
     import torch
     return not torch.cuda.is_available()
