@@ -109,15 +109,32 @@ def test_signature_thresholds_for_rows_beyond_the_register_kernel(B):
 
 
 @pytest.mark.parametrize("Hq,L,b_imp,b_rep,ties", [
-    (4, 13088, 900, 1300, 0), (4, 13216, 900, 1300, 0),      # the last segment staged whole, the first that is not
-    (128, 7488, 300, 1500, 0), (128, 7680, 300, 1500, 0),    # the same with four signature words; buckets of 5
-    (4, 33000, 2000, 3300, 0),                               # signatures and 16-bit order in shared memory; buckets of 10
-    (4, 45000, 500, 9000, 0),                                # order in global memory; buckets of 5
-    (4, 66000, 100, 300, 0),                                 # nothing staged, buckets of 220
+    (4, 13088, 900, 1300, 0), (4, 13216, 900, 1300, 0),      # a cluster of four blocks
+    (128, 7488, 300, 1500, 0), (128, 7680, 300, 1500, 0),    # one block, the last segment staged whole and the first that is not
+    (4, 33000, 2000, 3300, 0),                               # a cluster of eight: buckets of 10
+    (4, 45000, 500, 9000, 0),                                # buckets of 5
+    (4, 66000, 100, 300, 0),                                 # buckets of 220
     (4, 20000, 700, 1700, 3), (4, 300, 40, 60, 2),           # more than 256 candidates after the first round, ties cut
 ])
 def test_select_at_the_edges_of_its_staging(B, Hq, L, b_imp, b_rep, ties):
     _select_case(B, Hq, Hq, [L], [(b_imp, b_rep)], 1, ties, 0, seed=330 + L % 97)
+
+
+@pytest.mark.parametrize("Hq,L,n_short,b_imp,b_rep,ties,share", [
+    (4, 13088, 32, 900, 1300, 0, True), (4, 13216, 32, 900, 1300, 0, True),     # the last segment staged whole, the first that is not
+    (40, 12288, 32, 700, 1000, 0, True), (128, 9000, 32, 300, 1500, 2, True),   # two and four signature words
+    (4, 20000, 32, 700, 1700, 3, False),                     # more than 256 candidates after the first round, ties cut
+    (4, 33000, 64, 2000, 3300, 0, True),                     # signatures and 16-bit order in shared memory; buckets of 10
+    (4, 45000, 64, 500, 9000, 0, False),                     # order in global memory; buckets of 5
+    (4, 66000, 64, 100, 300, 2, True),                       # nothing staged, buckets of 220
+])
+def test_select_of_one_long_segment_among_many(B, Hq, L, n_short, b_imp, b_rep, ties, share):
+    """One block a segment, because there are too many for clusters, and one of them too long to be staged whole."""
+    seqlens = [L] + [33 + 7 * (i % 5) for i in range(n_short)]
+    budgets = [(b_imp, b_rep)] + [(n // 6, n // 5) for n in seqlens[1:]]
+    prob = B.Problem(1, Hq, Hq, 16, seqlens, device=_dev())
+    assert B.lib().kvcrush_diag_select_blocks(prob.ref, 148, 8) == 1
+    _select_case(B, Hq, Hq, seqlens, budgets, 1, ties, 0, seed=450 + L % 89, share_importance=share)
 
 
 @pytest.mark.parametrize("Hq,seqlens,mode,ties", [
@@ -630,8 +647,9 @@ def test_cuda_core_scores_at_the_edges_of_their_tiles(B, dtype, D, Hq, Hkv, seql
     (2, 32, 8, 96, [1500, 1100], "bfloat16"),                                               # by the counter
 ])
 def test_a_pass_follows_inputs_written_just_before_it(B, layers, Hq, Hkv, D, seqlens, dtype):
-    """Kernels of a call that read its inputs before the kernel in front of them has ended: queries, keys and scores written by
-    the launch before the call give what they give after a synchronisation, bit for bit."""
+    """A whole pass right behind copies into its inputs gives what it gives after a synchronisation, bit for bit, also while the
+    caches hold the old inputs.  (Its column sweep and its packing read before they wait, each behind a kernel of the same pass.
+    The copies let nothing start early; launches that do come before the packing in the next test.)"""
     import torch
     dev, dt = _dev(), getattr(torch, dtype)
     T = sum(seqlens)
@@ -655,3 +673,53 @@ def test_a_pass_follows_inputs_written_just_before_it(B, layers, Hq, Hkv, D, seq
         cp.check_status()
         for a, b in zip(got, outs()):
             assert torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
+
+
+@pytest.mark.parametrize("writer", ["decode", "pool", "gather"])
+@pytest.mark.parametrize("layers,Hq,seqlens", [
+    (1, 32, [1001]), (2, 8, [130, 1, 257, 30, 7, 90]),       # tokens no multiple of 4; several sequences in 128 tokens
+    (3, 8, [8192]), (1, 4, [33000]), (20, 32, [700, 900]),   # every kernel of the thresholds
+])
+def test_signatures_follow_scores_written_by_the_launch_before(B, writer, layers, Hq, seqlens):
+    """Scores written by a kernel that lets the thresholds' kernel be set up early, which does the same for the packing: that reads
+    the scores before it waits.  Bit for bit what the same calls give with a synchronisation after each."""
+    import torch
+    dev = _dev()
+    g = torch.Generator(device=dev).manual_seed(13)
+    T, D = sum(seqlens), 64
+    prob = B.Problem(layers, Hq, Hq, D, seqlens, device=dev)
+    keep = np.asarray([[max(1, L // 8) for L in seqlens]], dtype=np.int32)
+    cp = B.CompressionPass(prob, keep, keep)
+    scores = torch.zeros((layers, Hq, T), device=dev)
+    status = torch.zeros(4, dtype=torch.int32, device=dev)
+    if writer == "decode":
+        q = torch.randn((layers, len(seqlens), Hq, D), generator=g, device=dev).to(torch.bfloat16)
+        k = torch.randn((layers, T, Hq, D), generator=g, device=dev).to(torch.bfloat16)
+        write = lambda x: (scores.copy_(x), B.kvcrush_score_decode(prob, q, k, scores, status=status))
+        source = lambda: torch.rand((layers, Hq, T), generator=g, device=dev)
+    elif writer == "pool":
+        write = lambda x: B.kvcrush_pool_scores(prob, x, 5, scores, status=status)
+        source = lambda: torch.rand((layers, Hq, T), generator=g, device=dev)
+    else:                                                    # every other token of a cache of twice the lengths
+        before = B.Problem(layers, Hq, Hq, D, [2 * L for L in seqlens], device=dev)
+        idx = torch.cat([2 * torch.arange(L, dtype=torch.int32, device=dev) for L in seqlens]).repeat(layers)
+        cu_kept = torch.tensor(np.concatenate([[0], np.cumsum(list(seqlens) * layers)]), dtype=torch.int32, device=dev)
+        write = lambda x: B.kvcrush_compact_scores(before, x, 0, cu_kept, idx, layers * T, scores, status=status)
+        source = lambda: torch.rand((layers, Hq, 2 * T), generator=g, device=dev)
+
+    def outputs(x, wait):
+        for call in (lambda: write(x), lambda: cp.signature(scores), lambda: cp.select(scores)):
+            call()
+            if wait:
+                torch.cuda.synchronize()
+        return [t.clone() for t in (cp.theta, cp.sigs, cp.importance, cp.idx)]
+
+    for _ in range(4):
+        old, new = source(), source()
+        outputs(old, False)                                  # the old scores are in every cache
+        got = outputs(new, False)
+        outputs(old, True)
+        for a, b in zip(got, outputs(new, True)):
+            assert torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
+    cp.check_status()
+    assert status.tolist()[0] == 0
