@@ -5,8 +5,9 @@
 // Two sweeps of one tiled kernel: row log-sum-exps, then column sums.  64 x 64 logit tiles from fp32 copies of both
 // operands in shared memory, 4 x 4 logits a thread, so that a 16-byte shared-memory read feeds eight FMAs (one warp
 // per row and one dot product per lane spent 170 us on 8 heads x 512 tokens of 64 channels, all of it waiting for loads,
-// and 2174 us on 4 layers of 1024 tokens; the two sweeps now take 26 and 180 us one after the other).  The column sweep
-// stages its tiles and forms its first logits while the row sweep ends: whole pass of 8 heads x 512 tokens 44.8 -> 39.8 us.
+// and 2174 us on 4 layers of 1024 tokens; the two sweeps now take 26 and 190 us).  Of a call of few blocks the column sweep
+// stages its tiles and forms its first logits while the row sweep ends: whole pass of 8 heads x 512 tokens 44.8 -> 39.8 us, with
+// operands that no cache holds half of that.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -23,19 +24,20 @@ constexpr int kRows = 64;                    // rows of both operands' tiles
 constexpr int kThreads = 256;
 constexpr int kMaxD = 256;
 
-template <typename T>
-__device__ __forceinline__ void load8(const T* p, float (&v)[8]);
+// kPastL1: a kernel that may read the operands before it waits for the one in front (see common.cuh).
+template <bool kPastL1, class V>
+__device__ __forceinline__ V load(const V* p) { if constexpr (kPastL1) return __ldcg(p); else return __ldg(p); }
 
-template <>
-__device__ __forceinline__ void load8<float>(const float* p, float (&v)[8]) {
-  const float4 a = __ldcg(reinterpret_cast<const float4*>(p));
-  const float4 b = __ldcg(reinterpret_cast<const float4*>(p) + 1);
+template <bool kPastL1>
+__device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
+  const float4 a = load<kPastL1>(reinterpret_cast<const float4*>(p));
+  const float4 b = load<kPastL1>(reinterpret_cast<const float4*>(p) + 1);
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 
-template <>
-__device__ __forceinline__ void load8<__nv_bfloat16>(const __nv_bfloat16* p, float (&v)[8]) {
-  const uint4 r = __ldcg(reinterpret_cast<const uint4*>(p));
+template <bool kPastL1>
+__device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8]) {
+  const uint4 r = load<kPastL1>(reinterpret_cast<const uint4*>(p));
   const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -44,9 +46,9 @@ __device__ __forceinline__ void load8<__nv_bfloat16>(const __nv_bfloat16* p, flo
   }
 }
 
-template <>
-__device__ __forceinline__ void load8<__half>(const __half* p, float (&v)[8]) {
-  const uint4 r = __ldcg(reinterpret_cast<const uint4*>(p));
+template <bool kPastL1>
+__device__ __forceinline__ void load8(const __half* p, float (&v)[8]) {
+  const uint4 r = load<kPastL1>(reinterpret_cast<const uint4*>(p));
   const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -61,13 +63,13 @@ __device__ __forceinline__ void load8<__half>(const __half* p, float (&v)[8]) {
 constexpr int kPad = 4;
 
 // Stages rows row0 .. row0+kStaged-1 of a sequence of L tokens (zeros past its end) as fp32.
-template <typename T, int kStaged>
+template <typename T, int kStaged, bool kPastL1>
 __device__ __forceinline__ void stage_tile(float* sh, const T* base, long long stride, int row0, int L, int D) {
   const int vec = D / 8;                                    // 8 channels at a time
   for (int e = threadIdx.x; e < kStaged * vec; e += kThreads) {
     const int r = e / vec, d = (e - r * vec) * 8;
     float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (row0 + r < L) load8<T>(base + (long long)(row0 + r) * stride + d, v);
+    if (row0 + r < L) load8<kPastL1>(base + (long long)(row0 + r) * stride + d, v);
     float4* out = reinterpret_cast<float4*>(sh + r * (D + kPad) + d);
     out[0] = make_float4(v[0], v[1], v[2], v[3]);
     out[1] = make_float4(v[4], v[5], v[6], v[7]);
@@ -81,11 +83,15 @@ __device__ __forceinline__ void stage_tile(float* sh, const T* base, long long s
 //   kColsum = true    stationary keys, streamed queries: sum of 2^(x - lse2(query)) of every key
 // 256 threads as 16 x 16; a thread holds N x N logits of a tile: 4 x 4, or 1 x 1 or 2 x 2 where no sequence is longer than
 // 16 or 32 tokens and the rest of the 64 x 64 would be zeros (300 sequences of 5 tokens, 2 layers x 8 heads: 237 -> 70 us).
+// kLate: the column sweep takes the row log-sum-exp behind a tile's products instead of beside its loads, so that it can start
+// while the row sweep ends (`early`).  Tiles of 64 x 64 do so in any case, which costs nothing there (100 sequences of 300 tokens
+// 1062 -> 1048 us, 8 heads x 8192 tokens 2394 -> 2382, 32 heads x 1024 of 128 channels 343.6 -> 347.4); smaller ones, a product
+// of a few steps between two barriers, only where they start early (300 sequences of 5 tokens 66.2 -> 64.2 us without).
 // Grid: (slot, layer, head) x the cluster's blocks.  In a batch of sequences of similar length slots are (tile, sequence)
 // pairs, the heaviest tiles of all sequences first (4 layers x 8 heads x 6 sequences of 600 tokens: 424 us, sequence by sequence
 // 453).  Otherwise (by_seq) sequence i owns the slots cu[i] / kRows + i up to the next one's first: at least as many as it has
 // tiles, and in all only T / kRows + n_seqs of them, found without a table.
-template <typename T, bool kColsum, int N>
+template <typename T, bool kColsum, int N, bool kLate>
 __global__ void __launch_bounds__(kThreads)
 simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const float* __restrict__ lse, float lse_mul,
                   float* __restrict__ lse2_out, float* __restrict__ lse_nat_out, float* __restrict__ scores, int normalize,
@@ -95,7 +101,7 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
   float* str_sh = fix_sh + 16 * N * (s.D + kPad);
   __shared__ float part[2][kRows];                          // this block's maximum (sweep 1) and sum of every row
   __shared__ float nlse_sh[kRows];                          // sweep 2: minus lse2 of the streamed queries that vote
-  if (!kColsum || !early) {                                 // early: sweep 1 of the same call is the launch before
+  if (!kLate || !early) {                                   // early: sweep 1 of the same call is the launch before
     chain_wait();
     chain_trigger();
   }
@@ -130,13 +136,17 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
   const size_t vec0 = ((size_t)layer * s.Hq + h) * s.T + t0;
   const float ninf = -INFINITY;
 
-  stage_tile<T, 16 * N>(fix_sh, kColsum ? kbase : qbase, kColsum ? K.st : Q.st, row0, L, s.D);
+  stage_tile<T, 16 * N, kLate || N == 4>(fix_sh, kColsum ? kbase : qbase, kColsum ? K.st : Q.st, row0, L, s.D);
   float m[N], sum[N];
 #pragma unroll
   for (int i = 0; i < N; ++i) { m[i] = ninf; sum[i] = 0.f; }
   for (int u = first + rank; u < last; u += n_blk) {
     __syncthreads();                                        // the previous tile is done with
-    stage_tile<T, 16 * N>(str_sh, kColsum ? qbase : kbase, kColsum ? Q.st : K.st, u * kRows, L, s.D);
+    stage_tile<T, 16 * N, kLate || N == 4>(str_sh, kColsum ? qbase : kbase, kColsum ? Q.st : K.st, u * kRows, L, s.D);
+    if (kColsum && !kLate && tid < kRows) {
+      const int j = u * kRows + tid;
+      nlse_sh[tid] = j < L && j >= ws ? -(__ldcg(lse + vec0 + j) * lse_mul) : ninf;
+    }
     __syncthreads();
     float acc[N][N];
 #pragma unroll
@@ -159,7 +169,7 @@ simt_sweep_kernel(Shape s, TensorView Q, TensorView K, float scale_log2, const f
         for (int j = 0; j < N; ++j)
           acc[i][j] = fmaf(a[i].w, b[j].w, fmaf(a[i].z, b[j].z, fmaf(a[i].y, b[j].y, fmaf(a[i].x, b[j].x, acc[i][j]))));
     }
-    if constexpr (kColsum) {                                // the row log-sum-exp is needed only now
+    if constexpr (kLate) {                                  // the row log-sum-exp is needed only now
       if (early && u == first + rank) {
         chain_wait();
         chain_trigger();
@@ -242,18 +252,19 @@ int launch_sweep(const Shape& s, const int32_t* cu_host, const TensorView& Q, co
   const long long slots = by_seq ? (long long)s.T / kRows + s.n_seqs : pairs, per_layer = slots * s.Hq * n_blk;
   if (per_layer > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
   const size_t dyn = (size_t)2 * 16 * N * (s.D + kPad) * sizeof(float);
-  auto kern = simt_sweep_kernel<T, kColsum, N>;
-  if (dyn > 40 * 1024 && allow_dynamic_smem(kern, 2 * 16 * N * (kMaxD + kPad) * (int)sizeof(float)) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
   // Blocks that are set up while the predecessor still runs are placed where there is room first, not evenly.  A grid of more
   // than a block an SM pays for that unless its blocks are short: 2 layers x 8 heads, 500 + 300 + 700 tokens, both sweeps 146
   // against 109 us; 8 heads x 512 tokens, two tiles a block, whole pass 46 against 47 us.
   const int streamed = s.window > 0 && s.window / kRows + 2 < max_tiles ? s.window / kRows + 2 : max_tiles;
   const bool overlap = per_layer * s.n_layers <= n_sms || (per_layer * s.n_layers <= 2 * n_sms && streamed <= 2 * n_blk);
+  early = early && overlap;                                 // (one launch then)
+  auto kern = kColsum && (N == 4 || early) ? simt_sweep_kernel<T, kColsum, N, kColsum> : simt_sweep_kernel<T, kColsum, N, kColsum && N == 4>;
+  if (dyn > 40 * 1024 && allow_dynamic_smem(kern, 2 * 16 * N * (kMaxD + kPad) * (int)sizeof(float)) != KVCRUSH_OK) return KVCRUSH_ERR_CUDA;
   const int layers = (int)(0x7FFFFFFFLL / per_layer < s.n_layers ? 0x7FFFFFFFLL / per_layer : s.n_layers);    // of one launch
   for (int layer0 = 0; layer0 < s.n_layers; layer0 += layers) {
     const int n = s.n_layers - layer0 < layers ? s.n_layers - layer0 : layers;
     const int rc = launch_kernel(overlap, kern, dim3((unsigned)(per_layer * n)), dim3(kThreads), dyn, stream, n_blk, s, Q, K, scale_log2,
-                                  lse, lse_mul, lse2_out, lse_nat_out, scores, normalize, layer0, n, by_seq, early && overlap && layer0 == 0);
+                                  lse, lse_mul, lse2_out, lse_nat_out, scores, normalize, layer0, n, by_seq, early);
     if (rc != KVCRUSH_OK) return rc;
   }
   return KVCRUSH_OK;
