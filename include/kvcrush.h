@@ -16,10 +16,10 @@
  *   - Pointers named *_dev (and every tensor / output pointer) are DEVICE pointers
  *     owned by the caller; pointers named *_host are host pointers read during the
  *     call only.  The library allocates and frees no memory and keeps no state
- *     between calls apart from three process-wide, write-once caches (the driver's
- *     tensor-map encoder entry point; how many thread block clusters of a size a
- *     device holds at once; for kvcrush_signature_static the device address of its
- *     array); scratch memory is the caller's `workspace` (device, 256-byte
+ *     between calls apart from four process-wide, write-once caches (the driver's
+ *     tensor-map encoder entry point; how many thread block clusters of the window
+ *     kernel a device holds at once, and whether it runs those of the selection; for
+ *     kvcrush_signature_static the device address of its array); scratch memory is the caller's `workspace` (device, 256-byte
  *     aligned, size from kvcrush_workspace_size).
  *   - Work is enqueued on `stream` (a cudaStream_t passed as void*, NULL = default
  *     stream) and the call returns without synchronising.  Inputs are never written.

@@ -64,7 +64,7 @@ __device__ __forceinline__ int warp_segment_of_row(const int32_t* __restrict__ c
 // ---- launches that overlap their predecessor's end --------------------------------------------------
 // A pass is a chain of short kernels, so every kernel is launched with programmatic stream serialization: its blocks are
 // set up while the kernel before it still runs.  The price is a rule: every kernel launched with launch_chained calls
-// chain_wait before its first access to global memory (the kernel before it, and with that everything earlier in the
+// chain_wait before its first access to global memory, but for what the last paragraph allows (the kernel before it, and with that everything earlier in the
 // stream, has then completed and its writes are visible) and chain_trigger after that, never before: a kernel that is
 // set up early must not find work older than its direct predecessor still running.  For the same reason a grid must not end
 // before the one in front of it, which only a chain_wait prevents: not on the path of an error either.

@@ -171,7 +171,7 @@ int launch_compact_scores(const Shape& s, const float* scores_in, int page_size,
   const long long blocks = (rows + 255) / 256;
   if (blocks > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
   // In pages a thread takes more groups of heads where the rows alone fill the chip: consecutive rows are read together, and
-  // finding a row costs as much as loading a group (16 x 736 tokens, 32 layers x 32 heads, pages of 32: 23.1 -> 19.3 us).  Single
+  // finding a row costs as much as loading a group (16 x 736 tokens, 32 layers x 32 heads, pages of 32: 24.6 -> 19.9 us).  Single
   // tokens of a long cache are bound by their sectors and gain nothing (32768 tokens, a fifth kept: 26.0 -> 26.4).
   unsigned head_blocks = (unsigned)((s.Hq + kScoreHeads - 1) / kScoreHeads);
   while (ps > 1 && head_blocks > 1 && blocks * head_blocks > 16LL * sm_count()) head_blocks = (head_blocks + 1) / 2;

@@ -6,8 +6,8 @@
 // operands in shared memory, 4 x 4 logits a thread, so that a 16-byte shared-memory read feeds eight FMAs (one warp
 // per row and one dot product per lane spent 170 us on 8 heads x 512 tokens of 64 channels, all of it waiting for loads,
 // and 2174 us on 4 layers of 1024 tokens; the two sweeps now take 26 and 190 us).  Of a call of few blocks the column sweep
-// stages its tiles and forms its first logits while the row sweep ends: whole pass of 8 heads x 512 tokens 44.8 -> 39.8 us, with
-// operands that no cache holds half of that.
+// stages its tiles and forms its first logits while the row sweep ends: whole pass of 8 heads x 512 tokens 45.2 -> 40.0 us, with
+// operands that no cache holds 47.7 -> 41.3.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>

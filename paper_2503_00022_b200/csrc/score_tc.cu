@@ -760,8 +760,9 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
   }
   if (!plan(false, counters + 1)) return KVCRUSH_ERR_CUDA;
   // The column sweep need not wait for the whole row sweep where that is the launch before it.  It saves 3 to 5 us a call (32
-  // heads over 8, 1001 tokens, whole pass 54.7 -> 49.8 us; 32 heads of 4096 tokens 199.2 -> 198.3), but this build of the kernel
-  // is 2 % slower in its loop (32 x 32 x 8192 tokens 20.0 -> 20.3 ms), so that only calls of one or two items a block take it.
+  // heads over 8, 1001 tokens, whole pass 54.8 -> 50.0 us, with operands that no cache holds 55.8 -> 51.2; 32 heads of 4096 tokens
+  // 192.3 -> 189.4), but this build of the kernel is 2 % slower in its loop (32 x 32 x 8192 tokens 20.0 -> 20.3 ms), so that only
+  // calls of one or two items a block take it.
   if (!lse_in && !a.counter) return a.tpb < kQ ? launch_persist<true, true, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<true, false, true>(mq, mk, a, sw, n_sms, stream);
   return a.tpb < kQ ? launch_persist<true, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<true, false>(mq, mk, a, sw, n_sms, stream);
 }
