@@ -124,6 +124,7 @@ struct Geo {
   int layer, h, hk, t0, L, first_stream, n_iter;
   int row0, tile0;             // first row of the stationary block inside the sequence, and row0 / kTile
   int ws;                      // first query row that votes (0 without an observation window)
+  bool last_seq;               // nothing is packed behind the sequence: TMA reads zeros past its end
   bool causal;
   int nq;                      // 128-row quarters of the block that hold rows of the sequence
   // The four accumulator slots normally hold four quarters.  When an item has only one or two (small blocks, the last
@@ -139,6 +140,7 @@ struct Geo {
     causal = s.causal != 0;
     nq = min(tpb, (L - row0 + kTile - 1) / kTile);
     ws = (s.window > 0 && L > s.window) ? L - s.window : 0;
+    last_seq = t0 + L == s.T;
     v0 = 0;
     if (kColsum) {                                                      // stationary keys, streamed query tiles
       first_stream = max(causal ? tile0 : 0, ws / kTile);
@@ -150,12 +152,12 @@ struct Geo {
     }
     rep = !kSplit ? 1 : nq - v0 == 1 ? 4 : nq - v0 == 2 ? 2 : 1;
   }
-  // Sweep 2: the rows [lo, end) of streamed tile i hold queries that vote; the others belong to the next sequence or come
-  // before the window.  Only the first and the last tile of an item can have such rows.
+  // Sweep 2: the rows [lo, end) of streamed tile i hold queries that vote (or zeros); the others belong to the next sequence or
+  // come before the window.  Only the first and the last tile of an item can have such rows.
   struct Voters { int lo, end; __device__ __forceinline__ bool all() const { return lo == 0 && end == kTile; } };
   __device__ __forceinline__ Voters voters(int i) const {
     const int j0 = (first_stream + i) * kTile;
-    return {max(0, ws - j0), min(kTile, L - j0)};
+    return {max(0, ws - j0), last_seq ? kTile : min(kTile, L - j0)};
   }
   __device__ __forceinline__ int quarter(int slot) const { return rep > 1 ? v0 + slot / rep : slot; }
   // Streamed tiles of a slot: first, first + rep, .. below end; `diag`: the one that holds the causal diagonal (-1: none).
@@ -178,8 +180,9 @@ struct Geo {
 // as a run-time bound it cost the full width 0.5 %).
 // kEarly: a column sweep right behind its row sweep.  Only its epilogue waits for the row log-sum-exp; items, loads and the
 // first products read the call's inputs and start as soon as an SM is free.
+// kEdge: a column sweep some of whose tiles hold queries that do not vote (see the edge warp).
 // kPolls: polls of every bounded barrier wait (a compile-time constant: the epilogue has no register to spare for it).
-template <int D, int kSteps, bool kColsum, bool kSplit, bool kEarly, uint32_t kPolls>
+template <int D, int kSteps, bool kColsum, bool kSplit, bool kEarly, bool kEdge, uint32_t kPolls>
 __global__ void __launch_bounds__(kThreads, 1)
 score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const PersistArgs a) {
@@ -207,7 +210,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       mbar_init(smem_u32(&aux->epi_bar), kEpiWarps);
       for (int i = 0; i < kSlots; ++i) {
         mbar_init(smem_u32(&aux->item_full[i]), 1);
-        mbar_init(smem_u32(&aux->item_empty[i]), kIssueWarps + kEpiWarps + (kColsum ? 1 : 0));
+        mbar_init(smem_u32(&aux->item_empty[i]), kIssueWarps + kEpiWarps + (kEdge ? 1 : 0));
       }
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -298,7 +301,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             ok = mbar_wait(smem_u32(&aux->empty[rs]), ring_phase ^ 1, abort_flag, kPolls);
             if (!ok) break;
             uint32_t landed = smem_u32(&aux->full[rs]);
-            if constexpr (kColsum) {               // edge_full first, the edge warp passes it on to `full`
+            if constexpr (kEdge) {                 // edge_full first, the edge warp passes it on to `full`
               edge_last &= ~(1u << rs);
               if (!g.voters(i).all()) {
                 landed = smem_u32(&aux->edge_full[rs]);
@@ -324,7 +327,7 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       // give the copies in flight a bounded time to land before the CTA's shared memory is released
       for (int q = max(0, n_stream - ring); q < n_stream; ++q) {
         const int slot = q % ring;
-        const bool edge = edge_last >> slot & 1u;
+        const bool edge = kEdge && (edge_last >> slot & 1u);
         const uint32_t bar = smem_u32(edge ? &aux->edge_full[slot] : &aux->full[slot]);
         const uint32_t parity = edge ? (edge_phase >> slot & 1u) ^ 1u : (uint32_t)(q / ring) & 1u;
         for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(bar, parity); ++i) {}
@@ -397,14 +400,17 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(smem_u32(&aux->drain[iw]), 0); ++i) {}
       }
     }
-  } else if (kColsum && warp == kEdgeWarp) {
+  } else if (kEdge && warp == kEdgeWarp) {
     // ------------------------------ queries that do not vote ------------------------------
     // A weight of 2^(x - inf) is 0 only while x is finite or -inf: a NaN or an infinite logit of the next sequence's first
     // queries, or of one before the window, would reach every key of the block.  So their rows take the values of the tile's
     // last query that votes before the products are formed: it sees every key whose sum this tile adds to, so that what is
     // not finite then is not finite in its own right.  (Masked in the epilogue instead, which has no instruction to spare:
-    // heads of 96, 5003 + 3117 tokens, both sweeps 2546 -> 2634 us, 64 sequences of 130 tokens 3895 -> 4380, and 1 % where there
-    // is nothing to mask.)
+    // heads of 96, 5003 + 3117 tokens, both sweeps 2546 -> 2634 us, 64 sequences of 130 tokens 3884 -> 4380, and 1 % where there
+    // is nothing to mask.)  The detour from the tile's landing over this warp to the issuers takes about half a us, which is
+    // seen where an item has one or two tiles: 22 layers x 32 heads, 383 tokens, window of 128, 71.9 -> 76.1 us, 27 layers of
+    // 269 + 110 tokens with a given log-sum-exp, whole pass, 82.3 -> 86.9; batches of 500 to 4000 tokens 0 to 1 %.  (The first
+    // tile loaded before the stationary ones hides it for windows, 74.1 us, and costs the others 1 %.)
     int n_item = 0, rs = 0;
     uint32_t phase = 0;               // bit per ring slot: phase of edge_full
     bool ok = true;
@@ -425,16 +431,19 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (!ok) break;
         phase ^= 1u << q;
         // a lane keeps one 16-byte piece of every 64 channels; the swizzle has piece c of row r at place c ^ (r & 7)
-        uint4* tile = reinterpret_cast<uint4*>(smem + (a.tpb + q) * SL::kTileBytes);
-        const int piece = lane & 7, from = v.end - 1, n_rows = v.lo + kTile - v.end;
+        const uint32_t tile = ring_addr + q * SL::kTileBytes;
+        const int piece = lane & 7, from = v.end - 1;
         uint4 val[D / 64];
 #pragma unroll
-        for (int kb = 0; kb < D / 64; ++kb) val[kb] = tile[kb * (SL::kBlockBytes / 16) + from * 8 + (piece ^ (from & 7))];
-        for (int e = lane >> 3; e < n_rows; e += 4) {
-          const int row = e < v.lo ? e : e - v.lo + v.end;
+        for (int kb = 0; kb < D / 64; ++kb) val[kb] = ld_shared16(tile + kb * SL::kBlockBytes + from * 128 + ((piece ^ (from & 7)) << 4));
+        auto fill = [&](int first, int end) {
+#pragma unroll 8
+          for (int row = first + (lane >> 3); row < end; row += 4)
 #pragma unroll
-          for (int kb = 0; kb < D / 64; ++kb) tile[kb * (SL::kBlockBytes / 16) + row * 8 + (piece ^ (row & 7))] = val[kb];
-        }
+            for (int kb = 0; kb < D / 64; ++kb) st_shared16(tile + kb * SL::kBlockBytes + row * 128 + ((piece ^ (row & 7)) << 4), val[kb]);
+        };
+        fill(0, v.lo);
+        fill(v.end, kTile);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // read by tcgen05.mma
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&aux->full[q]));
@@ -607,27 +616,29 @@ score_persist_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   if (tid == 0 && !dead && *abort_flag) report(a.status, KVCRUSH_DEV_TIMEOUT, kColsum ? KID_SCORE_COLSUM : KID_SCORE_LSE, blockIdx.x, 0);
 }
 
-template <int D, int kSteps, bool kColsum, bool kSplit, bool kEarly, uint32_t kPolls>
+template <int D, int kSteps, bool kColsum, bool kSplit, bool kEarly, bool kEdge, uint32_t kPolls>
 int launch_persist_polls(const CUtensorMap& mq, const CUtensorMap& mk, const PersistArgs& a, int n_sms, cudaStream_t stream) {
-  auto kern = score_persist_kernel<D, kSteps, kColsum, kSplit, kEarly, kPolls>;
+  auto kern = score_persist_kernel<D, kSteps, kColsum, kSplit, kEarly, kEdge, kPolls>;
   constexpr int smem = PSmem<D>::kTotal;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return KVCRUSH_ERR_CUDA;
   const int blocks = a.total_items < n_sms ? a.total_items : n_sms;
   return launch_chained(kern, dim3((unsigned)blocks), dim3(kThreads), smem, stream, 1, mq, mk, a);
 }
 
-template <bool kColsum, bool kSplit, bool kEarly, uint32_t kPolls>
+template <bool kColsum, bool kSplit, bool kEarly, bool kEdge, uint32_t kPolls>
 int launch_persist_width(const CUtensorMap& mq, const CUtensorMap& mk, const PersistArgs& a, int n_sms, cudaStream_t stream) {
-  if (a.s.D <= 64) return launch_persist_polls<64, 4, kColsum, kSplit, kEarly, kPolls>(mq, mk, a, n_sms, stream);
-  if (a.s.D <= 96) return launch_persist_polls<128, 6, kColsum, kSplit, kEarly, kPolls>(mq, mk, a, n_sms, stream);
-  return launch_persist_polls<128, 8, kColsum, kSplit, kEarly, kPolls>(mq, mk, a, n_sms, stream);
+  if (a.s.D <= 64) return launch_persist_polls<64, 4, kColsum, kSplit, kEarly, kEdge, kPolls>(mq, mk, a, n_sms, stream);
+  if (a.s.D <= 96) return launch_persist_polls<128, 6, kColsum, kSplit, kEarly, kEdge, kPolls>(mq, mk, a, n_sms, stream);
+  return launch_persist_polls<128, 8, kColsum, kSplit, kEarly, kEdge, kPolls>(mq, mk, a, n_sms, stream);
 }
 
+// edge: some tile of the column sweep holds queries that do not vote (the diagnostic build takes that kernel always)
 template <bool kColsum, bool kSplit, bool kEarly = false>
-int launch_persist(const CUtensorMap& mq, const CUtensorMap& mk, const PersistArgs& a, bool short_waits, int n_sms,
+int launch_persist(const CUtensorMap& mq, const CUtensorMap& mk, const PersistArgs& a, bool edge, bool short_waits, int n_sms,
                    cudaStream_t stream) {
-  return short_waits ? launch_persist_width<kColsum, kSplit, kEarly, kShortWaitPolls>(mq, mk, a, n_sms, stream)
-                     : launch_persist_width<kColsum, kSplit, kEarly, kWaitPolls>(mq, mk, a, n_sms, stream);
+  if (short_waits) return launch_persist_width<kColsum, kSplit, kEarly, kColsum, kShortWaitPolls>(mq, mk, a, n_sms, stream);
+  return kColsum && edge ? launch_persist_width<kColsum, kSplit, kEarly, kColsum, kWaitPolls>(mq, mk, a, n_sms, stream)
+                         : launch_persist_width<kColsum, kSplit, kEarly, false, kWaitPolls>(mq, mk, a, n_sms, stream);
 }
 
 // Tiles of an item's stationary block.  Four 128-row tiles take the most out of every streamed tile, but a launch with
@@ -728,6 +739,13 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
   const long long items_all = count(1, false);
   if (items_all == 0) return KVCRUSH_OK;
   if (items_all * a.n_lh > 0x7FFFFFFFLL) return KVCRUSH_ERR_UNSUPPORTED;
+  // Tiles of the column sweep with queries that do not vote: behind a sequence's end, unless nothing is packed there, and before
+  // a window.  Without any (single sequences, lengths that are multiples of 128) the sweep does without the edge warp.
+  bool edge = false;
+  for (int i = 0; i < s.n_seqs; ++i) {
+    const int len = cu_host[i + 1] - cu_host[i];
+    edge = edge || (len % kTile != 0 && cu_host[i + 1] < s.T) || (s.window > 0 && len > s.window && (len - s.window) % kTile != 0);
+  }
   a.tpb = s.window > 0 ? kQ : block_tiles(s, cu_host, n_sms, !lse_in);
   bool zeroed = false;
   auto plan = [&](bool row_sweep, int* counter) {
@@ -752,7 +770,7 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
     if (!plan(true, counters)) return KVCRUSH_ERR_CUDA;
     a.lse2_out = lse2_ws; a.lse_nat_out = lse_out;
     // Sequences of one tile have nothing to split (4 layers x 32 heads x 64 of 64 tokens, both sweeps: 368 -> 302 us).
-    rc = s.max_seqlen > kTile ? launch_persist<false, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<false, false>(mq, mk, a, sw, n_sms, stream);
+    rc = s.max_seqlen > kTile ? launch_persist<false, true>(mq, mk, a, edge, sw, n_sms, stream) : launch_persist<false, false>(mq, mk, a, edge, sw, n_sms, stream);
     if (rc != KVCRUSH_OK) return rc;
     a.lse = lse2_ws; a.lse_mul = 1.f;
   } else {
@@ -763,8 +781,8 @@ int launch_score_tensor(const Shape& s, const int32_t* cu_host, const TensorView
   // heads over 8, 1001 tokens, whole pass 54.8 -> 50.0 us, with operands that no cache holds 55.8 -> 51.2; 32 heads of 4096 tokens
   // 192.3 -> 189.4), but this build of the kernel is 2 % slower in its loop (32 x 32 x 8192 tokens 20.0 -> 20.3 ms), so that only
   // calls of one or two items a block take it.
-  if (!lse_in && !a.counter) return a.tpb < kQ ? launch_persist<true, true, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<true, false, true>(mq, mk, a, sw, n_sms, stream);
-  return a.tpb < kQ ? launch_persist<true, true>(mq, mk, a, sw, n_sms, stream) : launch_persist<true, false>(mq, mk, a, sw, n_sms, stream);
+  if (!lse_in && !a.counter) return a.tpb < kQ ? launch_persist<true, true, true>(mq, mk, a, edge, sw, n_sms, stream) : launch_persist<true, false, true>(mq, mk, a, edge, sw, n_sms, stream);
+  return a.tpb < kQ ? launch_persist<true, true>(mq, mk, a, edge, sw, n_sms, stream) : launch_persist<true, false>(mq, mk, a, edge, sw, n_sms, stream);
 }
 
 }  // namespace kvc

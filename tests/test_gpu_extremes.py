@@ -94,6 +94,7 @@ def test_queries_that_do_not_vote_have_no_influence_on_the_cuda_cores(B):
 @pytest.mark.parametrize("lens,window,causal", [
     ((200, 150), 0, True), ((200, 150), 0, False), ((1001, 130, 77), 0, True),     # the next sequence's queries in the last tile
     ((1001, 600), 100, True), ((300, 400), 260, True),                             # and queries before the window in the first one
+    ((256, 150), 0, True), ((384, 77), 128, True),                                 # full tiles: none of either kind
 ])
 @pytest.mark.parametrize("layers,Hq", [(1, 2), (16, 32)])                          # blocks of one or two tiles, full blocks
 @pytest.mark.parametrize("bad", [float("nan"), 3e38])
